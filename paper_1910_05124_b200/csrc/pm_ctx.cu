@@ -890,7 +890,7 @@ static pm_status stage_forward(pm_ctx* ctx, const TickArgs& ta, int p) {
   if (sd.pre != PRE_NONE && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(ta, dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
   for (int l = 0; l < sd.n_lin; ++l) {
     prof_begin(ctx, PM_PROF_GEMM_FWD);
-    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, dt, 0, l, ctx->ls) : umma_launch(ctx->umma, ta, 0, l, ctx->ls);
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, 0, l, ctx->ls) : umma_launch(ctx->umma, ta, 0, l, ctx->ls);
     if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
   }
   const bool att = feeds_attention(sd.post);
@@ -920,12 +920,12 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     cudaError_t e;
     if (!grouped) {
       prof_begin(ctx, PM_PROF_WGRAD);
-      e = dt == PM_F32 ? launch_simt_gemm(ta, dt, 2, l, ctx->ls) : umma_launch(ctx->umma, ta, 2, l, ctx->ls);
+      e = dt == PM_F32 ? launch_simt_gemm(ta, 2, l, ctx->ls) : umma_launch(ctx->umma, ta, 2, l, ctx->ls);
       if ((s = check(ctx, e, "wgrad GEMM")) != PM_OK) return s;
     }
     if (p == 0 && l == 0 && sd.pre != PRE_EMBED) continue;          // raw network inputs need no gradient
     prof_begin(ctx, PM_PROF_DGRAD);
-    e = dt == PM_F32 ? launch_simt_gemm(ta, dt, 1, l, ctx->ls) : umma_launch(ctx->umma, ta, (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
+    e = dt == PM_F32 ? launch_simt_gemm(ta, 1, l, ctx->ls) : umma_launch(ctx->umma, ta, (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;
@@ -966,7 +966,7 @@ static pm_status grouped_wgrad(pm_ctx* ctx, int table, bool fused = false) {
   TickArgs ta = mb_args(ctx, table, -1);
   ta.fuse_upd = fused ? 1 : 0;
   prof_begin(ctx, PM_PROF_WGRAD);
-  cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, dt, 2, 0, ctx->ls) : umma_launch(ctx->umma, ta, 2, 0, ctx->ls);
+  cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, 2, 0, ctx->ls) : umma_launch(ctx->umma, ta, 2, 0, ctx->ls);
   return check(ctx, e, "wgrad GEMM");
 }
 
@@ -1167,7 +1167,7 @@ pm_status pm_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
       if (ctx->L.any_pre && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(ctx->ta, dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
       for (int l = 0; l < ctx->L.max_lin; ++l) {
         prof_begin(ctx, PM_PROF_GEMM_FWD);
-        cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, dt, 0, l, ctx->ls)
+        cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, 0, l, ctx->ls)
                                      : umma_launch(ctx->umma, ctx->ta, 0, l, ctx->ls);
         if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
       }
@@ -1204,12 +1204,12 @@ pm_status pm_backward(pm_ctx* ctx) {
         cudaError_t e = cudaSuccess;
         if (!ctx->L.fuse) {                                           // fused update: formed in the update phase
           prof_begin(ctx, PM_PROF_WGRAD);
-          e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, dt, 2, l, ctx->ls)
+          e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, 2, l, ctx->ls)
                            : umma_launch(ctx->umma, ctx->ta, 2, l, ctx->ls);
           if ((s = check(ctx, e, "wgrad GEMM")) != PM_OK) return s;
         }
         prof_begin(ctx, PM_PROF_DGRAD);
-        e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, dt, 1, l, ctx->ls)
+        e = dt == PM_F32 ? launch_simt_gemm(ctx->ta, 1, l, ctx->ls)
                          : umma_launch(ctx->umma, ctx->ta, 1, l, ctx->ls);
         if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
       }

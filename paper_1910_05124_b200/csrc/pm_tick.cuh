@@ -193,6 +193,6 @@ size_t attention_smem_bytes(int S, int dk, int dtype);
 cudaError_t attention_set_smem_limits(int S, int dk, int dtype);
 
 // fp32 SIMT grouped GEMMs (PM_F32 path).  mode: 0 forward, 1 dgrad (corrected weights), 2 wgrad.
-cudaError_t launch_simt_gemm(const TickArgs& t, int dtype, int mode, int lvl, cudaStream_t stream);
+cudaError_t launch_simt_gemm(const TickArgs& t, int mode, int lvl, cudaStream_t stream);
 
 }  // namespace pm
