@@ -333,8 +333,8 @@ cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t st
 // them into its own part of shared memory with asynchronous copies (kF32Buf chunks ahead, so a reduction of up to
 // 16 * 8 * kF32Buf is in flight at once) and multiplies without any block-wide barrier; the eight partial tiles are added
 // in warp order at the end.  Warp tile (4 TM) x (8 TN), TM x TN outputs per lane.  Measured against a 64 x 64 tile with a
-serial k loop: a tick of the 4-stage 256-wide MLP at 32 rows 87.6 -> 44.4 us, an update of the 6-stage 200-wide MLP (two
-Linears per stage, two microbatches of 50 rows, microbatch-major order) 1483 -> 562 us.
+// serial k loop: a tick of the 4-stage 256-wide MLP at 32 rows 87.6 -> 44.4 us, an update of the 6-stage 200-wide MLP (two
+// Linears per stage, two microbatches of 50 rows, microbatch-major order) 1483 -> 562 us.
 constexpr int kF32KC = 16;
 
 template <int TM, int TN, int NBUF, int MODE> struct F32Cfg {
