@@ -11,9 +11,9 @@ enum { PRE_NONE = 0, PRE_EMBED = 1, PRE_LN = 2 };
 enum { POST_NONE = 0, POST_ATTENTION = 1, POST_SKIP_OUT = 2, POST_RESIDUAL = 3, POST_CROSS_ATTENTION = 4 };
 // LF_ACT_FROM_Y: a ReLU whose pre-activation is not stashed: the backward takes the mask from the stashed output
 // (y > 0 exactly where z > 0), which the next Linear keeps for its weight gradient anyway
-// LF_DZ_FUSED: a ReLU at the end of a stage whose output is the next stage's stashed input (bf16 tensor-core path): the
-// next stage's dgrad epilogue applies the mask (its own stashed input > 0) to the gradient it sends back, so this
-// Linear receives dz itself and its backward pass treats it as a Linear without activation
+// LF_DZ_FUSED: whoever produces the gradient of this Linear's output (the next Linear's dgrad epilogue, the MSE loss) has
+// multiplied it by act'(z) already, so this Linear receives dz itself and its backward pass treats it as a Linear without
+// activation
 enum { LF_WRITE_Z = 1, LF_WRITE_Y = 2, LF_OUT_F32 = 4, LF_ACT_FROM_Y = 8, LF_DZ_FUSED = 16 };
 
 // Static description of one Linear inside a stage (device copy).
@@ -25,6 +25,8 @@ struct LinDev {
   uint64_t h_ring;            // byte offset of this Linear's output stash h[depth][T*n_out] (unused for the last Linear)
   uint32_t b_soff;            // offset of the bias inside a slot of the stage's small-tensor version ring
   uint32_t _pad;
+  uint64_t dz_off;            // ws: dz = dy * act'(z) [T*n_out] (a Linear whose backward applies its activation itself)
+  uint64_t dy_off;            // ws: gradient w.r.t. this Linear's output [T*n_out] (a Linear inside a stage)
 };
 
 // Static description of one stage (device copy).  A stage is [pre-op] Linear{1..4} [post-op]:
@@ -75,8 +77,7 @@ struct StageDev {
   uint64_t ytmp;              // ws: Linear output awaiting the residual add [T*n_out]
   uint64_t gin;               // ws: incoming gradient w.r.t. the main output [3][T*d_out_main], slot = writer's tick % 3
   uint64_t dy;                // ws: gradient w.r.t. the Linear output when a post-op produces it [T*n_out] (attention)
-  uint64_t dz;                // ws: dz scratch [T*max_dim]
-  uint64_t dh;                // ws: dgrad output scratch [T*max_dim] (du of the first Linear, dh between Linears)
+  uint64_t dh;                // ws: gradient w.r.t. the pre-op's output u [T*d_in] (stages with a pre-op)
   LinDev lin[PM_MAX_LINEARS];
 };
 

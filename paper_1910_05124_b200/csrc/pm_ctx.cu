@@ -49,6 +49,7 @@ struct Layout {
   int32_t pe_seq = 0, pe_d = 0;
   int64_t loss_cap = 0;
   int32_t max_lin = 0, max_dim = 0, n_in_first = 0, n_out_last = 0;
+  int32_t act_levels = 0;               // bit l: some stage's Linear l applies its activation's derivative in its own backward
   // microbatch-major order
   bool mb = false;
   bool queue = false;                   // the forward pass reads its weights from per-stage version queues (mb, or entry period > 1)
@@ -313,6 +314,13 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
           stages[p + 1].ops[0].kind == PM_OP_LINEAR && !(sd.tau_fwd > 0 && sd.tau_bkwd == sd.tau_fwd) &&
           !(stages[p + 1].tau_fwd > 0 && stages[p + 1].tau_bkwd == stages[p + 1].tau_fwd))
         ld.flags |= LF_DZ_FUSED;
+      // fp32 networks: the gradient of a Linear's output is multiplied by act'(z) where it is formed (the next Linear's dgrad,
+      // the MSE loss), which saves a launch per Linear.  Not across a recompute segment's edge: there the z of the earlier
+      // stage is formed again only after the later stage's dgrad has run.
+      if (cfg->compute_dtype == PM_F32 && ld.act != PM_ACT_NONE &&
+          (!last || (p == P - 1 ? (!ce && s.post == POST_NONE) : (next_takes_y && stages[p + 1].n_ops > 0 && stages[p + 1].ops && stages[p + 1].ops[0].kind == PM_OP_LINEAR && (S == 0 || (p + 1) % S != 0)))))
+        ld.flags |= LF_DZ_FUSED;
+      if (bwd_act(ld) != PM_ACT_NONE) L.act_levels |= 1 << l;
     }
     if (p > 0 && (L.st[p - 1].lin[L.st[p - 1].n_lin - 1].flags & LF_DZ_FUSED)) s.mask_dx = 1;
     // ---- rings
@@ -470,16 +478,18 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   for (int p = 0; p < P; ++p) {
     StageDev& s = L.st[p];
     const uint64_t n_out_last = s.lin[s.n_lin - 1].n_out;
-    uint64_t mo = 0, mi = 0;
-    for (int l = 0; l < s.n_lin; ++l) { mo = std::max<uint64_t>(mo, s.lin[l].n_out); mi = std::max<uint64_t>(mi, s.lin[l].n_in); }
     s.gin = w; w = align_up(w + (uint64_t)s.gin_depth * T * s.d_out_main * esz, 256);
     if (s.post == POST_RESIDUAL) {
       s.skip_in = w; w = align_up(w + (uint64_t)s.skip_depth * T * n_out_last * esz, 256);
       s.ytmp = w; w = align_up(w + T * n_out_last * esz, 256);
     }
     if (s.post == POST_ATTENTION || s.post == POST_CROSS_ATTENTION) { s.dy = w; w = align_up(w + T * n_out_last * esz, 256); }
-    s.dz = w; w = align_up(w + T * mo * esz, 256);
-    s.dh = w; w = align_up(w + T * mi * esz, 256);
+    // every Linear keeps its dz until the grouped weight-gradient launches at the end of a backward pass
+    for (int l = 0; l < s.n_lin; ++l) {
+      if (bwd_act(s.lin[l]) != PM_ACT_NONE) { s.lin[l].dz_off = w; w = align_up(w + T * s.lin[l].n_out * esz, 256); }
+      if (l < s.n_lin - 1) { s.lin[l].dy_off = w; w = align_up(w + T * s.lin[l].n_out * esz, 256); }
+    }
+    if (s.pre != PRE_NONE) { s.dh = w; w = align_up(w + T * s.d_in * esz, 256); }
   }
   L.ws_bytes = w;
   return PM_OK;
@@ -690,7 +700,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   t.max_lin = L.max_lin; t.max_dim = L.max_dim;
   t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0;
   t.res_fused = cfg->compute_dtype == PM_BF16 ? 1 : 0;
-  t.ln_li0 = 0; t.defer_finish = 0; t.colsum_only = 0; t.ln_stage = 0; t.fin_deferred = 0;
+  t.ln_li0 = 0; t.defer_finish = 0; t.colsum_only = 0; t.dz_only = 0; t.ln_stage = 0;
   t.dgrad_split_below = 0;
   t.loss_scale = 1.0f / (float)(cfg->n_micro > 1 ? cfg->n_micro : 1);
   t.stash = (L.stash || L.materialize) ? 1 : 0;     // the backward pass reads its table entry's version slot
@@ -900,8 +910,15 @@ static pm_status stage_forward(pm_ctx* ctx, const TickArgs& ta, int p) {
   return PM_OK;
 }
 
-// The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradient, the bias column sums of
-// Linears without activation and the finishing passes are left to grouped launches over all stages (ta.defer_finish set).
+// does a launch of the activation backward at level l have anything to do (all stages, or stage p): the bias gradients of
+// bf16 networks are summed there, those of fp32 networks by the weight-gradient GEMM
+static bool need_actbwd(const pm_ctx* ctx, int l, int p, bool dz_only) {
+  if (!dz_only && ctx->cfg.compute_dtype == PM_BF16) return true;
+  return p >= 0 ? bwd_act(ctx->L.st[p].lin[l]) != PM_ACT_NONE : (ctx->L.act_levels >> l & 1) != 0;
+}
+
+// The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradients, the bias column sums and
+// the finishing passes are left to grouped launches over all stages (ta.dz_only and ta.defer_finish set).
 static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool grouped) {
   const int dt = ctx->cfg.compute_dtype;
   const int P = ctx->cfg.n_stages;
@@ -913,10 +930,9 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     else if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(ta, dt, ctx->ls), "attention backward"))) != PM_OK) return s;
   }
   for (int l = sd.n_lin - 1; l >= 0; --l) {
-    // dz = dy * act'(z) must exist before this stage's dgrad; a Linear without activation needs only the column sums
-    // of its incoming gradient (the bias gradient), which can wait for one grouped launch
-    if ((!grouped || bwd_act(sd.lin[l]) != PM_ACT_NONE) &&
-        (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ta, dt, l, ctx->ls), "activation backward", actbwd_launches(ta)))) != PM_OK) return s;
+    // dz = dy * act'(z) must exist before this stage's dgrad; the column sums (the bias gradient) can wait for one grouped launch
+    if (need_actbwd(ctx, l, p, grouped) &&
+        (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ta, dt, l, ctx->ls), "activation backward", actbwd_launches(ta, dt)))) != PM_OK) return s;
     cudaError_t e;
     if (!grouped) {
       prof_begin(ctx, PM_PROF_WGRAD);
@@ -960,23 +976,25 @@ static pm_status mb_forward(pm_ctx* ctx, const void* inputs, const void* targets
 }
 
 // The grouped launches that close a backward pass over the stages table `table` marks (all of them, or one recompute
-// segment): the weight gradients as one launch.
+// segment): the weight gradients as one launch per Linear of a stage.
 static pm_status grouped_wgrad(pm_ctx* ctx, int table, bool fused = false) {
   const int dt = ctx->cfg.compute_dtype;
   TickArgs ta = mb_args(ctx, table, -1);
   ta.fuse_upd = fused ? 1 : 0;
-  prof_begin(ctx, PM_PROF_WGRAD);
-  cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, 2, 0, ctx->ls) : umma_launch(ctx->umma, ta, 2, 0, ctx->ls);
-  return check(ctx, e, "wgrad GEMM");
+  for (int l = 0; l < ctx->L.max_lin; ++l) {
+    prof_begin(ctx, PM_PROF_WGRAD);
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, 2, l, ctx->ls) : umma_launch(ctx->umma, ta, 2, l, ctx->ls);
+    pm_status s = check(ctx, e, "wgrad GEMM");
+    if (s != PM_OK) return s;
+  }
+  return PM_OK;
 }
 
 static pm_status mb_backward(pm_ctx* ctx) {
   const int dt = ctx->cfg.compute_dtype;
   const int P = ctx->cfg.n_stages;
-  // With one Linear per stage nothing overwrites a stage's dz before the end of the backward chain, so the weight
-  // gradients of all stages run as ONE grouped launch (the tick schedule's launch, which fills the GPU); stages
-  // with several Linears reuse their dz scratch from level to level and form each weight gradient on the spot.
-  const bool grouped = ctx->L.max_lin == 1;
+  // Nothing overwrites a Linear's dz before the end of the backward chain, so the weight gradients of all stages run as
+  // ONE grouped launch per Linear of a stage (the tick schedule's launches, which fill the GPU).
   // PipeMare Recompute (Appendix A.2): segments from the last to the first; before a segment's backward its stages run
   // forward again from the input the forward pass left at the segment's first stage, with the recompute weights
   // (table 2P + 1), overwriting every stash the backward reads.  The last segment's backward follows its forward
@@ -993,20 +1011,21 @@ static pm_status mb_backward(pm_ctx* ctx) {
           if ((s = stage_forward(ctx, mb_args(ctx, 2 * P + 1, p), p)) != PM_OK) return s;
       for (int p = hi - 1; p >= lo; --p) {
         TickArgs ta = mb_args(ctx, 2 * P - 1 - p, p);
-        ta.defer_finish = grouped ? 1 : 0;      // the partial sums of bias and LayerNorm gradients are added up once, below
-        if ((s = stage_backward(ctx, ta, p, grouped)) != PM_OK) return s;
+        ta.dz_only = 1; ta.defer_finish = 1;    // bias and LayerNorm gradients are summed once, below
+        if ((s = stage_backward(ctx, ta, p, true)) != PM_OK) return s;
       }
-      if (grouped && S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
+      if (S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
     }
-    if (grouped) {
-      TickArgs ta = mb_args(ctx, 2 * P, -1);
-      ta.colsum_only = 1; ta.defer_finish = 1;                  // bias gradients of the Linears without activation, all stages at once
-      if ((s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ta, dt, 0, ctx->ls), "bias gradient column sums", actbwd_launches(ta)))) != PM_OK) return s;
-      ta.colsum_only = 0; ta.defer_finish = 0;
-      if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
-      const int n_fin = deferred_finish_launches(ta);
-      if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_deferred_finish(ta, dt, ctx->ls), "bias / LayerNorm gradient sums", n_fin))) != PM_OK) return s;
+    TickArgs ta = mb_args(ctx, 2 * P, -1);
+    if (dt == PM_BF16) {
+      ta.colsum_only = 1;                                       // bias gradients of all stages
+      for (int l = 0; l < ctx->L.max_lin; ++l)
+        if ((s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ta, dt, l, ctx->ls), "bias gradient column sums", actbwd_launches(ta, dt)))) != PM_OK) return s;
+      ta.colsum_only = 0;
     }
+    if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
+    const int n_fin = ln_finish_launches(ta);
+    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
     return PM_OK;
   });
   if (s != PM_OK) return s;
@@ -1200,7 +1219,8 @@ pm_status pm_backward(pm_ctx* ctx) {
       if (ctx->attn) { if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, attn_tc_launch(ctx->attn, ctx->ta, false, ctx->ls), "attention backward"))) != PM_OK) return s; }
       else if (ctx->L.att_blocks > 0 && (s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(ctx->ta, dt, ctx->ls), "attention backward"))) != PM_OK) return s;
       for (int l = ctx->L.max_lin - 1; l >= 0; --l) {
-        if ((s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ctx->ta, dt, l, ctx->ls), "activation backward", actbwd_launches(ctx->ta)))) != PM_OK) return s;
+        if (need_actbwd(ctx, l, -1, false) &&
+            (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(ctx->ta, dt, l, ctx->ls), "activation backward", actbwd_launches(ctx->ta, dt)))) != PM_OK) return s;
         cudaError_t e = cudaSuccess;
         if (!ctx->L.fuse) {                                           // fused update: formed in the update phase
           prof_begin(ctx, PM_PROF_WGRAD);

@@ -70,13 +70,18 @@ __global__ void __launch_bounds__(kLossThreads) mse_loss_kernel(TickArgs t) {
   float* partial = ws_ptr<float>(t, t.lossred_off);
   unsigned int* counter = reinterpret_cast<unsigned int*>(partial + kLossBlocks);
   const float scale = (float)(2.0 / (double)n * (double)t.loss_scale);
+  const LinDev& Ll = sl.lin[sl.n_lin - 1];
+  const int act = (Ll.flags & LF_DZ_FUSED) ? Ll.act : PM_ACT_NONE;       // the last Linear receives dz itself
+  const AT* z = act != PM_ACT_NONE ? ring_ptr<AT>(t, Ll.z_ring, d.b_slot, n) : nullptr;
   const uint64_t chunk = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
   float part = 0.f;
   for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     float r = __fsub_rn(to_f<AT>(y[i]), tg[i]);
     part = __fadd_rn(part, __fmul_rn(r, r));
-    dy[i] = from_f<AT>(__fmul_rn(scale, r));
+    AT g = from_f<AT>(__fmul_rn(scale, r));
+    if (act != PM_ACT_NONE) g = from_f<AT>(__fmul_rn(to_f<AT>(g), act_grad(to_f<AT>(z[i]), act)));
+    dy[i] = g;
   }
   __shared__ float red[kLossThreads];
   __shared__ bool last;
@@ -112,23 +117,15 @@ cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
 
 // ---- activation backward + bias gradient ---------------------------------------------------------
 // dz = dy * act'(z) (stored in the activation type); db[c] = sum over rows of the stored dz.
-// A block owns 64 columns; warp w takes rows w, w+8, ... (ascending), two columns per thread; the eight
-// per-warp partial sums of a column are added in warp order.
-constexpr int kActCols = 64, kActWarps = 8;
-
-template <typename AT> struct Pair;
-template <> struct Pair<float> {
-  static __device__ __forceinline__ float2 ld(const float* p) { return *reinterpret_cast<const float2*>(p); }
-  static __device__ __forceinline__ void st(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
-};
-template <> struct Pair<__nv_bfloat16> {
-  static __device__ __forceinline__ float2 ld(const __nv_bfloat16* p) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p)); }
-  static __device__ __forceinline__ void st(__nv_bfloat16* p, float2 v) { *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v.x, v.y); }
-};
+// A block owns 256 columns; warp w takes rows w, w + NW, ... (ascending), eight columns per lane; the per-warp partial sums of
+// a column are added in warp order.  (fp32 networks: dz only, the weight-gradient GEMM sums the columns of its operand.)
+constexpr int kActWarps = 8;
 
 constexpr int kActColsV = 256;                        // columns per block: 8 per lane
 constexpr int kColsumGroup = 8;                       // row chunks per block in a launch that only sums columns
 constexpr int kStageGroup = 4;                        // ... and in a launch of one stage
+constexpr int kSmallRows = 512;                       // microbatches of up to this many rows: a block takes all rows of its columns
+constexpr int kSmallCols = 64;
 // Row chunks one block of the activation-backward launch covers; its sum is partial row (first chunk / group) of the stage.
 __host__ __device__ inline int act_chunk_group(const TickArgs& t) {
   return t.row_chunks > 1 ? (t.colsum_only ? kColsumGroup : (t.sel_p >= 0 ? kStageGroup : 1)) : 1;
@@ -198,15 +195,17 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = c0 + 8 * lane;
   const uint64_t n = (uint64_t)t.T * L.n_out;
-  const AT* dy = (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, s.dh)
+  const bool has_act = bwd_act(L) != PM_ACT_NONE && !t.colsum_only;   // without an activation (or with one applied upstream) dz = dy: nothing is stored
+  const bool sums = sizeof(AT) == 2 && !t.dz_only;
+  if (!has_act && !sums) return;
+  const AT* dy = t.colsum_only ? dz_src<AT>(t, s, d, lvl)
+                 : (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off)
                  : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
-  const bool has_act = bwd_act(L) != PM_ACT_NONE;           // without an activation (or with one applied upstream) dz = dy: nothing is stored
-  if (t.colsum_only && has_act) return;
   // the pre-activation stash, or for a ReLU without one the stashed output (same sign pattern)
   const AT* z = !has_act ? dy
                 : !(L.flags & LF_ACT_FROM_Y) ? ring_ptr<AT>(t, L.z_ring, d.b_slot, n)
                 : (lvl < s.n_lin - 1 ? ring_ptr<AT>(t, L.h_ring, d.b_slot, n) : ring_ptr<AT>(t, t.st[p + 1].x_ring, d.b_next_xslot, n));
-  AT* dz = ws_ptr<AT>(t, s.dz);
+  AT* dz = ws_ptr<AT>(t, L.dz_off);
   const bool vec = (L.n_out & 7) == 0;                      // vector path needs 8-element alignment of every row
   float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (vec) {
@@ -227,6 +226,7 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
         }
     }
   }
+  if (!sums) return;
   __shared__ float red[NW][kActColsV];
 #pragma unroll
   for (int k = 0; k < 8; ++k) red[warp][8 * lane + k] = sum[k];
@@ -238,6 +238,71 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
     for (int w = 0; w < NW; ++w) a = __fadd_rn(a, red[w][threadIdx.x]);
     if (t.row_chunks == 1) t.a.grad[L.b_off + cc] = d.accum ? __fadd_rn(t.a.grad[L.b_off + cc], a) : a;
     else ws_ptr<float>(t, t.colred_off)[((uint64_t)p * t.row_chunks + blockIdx.y) * (2 * (uint64_t)t.max_dim) + cc] = a;   // partial rows are dense: one per block
+  }
+}
+
+// The same for microbatches of at most kSmallRows rows: a block takes 64 columns of ALL rows (eight columns per lane, four
+// rows per warp and step), so there are no partial sums to finish in a second launch.  What bounds these launches is the
+// number of rows a block walks one after the other and the launches themselves, not the bytes: with 256-column blocks of 32
+// rows and a finishing launch a level of the 32-stage 1024-wide MLP (128 rows) took 17.6 + 12.7 us.
+template <typename AT>
+__global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) {
+  constexpr int kPer = kActColsV / kSmallCols;
+  const int* start = t.act_start + (size_t)lvl * (t.P + 1);
+  const int blk = (int)(blockIdx.x / kPer) + t.act_first[lvl];
+  int lo = 0, hi = t.P - 1;
+  if (t.sel_p >= 0) lo = hi = t.sel_p;
+  while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (start[mid] <= blk) lo = mid; else hi = mid - 1; }
+  const int p = lo;
+  const StageDyn& d = t.dyn[p];
+  const StageDev& s = t.st[p];
+  if (d.b_mb < 0 || lvl >= s.n_lin) return;
+  const LinDev& L = s.lin[lvl];
+  const int c0 = (blk - start[p]) * kActColsV + (int)(blockIdx.x % kPer) * kSmallCols;
+  if (c0 >= L.n_out) return;
+  const bool has_act = bwd_act(L) != PM_ACT_NONE && !t.colsum_only;
+  const bool sums = sizeof(AT) == 2 && !t.dz_only;
+  if (!has_act && !sums) return;
+  const AT* dy = t.colsum_only ? dz_src<AT>(t, s, d, lvl)
+                 : (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off)
+                 : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
+  const uint64_t n = (uint64_t)t.T * L.n_out;
+  const AT* z = !has_act ? dy
+                : !(L.flags & LF_ACT_FROM_Y) ? ring_ptr<AT>(t, L.z_ring, d.b_slot, n)
+                : (lvl < s.n_lin - 1 ? ring_ptr<AT>(t, L.h_ring, d.b_slot, n) : ring_ptr<AT>(t, t.st[p + 1].x_ring, d.b_next_xslot, n));
+  AT* dz = ws_ptr<AT>(t, L.dz_off);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if ((L.n_out & 7) == 0) {
+    const int c = c0 + 8 * (lane & 7), r = 4 * warp + (lane >> 3);
+    if (c < L.n_out) {
+      if (!has_act) actbwd_rows<AT, PM_ACT_NONE, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
+      else if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
+      else actbwd_rows<AT, PM_ACT_GELU, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
+    }
+  } else if (has_act) {                                     // fp32 only: bf16 Linears have widths that are multiples of 8
+    const int c = c0 + (int)(threadIdx.x & 63);
+    if (c < L.n_out)
+      for (int r = threadIdx.x >> 6; r < t.T; r += 4) {
+        const uint64_t i = (uint64_t)r * L.n_out + c;
+        dz[i] = from_f<AT>(round_as<AT>(__fmul_rn(to_f<AT>(dy[i]), act_grad(to_f<AT>(z[i]), L.act))));
+      }
+  }
+  if (!sums) return;
+  __shared__ float red[8][kSmallCols];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {                             // the four rows of the warp, in a fixed order
+    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 8));
+    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 16));
+    if (lane < 8) red[warp][8 * lane + k] = sum[k];
+  }
+  __syncthreads();
+  const int cc = c0 + threadIdx.x;
+  if (threadIdx.x < kSmallCols && cc < L.n_out) {
+    float a = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) a = __fadd_rn(a, red[w][threadIdx.x]);
+    t.a.grad[L.b_off + cc] = d.accum ? __fadd_rn(t.a.grad[L.b_off + cc], a) : a;
   }
 }
 
@@ -268,7 +333,7 @@ __global__ void __launch_bounds__(256) bias_finish_kernel(TickArgs t, int lvl) {
   const uint64_t ps = 2 * (uint64_t)t.max_dim;
   const float* part = ws_ptr<float>(t, t.colred_off) + (uint64_t)p * t.row_chunks * ps + (c < L.n_out ? c : 0);
   // partial rows the activation-backward launch of this Linear wrote: one per block of that launch
-  const int cg = t.fin_deferred ? (t.row_chunks > 1 ? (bwd_act(L) != PM_ACT_NONE ? kStageGroup : kColsumGroup) : 1) : act_chunk_group(t);
+  const int cg = act_chunk_group(t);
   const int n_rows = (t.row_chunks + cg - 1) / cg;
   float sum = 0.f;
   for (int k0 = warp; k0 < n_rows; k0 += 8 * kFinMaxPer) {
@@ -289,24 +354,15 @@ __global__ void __launch_bounds__(256) bias_finish_kernel(TickArgs t, int lvl) {
   }
 }
 
-int actbwd_launches(const TickArgs& t) { return (t.row_chunks == 1 || t.defer_finish) ? 1 : 2; }
-
-int deferred_finish_launches(const TickArgs& t) { return (t.row_chunks > 1 ? t.max_lin : 0) + ln_finish_launches(t); }
-cudaError_t launch_deferred_finish(const TickArgs& t, int dtype, cudaStream_t stream) {
-  (void)dtype;
-  if (t.row_chunks > 1) {
-    TickArgs tf = t;
-    tf.fin_deferred = 1;
-    for (int lvl = 0; lvl < t.max_lin; ++lvl)
-      if (t.act_blocks[lvl] > 0) bias_finish_kernel<<<t.act_blocks[lvl] * (kActColsV / kFinCols), 256, 0, stream>>>(tf, lvl);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return launch_ln_finish(t, stream);
-}
+int actbwd_launches(const TickArgs& t, int dtype) { return (t.T <= kSmallRows || t.row_chunks == 1 || t.dz_only || dtype == PM_F32) ? 1 : 2; }
 
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream) {
   if (t.act_blocks[lvl] == 0) return cudaSuccess;
+  if (t.T <= kSmallRows) {
+    if (dtype == PM_F32) actbwd_small_kernel<float><<<t.act_blocks[lvl] * (kActColsV / kSmallCols), 256, 0, stream>>>(t, lvl);
+    else actbwd_small_kernel<__nv_bfloat16><<<t.act_blocks[lvl] * (kActColsV / kSmallCols), 256, 0, stream>>>(t, lvl);
+    return cudaGetLastError();
+  }
   const int cg = act_chunk_group(t);
   dim3 grid(t.act_blocks[lvl], (t.row_chunks + cg - 1) / cg);
   if (t.sel_p >= 0 && t.row_chunks > 1) {
@@ -317,7 +373,7 @@ cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t st
     else actbwd_kernel<__nv_bfloat16, kActWarps><<<grid, kActWarps * 32, 0, stream>>>(t, lvl);
   }
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || t.row_chunks == 1 || t.defer_finish) return e;
+  if (e != cudaSuccess || actbwd_launches(t, dtype) == 1) return e;
   bias_finish_kernel<<<t.act_blocks[lvl] * (kActColsV / kFinCols), 256, 0, stream>>>(t, lvl);
   return cudaGetLastError();
 }
@@ -325,8 +381,9 @@ cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t st
 // ---- fp32 SIMT grouped GEMM ------------------------------------------------------------------------
 // C[M,N] = sum_k A(m,k) B(k,n) with fused multiply-adds in fp32.
 //   mode 0 forward:  A = x [T,in],        B(k,n) = W[n,k]            -> z = C + b, y = act(z)
-//   mode 1 dgrad:    A = dz [T,out],      B(k,n) = W[k,n]-gap*delta  -> dx = C
-//   mode 2 wgrad:    A(m,k) = dz[k,m],    B(k,n) = x[k,n]            -> dW = C
+//   mode 1 dgrad:    A = dz [T,out],      B(k,n) = W[k,n]-gap*delta  -> dx = C, times act'(z) of the Linear that receives it
+//   mode 2 wgrad:    A(m,k) = dz[k,m],    B(k,n) = x[k,n]            -> dW = C; db = the row sums of A (the bias gradient
+//                    without a launch of its own)
 // What bounds it: latency.  The fp32 workloads have a few hundred rows and columns and a reduction of as many, so a
 // launch is a handful of loads deep; a k loop that loads, synchronises and multiplies in turn paid one L2 round trip
 // per 16 k.  Here the eight warps of a block split the reduction: warp w owns the 16-deep k chunks w, w + 8, ..., brings
@@ -345,7 +402,7 @@ template <int TM, int TN, int NBUF, int MODE> struct F32Cfg {
   static constexpr int kB = MODE == 0 ? BN * (kF32KC + 4) : kF32KC * (BN + 4);
   static constexpr int kBuf = kA + kB * (MODE == 1 ? 2 : 1);                     // mode 1: w and delta
   static constexpr int kPanels = 8 * NBUF * kBuf;
-  static constexpr int kRed = 8 * BM * (BN + 4);
+  static constexpr int kRed = 8 * BM * (BN + 4) + (MODE == 2 ? 8 * BM : 0);      // partial tiles; mode 2: partial row sums of A
   static constexpr int kBytes = 4 * (kPanels > kRed ? kPanels : kRed);
 };
 
@@ -442,6 +499,10 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+  float rows[TM];                                          // mode 2, first column of tiles: row sums of A over this warp's k
+#pragma unroll
+  for (int i = 0; i < TM; ++i) rows[i] = 0.f;
+  const bool bias_tile = MODE == 2 && n0 == 0;
 
 #pragma unroll
   for (int b = 0; b < NBUF; ++b) load(warp + 8 * b, mine + b * C::kBuf);
@@ -490,6 +551,12 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
             bv[j][kk] = v.x; bv[j + 1][kk] = v.y;
           }
       }
+      if (bias_tile) {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int i = 0; i < TM; ++i) rows[i] = __fadd_rn(rows[i], av[i][kk]);
+      }
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
@@ -512,8 +579,18 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
         const int m = MODE == 2 ? ty * TM + i : ty + 4 * i, n = MODE == 0 ? tx + 8 * j : tx * TN + j;
         red[m * (BN + 4) + n] = acc[i][j];
       }
+    if (bias_tile && tx == 0)
+#pragma unroll
+      for (int i = 0; i < TM; ++i) f32_sm[8 * BM * (BN + 4) + warp * BM + ty * TM + i] = rows[i];
   }
   __syncthreads();
+  if (bias_tile && tid < BM && m0 + tid < M) {
+    float v = f32_sm[8 * BM * (BN + 4) + tid];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v = __fadd_rn(v, f32_sm[8 * BM * (BN + 4) + w * BM + tid]);
+    float* db = t.a.grad + L.b_off + m0 + tid;
+    *db = d.accum ? __fadd_rn(*db, v) : v;
+  }
 
   // epilogue: consecutive threads take consecutive columns of a row
   const uint64_t n_xout = (uint64_t)T * L.n_out;
@@ -521,7 +598,9 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
   float* yout = MODE == 0 ? y_dest<float>(t, p, s, d, lvl) : nullptr;
   float* lout = MODE == 0 && (L.flags & LF_OUT_F32) ? ws_ptr<float>(t, t.yout_off) + (uint64_t)(d.tick & 1) * n_xout : nullptr;
   const float* bias = fwd_small<float>(t, s, d, L.b_off, L.b_soff);
-  float* dx = MODE == 1 ? ((lvl == 0 && s.pre == PRE_NONE) ? gin_write_prev<float>(t, p, d) : ws_ptr<float>(t, s.dh)) : nullptr;
+  float* dx = MODE == 1 ? dx_dest<float>(t, p, s, d, lvl) : nullptr;
+  const float* z = nullptr;
+  const int dact = MODE == 1 ? dx_fused_act<float>(t, p, s, d, lvl, &z) : PM_ACT_NONE;
   float* dW = t.a.grad + L.w_off;
 #pragma unroll
   for (int o = tid; o < BM * BN; o += 256) {
@@ -536,7 +615,7 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
       if (lout) lout[i] = v;
       if (zout) zout[i] = v;
       if (yout) yout[i] = act_fwd(v, L.act);
-    } else if (MODE == 1) dx[i] = v;
+    } else if (MODE == 1) dx[i] = dact != PM_ACT_NONE ? __fmul_rn(v, act_grad(z[i], dact)) : v;
     else dW[i] = d.accum ? __fadd_rn(dW[i], v) : v;
   }
 }

@@ -58,15 +58,14 @@ struct TickArgs {
                                // group (0: always two); launches of one stage need enough groups for the CTA pairs
   float loss_scale;       // factor on dL/dy: 1/N with N microbatches per update (the minibatch loss is their mean), else 1
   int32_t ln_li0;         // first entry of ln_ids a launch covers (its grid counts entries from there)
-  int32_t colsum_only;    // activation-backward launch that only sums columns (bias gradients) of Linears WITHOUT activation:
-                          // stages with an activation were handled by their own launch (microbatch-major order)
-  int32_t defer_finish;   // launches of one stage leave the per-chunk partial sums of bias / LayerNorm gradients in place;
+  int32_t colsum_only;    // activation-backward launch that only sums the columns of every Linear's dz (bias gradients), all stages at
+                          // once at the end of a microbatch-major backward pass; dz was formed on the way
+  int32_t dz_only;        // ... and the launches of one stage on the way: dz, no sums
+  int32_t defer_finish;   // launches of one stage leave the per-chunk partial sums of LayerNorm gradients in place;
                           // one grouped launch over all stages adds them up at the end of the backward pass
   // weight-gradient launch that applies the PipeMare update to the Linear matrices in its epilogue (bf16 tensor-core
   // path): dW never reaches the grad arena; the stage's step size, T2 decay and bias corrections come from its table
   // entry, the optimiser constants from here, and the operand-type copy of the new weights goes to lp_base
-  int32_t fin_deferred;   // bias finishing pass launched once for all stages at the end of a microbatch-major backward pass: the partial
-                          // rows were written by launches of one stage (Linears with activation) or by the column-sum-only launch
   int32_t ln_stage;       // LayerNorm backward: a block first brings its rows of x, du and the skip gradient into shared memory
                           // with asynchronous copies (all in flight at once), then works from there (set by the launcher)
   int32_t stash;          // weight stashing (tau_bkwd = tau_fwd for every stage): the backward pass reads the queued version the
@@ -145,10 +144,28 @@ template <typename AT> __device__ __forceinline__ AT* mem_at(const TickArgs& t, 
 }
 // dz = dy * act'(z) of Linear lvl as the wgrad / dgrad operand: without an activation it IS the incoming gradient
 template <typename AT> __device__ __forceinline__ const AT* dz_src(const TickArgs& t, const StageDev& s, const StageDyn& d, int lvl) {
-  if (bwd_act(s.lin[lvl]) != PM_ACT_NONE) return ws_at<AT>(t, s.dz);
-  if (lvl < s.n_lin - 1) return ws_at<AT>(t, s.dh);
+  if (bwd_act(s.lin[lvl]) != PM_ACT_NONE) return ws_at<AT>(t, s.lin[lvl].dz_off);
+  if (lvl < s.n_lin - 1) return ws_at<AT>(t, s.lin[lvl].dy_off);
   if (feeds_attention(s.post)) return ws_at<AT>(t, s.dy);
   return gin_read<AT>(t, s, d);
+}
+// where the dgrad of Linear lvl of stage p writes: the previous Linear's output gradient (inside the stage, or through the
+// previous stage's mailbox), or the gradient of the pre-op's output
+template <typename AT> __device__ __forceinline__ AT* dx_dest(const TickArgs& t, int p, const StageDev& s, const StageDyn& d, int lvl) {
+  if (lvl > 0) return ws_at<AT>(t, s.lin[lvl - 1].dy_off);
+  return s.pre == PRE_NONE ? gin_write_prev<AT>(t, p, d) : ws_at<AT>(t, s.dh);
+}
+// the activation the dgrad of Linear lvl of stage p applies to what it writes (LF_DZ_FUSED of the Linear that receives it),
+// and the stash its derivative comes from: that Linear's z, or its output y = this Linear's own stashed input
+template <typename AT> __device__ __forceinline__ int dx_fused_act(const TickArgs& t, int p, const StageDev& s, const StageDyn& d, int lvl, const AT** z) {
+  *z = nullptr;
+  if (lvl == 0 && (p == 0 || s.pre != PRE_NONE)) return PM_ACT_NONE;
+  const StageDev& q = lvl > 0 ? s : t.st[p - 1];
+  const LinDev& L = q.lin[lvl > 0 ? lvl - 1 : q.n_lin - 1];
+  if (!(L.flags & LF_DZ_FUSED)) return PM_ACT_NONE;
+  if (L.flags & LF_ACT_FROM_Y) *z = lin_input<AT>(t, s, d, lvl, false);
+  else *z = ring_at<AT>(t, L.z_ring, lvl > 0 ? d.b_slot : (int)(d.b_mb % q.depth), (uint64_t)t.T * L.n_out);
+  return L.act;
 }
 // destination of Linear lvl's activation y in the forward pass (nullptr: not written)
 template <typename AT> __device__ __forceinline__ AT* y_dest(const TickArgs& t, int p, const StageDev& s, const StageDyn& d, int lvl) {
@@ -168,11 +185,8 @@ cudaError_t launch_ingest(const TickArgs& t, int dtype, const void* inputs, cons
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream);
 // dz = dy * act'(z) and db = column sums, level `lvl` of every stage that runs backward this tick.
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream);
-int actbwd_launches(const TickArgs& t);
-// the finishing passes that launches with defer_finish left out, grouped over all stages (bias column sums, LayerNorm
-// parameter gradients)
-cudaError_t launch_deferred_finish(const TickArgs& t, int dtype, cudaStream_t stream);
-int deferred_finish_launches(const TickArgs& t);
+int actbwd_launches(const TickArgs& t, int dtype);
+// the finishing pass that launches with defer_finish left out, grouped over all stages (LayerNorm parameter gradients)
 cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream);      // pm_xfmr.cu
 int ln_finish_launches(const TickArgs& t);
 

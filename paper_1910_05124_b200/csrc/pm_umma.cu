@@ -1963,10 +1963,10 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
         okm = okm && encode(fn, m + MAP_D_F32H, 3, (void*)(t.a.delta + L.w_off), 2, dims, strides4, box4h, err);
       }
       {
-        // dz operand (same rule as dz_src): dz scratch | dh scratch | attention's dy | rotating incoming-gradient mailbox
+        // dz operand (same rule as dz_src): dz scratch | gradient inside the stage | attention's dy | rotating incoming-gradient mailbox
         char* dzb; uint64_t dz_slots = 1;
-        if (bwd_act(L) != PM_ACT_NONE) dzb = t.ws + s.dz;
-        else if (l < s.n_lin - 1) dzb = t.ws + s.dh;
+        if (bwd_act(L) != PM_ACT_NONE) dzb = t.ws + L.dz_off;
+        else if (l < s.n_lin - 1) dzb = t.ws + L.dy_off;
         else if (feeds_attention(s.post)) dzb = t.ws + s.dy;
         else if (s.emit_memory) { dzb = t.ws + t.gmem_off; dz_slots = (uint64_t)t.gmem_depth; }
         else { dzb = t.ws + s.gin; dz_slots = (uint64_t)s.gin_depth; }
@@ -1995,7 +1995,7 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
         }
         if (!(p == 0 && l == 0 && s.pre != PRE_EMBED)) {
           const bool to_prev = l == 0 && s.pre == PRE_NONE;
-          char* xbase = to_prev ? t.ws + st[p - 1].gin : t.ws + s.dh;
+          char* xbase = to_prev ? t.ws + st[p - 1].gin : t.ws + (l > 0 ? s.lin[l - 1].dy_off : s.dh);
           uint64_t xd[3] = {n_in, T, (uint64_t)(to_prev ? st[p - 1].gin_depth : 1)}, xs[2] = {n_in * 2, T * n_in * 2};
           okm = okm && encode(fn, m + MAP_DX_OUT, 1, xbase, 3, xd, xs, box_bf, err);
         }
