@@ -320,6 +320,14 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       if (cfg->compute_dtype == PM_F32 && ld.act != PM_ACT_NONE &&
           (!last || (p == P - 1 ? (!ce && s.post == POST_NONE) : (next_takes_y && stages[p + 1].n_ops > 0 && stages[p + 1].ops && stages[p + 1].ops[0].kind == PM_OP_LINEAR && (S == 0 || (p + 1) % S != 0)))))
         ld.flags |= LF_DZ_FUSED;
+      // bf16, microbatch-major order: the same where the consuming dgrad runs on the kernel for few tiles
+      if (mb && cfg->compute_dtype == PM_BF16 && ld.act != PM_ACT_NONE) {
+        const pm_op_desc* nx = !last ? &sd.ops[s.pre == PRE_NONE ? l + 1 : l + 2]
+                               : (next_takes_y && stages[p + 1].n_ops > 0 && stages[p + 1].ops && stages[p + 1].ops[0].kind == PM_OP_LINEAR && (S == 0 || (p + 1) % S != 0)) ? &stages[p + 1].ops[0] : nullptr;
+        LinDev nl{};
+        if (nx) { nl.n_in = nx->n_in; nl.n_out = nx->n_out; }
+        if (nx ? umma_row_dgrad((int)T, nl) : (last && p == P - 1 && !ce && s.post == POST_NONE)) ld.flags |= LF_DZ_FUSED;
+      }
       if (bwd_act(ld) != PM_ACT_NONE) L.act_levels |= 1 << l;
     }
     if (p > 0 && (L.st[p - 1].lin[L.st[p - 1].n_lin - 1].flags & LF_DZ_FUSED)) s.mask_dx = 1;
@@ -530,6 +538,7 @@ struct pm_ctx {
   std::vector<int32_t> h_delays;           // stochastic delay model: host copy of the delays in force
   bool graphs = true;
   cudaStream_t cap_stream = nullptr;
+  bool chained = false;                 // a launch of the running phase body precedes: the next may be a programmatic dependent of it
   cudaStream_t ls = nullptr;            // the stream the phase bodies launch on: `stream`, or `cap_stream` while capturing
   ~pm_ctx() {
     for (PhaseGraph* g : {&g_fwd, &g_bwd, &g_upd}) if (g->exec) cudaGraphExecDestroy(g->exec);
@@ -698,7 +707,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   t.n_in_first = L.n_in_first; t.n_out_last = L.n_out_last;
   t.yout_off = L.off_yout; t.tgt_off = L.off_tgt; t.loss_off = L.off_loss; t.loss_cap = L.loss_cap; t.lossred_off = L.off_lossred;
   t.max_lin = L.max_lin; t.max_dim = L.max_dim;
-  t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0;
+  t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0; t.pdl = 0;
   t.res_fused = cfg->compute_dtype == PM_BF16 ? 1 : 0;
   t.ln_li0 = 0; t.defer_finish = 0; t.colsum_only = 0; t.dz_only = 0; t.ln_stage = 0;
   t.dgrad_split_below = 0;
@@ -746,6 +755,10 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
     if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "attention shared-memory limit"); delete c; return r; }
   }
 
+  if (cfg->compute_dtype == PM_F32) {
+    e = simt_gemm_set_limits();
+    if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "GEMM shared-memory limit"); delete c; return r; }
+  }
   if (cfg->compute_dtype == PM_BF16) {
     std::string uerr;
     pm_status us = umma_plan_create(&c->umma, t, c->L.st, c->ws + L.off_umma, c->stream, uerr);
@@ -791,6 +804,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
 // every call checked here enqueued `kernels` kernels
 static pm_status check(pm_ctx* ctx, cudaError_t e, const char* what, int kernels = 1) {
   ctx->launches += kernels;
+  ctx->chained = true;
   if (ctx->prof_on && ctx->prof_cls >= 0 && ctx->prof_used < ctx->prof_pair_cls.size()) {
     cudaEventRecord(ctx->prof_ev[2 * ctx->prof_used + 1], ctx->stream);
     ctx->prof_pair_cls[ctx->prof_used] = ctx->prof_cls;
@@ -812,6 +826,7 @@ static inline void prof_begin(pm_ctx* ctx, int cls) {
 static pm_status run_phase(pm_ctx* ctx, pm_ctx::PhaseGraph& g, const std::function<pm_status()>& body, cudaStream_t run_on = nullptr) {
   if (!run_on) run_on = ctx->stream;
   ctx->ls = run_on;
+  ctx->chained = false;
   if (!ctx->graphs || ctx->prof_on || g.failed || !ctx->cap_stream) return body();
   if (g.exec) {
     ctx->launches += g.launches;
@@ -835,6 +850,7 @@ static pm_status run_phase(pm_ctx* ctx, pm_ctx::PhaseGraph& g, const std::functi
     cudaGetLastError();
     g.failed = true; g.exec = nullptr;
     ctx->launches = l0;
+    ctx->chained = false;
     return body();
   }
   e = cudaGraphLaunch(g.exec, run_on);
@@ -900,7 +916,9 @@ static pm_status stage_forward(pm_ctx* ctx, const TickArgs& ta, int p) {
   if (sd.pre != PRE_NONE && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(ta, dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
   for (int l = 0; l < sd.n_lin; ++l) {
     prof_begin(ctx, PM_PROF_GEMM_FWD);
-    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(ta, 0, l, ctx->ls) : umma_launch(ctx->umma, ta, 0, l, ctx->ls);
+    TickArgs tl = ta;
+    tl.pdl = ctx->chained ? 1 : 0;
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(tl, 0, l, ctx->ls) : umma_launch(ctx->umma, tl, 0, l, ctx->ls);
     if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
   }
   const bool att = feeds_attention(sd.post);
@@ -941,7 +959,9 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     }
     if (p == 0 && l == 0 && sd.pre != PRE_EMBED) continue;          // raw network inputs need no gradient
     prof_begin(ctx, PM_PROF_DGRAD);
-    e = dt == PM_F32 ? launch_simt_gemm(ta, 1, l, ctx->ls) : umma_launch(ctx->umma, ta, (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
+    TickArgs tl = ta;
+    tl.pdl = ctx->chained ? 1 : 0;
+    e = dt == PM_F32 ? launch_simt_gemm(tl, 1, l, ctx->ls) : umma_launch(ctx->umma, tl, (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;

@@ -623,12 +623,20 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
 template <int TM, int TN, int NBUF, int MODE>
 static cudaError_t launch_f32_t(const TickArgs& t, int lvl, int grid_m, cudaStream_t stream) {
   using C = F32Cfg<TM, TN, NBUF, MODE>;
-  static const cudaError_t attr = cudaFuncSetAttribute((const void*)f32_gemm_kernel<TM, TN, NBUF, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes);
-  if (attr != cudaSuccess) return attr;
   const int tiles_n = (t.max_dim + C::BN - 1) / C::BN, tiles_m = (grid_m + C::BM - 1) / C::BM;
   dim3 grid((unsigned)tiles_m * (unsigned)tiles_n, t.sel_p >= 0 ? 1 : t.P);
   f32_gemm_kernel<TM, TN, NBUF, MODE><<<grid, 256, C::kBytes, stream>>>(t, lvl, tiles_n);
   return cudaGetLastError();
+}
+
+// opt-in shared-memory sizes, on the current device
+cudaError_t simt_gemm_set_limits() {
+  cudaError_t e = cudaSuccess;
+#define PM_F32_LIMIT(TM, TN, NB, MODE) if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)f32_gemm_kernel<TM, TN, NB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Cfg<TM, TN, NB, MODE>::kBytes)
+  PM_F32_LIMIT(4, 2, 4, 0); PM_F32_LIMIT(4, 2, 3, 1); PM_F32_LIMIT(4, 2, 4, 2);
+  PM_F32_LIMIT(8, 4, 2, 0); PM_F32_LIMIT(8, 4, 2, 1); PM_F32_LIMIT(8, 4, 2, 2);
+#undef PM_F32_LIMIT
+  return e;
 }
 
 // 16 x 16 tiles while 32 x 32 ones would number no more than the 148 SMs: a smaller tile has a quarter of the multiplies on

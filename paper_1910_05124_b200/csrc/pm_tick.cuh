@@ -51,6 +51,8 @@ struct TickArgs {
   // the stage from a block coordinate use sel_p instead (-1: all stages, the coordinate); the stage lists above then
   // point at that stage's entry; act_first[lvl] is added to the block index of the activation-backward walk
   int32_t sel_p;
+  int32_t pdl;            // the launch may start before its predecessor in the phase has ended (programmatic dependent launch): kernels
+                          // that honour it read only weights and tables before they wait
   int32_t sel_tile0;      // GEMM launches of one stage: flattened id of the stage's first tile (set by the launcher)
   int32_t act_first[PM_MAX_LINEARS];
   int32_t res_fused;      // the forward GEMM's epilogue adds the skip tensor (bf16 tensor-core path): no residual kernel
@@ -207,6 +209,7 @@ size_t attention_smem_bytes(int S, int dk, int dtype);
 cudaError_t attention_set_smem_limits(int S, int dk, int dtype);
 
 // fp32 SIMT grouped GEMMs (PM_F32 path).  mode: 0 forward, 1 dgrad (corrected weights), 2 wgrad.
+cudaError_t simt_gemm_set_limits();
 cudaError_t launch_simt_gemm(const TickArgs& t, int mode, int lvl, cudaStream_t stream);
 
 }  // namespace pm

@@ -49,7 +49,10 @@ template <int MODE> struct Cfg {                           // MODE 0 forward, 2 
 };
 
 enum { MAP_ACT_K = 0, MAP_W_K = 1, MAP_DZ_K = 2, MAP_DZ_MN = 3, MAP_ACT_MN = 4, MAP_W_F32 = 5, MAP_D_F32 = 6,
-       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_F32Q = 11, MAP_D_F32Q = 12, MAP_W_F32H = 13, MAP_D_F32H = 14, MAP_W_MN = 15, MAPS_PER_LINEAR = 16 };
+       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_F32Q = 11, MAP_D_F32Q = 12, MAP_W_F32H = 13, MAP_D_F32H = 14, MAP_W_MN = 15, MAP_W_K32 = 16, MAPS_PER_LINEAR = 17 };
+}  // namespace pm
+#include "pm_umma_row.cuh"     // the kernel of launches with few tiles; uses the tensor maps above
+namespace pm {
 
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = 128, operand majors as given.
 __device__ __forceinline__ uint32_t make_idesc(int a_mn_major, int b_mn_major) {
@@ -1779,6 +1782,7 @@ struct UmmaPlan {
   int P = 0;
   // launches of one stage (microbatch-major order): the stage's tiles in ascending order are a slice of the identity list
   std::vector<int> h_tile_start;         // host copy of the tile starts
+  std::vector<StageDev> st;              // host copy of the stages (launches of one stage with few tiles)
   const int* d_identity = nullptr;       // 0, 1, 2, ...
   int max_ctas = 148;
 };
@@ -1950,6 +1954,8 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
             wbase = (void*)(reinterpret_cast<__nv_bfloat16*>(t.ring + s.v_ring) + (L.w_off - s.begin));
           }
           okm = okm && encode(fn, m + MAP_W_K, 0, wbase, 3, dims3, strides3, box3, err);
+          uint32_t box32[3] = {TILE_K, 32, 1};                          // 32 columns of an output tile (launches with few tiles)
+          okm = okm && encode(fn, m + MAP_W_K32, 0, wbase, 3, dims3, strides3, box32, err);
           uint32_t box3mn[3] = {64, TILE_K, 1};                         // the same copies as an MN-major operand (dgrad against a queued version)
           okm = okm && encode(fn, m + MAP_W_MN, 0, wbase, 3, dims3, strides3, box3mn, err);
         }
@@ -2036,6 +2042,9 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DP_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D1_SMEM_BYTES);
+  if (e == cudaSuccess) e = row_set_limits<0>();
+  if (e == cudaSuccess) e = row_set_limits<1>();
+  if (e == cudaSuccess) e = row_set_limits<2>();
   if (e != cudaSuccess) { err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); delete plan; return PM_ERR_CUDA; }
   plan->d_status = (int*)region;
   plan->d_maps = (const CUtensorMap*)(region + 256);
@@ -2044,6 +2053,7 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   plan->d_identity = (const int*)id_dev;
   plan->h_tile_start = tt.tile_start;
   plan->max_ctas = device_sms();
+  plan->st = st;
   *out = plan;
   return PM_OK;
 }
@@ -2073,7 +2083,18 @@ cudaError_t umma_clear_status(UmmaPlan* plan, cudaStream_t stream) { return cuda
 
 int* umma_status_word(UmmaPlan* plan) { return plan ? plan->d_status : nullptr; }
 
+bool umma_row_dgrad(int T, const LinDev& L) { return row_shape(T, L.n_in, L.n_out, 1).bn != 0; }
+
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream) {
+  if (t.sel_p >= 0 && mode != 2) {
+    const LinDev& L = plan->st[t.sel_p].lin[lvl];
+    const int N = mode == 0 ? L.n_out : L.n_in;
+    const RowShape r = row_shape(t.T, N, mode == 0 ? L.n_in : L.n_out, 1);
+    if (r.bn != 0)
+      return mode == 0 ? row_launch<0>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
+             : mode == 1 ? row_launch<1>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
+                         : row_launch<2>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream);
+  }
   int n_slots = plan->n_slots[mode][lvl];
   if (n_slots == 0) return cudaSuccess;
   int grid = plan->grid[mode][lvl];                                   // one persistent CTA per SM

@@ -21,6 +21,8 @@ int* umma_status_word(UmmaPlan* plan);
 // word like a real expiry would and writes 2 to *d_returned.  umma_clear_status resets the status word.
 cudaError_t umma_wait_timeout_probe(UmmaPlan* plan, long long limit_cycles, int* d_returned, cudaStream_t stream);
 cudaError_t umma_clear_status(UmmaPlan* plan, cudaStream_t stream);
+// does the dgrad of this Linear, launched for its stage alone, run on the kernel for few tiles (pm_umma_row.cuh)?
+bool umma_row_dgrad(int T, const LinDev& L);
 // mode: 0 forward, 1 dgrad (corrected weights formed in the operand-load path), 2 wgrad.
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream);
 
