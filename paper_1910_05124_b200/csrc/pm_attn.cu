@@ -1,5 +1,5 @@
 // Multi-head self-attention on the tensor cores (tcgen05 + TMEM + TMA), forward and backward, for
-// sequences of 128 tokens and heads of width 64 (bf16).  One CTA of 128 threads handles one (sequence, head):
+// sequences of up to 128 tokens and heads of width 64 (bf16).  One CTA of 128 threads handles one (sequence, head):
 // thread r owns query row r = TMEM lane r, so the softmax needs no cross-thread traffic.
 //
 // forward :  S = Q K^T (128x128x64)  ->  p~ = exp(S/8 - rowmax), l = sum p~  ->  O = (bf16(p~) V) / l  (128x64x128);
@@ -103,6 +103,20 @@ __device__ __forceinline__ void attn_store32(__nv_bfloat16* dst, const uint32_t 
   }
 }
 
+// Rows S .. 127 of a [128 x 64] tile, which a sequence of S < 128 tokens leaves untouched, become zeros (the copies bring S rows,
+// so nothing of a neighbouring sequence is ever multiplied).  Zero rows of K give scores that the key mask drops, zero
+// rows of V, Q and dO contribute nothing to a product, and the rows of the results beyond S are not stored.
+__device__ __forceinline__ void zero_rows(uint8_t* tiles, int n_tiles, int S) {
+  const int per = (AT_S - S) * 8;                             // 16-byte chunks of a tile
+  for (int i = threadIdx.x; i < n_tiles * per; i += blockDim.x)
+    *reinterpret_cast<uint4*>(tiles + (i / per) * AT_TILE + S * 128 + (i % per) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  fence_async_smem();
+  __syncthreads();
+}
+
+// FULL: sequences of exactly 128 tokens; otherwise S < 128 (one sequence per tile all the same: a launch is bound by the length
+// of one block's chain of products, not by their number)
+template <bool FULL>
 __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ stage_ids, int* status) {
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
@@ -111,7 +125,8 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
   const bool cross = s.post == POST_CROSS_ATTENTION;         // q = the stage's main input; the Linear gave [k | v]
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
-  if ((int)blockIdx.x >= (t.T / AT_S) * H) return;
+  const int S = FULL ? AT_S : s.seq_len;
+  if ((int)blockIdx.x >= (t.T / S) * H) return;
   const int b = blockIdx.x / H, h = blockIdx.x % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, 3 * AT_TILE, 128);
@@ -121,13 +136,14 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
   const CUtensorMap* lm = maps + (size_t)p * AMAPS_PER_STAGE;
   const int r = threadIdx.x;                                 // query row = TMEM lane
   const int warp = r >> 5;
+  if (!FULL) zero_rows(c.sptr, 3, S);
 
   if (r == 0) {
     const int ko = cross ? 0 : dm;                           // column of k inside the Linear's output
-    mbar_arrive_expect_tx(c.bar_load, 3 * AT_TILE);
-    tma_load_3d(sQ, lm + AMAP_Q, c.bar_load, h * AT_DK, b * AT_S, cross ? d.f_xslot : d.f_slot);
-    tma_load_3d(sK, lm + AMAP_KV, c.bar_load, ko + h * AT_DK, b * AT_S, d.f_slot);
-    tma_load_3d(sV, lm + AMAP_KV, c.bar_load, ko + dm + h * AT_DK, b * AT_S, d.f_slot);
+    mbar_arrive_expect_tx(c.bar_load, 3 * S * AT_DK * 2);
+    tma_load_3d(sQ, lm + AMAP_Q, c.bar_load, h * AT_DK, b * S, cross ? d.f_xslot : d.f_slot);
+    tma_load_3d(sK, lm + AMAP_KV, c.bar_load, ko + h * AT_DK, b * S, d.f_slot);
+    tma_load_3d(sV, lm + AMAP_KV, c.bar_load, ko + dm + h * AT_DK, b * S, d.f_slot);
     if (mbar_wait(c.bar_load, 0, c.abort_flag, status, 11)) {
       tc_fence_after();
       issue_k64(tmem_base, sQ, sK, make_idesc_mn(128, 128, 0, 0), true, true, 0, 0, false);   // S = Q K^T
@@ -145,7 +161,7 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
       tmem_ld_wait();
 #pragma unroll
       for (int j = 0; j < 32; ++j)
-        if (!causal || cc * 32 + j <= r) mx = fmaxf(mx, __uint_as_float(v[j]) * scale);
+        if ((FULL || cc * 32 + j < S) && (!causal || cc * 32 + j <= r)) mx = fmaxf(mx, __uint_as_float(v[j]) * scale);
     }
     float l = 0.f;
 #pragma unroll 1
@@ -156,7 +172,7 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
       float e[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        e[j] = (!causal || cc * 32 + j <= r) ? __expf(__uint_as_float(v[j]) * scale - mx) : 0.f;
+        e[j] = ((FULL || cc * 32 + j < S) && (!causal || cc * 32 + j <= r)) ? __expf(__uint_as_float(v[j]) * scale - mx) : 0.f;
         l += e[j];
       }
 #pragma unroll
@@ -181,7 +197,8 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
       tmem_ld_wait();
       const float inv = 1.0f / l;
       __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(t.ring + t.st[p + 1].x_ring) + (size_t)d.f_next_xslot * ((size_t)t.T * dm) +
-                           (size_t)(b * AT_S + r) * dm + h * AT_DK;
+                           (size_t)(b * S + r) * dm + h * AT_DK;
+      if (FULL || r < S)
 #pragma unroll
       for (int g = 0; g < 8; ++g) {
         const uint32_t* src = g < 4 ? o0 + (g & 3) * 8 : o1 + (g & 3) * 8;
@@ -205,6 +222,7 @@ constexpr int AT_BWD_THREADS = 256;
 constexpr int AT_BWD_TILES = 5;
 constexpr int AT_XCH_BYTES = 3 * 2 * AT_S * 4;
 
+template <bool FULL>
 __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ stage_ids, int* status) {
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
@@ -213,7 +231,8 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
   const bool cross = s.post == POST_CROSS_ATTENTION;
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
-  if ((int)blockIdx.x >= (t.T / AT_S) * H) return;
+  const int S = FULL ? AT_S : s.seq_len;
+  if ((int)blockIdx.x >= (t.T / S) * H) return;
   const int b = blockIdx.x / H, h = blockIdx.x % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, AT_BWD_TILES * AT_TILE);
@@ -225,14 +244,15 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
   const int tid = threadIdx.x;
   const int r = tid & 127, hf = tid >> 7;                    // query row (TMEM lane), key half
   const int warp = tid >> 5;
+  if (!FULL) zero_rows(c.sptr, 4, S);
 
   if (tid == 0) {
     const int ko = cross ? 0 : dm;
-    mbar_arrive_expect_tx(c.bar_load, 4 * AT_TILE);
-    tma_load_3d(sQ, lm + AMAP_Q, c.bar_load, h * AT_DK, b * AT_S, cross ? d.b_xslot : d.b_slot);
-    tma_load_3d(sK, lm + AMAP_KV, c.bar_load, ko + h * AT_DK, b * AT_S, d.b_slot);
-    tma_load_3d(sV, lm + AMAP_KV, c.bar_load, ko + dm + h * AT_DK, b * AT_S, d.b_slot);
-    tma_load_3d(sdO, lm + AMAP_DO, c.bar_load, h * AT_DK, b * AT_S, gin_slot_read(s, d));
+    mbar_arrive_expect_tx(c.bar_load, 4 * S * AT_DK * 2);
+    tma_load_3d(sQ, lm + AMAP_Q, c.bar_load, h * AT_DK, b * S, cross ? d.b_xslot : d.b_slot);
+    tma_load_3d(sK, lm + AMAP_KV, c.bar_load, ko + h * AT_DK, b * S, d.b_slot);
+    tma_load_3d(sV, lm + AMAP_KV, c.bar_load, ko + dm + h * AT_DK, b * S, d.b_slot);
+    tma_load_3d(sdO, lm + AMAP_DO, c.bar_load, h * AT_DK, b * S, gin_slot_read(s, d));
     if (mbar_wait(c.bar_load, 0, c.abort_flag, status, 14)) {
       tc_fence_after();
       const uint32_t idesc = make_idesc_mn(128, 128, 0, 0);
@@ -254,7 +274,7 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
       tmem_ld_wait();
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        e[cc * 32 + j] = (!causal || hf * 64 + cc * 32 + j <= r) ? __uint_as_float(v[j]) * scale : -INFINITY;
+        e[cc * 32 + j] = ((FULL || hf * 64 + cc * 32 + j < S) && (!causal || hf * 64 + cc * 32 + j <= r)) ? __uint_as_float(v[j]) * scale : -INFINITY;
         mx = fmaxf(mx, e[cc * 32 + j]);
       }
     }
@@ -327,23 +347,23 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
       // self-attention: the stage's dy buffer receives [dq | dk | dv]; cross-attention: dy = [dk | dv] and dq goes
       // to the previous stage's gradient mailbox.  This thread stores 32 of the 64 head columns.
       const int wz = cross ? 2 * dm : 3 * dm, ko = cross ? 0 : dm;
-      __nv_bfloat16* dy = reinterpret_cast<__nv_bfloat16*>(t.ws + s.dy) + (size_t)(b * AT_S + r) * wz + h * AT_DK + hf * 32;
-      __nv_bfloat16* dq = cross ? gin_write_prev<__nv_bfloat16>(t, p, d) + (size_t)(b * AT_S + r) * dm + h * AT_DK + hf * 32 : dy;
+      __nv_bfloat16* dy = reinterpret_cast<__nv_bfloat16*>(t.ws + s.dy) + (size_t)(b * S + r) * wz + h * AT_DK + hf * 32;
+      __nv_bfloat16* dq = cross ? gin_write_prev<__nv_bfloat16>(t, p, d) + (size_t)(b * S + r) * dm + h * AT_DK + hf * 32 : dy;
       {
         uint32_t o[32];
         tc_fence_after();
         tmem_ld32(lane_addr + hf * 32, o);                   // dV while dQ and dK are being computed
         tmem_ld_wait();
-        attn_store32(dy + ko + dm, o, 1.0f);
+        if (FULL || r < S) attn_store32(dy + ko + dm, o, 1.0f);
       }
       if (wait_mma(c, 0, status, 17)) {
         uint32_t o[32];
         tmem_ld32(lane_addr + 64 + hf * 32, o);
         tmem_ld_wait();
-        attn_store32(dq, o, scale);
+        if (FULL || r < S) attn_store32(dq, o, scale);
         tmem_ld32(lane_addr + 128 + hf * 32, o);
         tmem_ld_wait();
-        attn_store32(dy + ko, o, scale);
+        if (FULL || r < S) attn_store32(dy + ko, o, scale);
       }
     }
   }
@@ -660,7 +680,7 @@ struct AttnPlan {
 static uint64_t attn_maps_bytes(int n_stages) { return (uint64_t)n_stages * AMAPS_PER_STAGE * sizeof(CUtensorMap); }
 uint64_t attn_workspace_bytes(int n_stages) { return 256 + attn_maps_bytes(n_stages) + ((uint64_t)n_stages * sizeof(int) + 255) / 256 * 256; }
 
-bool attn_tc_supported(int dtype, int S, int dk) { return dtype == PM_BF16 && (S == AT_S || S == AT2_S) && dk == AT_DK; }
+bool attn_tc_supported(int dtype, int S, int dk) { return dtype == PM_BF16 && ((S >= 1 && S <= AT_S) || S == AT2_S) && dk == AT_DK; }
 
 pm_status attn_plan_create(AttnPlan** out, const TickArgs& t, const std::vector<StageDev>& st, void* ws_region, cudaStream_t stream, std::string& err) {
   *out = nullptr;
@@ -679,7 +699,7 @@ pm_status attn_plan_create(AttnPlan** out, const TickArgs& t, const std::vector<
     if (!feeds_attention(s.post)) continue;
     const bool cross = s.post == POST_CROSS_ATTENTION;
     const cuuint64_t dz = (cuuint64_t)s.lin[0].n_out, dm = (cuuint64_t)s.d_out_main;
-    cuuint32_t box[3] = {AT_DK, AT_S, 1}, es[3] = {1, 1, 1};
+    cuuint32_t box[3] = {AT_DK, (cuuint32_t)(t.att_S < AT_S ? t.att_S : AT_S), 1}, es[3] = {1, 1, 1};
     auto enc = [&](int which, void* base, cuuint64_t width, cuuint64_t slots, const char* what) -> bool {
       cuuint64_t dims[3] = {width, T, slots}, strides[2] = {width * 2, T * width * 2};
       CUresult r = fn(&maps[(size_t)p * AMAPS_PER_STAGE + which], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides,
@@ -697,8 +717,10 @@ pm_status attn_plan_create(AttnPlan** out, const TickArgs& t, const std::vector<
   if (e == cudaSuccess && !ids.empty()) e = cudaMemcpyAsync(region + 256 + attn_maps_bytes(t.P), ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(region, 0, 256, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_fwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_FWD_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_bwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_BWD_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_fwd_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_FWD_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_fwd_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_FWD_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_bwd_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_BWD_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_bwd_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_BWD_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_fwd_tc256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT2_FWD_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attn_bwd_tc256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT2_BWD_SMEM);
   if (e != cudaSuccess) { err = std::string("attention plan: ") + cudaGetErrorString(e); return PM_ERR_CUDA; }
@@ -731,8 +753,14 @@ cudaError_t attn_tc_launch(AttnPlan* plan, const TickArgs& t, bool forward, cuda
     else attn_bwd_tc256_kernel<<<grid, AT2_BWD_THREADS, AT2_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
     return cudaGetLastError();
   }
-  if (forward) attn_fwd_tc_kernel<<<grid, 128, AT_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-  else attn_bwd_tc_kernel<<<grid, AT_BWD_THREADS, AT_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
+  const bool full = t.att_S == AT_S;
+  if (forward) {
+    if (full) attn_fwd_tc_kernel<true><<<grid, 128, AT_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
+    else attn_fwd_tc_kernel<false><<<grid, 128, AT_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
+  } else {
+    if (full) attn_bwd_tc_kernel<true><<<grid, AT_BWD_THREADS, AT_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
+    else attn_bwd_tc_kernel<false><<<grid, AT_BWD_THREADS, AT_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
+  }
   return cudaGetLastError();
 }
 

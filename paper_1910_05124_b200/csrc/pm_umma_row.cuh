@@ -107,6 +107,20 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
   const uint32_t tmem = *tmem_slot;
   const CUtensorMap* lm = maps + ((size_t)p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
 
+  // What the epilogue will need (256 threads, groups of four columns of the rows this CTA owns): addresses come from the
+  // stage tables by dependent loads, so they are formed, and the operands fetched, before the accumulators are awaited.
+  using bf16 = __nv_bfloat16;
+  const int tid = (int)threadIdx.x - 64;
+  const int c4 = tid % (BN / 4) * 4, n = n0 + c4;
+  const uint64_t nx = (uint64_t)M * N;
+  const bf16* aux = nullptr;                                   // skip tensor (forward, residual) or act' stash (dgrad)
+  bf16 *out = nullptr, *zout = nullptr;
+  float* lout = nullptr;
+  int act = PM_ACT_NONE;
+  bool resid = false;
+  float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  uint2 ax[C::kGroups];
+
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
@@ -216,7 +230,29 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
       }
     }
     // ---------------- partial accumulators -> the CTA that finishes their rows ----------------
+    if (MODE == 0) {
+      act = L.act;
+      resid = s.post == POST_RESIDUAL && lvl == s.n_lin - 1;
+      if (n < N) b4 = *reinterpret_cast<const float4*>(fwd_small<bf16>(t, s, d, L.b_off, L.b_soff) + n);
+      if (L.flags & LF_OUT_F32) lout = ws_at<float>(t, t.yout_off) + (uint64_t)(d.tick & 1) * nx;
+      if (L.flags & LF_WRITE_Z) zout = ring_at<bf16>(t, L.z_ring, d.f_slot, nx);
+      if (L.flags & LF_WRITE_Y) {
+        if (!resid) out = y_dest<bf16>(t, p, s, d, lvl);
+        else if (s.emit_memory) out = mem_at<bf16>(t, d.f_mb);
+        else if (p < t.P - 1) out = ring_at<bf16>(t, t.st[p + 1].x_ring, d.f_next_xslot, nx);
+        else out = ws_at<bf16>(t, t.yout_off) + (uint64_t)(d.tick & 1) * nx;
+      }
+      if (resid) aux = ws_at<bf16>(t, s.skip_in) + (uint64_t)d.skip_rslot * nx;
+    } else {
+      out = dx_dest<bf16>(t, p, s, d, lvl);
+      act = dx_fused_act<bf16>(t, p, s, d, lvl, &aux);
+    }
     pdl_wait();
+#pragma unroll
+    for (int g = 0; g < C::kGroups; ++g) {
+      const int m = m0 + rank * C::kRows + (tid + 256 * g) / (BN / 4);
+      ax[g] = (aux && m < M && n < N) ? *reinterpret_cast<const uint2*>(aux + (uint64_t)m * N + n) : make_uint2(0u, 0u);
+    }
     const int q = warp & 3, half = w >> 2;                     // TMEM lane group (32 rows), half of the columns
     bool ready = mbar_wait(bar_acc, 0, abort_flag, status, 64);
     ready = __all_sync(0xffffffffu, ready);
@@ -258,41 +294,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
   }
   if (warp < 2) return;
 
-  // ---------------- epilogue: 256 threads, groups of four columns of the rows this CTA owns ----------------
-  const int tid = threadIdx.x - 64;
-  const int c4 = tid % (BN / 4) * 4, n = n0 + c4;
+  // ---------------- epilogue ----------------
   if (n >= N) return;                                          // widths are multiples of 8
-  using bf16 = __nv_bfloat16;
-  const uint64_t nx = (uint64_t)M * N;
-  const bf16* aux = nullptr;                                   // skip tensor (forward, residual) or act' stash (dgrad)
-  bf16 *out = nullptr, *zout = nullptr;
-  float* lout = nullptr;
-  int act = PM_ACT_NONE;
-  bool resid = false;
-  float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (MODE == 0) {
-    act = L.act;
-    resid = s.post == POST_RESIDUAL && lvl == s.n_lin - 1;
-    b4 = *reinterpret_cast<const float4*>(fwd_small<bf16>(t, s, d, L.b_off, L.b_soff) + n);
-    if (L.flags & LF_OUT_F32) lout = ws_at<float>(t, t.yout_off) + (uint64_t)(d.tick & 1) * nx;
-    if (L.flags & LF_WRITE_Z) zout = ring_at<bf16>(t, L.z_ring, d.f_slot, nx);
-    if (L.flags & LF_WRITE_Y) {
-      if (!resid) out = y_dest<bf16>(t, p, s, d, lvl);
-      else if (s.emit_memory) out = mem_at<bf16>(t, d.f_mb);
-      else if (p < t.P - 1) out = ring_at<bf16>(t, t.st[p + 1].x_ring, d.f_next_xslot, nx);
-      else out = ws_at<bf16>(t, t.yout_off) + (uint64_t)(d.tick & 1) * nx;
-    }
-    if (resid) aux = ws_at<bf16>(t, s.skip_in) + (uint64_t)d.skip_rslot * nx;
-  } else {
-    out = dx_dest<bf16>(t, p, s, d, lvl);
-    act = dx_fused_act<bf16>(t, p, s, d, lvl, &aux);
-  }
-  uint2 ax[C::kGroups];
-#pragma unroll
-  for (int g = 0; g < C::kGroups; ++g) {
-    const int m = m0 + rank * C::kRows + (tid + 256 * g) / (BN / 4);
-    ax[g] = (aux && m < M) ? *reinterpret_cast<const uint2*>(aux + (uint64_t)m * N + n) : make_uint2(0u, 0u);
-  }
 #pragma unroll
   for (int g = 0; g < C::kGroups; ++g) {
     const int rl = (tid + 256 * g) / (BN / 4), m = m0 + rank * C::kRows + rl;
