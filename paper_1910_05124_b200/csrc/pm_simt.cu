@@ -55,7 +55,7 @@ cudaError_t launch_ingest(const TickArgs& t, int dtype, const void* inputs, cons
 // loss = mean over T*out of (y - y*)^2 ;  dy = 2 (y - y*) / (T*out), stored in the activation type.
 // Fixed summation order: each block sums a contiguous chunk (strided per-thread partials, fixed tree),
 // the last block to finish adds the per-block partials in block order.
-constexpr int kLossBlocks = 64, kLossThreads = 256;
+constexpr int kLossBlocks = 96, kLossThreads = 256;     // partial sums and the counter share a 512-byte block of the workspace
 
 template <typename AT>
 __global__ void __launch_bounds__(kLossThreads) mse_loss_kernel(TickArgs t) {
@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kLossThreads) mse_loss_kernel(TickArgs t) {
   const uint64_t chunk = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
   float part = 0.f;
+#pragma unroll 4
   for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     float r = __fsub_rn(to_f<AT>(y[i]), tg[i]);
     part = __fadd_rn(part, __fmul_rn(r, r));
@@ -97,12 +98,17 @@ __global__ void __launch_bounds__(kLossThreads) mse_loss_kernel(TickArgs t) {
     last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last && threadIdx.x < 32) {                     // lane l adds partials l, l + 32, l + 64, then a fixed tree
     __threadfence();
     float sum = 0.f;
-    for (int b = 0; b < (int)gridDim.x; ++b) sum = __fadd_rn(sum, reinterpret_cast<volatile float*>(partial)[b]);
-    ws_ptr<float>(t, t.loss_off)[d.b_mb % t.loss_cap] = sum / (float)n;
-    *counter = 0;                                     // ready for the next tick
+#pragma unroll
+    for (int b = 0; b < kLossBlocks / 32; ++b) sum = __fadd_rn(sum, __ldcg(partial + 32 * b + threadIdx.x));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sum = __fadd_rn(sum, __shfl_xor_sync(0xffffffffu, sum, off));
+    if (threadIdx.x == 0) {
+      ws_ptr<float>(t, t.loss_off)[d.b_mb % t.loss_cap] = sum / (float)n;
+      *counter = 0;                                   // ready for the next tick
+    }
   }
 }
 
@@ -125,7 +131,7 @@ constexpr int kActColsV = 256;                        // columns per block: 8 pe
 constexpr int kColsumGroup = 8;                       // row chunks per block in a launch that only sums columns
 constexpr int kStageGroup = 4;                        // ... and in a launch of one stage
 constexpr int kSmallRows = 512;                       // microbatches of up to this many rows: a block takes all rows of its columns
-constexpr int kSmallCols = 64;
+constexpr int kSmallCols = 32;
 // Row chunks one block of the activation-backward launch covers; its sum is partial row (first chunk / group) of the stage.
 __host__ __device__ inline int act_chunk_group(const TickArgs& t) {
   return t.row_chunks > 1 ? (t.colsum_only ? kColsumGroup : (t.sel_p >= 0 ? kStageGroup : 1)) : 1;
@@ -241,7 +247,7 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
   }
 }
 
-// The same for microbatches of at most kSmallRows rows: a block takes 64 columns of ALL rows (eight columns per lane, four
+// The same for microbatches of at most kSmallRows rows: a block takes 32 columns of ALL rows (eight columns per lane, eight
 // rows per warp and step), so there are no partial sums to finish in a second launch.  What bounds these launches is the
 // number of rows a block walks one after the other and the launches themselves, not the bytes: with 256-column blocks of 32
 // rows and a finishing launch a level of the 32-stage 1024-wide MLP (128 rows) took 17.6 + 12.7 us.
@@ -274,16 +280,16 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if ((L.n_out & 7) == 0) {
-    const int c = c0 + 8 * (lane & 7), r = 4 * warp + (lane >> 3);
+    const int c = c0 + 8 * (lane & 3), r = 8 * warp + (lane >> 2);
     if (c < L.n_out) {
-      if (!has_act) actbwd_rows<AT, PM_ACT_NONE, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
-      else if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
-      else actbwd_rows<AT, PM_ACT_GELU, 32>(dy, z, dz, L.n_out, c, r, t.T, sum);
+      if (!has_act) actbwd_rows<AT, PM_ACT_NONE, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
+      else if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
+      else actbwd_rows<AT, PM_ACT_GELU, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
     }
   } else if (has_act) {                                     // fp32 only: bf16 Linears have widths that are multiples of 8
-    const int c = c0 + (int)(threadIdx.x & 63);
+    const int c = c0 + (int)(threadIdx.x & 31);
     if (c < L.n_out)
-      for (int r = threadIdx.x >> 6; r < t.T; r += 4) {
+      for (int r = threadIdx.x >> 5; r < t.T; r += 8) {
         const uint64_t i = (uint64_t)r * L.n_out + c;
         dz[i] = from_f<AT>(round_as<AT>(__fmul_rn(to_f<AT>(dy[i]), act_grad(to_f<AT>(z[i]), L.act))));
       }
@@ -291,10 +297,11 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
   if (!sums) return;
   __shared__ float red[8][kSmallCols];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {                             // the four rows of the warp, in a fixed order
+  for (int k = 0; k < 8; ++k) {                             // the eight rows of the warp, in a fixed order
+    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 4));
     sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 8));
     sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 16));
-    if (lane < 8) red[warp][8 * lane + k] = sum[k];
+    if (lane < 4) red[warp][8 * lane + k] = sum[k];
   }
   __syncthreads();
   const int cc = c0 + threadIdx.x;

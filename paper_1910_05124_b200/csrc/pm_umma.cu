@@ -2083,13 +2083,13 @@ cudaError_t umma_clear_status(UmmaPlan* plan, cudaStream_t stream) { return cuda
 
 int* umma_status_word(UmmaPlan* plan) { return plan ? plan->d_status : nullptr; }
 
-bool umma_row_dgrad(int T, const LinDev& L) { return row_shape(T, L.n_in, L.n_out, 1).bn != 0; }
+bool umma_row_dgrad(int T, const LinDev& L) { return row_dgrad_shape(T, L.n_in, L.n_out).bn != 0; }
 
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream) {
   if (t.sel_p >= 0 && mode != 2) {
     const LinDev& L = plan->st[t.sel_p].lin[lvl];
     const int N = mode == 0 ? L.n_out : L.n_in;
-    const RowShape r = row_shape(t.T, N, mode == 0 ? L.n_in : L.n_out, 1);
+    const RowShape r = mode == 0 ? row_shape(t.T, N, L.n_in, 1) : row_dgrad_shape(t.T, N, L.n_out);
     if (r.bn != 0)
       return mode == 0 ? row_launch<0>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
              : mode == 1 ? row_launch<1>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)

@@ -359,6 +359,17 @@ static cudaError_t row_launch_t(const TickArgs& t, const CUtensorMap* maps, int 
   return cudaLaunchKernelEx(&cfg, umma_row_kernel<MODE, BN, S>, t, maps, lvl, tiles_n, status);
 }
 
+// dgrad: every row tile forms its operand again, four 64 x 32 pieces per round trip of its loads, so many row tiles of a deep
+// reduction belong to the CTA-pair kernels where those apply (256 rows and columns).  An update of a 3-layer encoder at width
+// 512 takes 1202 us with this kernel everywhere and 1022 without it at 4096 rows (K = 512 to 2048, 32 row tiles); at 1024
+// rows 680 with it and 702 without.
+inline RowShape row_dgrad_shape(int T, int N, int K) {
+  RowShape r = row_shape(T, N, K, 1);
+  const int items = ((K + ROW_K - 1) / ROW_K + r.split - 1) / r.split * (r.bn / 32);
+  if (T >= 256 && N >= 256 && items * ((T + ROW_M - 1) / ROW_M) > 200) r.bn = 0;
+  return r;
+}
+
 template <int MODE>
 static cudaError_t row_set_limits() {
   cudaError_t e = cudaSuccess;
