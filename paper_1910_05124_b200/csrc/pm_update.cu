@@ -206,103 +206,93 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
               const StageDyn* __restrict__ dyn, int64_t* __restrict__ nupd, int n_stages, uint64_t total_vec4,
               float beta1, float beta2, float eps, uint64_t first_vec4, const uint32_t* __restrict__ skip_b64, const uint32_t* __restrict__ skip_e64,
               const float* __restrict__ gsrc) {
-  extern __shared__ uint32_t sm_bounds[];           // [n_stages] begins, then [n_stages] ends, then the skipped ranges' begins and ends
-  uint32_t* sb = sm_bounds;
-  uint32_t* se = sm_bounds + n_stages;
   // ranges (one per stage, in 64-element groups) that another kernel has updated already: the Linear matrices, when the
   // weight-gradient GEMM applies the update in its epilogue
-  uint32_t* kb = sm_bounds + 2 * n_stages;
-  uint32_t* ke = sm_bounds + 3 * n_stages;
   const bool skip = skip_b64 != nullptr;
-  for (int i = threadIdx.x; i < n_stages; i += blockDim.x) {
-    sb[i] = begin64[i]; se[i] = end64[i];
-    kb[i] = skip ? skip_b64[i] : 0u; ke[i] = skip ? skip_e64[i] : 0u;
-  }
-  __syncthreads();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
-  const uint64_t stride = (uint64_t)gridDim.x * kUpdThreads * kUpdUnroll;
-  for (uint64_t base = first_vec4 + (uint64_t)blockIdx.x * kUpdThreads * kUpdUnroll; base < total_vec4; base += stride) {
-    if (skip) {
-      // the whole span of this block lies inside a skipped range (and past the stage's first group): nothing to do
-      const uint32_t g0 = (uint32_t)(base >> 4), g1 = (uint32_t)((base + (uint64_t)kUpdThreads * kUpdUnroll - 1) >> 4);
-      int lo = 0, hi = n_stages - 1;
-      while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sb[mid] <= g0) lo = mid; else hi = mid - 1; }
-      if (kb[lo] <= g0 && g1 < ke[lo] && g0 > sb[lo]) continue;
-    }
-    uint64_t v[kUpdUnroll];
-    int stage[kUpdUnroll];
-    UpdScalars sc[kUpdUnroll];
-    float4 g[kUpdUnroll], w[kUpdUnroll], m[kUpdUnroll], dl[kUpdUnroll], s[kUpdUnroll];
+  const uint64_t base = first_vec4 + (uint64_t)blockIdx.x * kUpdThreads * kUpdUnroll;
+  // the stage of the block's first group: the largest i with begin64[i] <= g0 (every thread searches, on the same addresses)
+  const uint32_t g0 = (uint32_t)(base >> 4);
+  int lo0 = 0, hi = n_stages - 1;
+  while (lo0 < hi) { const int mid = (lo0 + hi + 1) >> 1; if (__ldg(begin64 + mid) <= g0) lo0 = mid; else hi = mid - 1; }
+  if (skip) {
+    // the whole span of this block lies inside a skipped range (and past the stage's first group): nothing to do
+    const uint32_t g1 = (uint32_t)((base + (uint64_t)kUpdThreads * kUpdUnroll - 1) >> 4);
+    if (skip_b64[lo0] <= g0 && g1 < skip_e64[lo0] && g0 > begin64[lo0]) return;
+  }
+  uint64_t v[kUpdUnroll];
+  int stage[kUpdUnroll];
+  UpdScalars sc[kUpdUnroll];
+  float4 g[kUpdUnroll], w[kUpdUnroll], m[kUpdUnroll], dl[kUpdUnroll], s[kUpdUnroll];
 #pragma unroll
-    for (int u = 0; u < kUpdUnroll; ++u) {
-      v[u] = base + (uint64_t)u * kUpdThreads + threadIdx.x;
-      stage[u] = -1;
-      if (v[u] < total_vec4) {
-        uint32_t e64 = (uint32_t)(v[u] >> 4);
-        int lo = 0, hi = n_stages - 1;               // largest i with sb[i] <= e64
-        while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (sb[mid] <= e64) lo = mid; else hi = mid - 1; }
-        if (sb[lo] <= e64 && e64 < se[lo] && dyn[lo].active_update) {
-          if (skip && kb[lo] <= e64 && e64 < ke[lo]) {                     // updated elsewhere; the stage's counter is still kept here
-            if (e64 == sb[lo] && (v[u] & 15) == 0) nupd[lo] += 1;
-          } else stage[u] = lo;
-        }
-      }
-      if (stage[u] >= 0) {
-        const uint64_t e = v[u] * 4;
-        const StageDyn& d = dyn[stage[u]];
-        g[u] = ld_stream(gsrc + (d.g_shift + (int64_t)e));
-        w[u] = ld_stream(a.w + e);
-        m[u] = ld_stream(a.m + e);
-        sc[u].alpha = d.alpha; sc[u].gamma = d.gamma; sc[u].omg = d.one_minus_gamma;
-        sc[u].bc1 = d.bc1; sc[u].bc2 = d.bc2; sc[u].use_delta = d.use_delta;
-        if (LP != 0) { sc[u].lp_shift = d.lp_shift; sc[u].rc_shift = d.rc_uslot >= 0 ? d.rc_shift : -1; sc[u].rc_gap = d.rc_gap; }
-        if (sc[u].use_delta || (LP != 0 && sc[u].rc_shift >= 0)) dl[u] = ld_stream(a.delta + e);
-        if (OPT == PM_ADAM) s[u] = ld_stream(a.s + e);
+  for (int u = 0; u < kUpdUnroll; ++u) {
+    v[u] = base + (uint64_t)u * kUpdThreads + threadIdx.x;
+    stage[u] = -1;
+    if (v[u] < total_vec4) {
+      const uint32_t e64 = (uint32_t)(v[u] >> 4);
+      int lo = lo0;
+      while (lo + 1 < n_stages && __ldg(begin64 + lo + 1) <= e64) ++lo;      // a block spans 32 groups: rarely more than one stage on
+      if (__ldg(begin64 + lo) <= e64 && e64 < __ldg(end64 + lo) && dyn[lo].active_update) {
+        if (skip && skip_b64[lo] <= e64 && e64 < skip_e64[lo]) {             // updated elsewhere; the stage's counter is still kept here
+          if (e64 == begin64[lo] && (v[u] & 15) == 0) nupd[lo] += 1;
+        } else stage[u] = lo;
       }
     }
-#pragma unroll
-    for (int u = 0; u < kUpdUnroll; ++u) {
-      if (stage[u] < 0) continue;
+    if (stage[u] >= 0) {
       const uint64_t e = v[u] * 4;
-      float4 wn;
-      wn.x = upd_one<OPT>(g[u].x, w[u].x, m[u].x, s[u].x, dl[u].x, sc[u], beta1, beta2, omb1, omb2, eps);
-      wn.y = upd_one<OPT>(g[u].y, w[u].y, m[u].y, s[u].y, dl[u].y, sc[u], beta1, beta2, omb1, omb2, eps);
-      wn.z = upd_one<OPT>(g[u].z, w[u].z, m[u].z, s[u].z, dl[u].z, sc[u], beta1, beta2, omb1, omb2, eps);
-      wn.w = upd_one<OPT>(g[u].w, w[u].w, m[u].w, s[u].w, dl[u].w, sc[u], beta1, beta2, omb1, omb2, eps);
-      st_stream(a.w + e, wn);
-      st_stream(a.m + e, m[u]);
-      if (OPT == PM_ADAM) st_stream(a.s + e, s[u]);
-      if (sc[u].use_delta) st_stream(a.delta + e, dl[u]);
+      const StageDyn& d = dyn[stage[u]];
+      g[u] = ld_stream(gsrc + (d.g_shift + (int64_t)e));
+      w[u] = ld_stream(a.w + e);
+      m[u] = ld_stream(a.m + e);
+      sc[u].alpha = d.alpha; sc[u].gamma = d.gamma; sc[u].omg = d.one_minus_gamma;
+      sc[u].bc1 = d.bc1; sc[u].bc2 = d.bc2; sc[u].use_delta = d.use_delta;
+      if (LP != 0) { sc[u].lp_shift = d.lp_shift; sc[u].rc_shift = d.rc_uslot >= 0 ? d.rc_shift : -1; sc[u].rc_gap = d.rc_gap; }
+      if (sc[u].use_delta || (LP != 0 && sc[u].rc_shift >= 0)) dl[u] = ld_stream(a.delta + e);
+      if (OPT == PM_ADAM) s[u] = ld_stream(a.s + e);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kUpdUnroll; ++u) {
+    if (stage[u] < 0) continue;
+    const uint64_t e = v[u] * 4;
+    float4 wn;
+    wn.x = upd_one<OPT>(g[u].x, w[u].x, m[u].x, s[u].x, dl[u].x, sc[u], beta1, beta2, omb1, omb2, eps);
+    wn.y = upd_one<OPT>(g[u].y, w[u].y, m[u].y, s[u].y, dl[u].y, sc[u], beta1, beta2, omb1, omb2, eps);
+    wn.z = upd_one<OPT>(g[u].z, w[u].z, m[u].z, s[u].z, dl[u].z, sc[u], beta1, beta2, omb1, omb2, eps);
+    wn.w = upd_one<OPT>(g[u].w, w[u].w, m[u].w, s[u].w, dl[u].w, sc[u], beta1, beta2, omb1, omb2, eps);
+    st_stream(a.w + e, wn);
+    st_stream(a.m + e, m[u]);
+    if (OPT == PM_ADAM) st_stream(a.s + e, s[u]);
+    if (sc[u].use_delta) st_stream(a.delta + e, dl[u]);
+    if (LP == 1) {
+      __nv_bfloat162 lo2 = __floats2bfloat162_rn(wn.x, wn.y);
+      __nv_bfloat162 hi2 = __floats2bfloat162_rn(wn.z, wn.w);
+      uint2 packed;
+      packed.x = *reinterpret_cast<uint32_t*>(&lo2);
+      packed.y = *reinterpret_cast<uint32_t*>(&hi2);
+      *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(lp_base) + (sc[u].lp_shift + (int64_t)e)) = packed;   // re-read by a later forward: default caching
+    } else if (LP == 2) {
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(lp_base) + (sc[u].lp_shift + (int64_t)e)) = wn;
+    }
+    if (LP != 0 && sc[u].rc_shift >= 0) {
+      // T2 for recompute (Appendix D): the weights a recomputation tau_recomp updates from now reads, corrected with the
+      // accumulator as it stands with this version: w' - (tau_fwd - tau_recomp) * delta'
+      const float gp = sc[u].rc_gap;
+      float4 r;
+      r.x = __fsub_rn(wn.x, __fmul_rn(gp, dl[u].x)); r.y = __fsub_rn(wn.y, __fmul_rn(gp, dl[u].y));
+      r.z = __fsub_rn(wn.z, __fmul_rn(gp, dl[u].z)); r.w = __fsub_rn(wn.w, __fmul_rn(gp, dl[u].w));
       if (LP == 1) {
-        __nv_bfloat162 lo2 = __floats2bfloat162_rn(wn.x, wn.y);
-        __nv_bfloat162 hi2 = __floats2bfloat162_rn(wn.z, wn.w);
+        __nv_bfloat162 lo2 = __floats2bfloat162_rn(r.x, r.y);
+        __nv_bfloat162 hi2 = __floats2bfloat162_rn(r.z, r.w);
         uint2 packed;
         packed.x = *reinterpret_cast<uint32_t*>(&lo2);
         packed.y = *reinterpret_cast<uint32_t*>(&hi2);
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(lp_base) + (sc[u].lp_shift + (int64_t)e)) = packed;   // re-read by a later forward: default caching
-      } else if (LP == 2) {
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(lp_base) + (sc[u].lp_shift + (int64_t)e)) = wn;
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(lp_base) + (sc[u].rc_shift + (int64_t)e)) = packed;
+      } else {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(lp_base) + (sc[u].rc_shift + (int64_t)e)) = r;
       }
-      if (LP != 0 && sc[u].rc_shift >= 0) {
-        // T2 for recompute (Appendix D): the weights a recomputation tau_recomp updates from now reads, corrected with the
-        // accumulator as it stands with this version: w' - (tau_fwd - tau_recomp) * delta'
-        const float gp = sc[u].rc_gap;
-        float4 r;
-        r.x = __fsub_rn(wn.x, __fmul_rn(gp, dl[u].x)); r.y = __fsub_rn(wn.y, __fmul_rn(gp, dl[u].y));
-        r.z = __fsub_rn(wn.z, __fmul_rn(gp, dl[u].z)); r.w = __fsub_rn(wn.w, __fmul_rn(gp, dl[u].w));
-        if (LP == 1) {
-          __nv_bfloat162 lo2 = __floats2bfloat162_rn(r.x, r.y);
-          __nv_bfloat162 hi2 = __floats2bfloat162_rn(r.z, r.w);
-          uint2 packed;
-          packed.x = *reinterpret_cast<uint32_t*>(&lo2);
-          packed.y = *reinterpret_cast<uint32_t*>(&hi2);
-          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(lp_base) + (sc[u].rc_shift + (int64_t)e)) = packed;
-        } else {
-          *reinterpret_cast<float4*>(reinterpret_cast<float*>(lp_base) + (sc[u].rc_shift + (int64_t)e)) = r;
-        }
-      }
-      if ((uint32_t)(v[u] >> 4) == sb[stage[u]] && (v[u] & 15) == 0) nupd[stage[u]] += 1;
     }
+    if ((uint32_t)(v[u] >> 4) == __ldg(begin64 + stage[u]) && (v[u] & 15) == 0) nupd[stage[u]] += 1;
   }
 }
 
@@ -314,18 +304,12 @@ cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* 
   uint64_t total_vec4 = total64 * 16;
   const uint64_t first_vec4 = first64 * 16;
   uint64_t per_block = (uint64_t)kUpdThreads * kUpdUnroll;
-  uint64_t need = (total_vec4 - first_vec4 + per_block - 1) / per_block;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  uint64_t cap = (uint64_t)sms * 8;                 // whole waves of resident blocks
-  int blocks = (int)(need < cap ? need : cap);
-  size_t smem = sizeof(uint32_t) * 4 * (size_t)n_stages;
+  const unsigned blocks = (unsigned)((total_vec4 - first_vec4 + per_block - 1) / per_block);   // 2048 elements per block: 2^31 blocks are 4e12 elements
   // the operand-type copy: the w_lp arena (bfloat16) unless the caller names a version ring and its element size
   if (lp_base == nullptr) { lp_base = a.w_lp; lp_elem = 2; }
   if (gsrc == nullptr) gsrc = a.grad;
   const int lp = lp_base == nullptr ? 0 : (lp_elem == 4 ? 2 : 1);
-#define PM_UPD(OPT, LP) update_kernel<OPT, LP><<<blocks, kUpdThreads, smem, stream>>>(a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc)
+#define PM_UPD(OPT, LP) update_kernel<OPT, LP><<<blocks, kUpdThreads, 0, stream>>>(a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc)
   if (optimizer == PM_SGDM) { if (lp == 0) PM_UPD(PM_SGDM, 0); else if (lp == 1) PM_UPD(PM_SGDM, 1); else PM_UPD(PM_SGDM, 2); }
   else { if (lp == 0) PM_UPD(PM_ADAM, 0); else if (lp == 1) PM_UPD(PM_ADAM, 1); else PM_UPD(PM_ADAM, 2); }
 #undef PM_UPD
