@@ -7,6 +7,25 @@
 
 namespace pm {
 
+// Programmatic dependent launch: a kernel launched with pdl may start once every block of its predecessor has triggered (or
+// ended); pdl_wait returns when that predecessor has ended and its writes are visible, and at once in a kernel launched plainly.
+// A kernel that may be launched this way calls pdl_wait in every block before it ends, so that "its predecessor has ended"
+// holds for everything before it, too.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... K, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool pdl, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
 enum { PRE_NONE = 0, PRE_EMBED = 1, PRE_LN = 2 };
 enum { POST_NONE = 0, POST_ATTENTION = 1, POST_SKIP_OUT = 2, POST_RESIDUAL = 3, POST_CROSS_ATTENTION = 4 };
 // LF_ACT_FROM_Y: a ReLU whose pre-activation is not stashed: the backward takes the mask from the stashed output

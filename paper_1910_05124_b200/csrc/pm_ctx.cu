@@ -976,12 +976,9 @@ static pm_status mb_forward(pm_ctx* ctx, const void* inputs, const void* targets
   const int64_t mb = ctx->n_fed;
   pm_status s;
   const bool stoch = ctx->L.stochastic > 0;
-  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_schedule_mb((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn),
-                                                            ctx->hp, mb, ctx->stream,
-                                                            stoch ? (const int32_t*)(ctx->ws + ctx->L.off_delays) : nullptr,
-                                                            stoch ? (const int64_t*)(ctx->ws + ctx->L.off_nupd) : nullptr), "schedule"));
-  if (s != PM_OK) return s;
-  s = TIMED(PM_PROF_INGEST, check(ctx, launch_ingest(ctx->ta, dt, inputs, (const float*)targets, mb, ctx->stream), "ingest"));
+  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn),
+                                                      ctx->hp, 0, 0, true, stoch ? (const int32_t*)(ctx->ws + ctx->L.off_delays) : nullptr,
+                                                      (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, dt, inputs, targets, mb, ctx->stream), "schedule and ingest"));
   if (s != PM_OK) return s;
   s = run_phase(ctx, ctx->g_fwd, [&]() -> pm_status {
     pm_status s;
@@ -1187,13 +1184,9 @@ pm_status pm_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
     if (ew != cudaSuccess) return cuda_fail(ctx, ew, "forward stream");
     ctx->fwd_pending = false;
   }
-  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_schedule((const StageSched*)(ctx->ws + ctx->L.off_sched), (const int64_t*)(ctx->ws + ctx->L.off_nupd),
-                                 (StageDyn*)(ctx->ws + ctx->L.off_dyn), ctx->hp, ctx->tick, ctx->n_fed, -1, ctx->stream), "schedule"));
+  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn), ctx->hp, ctx->tick, ctx->n_fed, false, nullptr,
+                                                      (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, dt, inputs, targets, mb, ctx->stream), "schedule and ingest"));
   if (s != PM_OK) return s;
-  if (inputs) {
-    s = TIMED(PM_PROF_INGEST, check(ctx, launch_ingest(ctx->ta, dt, inputs, (const float*)targets, mb, ctx->stream), "ingest"));
-    if (s != PM_OK) return s;
-  }
   if (sparse_ticks(ctx)) {
     if (any_stage_active(ctx, 0, ctx->cfg.n_stages - 1) && (s = sparse_forward_phase(ctx)) != PM_OK) return s;
     ctx->phase = 1;
@@ -1483,15 +1476,11 @@ pm_status pm_update_flat(const pm_arenas* arenas, const uint64_t* stage_offsets,
   const uint64_t need = pm_update_flat_workspace_bytes(n_stages);
   if (!workspace || workspace_bytes < need) return fail(nullptr, PM_ERR_NOMEM, "workspace too small: need " + std::to_string(need) + " bytes");
   const uint64_t P = (uint64_t)n_stages;
-  thread_local std::vector<char> host;             // staging for the stage table: no allocation after the first call of a thread
-  host.assign(need, 0);
-  uint64_t off_sched = 0, off_dyn = align_up(sizeof(StageSched) * P, 256);
-  uint64_t off_nupd = align_up(off_dyn + sizeof(StageDyn) * P, 256);
-  uint64_t off_b = align_up(off_nupd + sizeof(int64_t) * P, 256);
-  uint64_t off_e = align_up(off_b + sizeof(uint32_t) * P, 256);
-  StageSched* sc = (StageSched*)(host.data() + off_sched);
-  uint32_t* b64 = (uint32_t*)(host.data() + off_b);
-  uint32_t* e64 = (uint32_t*)(host.data() + off_e);
+  const uint64_t off_dyn = align_up(sizeof(StageSched) * P, 256);
+  const uint64_t off_nupd = align_up(off_dyn + sizeof(StageDyn) * P, 256);
+  const uint64_t off_b = align_up(off_nupd + sizeof(int64_t) * P, 256);
+  const uint64_t off_e = align_up(off_b + sizeof(uint32_t) * P, 256);
+  FlatStage st[PM_MAX_STAGES];
   uint64_t prev_end = 0;
   for (int i = 0; i < n_stages; ++i) {
     if (stage_offsets[i] % PM_ALIGN_ELEMS) return fail(nullptr, PM_ERR_INVALID_ARG, "stage offsets must be multiples of 64 elements");
@@ -1502,14 +1491,10 @@ pm_status pm_update_flat(const pm_arenas* arenas, const uint64_t* stage_offsets,
     uint64_t end = align_up(stage_offsets[i] + stage_counts[i], PM_ALIGN_ELEMS);
     if (end > arenas->count) return fail(nullptr, PM_ERR_NOMEM, "stage slice exceeds the arenas");
     prev_end = end;
-    sc[i] = StageSched{tau_fwd[i], tau_fwd[i] - tau_bkwd[i], 1, 1, 0, 0};
-    b64[i] = (uint32_t)(stage_offsets[i] / 64);
-    e64[i] = (uint32_t)(end / 64);
+    st[i] = FlatStage{(uint32_t)(stage_offsets[i] / 64), (uint32_t)(end / 64), tau_fwd[i], tau_fwd[i] - tau_bkwd[i]};
   }
-  cudaStream_t st = (cudaStream_t)stream;
+  cudaStream_t cs = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  cudaError_t e = cudaMemcpyAsync(ws, host.data(), need, cudaMemcpyHostToDevice, st);   // pageable source: staged before the call returns
-  if (e != cudaSuccess) return cuda_fail(nullptr, e, "stage table upload");
   HyperDev hp{};
   hp.optimizer = cfg->optimizer; hp.t1 = cfg->t1_enable; hp.t2 = cfg->t2_enable; hp.n_stages = n_stages;
   hp.K = cfg->t1_K > 0 ? cfg->t1_K : 1; hp.D = cfg->t2_D;
@@ -1517,11 +1502,11 @@ pm_status pm_update_flat(const pm_arenas* arenas, const uint64_t* stage_offsets,
   hp.alpha_tab = nullptr; hp.alpha_len = 0;
   hp.beta1 = cfg->beta1; hp.beta2 = cfg->beta2; hp.eps = cfg->eps;
   hp.warm = 0; hp.period = 1;
-  e = launch_schedule((const StageSched*)(ws + off_sched), (const int64_t*)(ws + off_nupd), (StageDyn*)(ws + off_dyn), hp, 0, 0, k, st);
+  cudaError_t e = launch_flat_table(st, hp, k, (uint32_t*)(ws + off_b), (uint32_t*)(ws + off_e), (StageDyn*)(ws + off_dyn), (int64_t*)(ws + off_nupd), cs);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "schedule");
   ArenasDev a{arenas->w, arenas->m, arenas->s, arenas->delta, arenas->grad, (__nv_bfloat16*)arenas->w_lp, arenas->count};
-  e = launch_update(a, (const uint32_t*)(ws + off_b), (const uint32_t*)(ws + off_e), (const StageDyn*)(ws + off_dyn),
-                    (int64_t*)(ws + off_nupd), n_stages, e64[n_stages - 1], cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, st);
+  e = launch_update(a, (const uint32_t*)(ws + off_b), (const uint32_t*)(ws + off_e), (const StageDyn*)(ws + off_dyn), (int64_t*)(ws + off_nupd), n_stages,
+                    st[n_stages - 1].end64, cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, cs, nullptr, 0, 0, nullptr, nullptr, nullptr, true);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "update");
   return PM_OK;
 }

@@ -1,4 +1,4 @@
-// Element-wise tick kernels (ingest, loss, activation backward) and the fp32 SIMT grouped GEMMs.
+// Element-wise tick kernels (loss, activation backward) and the fp32 SIMT grouped GEMMs.
 //
 // Every kernel is "grouped": blockIdx.z (or .y) selects the stage, the per-tick table says
 // whether that stage is active and which ring slots it touches.  Within a tick the stages
@@ -11,45 +11,6 @@ template <typename AT> __device__ __forceinline__ AT* ring_ptr(const TickArgs& t
   return ring_at<AT>(t, off, slot, slot_elems);
 }
 template <typename AT> __device__ __forceinline__ AT* ws_ptr(const TickArgs& t, uint64_t off) { return ws_at<AT>(t, off); }
-
-// ---- ingest -----------------------------------------------------------------------------------
-// MLP: inputs [T, n_in] (activation type) -> stage 1's input ring slot; targets [T, n_out] float -> target ring.
-// Encoder: token ids [T] int32 -> stage 1's id ring slot; target ids [T] int32 -> target ring.
-template <typename AT>
-__global__ void ingest_kernel(TickArgs t, const void* __restrict__ inputs, const void* __restrict__ targets, int64_t mb) {
-  const StageDev& s0 = t.st[0];
-  const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
-  if (s0.pre == PRE_EMBED) {
-    int32_t* idst = ring_ptr<int32_t>(t, s0.ids_ring, (int)(mb % s0.ids_depth), (uint64_t)t.T);
-    for (uint64_t i = gid; i < (uint64_t)t.T; i += stride) idst[i] = reinterpret_cast<const int32_t*>(inputs)[i];
-    if (t.n_streams > 1) {                                    // second token stream -> the stage that embeds it
-      const StageDev& s1 = t.st[t.second_embed_stage];
-      int32_t* d1 = ring_ptr<int32_t>(t, s1.ids_ring, (int)(mb % s1.ids_depth), (uint64_t)t.T);
-      for (uint64_t i = gid; i < (uint64_t)t.T; i += stride) d1[i] = reinterpret_cast<const int32_t*>(inputs)[(uint64_t)t.T + i];
-    }
-  } else {
-    const uint64_t n_x = (uint64_t)t.T * t.n_in_first;
-    AT* xdst = ring_ptr<AT>(t, s0.x_ring, (int)(mb % s0.xdepth), n_x);
-    for (uint64_t i = gid; i < n_x; i += stride) xdst[i] = reinterpret_cast<const AT*>(inputs)[i];
-  }
-  if (t.loss_kind == PM_LOSS_CE) {
-    int32_t* tdst = ws_ptr<int32_t>(t, t.tgt_off) + (uint64_t)(mb % (t.P + 1)) * t.T;
-    for (uint64_t i = gid; i < (uint64_t)t.T; i += stride) tdst[i] = reinterpret_cast<const int32_t*>(targets)[i];
-  } else {
-    const uint64_t n_t = (uint64_t)t.T * t.n_out_last;
-    float* tdst = ws_ptr<float>(t, t.tgt_off) + (uint64_t)(mb % (t.P + 1)) * n_t;
-    for (uint64_t i = gid; i < n_t; i += stride) tdst[i] = reinterpret_cast<const float*>(targets)[i];
-  }
-}
-
-cudaError_t launch_ingest(const TickArgs& t, int dtype, const void* inputs, const float* targets, int64_t mb, cudaStream_t stream) {
-  uint64_t n = (uint64_t)t.T * (t.n_in_first > t.n_out_last ? t.n_in_first : t.n_out_last);
-  int blocks = (int)((n + 255) / 256);
-  if (blocks > 1184) blocks = 1184;
-  if (dtype == PM_F32) ingest_kernel<float><<<blocks, 256, 0, stream>>>(t, inputs, targets, mb);
-  else ingest_kernel<__nv_bfloat16><<<blocks, 256, 0, stream>>>(t, inputs, targets, mb);
-  return cudaGetLastError();
-}
 
 // ---- MSE loss at the last stage ------------------------------------------------------------------
 // loss = mean over T*out of (y - y*)^2 ;  dy = 2 (y - y*) / (T*out), stored in the activation type.

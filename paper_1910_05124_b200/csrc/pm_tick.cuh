@@ -180,9 +180,6 @@ template <typename AT> __device__ __forceinline__ AT* y_dest(const TickArgs& t, 
   return ws_at<AT>(t, t.yout_off) + (uint64_t)(d.tick & 1) * n;
 }
 
-// inputs/targets -> stage 1's input ring slot and the target ring (activation type AT = float | bf16).
-cudaError_t launch_ingest(const TickArgs& t, int dtype, const void* inputs, const float* targets, int64_t mb,
-                          cudaStream_t stream);
 // MSE loss of the microbatch whose backward starts this tick, and dL/dy into the last stage's mailbox.
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream);
 // dz = dy * act'(z) and db = column sums, level `lvl` of every stage that runs backward this tick.

@@ -14,6 +14,7 @@
 //          w' = w - (alpha*(m'/bc1)) / (sqrt(s'/bc2) + eps)
 //   T2 (Section 3.2):      delta' = gamma*delta + (1-gamma)*(w' - w)
 #include "pm_update.cuh"
+#include "pm_tick.cuh"
 #include "pm_update_math.cuh"
 
 namespace pm {
@@ -26,77 +27,100 @@ namespace pm {
 // float once.
 // Per-stage state of one tick: forward microbatch a and backward microbatch b (-1: idle), `ver` updates applied to the
 // stage so far, the version `fver` its forward reads; k >= 0 activates the update with that index.
+// non-negative a modulo d, without the 64-bit division while a fits 32 bits
+__device__ __forceinline__ int32_t slot_of(int64_t a, int32_t d) {
+  return ((uint64_t)a >> 32) == 0 ? (int32_t)((uint32_t)a % (uint32_t)d) : (int32_t)(a % d);
+}
+
+// The launch is as long as one thread's chain of double-precision powers, so four neighbouring lanes share a stage: lane r of
+// the quad evaluates scalar r (step size, T2 decay, Adam's two bias corrections) of update index kk, and all four are
+// handed round.  Every lane of the warp must come here.
+struct DynScalars { float alpha, gamma, bc1, bc2; };
+__device__ __forceinline__ DynScalars quad_scalars(const StageSched& s, const HyperDev& hp, int64_t kk) {
+  const int lane = threadIdx.x & 31, r = lane & 3;
+  // warm-up microbatches (Section 4) are synchronous: standard step size, no correction, delta left alone; the T1
+  // annealing counts from the first PipeMare step
+  const bool sync = kk < hp.warm;
+  float v = r == 0 ? 0.f : (r == 1 ? 0.f : 1.f);
+  if (kk >= 0) {
+    // v = scale * base^expo (alpha: base step / tau^p), 1 - base^expo (bias corrections) or base^expo (gamma): one call of pow
+    double base = 1.0, expo = 0.0, step = hp.alpha_const;
+    if (r == 0) {
+      if (hp.alpha_tab != nullptr) step = hp.alpha_tab[kk < hp.alpha_len ? kk : hp.alpha_len - 1];
+      if (hp.t1 && !sync) {
+        const double q = (double)(kk - hp.warm) / (double)hp.K;
+        base = (double)(s.tau_f > 1 ? s.tau_f : 1);
+        expo = 1.0 - (q < 1.0 ? q : 1.0);
+      }
+    } else if (r == 1) {
+      if (hp.t2 && s.gap > 0 && !sync) { base = hp.D; expo = 1.0 / (double)s.gap; }
+    } else {
+      base = r == 2 ? (double)hp.beta1 : (double)hp.beta2;
+      expo = (double)(kk + 1);
+    }
+    const double pw = pow(base, expo);
+    if (r == 0) v = (float)((hp.t1 && !sync) ? step / pw : step);
+    else if (r == 1) v = (hp.t2 && s.gap > 0 && !sync) ? (float)pw : 0.f;
+    else v = hp.optimizer == PM_ADAM ? (float)(1.0 - pw) : 1.f;
+  }
+  DynScalars o;
+  o.alpha = __shfl_sync(0xffffffffu, v, lane & ~3);
+  o.gamma = __shfl_sync(0xffffffffu, v, (lane & ~3) + 1);
+  o.bc1 = __shfl_sync(0xffffffffu, v, (lane & ~3) + 2);
+  o.bc2 = __shfl_sync(0xffffffffu, v, (lane & ~3) + 3);
+  return o;
+}
+
+// kb: the update index the microbatch in backward belongs to (one microbatch per update: itself)
 __device__ StageDyn make_dyn(const StageSched& s, const HyperDev& hp, int64_t tick, int64_t a, int64_t b, int64_t k,
-                             int64_t ver, int64_t fver, bool slots, int64_t kb = -2) {
+                             int64_t ver, int64_t fver, bool slots, int64_t kb) {
   StageDyn d;
   d.tick = tick;
   d.accum = 0; d._pad2 = 0;
   d.rc_uslot = -1; d.rc_shift = 0; d.r_ver = fver; d.rc_gap = 0.f; d.g_shift = 0;
-  if (kb == -2) kb = b;                               // update index the microbatch in backward belongs to (N = 1: itself)
   const bool fa = a >= 0, ba = b >= 0;
   d.f_mb = a; d.b_mb = b; d.k = k;
-  d.f_slot = (fa && slots) ? (int32_t)(a % s.depth) : 0;
-  d.f_xslot = (fa && slots) ? (int32_t)(a % s.xdepth) : 0;
-  d.f_next_xslot = (fa && slots && s.next_xdepth > 0) ? (int32_t)(a % s.next_xdepth) : 0;
-  d.b_slot = (ba && slots) ? (int32_t)(b % s.depth) : 0;
-  d.b_xslot = (ba && slots) ? (int32_t)(b % s.xdepth) : 0;
-  d.gin_rslot = s.gin_depth > 0 ? (int32_t)((tick + s.gin_depth - 1) % s.gin_depth) : 0;
-  d.prev_wslot = s.prev_gin_depth > 0 ? (int32_t)(tick % s.prev_gin_depth) : 0;
-  d.gmem_slot = (s.gmem_depth > 0 && ba) ? (int32_t)(b % s.gmem_depth) : 0;
-  d.skip_wslot = s.skip_dst_depth > 0 ? (int32_t)(tick % s.skip_dst_depth) : 0;
-  d.skip_rslot = s.skip_depth > 0 ? (int32_t)((tick + 1) % s.skip_depth) : 0;
-  d.b_next_xslot = (ba && slots && s.next_xdepth > 0) ? (int32_t)(b % s.next_xdepth) : 0;
+  d.f_slot = (fa && slots) ? slot_of(a, s.depth) : 0;
+  d.f_xslot = (fa && slots) ? slot_of(a, s.xdepth) : 0;
+  d.f_next_xslot = (fa && slots && s.next_xdepth > 0) ? slot_of(a, s.next_xdepth) : 0;
+  d.b_slot = (ba && slots) ? slot_of(b, s.depth) : 0;
+  d.b_xslot = (ba && slots) ? slot_of(b, s.xdepth) : 0;
+  d.gin_rslot = s.gin_depth > 0 ? slot_of(tick + s.gin_depth - 1, s.gin_depth) : 0;
+  d.prev_wslot = s.prev_gin_depth > 0 ? slot_of(tick, s.prev_gin_depth) : 0;
+  d.gmem_slot = (s.gmem_depth > 0 && ba) ? slot_of(b, s.gmem_depth) : 0;
+  d.skip_wslot = s.skip_dst_depth > 0 ? slot_of(tick, s.skip_dst_depth) : 0;
+  d.skip_rslot = s.skip_depth > 0 ? slot_of(tick + 1, s.skip_depth) : 0;
+  d.b_next_xslot = (ba && slots && s.next_xdepth > 0) ? slot_of(b, s.next_xdepth) : 0;
   d.f_ver = fver;
   d.b_ver = ver;
   // version rings (microbatch-major order): version v sits in slot v % vdepth
-  d.f_vslot = s.vdepth > 1 ? (int32_t)(fver % s.vdepth) : 0;
-  d.u_vslot = s.vdepth > 1 ? (int32_t)((ver + 1) % s.vdepth) : 0;
+  d.f_vslot = s.vdepth > 1 ? slot_of(fver, s.vdepth) : 0;
+  d.u_vslot = s.vdepth > 1 ? slot_of(ver + 1, s.vdepth) : 0;
   d.lp_shift = hp.mb_major ? (int64_t)(s.v_ring / (uint64_t)hp.lp_elem) + (int64_t)d.u_vslot * (int64_t)s.count - (int64_t)s.begin : 0;
   if (hp.mb_major && s.rdepth > 0) {
     // corrected recompute weights of version ver + 1: slot vdepth + (ver + 1) % rdepth of the same rings
-    d.rc_uslot = s.vdepth + (int32_t)((ver + 1) % s.rdepth);
+    d.rc_uslot = s.vdepth + slot_of(ver + 1, s.rdepth);
     d.rc_shift = (int64_t)(s.v_ring / (uint64_t)hp.lp_elem) + (int64_t)d.rc_uslot * (int64_t)s.count - (int64_t)s.begin;
     d.rc_gap = (float)(s.tau_f - s.tau_r);
   }
   d.active_update = k >= 0 ? 1 : 0;
-  d.alpha = 0.f; d.gamma = 0.f; d.one_minus_gamma = 1.f; d.bc1 = 1.f; d.bc2 = 1.f; d.use_delta = 0;
   const int64_t kk = k >= 0 ? k : kb;                 // the update index of the microbatch in backward
-  if (kk >= 0) {
-    double base = hp.alpha_const;
-    if (hp.alpha_tab != nullptr) base = hp.alpha_tab[kk < hp.alpha_len ? kk : hp.alpha_len - 1];
-    double alpha = base;
-    // warm-up microbatches (Section 4) are synchronous: standard step size, no correction, delta left alone; the T1
-    // annealing counts from the first PipeMare step
-    const bool sync = kk < hp.warm;
-    if (hp.t1 && !sync) {
-      double r = (double)(kk - hp.warm) / (double)hp.K;
-      double p = 1.0 - (r < 1.0 ? r : 1.0);
-      int tau = s.tau_f > 1 ? s.tau_f : 1;
-      alpha = base / pow((double)tau, p);
-    }
-    d.alpha = (float)alpha;
-    if (hp.t2 && s.gap > 0 && !sync) {
-      d.gamma = (float)pow(hp.D, 1.0 / (double)s.gap);
-      d.one_minus_gamma = 1.0f - d.gamma;
-      d.use_delta = 1;
-    }
-    if (hp.optimizer == PM_ADAM) {
-      d.bc1 = (float)(1.0 - pow((double)hp.beta1, (double)(kk + 1)));
-      d.bc2 = (float)(1.0 - pow((double)hp.beta2, (double)(kk + 1)));
-    }
-  }
+  const DynScalars sc = quad_scalars(s, hp, kk);
+  d.use_delta = (kk >= 0 && hp.t2 && s.gap > 0 && !(kk < hp.warm)) ? 1 : 0;
+  d.alpha = kk >= 0 ? sc.alpha : 0.f;
+  d.gamma = d.use_delta ? sc.gamma : 0.f;
+  d.one_minus_gamma = d.use_delta ? 1.0f - sc.gamma : 1.f;
+  d.bc1 = sc.bc1; d.bc2 = sc.bc2;
   return d;
 }
 
-__global__ void schedule_kernel(const StageSched* __restrict__ sched, const int64_t* __restrict__ nupd,
-                                StageDyn* __restrict__ dyn, HyperDev hp, int64_t tick, int64_t n_fed,
-                                int64_t flat_k) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= hp.n_stages) return;
+// one quad of lanes per stage; every lane of the block must come here
+__device__ __forceinline__ void schedule_tick(const StageSched* __restrict__ sched, const int64_t* __restrict__ nupd,
+                                              StageDyn* __restrict__ dyn, const HyperDev& hp, int64_t tick, int64_t n_fed, int block) {
+  const int quad = (block * (int)blockDim.x + (int)threadIdx.x) >> 2;
+  const int P = hp.n_stages, i = quad < P ? quad : P - 1;
   const StageSched s = sched[i];
-  const int P = hp.n_stages;
   const int64_t ver = nupd[i];
-  if (flat_k >= 0) { dyn[i] = make_dyn(s, hp, tick, -1, -1, flat_k, ver, ver, false); return; }
   int64_t a = mb_at_tick(tick - i, hp.warm, hp.period, hp.entry_period);
   int64_t b = mb_at_tick(tick - (2 * (int64_t)P - (i + 1)), hp.warm, hp.period, hp.entry_period);
   if (!(a >= 0 && a < n_fed)) a = -1;
@@ -106,15 +130,8 @@ __global__ void schedule_kernel(const StageSched* __restrict__ sched, const int6
   // names from the stage's queue.
   int64_t fver = ver;
   if (hp.entry_period > 1 && a >= 0) { fver = a - s.tau_f; if (fver < 0) fver = 0; }
-  dyn[i] = make_dyn(s, hp, tick, a, b, b, ver, fver, true);
-}
-
-cudaError_t launch_schedule(const StageSched* sched, const int64_t* nupd, StageDyn* dyn, HyperDev hp,
-                            int64_t tick, int64_t n_fed, int64_t flat_k, cudaStream_t stream) {
-  int threads = 128;
-  int blocks = (hp.n_stages + threads - 1) / threads;
-  schedule_kernel<<<blocks, threads, 0, stream>>>(sched, nupd, dyn, hp, tick, n_fed, flat_k);
-  return cudaGetLastError();
+  const StageDyn d = make_dyn(s, hp, tick, a, b, b, ver, fver, true, b);
+  if (quad < P && (threadIdx.x & 3) == 0) dyn[i] = d;
 }
 
 // Microbatch-major order (the paper's own statement of the method, Section 2.1: a queue of weight versions per
@@ -124,11 +141,11 @@ cudaError_t launch_schedule(const StageSched* sched, const int64_t* nupd, StageD
 // older than the end of the warm-up), the backward the live weights (version t).  Table v in 0..2P-1 serves the
 // launches of sub-tick v; table 2P marks every stage in backward with its own backward sub-tick's slots and an
 // active update: it serves the grouped weight-gradient launch and the fused update.
-__global__ void schedule_mb_kernel(const StageSched* __restrict__ sched, StageDyn* __restrict__ tables, HyperDev hp, int64_t t,
-                                   const int32_t* __restrict__ delays, const int64_t* __restrict__ nupd) {
+__device__ __forceinline__ void schedule_mb(const StageSched* __restrict__ sched, StageDyn* __restrict__ tables, const HyperDev& hp, int64_t t,
+                                            const int32_t* __restrict__ delays, const int64_t* __restrict__ nupd, int block, int v) {
   const int P = hp.n_stages;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y;
-  if (i >= P) return;
+  const int quad = (block * (int)blockDim.x + (int)threadIdx.x) >> 2, i = quad < P ? quad : P - 1;
+  const bool store = quad < P && (threadIdx.x & 3) == 0;
   const StageSched s = sched[i];
   const int64_t base = 2 * (int64_t)P * t;
   // N microbatches per update (Section 2.1): versions, delays and step indices count updates; microbatch t belongs to
@@ -152,7 +169,7 @@ __global__ void schedule_mb_kernel(const StageSched* __restrict__ sched, StageDy
       d.g_shift = src >= 0 ? (src % hp.stochastic) * (int64_t)hp.total : 0;
     }
     d.r_ver = src >= 0 ? src : -1;
-    tables[(size_t)v * P + i] = d;
+    if (store) tables[(size_t)v * P + i] = d;
     return;
   }
   // PipeMare Recompute (Appendix A.2, Appendix D): the version the recomputation reads, clamped like the forward's
@@ -179,15 +196,105 @@ __global__ void schedule_mb_kernel(const StageSched* __restrict__ sched, StageDy
     d.f_vslot = s.rdepth > 0 ? s.vdepth : (s.vdepth > 1 ? (int32_t)(u % s.vdepth) : 0);
   }
   d.accum = (t % N != 0) ? 1 : 0;
-  tables[(size_t)v * P + i] = d;
+  if (store) tables[(size_t)v * P + i] = d;
 }
 
-cudaError_t launch_schedule_mb(const StageSched* sched, StageDyn* tables, HyperDev hp, int64_t t, cudaStream_t stream,
-                               const int32_t* delays, const int64_t* nupd) {
-  const int threads = 128;
-  dim3 grid((hp.n_stages + threads - 1) / threads, mb_table_count(hp.n_stages, hp.segment));
-  schedule_mb_kernel<<<grid, threads, 0, stream>>>(sched, tables, hp, t, delays, nupd);
+// ---- start of a tick ------------------------------------------------------------------------------
+// One launch writes the schedule table(s) and copies the microbatch in, which depend on nothing of each other: the first
+// `sched_blocks` blocks schedule, the rest copy.
+// MLP: inputs [T, n_in] (activation type) -> stage 1's input ring slot; targets [T, n_out] float -> target ring.
+// Encoder: token ids [T] int32 per stream -> the id ring slots of the embedding stages; target ids [T] int32 -> target ring.
+template <typename E>
+__device__ __forceinline__ void copy_in(E* __restrict__ dst, const E* __restrict__ src, uint64_t n, uint64_t gid, uint64_t stride) {
+  constexpr uint64_t V = 16 / sizeof(E);
+  uint64_t done = 0;
+  if ((((uintptr_t)dst | (uintptr_t)src) & 15) == 0) {      // the caller's pointer and an odd-sized slot may start anywhere
+    done = n / V * V;
+    for (uint64_t i = gid; i < n / V; i += stride) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
+  }
+  for (uint64_t i = done + gid; i < n; i += stride) dst[i] = src[i];
+}
+
+constexpr int kBeginThreads = 128;
+
+template <typename AT, bool MB>
+__global__ void __launch_bounds__(kBeginThreads) begin_kernel(const StageSched* __restrict__ sched, StageDyn* __restrict__ dyn, HyperDev hp, int64_t tick, int64_t n_fed,
+                                                              const int32_t* __restrict__ delays, const int64_t* __restrict__ nupd, int sched_blocks, int per_table,
+                                                              TickArgs t, const void* __restrict__ inputs, const void* __restrict__ targets, int64_t mb) {
+  if ((int)blockIdx.x < sched_blocks) {
+    if (MB) schedule_mb(sched, dyn, hp, mb, delays, nupd, (int)blockIdx.x % per_table, (int)blockIdx.x / per_table);
+    else schedule_tick(sched, nupd, dyn, hp, tick, n_fed, (int)blockIdx.x);
+    return;
+  }
+  const StageDev& s0 = t.st[0];
+  const uint64_t gid = (uint64_t)(blockIdx.x - sched_blocks) * blockDim.x + threadIdx.x, stride = (uint64_t)(gridDim.x - sched_blocks) * blockDim.x;
+  const uint64_t T = (uint64_t)t.T;
+  if (s0.pre == PRE_EMBED) {
+    const int32_t* ids = reinterpret_cast<const int32_t*>(inputs);
+    copy_in<int32_t>(ring_at<int32_t>(t, s0.ids_ring, (int)(mb % s0.ids_depth), T), ids, T, gid, stride);
+    if (t.n_streams > 1) {                                    // second token stream -> the stage that embeds it
+      const StageDev& s1 = t.st[t.second_embed_stage];
+      copy_in<int32_t>(ring_at<int32_t>(t, s1.ids_ring, (int)(mb % s1.ids_depth), T), ids + T, T, gid, stride);
+    }
+  } else {
+    const uint64_t n = T * t.n_in_first;
+    copy_in<AT>(ring_at<AT>(t, s0.x_ring, (int)(mb % s0.xdepth), n), reinterpret_cast<const AT*>(inputs), n, gid, stride);
+  }
+  if (t.loss_kind == PM_LOSS_CE) {
+    copy_in<int32_t>(ws_at<int32_t>(t, t.tgt_off) + (uint64_t)(mb % (t.P + 1)) * T, reinterpret_cast<const int32_t*>(targets), T, gid, stride);
+  } else {
+    const uint64_t n = T * t.n_out_last;
+    copy_in<float>(ws_at<float>(t, t.tgt_off) + (uint64_t)(mb % (t.P + 1)) * n, reinterpret_cast<const float*>(targets), n, gid, stride);
+  }
+}
+
+cudaError_t launch_begin(const StageSched* sched, StageDyn* dyn, HyperDev hp, int64_t tick, int64_t n_fed, bool mb_order, const int32_t* delays,
+                         const int64_t* nupd, const TickArgs& t, int dtype, const void* inputs, const void* targets, int64_t mb, cudaStream_t stream) {
+  const int per_table = (4 * hp.n_stages + kBeginThreads - 1) / kBeginThreads;
+  const int sched_blocks = per_table * (mb_order ? mb_table_count(hp.n_stages, hp.segment) : 1);
+  int copy_blocks = 0;
+  if (inputs) {
+    // 16 bytes per thread and array; the larger of the arrays decides, capped at a chip-full of blocks
+    const uint64_t x = t.n_in_first > 0 ? (uint64_t)t.T * t.n_in_first * (dtype == PM_F32 ? 4 : 2) : (uint64_t)t.T * 4;
+    const uint64_t y = t.loss_kind == PM_LOSS_CE ? (uint64_t)t.T * 4 : (uint64_t)t.T * t.n_out_last * 4;
+    const uint64_t need = ((x > y ? x : y) / 16 + kBeginThreads) / kBeginThreads;
+    copy_blocks = (int)(need < 1184 ? need : 1184);
+  }
+#define PM_BEGIN(AT, MB) begin_kernel<AT, MB><<<sched_blocks + copy_blocks, kBeginThreads, 0, stream>>>(sched, dyn, hp, tick, n_fed, delays, nupd, sched_blocks, per_table, t, inputs, targets, mb)
+  if (dtype == PM_F32) { if (mb_order) PM_BEGIN(float, true); else PM_BEGIN(float, false); }
+  else { if (mb_order) PM_BEGIN(__nv_bfloat16, true); else PM_BEGIN(__nv_bfloat16, false); }
+#undef PM_BEGIN
   return cudaGetLastError();
+}
+
+// ---- stand-alone update: stage tables ------------------------------------------------------------------------
+// The caller's stage split comes as a kernel argument (no copy from pageable host memory in front of the launch); the kernel
+// writes the bounds, the scalars of update index k and zeroed counters into the workspace.
+template <int N>
+__global__ void __launch_bounds__(128) flat_table_kernel(__grid_constant__ const FlatTable<N> tab, HyperDev hp, int64_t k, uint32_t* __restrict__ begin64,
+                                                         uint32_t* __restrict__ end64, StageDyn* __restrict__ dyn, int64_t* __restrict__ nupd) {
+  pdl_trigger();
+  const int quad = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+  const int P = hp.n_stages, i = quad < P ? quad : P - 1;
+  StageSched s{};
+  s.tau_f = tab.tau_f[i]; s.gap = tab.gap[i]; s.depth = 1; s.xdepth = 1;
+  const StageDyn d = make_dyn(s, hp, 0, -1, -1, k, 0, 0, false, -1);
+  if (quad < P && (threadIdx.x & 3) == 0) { dyn[i] = d; nupd[i] = 0; begin64[i] = tab.begin64[i]; end64[i] = tab.end64[i]; }
+}
+
+template <int N>
+static cudaError_t flat_table_t(const FlatStage* st, HyperDev hp, int64_t k, uint32_t* begin64, uint32_t* end64, StageDyn* dyn, int64_t* nupd, cudaStream_t stream) {
+  FlatTable<N> tab;
+  for (int i = 0; i < hp.n_stages; ++i) { tab.begin64[i] = st[i].begin64; tab.end64[i] = st[i].end64; tab.tau_f[i] = st[i].tau_f; tab.gap[i] = st[i].gap; }
+  flat_table_kernel<N><<<(4 * hp.n_stages + 127) / 128, 128, 0, stream>>>(tab, hp, k, begin64, end64, dyn, nupd);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_flat_table(const FlatStage* st, HyperDev hp, int64_t k, uint32_t* begin64, uint32_t* end64, StageDyn* dyn, int64_t* nupd, cudaStream_t stream) {
+  // argument sizes of 1, 4 and 16 KB: a launch copies all of them
+  if (hp.n_stages <= 64) return flat_table_t<64>(st, hp, k, begin64, end64, dyn, nupd, stream);
+  if (hp.n_stages <= 256) return flat_table_t<256>(st, hp, k, begin64, end64, dyn, nupd, stream);
+  return flat_table_t<PM_MAX_STAGES>(st, hp, k, begin64, end64, dyn, nupd, stream);
 }
 
 // ---- fused update ------------------------------------------------------------------------------
@@ -195,25 +302,36 @@ cudaError_t launch_schedule_mb(const StageSched* sched, StageDyn* tables, HyperD
 __device__ __forceinline__ float4 ld_stream(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ void st_stream(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
 
-constexpr int kUpdThreads = 256;
+constexpr int kUpdThreads = 128;
 constexpr int kUpdUnroll = 2;      // float4 groups per thread per array in flight
+
+// What bounds the kernel: HBM.  One block per 1024 elements, in ascending order, and not a persistent grid: resident blocks then
+// work on one moving window of the arenas, where grid-stride blocks drift apart and the nine streams lose their DRAM pages.
+// 100 M parameters, Adam, 64 stages: 674 us with eight persistent blocks of 256 threads per SM, 633 with a block of 256 threads
+// per chunk, 615 when the look-up tries the stage an even split would give before it searches, 598 with blocks of 128 threads
+// (6.36 TB/s; one float4 per array and thread instead of two: 602).
 
 // LP: operand-type copy of the new weights: 0 none, 1 bfloat16, 2 float (a version-ring slot of fp32 operands);
 // element e of the arenas goes to lp_base[lp_shift + e], lp_shift from the stage's table entry (0: the w_lp arena)
 template <int OPT, int LP>
-__global__ void __launch_bounds__(kUpdThreads, 3)
+__global__ void __launch_bounds__(kUpdThreads, 6)
 update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restrict__ begin64, const uint32_t* __restrict__ end64,
               const StageDyn* __restrict__ dyn, int64_t* __restrict__ nupd, int n_stages, uint64_t total_vec4,
               float beta1, float beta2, float eps, uint64_t first_vec4, const uint32_t* __restrict__ skip_b64, const uint32_t* __restrict__ skip_e64,
-              const float* __restrict__ gsrc) {
+              const float* __restrict__ gsrc, float stages_per_group) {
   // ranges (one per stage, in 64-element groups) that another kernel has updated already: the Linear matrices, when the
   // weight-gradient GEMM applies the update in its epilogue
   const bool skip = skip_b64 != nullptr;
+  pdl_wait();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
   const uint64_t base = first_vec4 + (uint64_t)blockIdx.x * kUpdThreads * kUpdUnroll;
   // the stage of the block's first group: the largest i with begin64[i] <= g0 (every thread searches, on the same addresses)
   const uint32_t g0 = (uint32_t)(base >> 4);
   int lo0 = 0, hi = n_stages - 1;
+  {
+    const int q = min(hi, (int)((float)g0 * stages_per_group));            // where it is if all stages have the same size
+    if (__ldg(begin64 + q) <= g0 && (q == hi || g0 < __ldg(begin64 + q + 1))) lo0 = hi = q;
+  }
   while (lo0 < hi) { const int mid = (lo0 + hi + 1) >> 1; if (__ldg(begin64 + mid) <= g0) lo0 = mid; else hi = mid - 1; }
   if (skip) {
     // the whole span of this block lies inside a skipped range (and past the stage's first group): nothing to do
@@ -299,21 +417,21 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
 cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* end64, const StageDyn* dyn,
                           int64_t* nupd, int n_stages, uint64_t total64, int optimizer, float beta1, float beta2,
                           float eps, cudaStream_t stream, void* lp_base, int lp_elem, uint64_t first64,
-                          const uint32_t* skip_b64, const uint32_t* skip_e64, const float* gsrc) {
+                          const uint32_t* skip_b64, const uint32_t* skip_e64, const float* gsrc, bool pdl) {
   if (total64 == 0 || n_stages == 0 || first64 >= total64) return cudaSuccess;
   uint64_t total_vec4 = total64 * 16;
   const uint64_t first_vec4 = first64 * 16;
-  uint64_t per_block = (uint64_t)kUpdThreads * kUpdUnroll;
-  const unsigned blocks = (unsigned)((total_vec4 - first_vec4 + per_block - 1) / per_block);   // 2048 elements per block: 2^31 blocks are 4e12 elements
+  const uint64_t per_block = (uint64_t)kUpdThreads * kUpdUnroll;
+  const unsigned blocks = (unsigned)((total_vec4 - first_vec4 + per_block - 1) / per_block);   // 1024 elements per block: 2^31 blocks are 2e12 elements
   // the operand-type copy: the w_lp arena (bfloat16) unless the caller names a version ring and its element size
   if (lp_base == nullptr) { lp_base = a.w_lp; lp_elem = 2; }
   if (gsrc == nullptr) gsrc = a.grad;
   const int lp = lp_base == nullptr ? 0 : (lp_elem == 4 ? 2 : 1);
-#define PM_UPD(OPT, LP) update_kernel<OPT, LP><<<blocks, kUpdThreads, 0, stream>>>(a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc)
-  if (optimizer == PM_SGDM) { if (lp == 0) PM_UPD(PM_SGDM, 0); else if (lp == 1) PM_UPD(PM_SGDM, 1); else PM_UPD(PM_SGDM, 2); }
-  else { if (lp == 0) PM_UPD(PM_ADAM, 0); else if (lp == 1) PM_UPD(PM_ADAM, 1); else PM_UPD(PM_ADAM, 2); }
+  const float per_group = (float)n_stages / (float)total64;
+#define PM_UPD(OPT, LP) launch_pdl(update_kernel<OPT, LP>, dim3(blocks), dim3(kUpdThreads), 0, stream, pdl, a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc, per_group)
+  if (optimizer == PM_SGDM) return lp == 0 ? PM_UPD(PM_SGDM, 0) : (lp == 1 ? PM_UPD(PM_SGDM, 1) : PM_UPD(PM_SGDM, 2));
+  return lp == 0 ? PM_UPD(PM_ADAM, 0) : (lp == 1 ? PM_UPD(PM_ADAM, 1) : PM_UPD(PM_ADAM, 2));
 #undef PM_UPD
-  return cudaGetLastError();
 }
 
 // ---- fp32 copies of the small forward-read tensors into the version rings -------------------------------------

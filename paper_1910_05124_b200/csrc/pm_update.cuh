@@ -15,18 +15,21 @@ struct StageSched {
   int32_t tau_r, rdepth;                // PipeMare Recompute: delay of the recomputation's weights, slots of their corrected queue
 };
 
-// Launches the scheduler for pipeline tick `tick` with `n_fed` microbatches fed so far.
-// flat_k >= 0 selects the stand-alone update mode: every stage is at update index flat_k.
-cudaError_t launch_schedule(const StageSched* sched, const int64_t* nupd, StageDyn* dyn, HyperDev hp,
-                            int64_t tick, int64_t n_fed, int64_t flat_k, cudaStream_t stream);
-// Microbatch-major order: fills the tables of microbatch t ([n_tables][P] entries): table v < 2P for the launches of
+struct TickArgs;
+// Starts a tick: fills the schedule table(s) and, with inputs, copies the microbatch `mb` into the rings.
+// Tick-major order: the table of pipeline tick `tick` with `n_fed` microbatches fed so far.
+// Microbatch-major order (mb_order): the tables of microbatch mb ([n_tables][P] entries): table v < 2P for the launches of
 // sub-tick v (stage i forward at v = i, backward at v = 2P - 1 - i), table 2P for the grouped weight-gradient launch
 // and the update.  With PipeMare Recompute (hp.segment > 0) table 2P + 1 holds every stage's recomputation (its forward
 // entry with the recompute weights' slot) and table 2P + 2 + k the backward entries of segment k alone (the grouped
 // weight-gradient launch of that segment).
-// delays / nupd (stochastic delay model only, else null): the step's per-stage delays and the stages' update counters.
-cudaError_t launch_schedule_mb(const StageSched* sched, StageDyn* tables, HyperDev hp, int64_t t, cudaStream_t stream,
-                               const int32_t* delays = nullptr, const int64_t* nupd = nullptr);
+// delays (stochastic delay model only, else null): the step's per-stage delays.  nupd: the stages' update counters.
+cudaError_t launch_begin(const StageSched* sched, StageDyn* dyn, HyperDev hp, int64_t tick, int64_t n_fed, bool mb_order, const int32_t* delays,
+                         const int64_t* nupd, const TickArgs& t, int dtype, const void* inputs, const void* targets, int64_t mb, cudaStream_t stream);
+// Stand-alone update: bounds, scalars of update index k and zeroed counters of hp.n_stages stages into device tables.
+struct FlatStage { uint32_t begin64, end64; int32_t tau_f, gap; };
+template <int N> struct FlatTable { uint32_t begin64[N], end64[N]; int32_t tau_f[N], gap[N]; };
+cudaError_t launch_flat_table(const FlatStage* st, HyperDev hp, int64_t k, uint32_t* begin64, uint32_t* end64, StageDyn* dyn, int64_t* nupd, cudaStream_t stream);
 inline int mb_table_count(int P, int segment) { return 2 * P + 1 + (segment > 0 ? 1 + (P + segment - 1) / segment : 0); }
 
 // Launches the fused update over all stages whose dyn[i].active_update is set.
@@ -34,7 +37,8 @@ inline int mb_table_count(int P, int segment) { return 2 * P + 1 + (segment > 0 
 cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* end64, const StageDyn* dyn,
                           int64_t* nupd, int n_stages, uint64_t total64, int optimizer, float beta1, float beta2,
                           float eps, cudaStream_t stream, void* lp_base = nullptr, int lp_elem = 0, uint64_t first64 = 0,
-                          const uint32_t* skip_b64 = nullptr, const uint32_t* skip_e64 = nullptr, const float* gsrc = nullptr);
+                          const uint32_t* skip_b64 = nullptr, const uint32_t* skip_e64 = nullptr, const float* gsrc = nullptr, bool pdl = false);
+// pdl: launched as a programmatic dependent of the launch before it.
 // gsrc: where the gradients are read (element e of stage i at gsrc[dyn[i].g_shift + e]); null: the grad arena.
 // skip_b64 / skip_e64: per stage, a range of 64-element groups this launch leaves alone (device arrays, or null): the
 // Linear matrices when the weight-gradient GEMM has applied their update in its epilogue.  The stage's update

@@ -8,7 +8,6 @@
 // needs only the arenas themselves.
 #include <mutex>
 #include <string>
-#include <cstring>
 
 #include "pm_update.cuh"
 
@@ -40,9 +39,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {nullptr};
 thread_local std::string g_static_error;
-
-// host staging for the table; fixed size so that the call performs no allocation of any kind
-thread_local unsigned char g_host_table[kScratchBytes];
 
 }  // namespace
 
@@ -85,16 +81,12 @@ pm_status pm_update_flat_static(const pm_arenas* arenas, const uint64_t* stage_o
   }
 
   const uint64_t P = (uint64_t)n_stages;
-  const uint64_t need = table_bytes(P);
-  const uint64_t off_sched = 0, off_dyn = align_up(sizeof(StageSched) * P, 256);
+  const uint64_t off_dyn = align_up(sizeof(StageSched) * P, 256);
   const uint64_t off_nupd = align_up(off_dyn + sizeof(StageDyn) * P, 256);
   const uint64_t off_b = align_up(off_nupd + sizeof(int64_t) * P, 256);
   const uint64_t off_e = align_up(off_b + sizeof(uint32_t) * P, 256);
-  // the array keeps whatever the previous call left: rebuild the whole table, zero counters included
-  std::memset(g_host_table, 0, need);
-  StageSched* sc = (StageSched*)(g_host_table + off_sched);
-  uint32_t* b64 = (uint32_t*)(g_host_table + off_b);
-  uint32_t* e64 = (uint32_t*)(g_host_table + off_e);
+  // the array keeps whatever the previous call left: the table kernel rewrites all of it that this call reads
+  FlatStage tab[PM_STATIC_MAX_STAGES];
   uint64_t prev_end = 0;
   for (int i = 0; i < n_stages; ++i) {
     if (stage_offsets[i] % PM_ALIGN_ELEMS) return fail(PM_ERR_INVALID_ARG, "stage offsets must be multiples of 64 elements");
@@ -105,25 +97,22 @@ pm_status pm_update_flat_static(const pm_arenas* arenas, const uint64_t* stage_o
     uint64_t end = align_up(stage_offsets[i] + stage_counts[i], PM_ALIGN_ELEMS);
     if (end > arenas->count) return fail(PM_ERR_NOMEM, "stage slice exceeds the arenas");
     prev_end = end;
-    sc[i] = StageSched{tau_fwd[i], tau_fwd[i] - tau_bkwd[i], 1, 1, 0, 0};
-    b64[i] = (uint32_t)(stage_offsets[i] / 64);
-    e64[i] = (uint32_t)(end / 64);
+    tab[i] = FlatStage{(uint32_t)(stage_offsets[i] / 64), (uint32_t)(end / 64), tau_fwd[i], tau_fwd[i] - tau_bkwd[i]};
   }
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)scratch;
-  e = cudaMemcpyAsync(ws, g_host_table, need, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return fail(PM_ERR_CUDA, cudaGetErrorString(e));
   HyperDev hp{};
   hp.optimizer = cfg->optimizer; hp.t1 = cfg->t1_enable; hp.t2 = cfg->t2_enable; hp.n_stages = n_stages;
   hp.K = cfg->t1_K > 0 ? cfg->t1_K : 1; hp.D = cfg->t2_D;
   hp.alpha_const = cfg->alpha_by_step ? cfg->alpha_by_step[k < cfg->alpha_len ? k : cfg->alpha_len - 1] : cfg->alpha_const;
   hp.alpha_tab = nullptr; hp.alpha_len = 0;
   hp.beta1 = cfg->beta1; hp.beta2 = cfg->beta2; hp.eps = cfg->eps;
-  e = launch_schedule((const StageSched*)(ws + off_sched), (const int64_t*)(ws + off_nupd), (StageDyn*)(ws + off_dyn), hp, 0, 0, k, st);
+  e = launch_flat_table(tab, hp, k, (uint32_t*)(ws + off_b), (uint32_t*)(ws + off_e), (StageDyn*)(ws + off_dyn), (int64_t*)(ws + off_nupd), st);
   if (e != cudaSuccess) return fail(PM_ERR_CUDA, cudaGetErrorString(e));
   ArenasDev a{arenas->w, arenas->m, arenas->s, arenas->delta, arenas->grad, (__nv_bfloat16*)arenas->w_lp, arenas->count};
   e = launch_update(a, (const uint32_t*)(ws + off_b), (const uint32_t*)(ws + off_e), (const StageDyn*)(ws + off_dyn),
-                    (int64_t*)(ws + off_nupd), n_stages, e64[n_stages - 1], cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, st);
+                    (int64_t*)(ws + off_nupd), n_stages, tab[n_stages - 1].end64, cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, st,
+                    nullptr, 0, 0, nullptr, nullptr, nullptr, true);
   if (e != cudaSuccess) return fail(PM_ERR_CUDA, cudaGetErrorString(e));
   return PM_OK;
 }
