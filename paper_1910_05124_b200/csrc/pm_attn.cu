@@ -121,16 +121,18 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
-  if (d.f_mb < 0 || !feeds_attention(s.post)) return;
+  if (d.f_mb < 0 || !feeds_attention(s.post)) { pdl_wait(); return; }
   const bool cross = s.post == POST_CROSS_ATTENTION;         // q = the stage's main input; the Linear gave [k | v]
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
   const int S = FULL ? AT_S : s.seq_len;
-  if ((int)blockIdx.x >= (t.T / S) * H) return;
+  if ((int)blockIdx.x >= (t.T / S) * H) { pdl_wait(); return; }
   const int b = blockIdx.x / H, h = blockIdx.x % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, 3 * AT_TILE, 128);
   const uint32_t tmem_base = *c.tmem_slot;
+  pdl_trigger();                                             // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
   const uint32_t sQ = c.sbase, sK = sQ + AT_TILE, sV = sK + AT_TILE, sP = sQ;   // P overwrites Q and K once S = Q K^T is done
   uint8_t* pP = c.sptr;
   const CUtensorMap* lm = maps + (size_t)p * AMAPS_PER_STAGE;
@@ -227,16 +229,18 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
-  if (d.b_mb < 0 || !feeds_attention(s.post)) return;
+  if (d.b_mb < 0 || !feeds_attention(s.post)) { pdl_wait(); return; }
   const bool cross = s.post == POST_CROSS_ATTENTION;
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
   const int S = FULL ? AT_S : s.seq_len;
-  if ((int)blockIdx.x >= (t.T / S) * H) return;
+  if ((int)blockIdx.x >= (t.T / S) * H) { pdl_wait(); return; }
   const int b = blockIdx.x / H, h = blockIdx.x % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, AT_BWD_TILES * AT_TILE);
   const uint32_t tmem_base = *c.tmem_slot;
+  pdl_trigger();                                             // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
   const uint32_t sQ = c.sbase, sK = sQ + AT_TILE, sdO = sK + AT_TILE, sV = sdO + AT_TILE, sP = sV;   // P and dS: tiles 3 and 4
   uint8_t* pP = c.sptr + 3 * AT_TILE;
   float* xch = reinterpret_cast<float*>(c.sptr + AT_BWD_TILES * AT_TILE + 128);                      // [3][2][128]
@@ -384,16 +388,18 @@ __global__ void __launch_bounds__(256, 2) attn_fwd_tc256_kernel(TickArgs t, cons
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
-  if (d.f_mb < 0 || !feeds_attention(s.post)) return;
+  if (d.f_mb < 0 || !feeds_attention(s.post)) { pdl_wait(); return; }
   const bool cross = s.post == POST_CROSS_ATTENTION;
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
-  if ((int)blockIdx.x >= (t.T / AT2_S) * H * 2) return;
+  if ((int)blockIdx.x >= (t.T / AT2_S) * H * 2) { pdl_wait(); return; }
   const int qb = blockIdx.x & 1, bh = blockIdx.x >> 1;
   const int b = bh / H, h = bh % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, AT2_FWD_TILES * AT_TILE, 256);
   const uint32_t tmem_base = *c.tmem_slot;
+  pdl_trigger();                                             // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
   const uint32_t sK = c.sbase, sQ = sK + 2 * AT_TILE, sV = sK + 4 * AT_TILE, sP = sK;
   uint8_t* pP = c.sptr;
   float* xch = reinterpret_cast<float*>(c.sptr + AT2_FWD_TILES * AT_TILE + 128);   // [2][2][128]
@@ -496,15 +502,17 @@ __global__ void __launch_bounds__(AT2_BWD_THREADS, 1) attn_bwd_tc256_kernel(Tick
   const int p = stage_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
-  if (d.b_mb < 0 || !feeds_attention(s.post)) return;
+  if (d.b_mb < 0 || !feeds_attention(s.post)) { pdl_wait(); return; }
   const bool cross = s.post == POST_CROSS_ATTENTION;
   const int causal = s.causal;
   const int H = s.n_heads, dm = s.d_out_main;
-  if ((int)blockIdx.x >= (t.T / AT2_S) * H) return;
+  if ((int)blockIdx.x >= (t.T / AT2_S) * H) { pdl_wait(); return; }
   const int b = blockIdx.x / H, h = blockIdx.x % H;
   extern __shared__ uint8_t smem_raw[];
   const AttnCommon c = attn_setup(smem_raw, AT2_BWD_TILES * AT_TILE, 512);
   const uint32_t tmem_base = *c.tmem_slot;
+  pdl_trigger();                                             // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
   const uint32_t sQ = c.sbase, sdO = sQ + AT_TILE, sK = sQ + 2 * AT_TILE, sV = sQ + 4 * AT_TILE, sP = sV, sdS = sQ + 8 * AT_TILE;
   uint8_t* pP = c.sptr + 4 * AT_TILE;
   uint8_t* pdS = c.sptr + 8 * AT_TILE;
@@ -749,19 +757,12 @@ cudaError_t attn_tc_launch(AttnPlan* plan, const TickArgs& t, bool forward, cuda
   }
   dim3 grid(t.att_blocks, n_att);                     // att_blocks = (sequence, head) pairs
   if (t.att_S == AT2_S) {
-    if (forward) attn_fwd_tc256_kernel<<<dim3(2 * t.att_blocks, n_att), 256, AT2_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-    else attn_bwd_tc256_kernel<<<grid, AT2_BWD_THREADS, AT2_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-    return cudaGetLastError();
+    if (forward) return launch_pdl(attn_fwd_tc256_kernel, dim3(2 * t.att_blocks, n_att), dim3(256), AT2_FWD_SMEM, stream, t.pdl, t, plan->d_maps, ids, plan->d_status);
+    return launch_pdl(attn_bwd_tc256_kernel, grid, dim3(AT2_BWD_THREADS), AT2_BWD_SMEM, stream, t.pdl, t, plan->d_maps, ids, plan->d_status);
   }
   const bool full = t.att_S == AT_S;
-  if (forward) {
-    if (full) attn_fwd_tc_kernel<true><<<grid, 128, AT_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-    else attn_fwd_tc_kernel<false><<<grid, 128, AT_FWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-  } else {
-    if (full) attn_bwd_tc_kernel<true><<<grid, AT_BWD_THREADS, AT_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-    else attn_bwd_tc_kernel<false><<<grid, AT_BWD_THREADS, AT_BWD_SMEM, stream>>>(t, plan->d_maps, ids, plan->d_status);
-  }
-  return cudaGetLastError();
+  if (forward) return launch_pdl(full ? attn_fwd_tc_kernel<true> : attn_fwd_tc_kernel<false>, grid, dim3(128), AT_FWD_SMEM, stream, t.pdl, t, plan->d_maps, ids, plan->d_status);
+  return launch_pdl(full ? attn_bwd_tc_kernel<true> : attn_bwd_tc_kernel<false>, grid, dim3(AT_BWD_THREADS), AT_BWD_SMEM, stream, t.pdl, t, plan->d_maps, ids, plan->d_status);
 }
 
 }  // namespace pm

@@ -20,6 +20,8 @@ constexpr int kLossBlocks = 96, kLossThreads = 256;     // partial sums and the 
 
 template <typename AT>
 __global__ void __launch_bounds__(kLossThreads) mse_loss_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const StageDyn& d = t.dyn[t.P - 1];
   if (d.b_mb < 0) return;
   const StageDev& sl = t.st[t.P - 1];
@@ -77,9 +79,7 @@ cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream);  
 
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
   if (t.loss_kind == PM_LOSS_CE) return launch_ce_loss(t, dtype, stream);
-  if (dtype == PM_F32) mse_loss_kernel<float><<<kLossBlocks, kLossThreads, 0, stream>>>(t);
-  else mse_loss_kernel<__nv_bfloat16><<<kLossBlocks, kLossThreads, 0, stream>>>(t);
-  return cudaGetLastError();
+  return launch_pdl(dtype == PM_F32 ? mse_loss_kernel<float> : mse_loss_kernel<__nv_bfloat16>, dim3(kLossBlocks), dim3(kLossThreads), 0, stream, t.pdl, t);
 }
 
 // ---- activation backward + bias gradient ---------------------------------------------------------
@@ -141,6 +141,8 @@ __device__ __forceinline__ void actbwd_rows(const AT* __restrict__ dy, const AT*
 // which has fewer blocks and needs more loads in flight per block
 template <typename AT, int NW>
 __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
+  pdl_trigger();
+  pdl_wait();
   const int* start = t.act_start + (size_t)lvl * (t.P + 1);
   int lo = 0, hi = t.P - 1;                                 // stage of this column block: largest p with start[p] <= its index
   const int blk = (int)blockIdx.x + t.act_first[lvl];
@@ -214,6 +216,8 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
 // rows and a finishing launch a level of the 32-stage 1024-wide MLP (128 rows) took 17.6 + 12.7 us.
 template <typename AT>
 __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) {
+  pdl_trigger();
+  pdl_wait();
   constexpr int kPer = kActColsV / kSmallCols;
   const int* start = t.act_start + (size_t)lvl * (t.P + 1);
   const int blk = (int)(blockIdx.x / kPer) + t.act_first[lvl];
@@ -281,6 +285,8 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
 constexpr int kFinCols = 32, kFinMaxPer = 32;            // columns per block; partials per warp held in registers at a time
 
 __global__ void __launch_bounds__(256) bias_finish_kernel(TickArgs t, int lvl) {
+  pdl_trigger();
+  pdl_wait();
   // the grid follows the list of 256-column blocks of the activation-backward launch (kActColsV / kFinCols blocks
   // here per entry there), so no block falls outside its Linear's columns however unequal the widths are
   constexpr int kPer = kActColsV / kFinCols;
@@ -326,24 +332,17 @@ int actbwd_launches(const TickArgs& t, int dtype) { return (t.T <= kSmallRows ||
 
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream) {
   if (t.act_blocks[lvl] == 0) return cudaSuccess;
-  if (t.T <= kSmallRows) {
-    if (dtype == PM_F32) actbwd_small_kernel<float><<<t.act_blocks[lvl] * (kActColsV / kSmallCols), 256, 0, stream>>>(t, lvl);
-    else actbwd_small_kernel<__nv_bfloat16><<<t.act_blocks[lvl] * (kActColsV / kSmallCols), 256, 0, stream>>>(t, lvl);
-    return cudaGetLastError();
-  }
+  if (t.T <= kSmallRows)
+    return launch_pdl(dtype == PM_F32 ? actbwd_small_kernel<float> : actbwd_small_kernel<__nv_bfloat16>, dim3(t.act_blocks[lvl] * (kActColsV / kSmallCols)), dim3(256), 0, stream, t.pdl, t, lvl);
   const int cg = act_chunk_group(t);
   dim3 grid(t.act_blocks[lvl], (t.row_chunks + cg - 1) / cg);
-  if (t.sel_p >= 0 && t.row_chunks > 1) {
-    if (dtype == PM_F32) actbwd_kernel<float, 16><<<grid, 16 * 32, 0, stream>>>(t, lvl);
-    else actbwd_kernel<__nv_bfloat16, 16><<<grid, 16 * 32, 0, stream>>>(t, lvl);
-  } else {
-    if (dtype == PM_F32) actbwd_kernel<float, kActWarps><<<grid, kActWarps * 32, 0, stream>>>(t, lvl);
-    else actbwd_kernel<__nv_bfloat16, kActWarps><<<grid, kActWarps * 32, 0, stream>>>(t, lvl);
-  }
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (t.sel_p >= 0 && t.row_chunks > 1)
+    e = launch_pdl(dtype == PM_F32 ? actbwd_kernel<float, 16> : actbwd_kernel<__nv_bfloat16, 16>, grid, dim3(16 * 32), 0, stream, t.pdl, t, lvl);
+  else
+    e = launch_pdl(dtype == PM_F32 ? actbwd_kernel<float, kActWarps> : actbwd_kernel<__nv_bfloat16, kActWarps>, grid, dim3(kActWarps * 32), 0, stream, t.pdl, t, lvl);
   if (e != cudaSuccess || actbwd_launches(t, dtype) == 1) return e;
-  bias_finish_kernel<<<t.act_blocks[lvl] * (kActColsV / kFinCols), 256, 0, stream>>>(t, lvl);
-  return cudaGetLastError();
+  return launch_pdl(bias_finish_kernel, dim3(t.act_blocks[lvl] * (kActColsV / kFinCols)), dim3(256), 0, stream, t.pdl, t, lvl);
 }
 
 // ---- fp32 SIMT grouped GEMM ------------------------------------------------------------------------
@@ -431,17 +430,19 @@ template <int TM, int TN, int NBUF, int MODE>
 __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int tiles_n) {
   using C = F32Cfg<TM, TN, NBUF, MODE>;
   constexpr int BM = C::BM, BN = C::BN, KC = kF32KC;
+  pdl_trigger();
   const int p = stage_of_block(t, blockIdx.y);
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
-  if (lvl >= s.n_lin) return;
-  if (MODE == 0 ? d.f_mb < 0 : d.b_mb < 0) return;
-  if (MODE == 1 && p == 0 && lvl == 0 && s.pre != PRE_EMBED) return;   // raw network inputs need no gradient
-  const LinDev& L = s.lin[lvl];
+  const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
   const int T = t.T;
   const int M = MODE == 2 ? L.n_out : T, N = MODE == 0 ? L.n_out : L.n_in, K = MODE == 0 ? L.n_in : (MODE == 1 ? L.n_out : T);
   const int m0 = (int)(blockIdx.x / tiles_n) * BM, n0 = (int)(blockIdx.x % tiles_n) * BN;
-  if (m0 >= M || n0 >= N) return;
+  if (lvl >= s.n_lin || (MODE == 0 ? d.f_mb < 0 : d.b_mb < 0) || m0 >= M || n0 >= N ||
+      (MODE == 1 && p == 0 && lvl == 0 && s.pre != PRE_EMBED)) {          // raw network inputs need no gradient
+    pdl_wait();
+    return;
+  }
 
   // operand sources
   const float* asrc = MODE == 0 ? lin_input<float>(t, s, d, lvl, true) : dz_src<float>(t, s, d, lvl);
@@ -458,14 +459,16 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = lane & 7, ty = lane >> 3;
   float* mine = f32_sm + warp * NBUF * C::kBuf;
   const int chunks = (K + KC - 1) / KC;
-  auto load = [&](int c, float* buf) {
+  auto load_b = [&](int c, float* buf) {
+    if (c >= chunks) return;
+    if (MODE == 0) f32_load_kc<BN>(buf + C::kA, bsrc, ldb, n0, N, c * KC, K, vb, lane);
+    else f32_load_nc<BN>(buf + C::kA, bsrc, ldb, n0, N, c * KC, K, vb, lane);
+    if (corr) f32_load_nc<BN>(buf + C::kA + C::kB, dl, ldb, n0, N, c * KC, K, vb, lane);
+  };
+  auto load_a = [&](int c, float* buf) {                   // closes the chunk's group of copies
     if (c < chunks) {
-      const int k0 = c * KC;
-      if (MODE == 0) f32_load_kc<BN>(buf + C::kA, bsrc, ldb, n0, N, k0, K, vb, lane);
-      else f32_load_nc<BN>(buf + C::kA, bsrc, ldb, n0, N, k0, K, vb, lane);
-      if (corr) f32_load_nc<BN>(buf + C::kA + C::kB, dl, ldb, n0, N, k0, K, vb, lane);
-      if (MODE == 2) f32_load_nc<BM>(buf, asrc, lda, m0, M, k0, K, va, lane);
-      else f32_load_kc<BM>(buf, asrc, lda, m0, M, k0, K, va, lane);
+      if (MODE == 2) f32_load_nc<BM>(buf, asrc, lda, m0, M, c * KC, K, va, lane);
+      else f32_load_kc<BM>(buf, asrc, lda, m0, M, c * KC, K, va, lane);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -479,8 +482,13 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
   for (int i = 0; i < TM; ++i) rows[i] = 0.f;
   const bool bias_tile = MODE == 2 && n0 == 0;
 
+  // weights and delta are written by no launch of this phase: their copies start before the predecessor has ended
+  if (MODE == 2) pdl_wait();
 #pragma unroll
-  for (int b = 0; b < NBUF; ++b) load(warp + 8 * b, mine + b * C::kBuf);
+  for (int b = 0; b < NBUF; ++b) load_b(warp + 8 * b, mine + b * C::kBuf);
+  if (MODE != 2) pdl_wait();
+#pragma unroll
+  for (int b = 0; b < NBUF; ++b) load_a(warp + 8 * b, mine + b * C::kBuf);
   int slot = 0;
   for (int c = warp; c < chunks; c += 8) {
     asm volatile("cp.async.wait_group %0;" :: "n"(NBUF - 1) : "memory");
@@ -540,7 +548,8 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
           acc[i][j] = __fadd_rn(acc[i][j], fmaf(av[i][3], bv[j][3], fmaf(av[i][2], bv[j][2], fmaf(av[i][1], bv[j][1], __fmul_rn(av[i][0], bv[j][0])))));
     }
     __syncwarp();
-    load(c + 8 * NBUF, buf);
+    load_b(c + 8 * NBUF, buf);
+    load_a(c + 8 * NBUF, buf);
     if (++slot == NBUF) slot = 0;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -596,8 +605,7 @@ static cudaError_t launch_f32_t(const TickArgs& t, int lvl, int grid_m, cudaStre
   using C = F32Cfg<TM, TN, NBUF, MODE>;
   const int tiles_n = (t.max_dim + C::BN - 1) / C::BN, tiles_m = (grid_m + C::BM - 1) / C::BM;
   dim3 grid((unsigned)tiles_m * (unsigned)tiles_n, t.sel_p >= 0 ? 1 : t.P);
-  f32_gemm_kernel<TM, TN, NBUF, MODE><<<grid, 256, C::kBytes, stream>>>(t, lvl, tiles_n);
-  return cudaGetLastError();
+  return launch_pdl(f32_gemm_kernel<TM, TN, NBUF, MODE>, grid, dim3(256), C::kBytes, stream, t.pdl, t, lvl, tiles_n);
 }
 
 // opt-in shared-memory sizes, on the current device

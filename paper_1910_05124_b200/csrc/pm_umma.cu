@@ -396,6 +396,8 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
@@ -613,6 +615,8 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
   cluster_sync_all();                                                 // barriers of both CTAs are initialised
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -844,6 +848,8 @@ umma_dgrad_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* _
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
@@ -1159,6 +1165,8 @@ umma_dgrad_pair_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const i
   cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
 
   // Two producer threads, each with its own cursor over the same (tile, k-block) sequence: warp 0 feeds the fp32
   // slab ring (w, delta), the last warp the dz ring.  Everything that is fixed for a tile is read once when the
@@ -1499,6 +1507,8 @@ umma_dgrad_pair128_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, cons
   cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+  pdl_wait();
 
   // Two producer threads, each with its own cursor over the same (tile, k-block) sequence: warp 0 feeds the fp32
   // staging ring (w, delta), the last warp the dz ring.  Their k-block loops are the critical path of the kernel
@@ -2120,19 +2130,20 @@ cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cu
   }
   TickArgs ta = t;
   ta.sel_tile0 = tile0;
+  auto go = [&](auto kernel, int threads, int smem) {
+    return launch_pdl(kernel, dim3(grid), dim3(threads), smem, stream, t.pdl, ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
+  };
   if (plan->pair[mode][lvl]) {
-    if (mode == 0) umma_pair_gemm_kernel<0><<<grid, P2_THREADS, P2_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-    else if (mode == 1) umma_dgrad_pair_kernel<<<grid, DP_THREADS, DP_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-    else if (mode == 3) umma_dgrad_pair128_kernel<<<grid, D1_THREADS, D1_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-    else if (mode == 4) umma_pair_gemm_kernel<1><<<grid, P2_THREADS, P2_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-    else umma_pair_gemm_kernel<2><<<grid, P2_THREADS, P2_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-    return cudaGetLastError();
+    if (mode == 0) return go(umma_pair_gemm_kernel<0>, P2_THREADS, P2_SMEM_BYTES);
+    if (mode == 1) return go(umma_dgrad_pair_kernel, DP_THREADS, DP_SMEM_BYTES);
+    if (mode == 3) return go(umma_dgrad_pair128_kernel, D1_THREADS, D1_SMEM_BYTES);
+    if (mode == 4) return go(umma_pair_gemm_kernel<1>, P2_THREADS, P2_SMEM_BYTES);
+    return go(umma_pair_gemm_kernel<2>, P2_THREADS, P2_SMEM_BYTES);
   }
-  if (mode == 0) umma_gemm_kernel<0><<<grid, Cfg<0>::kThreads, Cfg<0>::kSmemBytes, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-  else if (mode == 1) umma_dgrad_kernel<<<grid, DG_THREADS, DG_SMEM_BYTES, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-  else if (mode == 4) umma_gemm_kernel<1><<<grid, Cfg<1>::kThreads, Cfg<1>::kSmemBytes, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-  else umma_gemm_kernel<2><<<grid, Cfg<2>::kThreads, Cfg<2>::kSmemBytes, stream>>>(ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
-  return cudaGetLastError();
+  if (mode == 0) return go(umma_gemm_kernel<0>, Cfg<0>::kThreads, Cfg<0>::kSmemBytes);
+  if (mode == 1) return go(umma_dgrad_kernel, DG_THREADS, DG_SMEM_BYTES);
+  if (mode == 4) return go(umma_gemm_kernel<1>, Cfg<1>::kThreads, Cfg<1>::kSmemBytes);
+  return go(umma_gemm_kernel<2>, Cfg<2>::kThreads, Cfg<2>::kSmemBytes);
 }
 
 }  // namespace pm

@@ -71,7 +71,6 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (threadIdx.x == 0) pdl_trigger();
   const int p = stage_of_block(t, blockIdx.y);
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -101,6 +100,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();                                               // behind the tensor-memory allocation: a successor's must not come first
   if (S > 1) cluster_arrive();                                 // "this CTA runs": awaited before anything is written into it
   const uint32_t tmem = *tmem_slot;
   const CUtensorMap* lm = maps + ((size_t)p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;

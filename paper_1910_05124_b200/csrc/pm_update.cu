@@ -303,17 +303,17 @@ __device__ __forceinline__ float4 ld_stream(const float* p) { return __ldcs(rein
 __device__ __forceinline__ void st_stream(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
 
 constexpr int kUpdThreads = 128;
-constexpr int kUpdUnroll = 2;      // float4 groups per thread per array in flight
 
 // What bounds the kernel: HBM.  One block per 1024 elements, in ascending order, and not a persistent grid: resident blocks then
 // work on one moving window of the arenas, where grid-stride blocks drift apart and the nine streams lose their DRAM pages.
 // 100 M parameters, Adam, 64 stages: 674 us with eight persistent blocks of 256 threads per SM, 633 with a block of 256 threads
 // per chunk, 615 when the look-up tries the stage an even split would give before it searches, 598 with blocks of 128 threads
-// (6.36 TB/s; one float4 per array and thread instead of two: 602).
+// (6.36 TB/s).  U: float4 groups per thread and array.  Two while there are many waves of blocks (one: 602 us); one for small
+// networks, where a launch is as long as a thread's chain of divisions (a tick of the 4-stage MLP 36.9 -> 34.8 us).
 
 // LP: operand-type copy of the new weights: 0 none, 1 bfloat16, 2 float (a version-ring slot of fp32 operands);
 // element e of the arenas goes to lp_base[lp_shift + e], lp_shift from the stage's table entry (0: the w_lp arena)
-template <int OPT, int LP>
+template <int OPT, int LP, int U>
 __global__ void __launch_bounds__(kUpdThreads, 6)
 update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restrict__ begin64, const uint32_t* __restrict__ end64,
               const StageDyn* __restrict__ dyn, int64_t* __restrict__ nupd, int n_stages, uint64_t total_vec4,
@@ -322,9 +322,10 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
   // ranges (one per stage, in 64-element groups) that another kernel has updated already: the Linear matrices, when the
   // weight-gradient GEMM applies the update in its epilogue
   const bool skip = skip_b64 != nullptr;
+  pdl_trigger();
   pdl_wait();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
-  const uint64_t base = first_vec4 + (uint64_t)blockIdx.x * kUpdThreads * kUpdUnroll;
+  const uint64_t base = first_vec4 + (uint64_t)blockIdx.x * kUpdThreads * U;
   // the stage of the block's first group: the largest i with begin64[i] <= g0 (every thread searches, on the same addresses)
   const uint32_t g0 = (uint32_t)(base >> 4);
   int lo0 = 0, hi = n_stages - 1;
@@ -335,15 +336,15 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
   while (lo0 < hi) { const int mid = (lo0 + hi + 1) >> 1; if (__ldg(begin64 + mid) <= g0) lo0 = mid; else hi = mid - 1; }
   if (skip) {
     // the whole span of this block lies inside a skipped range (and past the stage's first group): nothing to do
-    const uint32_t g1 = (uint32_t)((base + (uint64_t)kUpdThreads * kUpdUnroll - 1) >> 4);
+    const uint32_t g1 = (uint32_t)((base + (uint64_t)kUpdThreads * U - 1) >> 4);
     if (skip_b64[lo0] <= g0 && g1 < skip_e64[lo0] && g0 > begin64[lo0]) return;
   }
-  uint64_t v[kUpdUnroll];
-  int stage[kUpdUnroll];
-  UpdScalars sc[kUpdUnroll];
-  float4 g[kUpdUnroll], w[kUpdUnroll], m[kUpdUnroll], dl[kUpdUnroll], s[kUpdUnroll];
+  uint64_t v[U];
+  int stage[U];
+  UpdScalars sc[U];
+  float4 g[U], w[U], m[U], dl[U], s[U];
 #pragma unroll
-  for (int u = 0; u < kUpdUnroll; ++u) {
+  for (int u = 0; u < U; ++u) {
     v[u] = base + (uint64_t)u * kUpdThreads + threadIdx.x;
     stage[u] = -1;
     if (v[u] < total_vec4) {
@@ -370,7 +371,7 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
     }
   }
 #pragma unroll
-  for (int u = 0; u < kUpdUnroll; ++u) {
+  for (int u = 0; u < U; ++u) {
     if (stage[u] < 0) continue;
     const uint64_t e = v[u] * 4;
     float4 wn;
@@ -421,14 +422,15 @@ cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* 
   if (total64 == 0 || n_stages == 0 || first64 >= total64) return cudaSuccess;
   uint64_t total_vec4 = total64 * 16;
   const uint64_t first_vec4 = first64 * 16;
-  const uint64_t per_block = (uint64_t)kUpdThreads * kUpdUnroll;
+  const bool small = total_vec4 - first_vec4 <= 4ull * 148 * 8 * kUpdThreads;      // up to four waves of blocks
+  const uint64_t per_block = (uint64_t)kUpdThreads * (small ? 1 : 2);
   const unsigned blocks = (unsigned)((total_vec4 - first_vec4 + per_block - 1) / per_block);   // 1024 elements per block: 2^31 blocks are 2e12 elements
   // the operand-type copy: the w_lp arena (bfloat16) unless the caller names a version ring and its element size
   if (lp_base == nullptr) { lp_base = a.w_lp; lp_elem = 2; }
   if (gsrc == nullptr) gsrc = a.grad;
   const int lp = lp_base == nullptr ? 0 : (lp_elem == 4 ? 2 : 1);
   const float per_group = (float)n_stages / (float)total64;
-#define PM_UPD(OPT, LP) launch_pdl(update_kernel<OPT, LP>, dim3(blocks), dim3(kUpdThreads), 0, stream, pdl, a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc, per_group)
+#define PM_UPD(OPT, LP) launch_pdl(small ? update_kernel<OPT, LP, 1> : update_kernel<OPT, LP, 2>, dim3(blocks), dim3(kUpdThreads), 0, stream, pdl, a, lp_base, begin64, end64, dyn, nupd, n_stages, total_vec4, beta1, beta2, eps, first_vec4, skip_b64, skip_e64, gsrc, per_group)
   if (optimizer == PM_SGDM) return lp == 0 ? PM_UPD(PM_SGDM, 0) : (lp == 1 ? PM_UPD(PM_SGDM, 1) : PM_UPD(PM_SGDM, 2));
   return lp == 0 ? PM_UPD(PM_ADAM, 0) : (lp == 1 ? PM_UPD(PM_ADAM, 1) : PM_UPD(PM_ADAM, 2));
 #undef PM_UPD
@@ -439,6 +441,8 @@ cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* 
 // order their versions sit in a ring of their own, filled here from the master weights after every update.
 __global__ void __launch_bounds__(128) push_small_kernel(const float* __restrict__ w, const float* __restrict__ delta, char* __restrict__ ring,
                                                          const SmallSeg* __restrict__ segs, int n_segs, const StageDyn* __restrict__ dyn, int slot_override) {
+  pdl_trigger();
+  pdl_wait();
   for (int sg = blockIdx.x; sg < n_segs; sg += gridDim.x) {
     const SmallSeg g = segs[sg];
     if (slot_override < 0 && !dyn[g.stage].active_update) continue;          // the stage was not updated this tick
@@ -468,10 +472,9 @@ __global__ void __launch_bounds__(128) push_small_kernel(const float* __restrict
 }
 
 cudaError_t launch_push_small(const float* w, const float* delta, char* ring, const SmallSeg* segs, int n_segs, const StageDyn* dyn,
-                              int slot_override, cudaStream_t stream) {
+                              int slot_override, cudaStream_t stream, bool pdl) {
   if (n_segs == 0) return cudaSuccess;
-  push_small_kernel<<<n_segs < 1184 ? n_segs : 1184, 128, 0, stream>>>(w, delta, ring, segs, n_segs, dyn, slot_override);
-  return cudaGetLastError();
+  return launch_pdl(push_small_kernel, dim3(n_segs < 1184 ? n_segs : 1184), dim3(128), 0, stream, pdl, w, delta, ring, segs, n_segs, dyn, slot_override);
 }
 
 }  // namespace pm

@@ -57,6 +57,6 @@ struct SmallSeg { uint64_t arena_off, ring_off; uint32_t count, slot_stride; int
 // corrected recompute weights, w - dyn[stage].rc_gap * delta into slot dyn[stage].rc_uslot.  slot_override >= 0 (the
 // initial fill, delta = 0): plain copies into that slot and into rc_base + slot_override.
 cudaError_t launch_push_small(const float* w, const float* delta, char* ring, const SmallSeg* segs, int n_segs, const StageDyn* dyn,
-                              int slot_override, cudaStream_t stream);
+                              int slot_override, cudaStream_t stream, bool pdl = false);
 
 }  // namespace pm

@@ -67,6 +67,8 @@ __device__ __forceinline__ void ln_fwd_row(const TickArgs& t, const StageDev& s,
 
 template <typename AT>
 __global__ void __launch_bounds__(256) pre_fwd_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = t.pre_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -159,14 +161,14 @@ __global__ void __launch_bounds__(256) pre_fwd_kernel(TickArgs t) {
 
 cudaError_t launch_pre_fwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   dim3 grid((t.T + 7) / 8, t.n_pre);
-  if (dtype == PM_F32) pre_fwd_kernel<float><<<grid, 256, 0, stream>>>(t);
-  else pre_fwd_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(t);
-  return cudaGetLastError();
+  return launch_pdl(dtype == PM_F32 ? pre_fwd_kernel<float> : pre_fwd_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, t.pdl, t);
 }
 
 // ---- residual add: next stage's input = skip + y --------------------------------------------------------------
 template <typename AT>
 __global__ void __launch_bounds__(256) residual_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = t.res_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -208,6 +210,8 @@ struct AttnShape { int S, dk, d; };
 
 template <typename AT>
 __global__ void __launch_bounds__(256) attention_fwd_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = stage_of_block(t, blockIdx.y);
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -283,16 +287,13 @@ cudaError_t launch_post_fwd(const TickArgs& t, int dtype, cudaStream_t stream, b
   cudaError_t e = cudaSuccess;
   if (any_att) {
     dim3 grid(nblk, t.sel_p >= 0 ? 1 : t.P);
-    if (dtype == PM_F32) attention_fwd_kernel<float><<<grid, 256, attn_fwd_smem(S, dk, 4), stream>>>(t);
-    else attention_fwd_kernel<__nv_bfloat16><<<grid, 256, attn_fwd_smem(S, dk, 2), stream>>>(t);
-    e = cudaGetLastError();
+    e = dtype == PM_F32 ? launch_pdl(attention_fwd_kernel<float>, grid, dim3(256), attn_fwd_smem(S, dk, 4), stream, t.pdl, t)
+                        : launch_pdl(attention_fwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_fwd_smem(S, dk, 2), stream, t.pdl, t);
     if (e != cudaSuccess) return e;
   }
   if (any_res) {
     dim3 grid(t.sel_p >= 0 ? 592 : 64, t.n_res);          // a launch of one stage brings all the blocks itself
-    if (dtype == PM_F32) residual_kernel<float><<<grid, 256, 0, stream>>>(t);
-    else residual_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(t);
-    e = cudaGetLastError();
+    e = launch_pdl(dtype == PM_F32 ? residual_kernel<float> : residual_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, t.pdl, t);
   }
   return e;
 }
@@ -302,6 +303,8 @@ cudaError_t launch_post_fwd(const TickArgs& t, int dtype, cudaStream_t stream, b
 // dQ = dS K / sqrt(d_k); dK = dS^T Q / sqrt(d_k).  Results go to the stage's dy buffer as [dq | dk | dv].
 template <typename AT>
 __global__ void __launch_bounds__(256) attention_bwd_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = stage_of_block(t, blockIdx.y);
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -382,9 +385,8 @@ __global__ void __launch_bounds__(256) attention_bwd_kernel(TickArgs t) {
 cudaError_t launch_post_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   if (t.att_blocks <= 0) return cudaSuccess;
   dim3 grid(t.att_blocks, t.sel_p >= 0 ? 1 : t.P);
-  if (dtype == PM_F32) attention_bwd_kernel<float><<<grid, 256, attn_bwd_smem(t.att_S, t.att_dk, 4), stream>>>(t);
-  else attention_bwd_kernel<__nv_bfloat16><<<grid, 256, attn_bwd_smem(t.att_S, t.att_dk, 2), stream>>>(t);
-  return cudaGetLastError();
+  return dtype == PM_F32 ? launch_pdl(attention_bwd_kernel<float>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 4), stream, t.pdl, t)
+                         : launch_pdl(attention_bwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 2), stream, t.pdl, t);
 }
 
 cudaError_t attention_set_smem_limits(int S, int dk, int dtype) {
@@ -400,14 +402,16 @@ cudaError_t attention_set_smem_limits(int S, int dk, int dtype) {
 }
 
 // ---- loss reduction shared by the cross-entropy kernels ----
-// per-token loss of this block's row; the last block to arrive adds all of them in a fixed order (strided per-thread
+// per-token losses of this block's rows (ce_row_loss); the last block to arrive adds all of them in a fixed order (strided per-thread
 // partials over the first 256 threads, then a fixed tree).  Called by every thread of the block.
-__device__ __forceinline__ void ce_finish(const TickArgs& t, const StageDyn& d, int row, float mx, float sum, float logit_tgt) {
+__device__ __forceinline__ void ce_row_loss(const TickArgs& t, int row, float mx, float sum, float logit_tgt) {
+  if (threadIdx.x == 0) ws_at<float>(t, t.rowloss_off)[row] = (mx + logf(sum)) - logit_tgt;
+}
+__device__ __forceinline__ void ce_finish(const TickArgs& t, const StageDyn& d) {
   float* rowloss = ws_at<float>(t, t.rowloss_off);
   unsigned int* counter = reinterpret_cast<unsigned int*>(ws_at<float>(t, t.lossred_off) + 64);
   __shared__ bool last;
   if (threadIdx.x == 0) {
-    rowloss[row] = (mx + logf(sum)) - logit_tgt;
     __threadfence();
     last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
@@ -448,6 +452,8 @@ template <> __device__ __forceinline__ float ce_div<__nv_bfloat16>(float e, floa
 // gradient.  The last block to finish adds the per-token losses in a fixed order.
 template <typename AT>
 __global__ void __launch_bounds__(256) ce_loss_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const StageDyn& d = t.dyn[t.P - 1];
   if (d.b_mb < 0) return;
   const StageDev& sl = t.st[t.P - 1];
@@ -542,7 +548,8 @@ __global__ void __launch_bounds__(256) ce_loss_kernel(TickArgs t) {
       dl[c] = from_f<AT>(pr * invT);
     }
   }
-  ce_finish(t, d, row, mx, sum, lg[tgt]);
+  ce_row_loss(t, row, mx, sum, lg[tgt]);
+  ce_finish(t, d);
 }
 
 // Rows longer than the register path holds (a vocabulary of tens of thousands): 512 threads read the fp32 row once
@@ -558,6 +565,8 @@ template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16*
 
 template <typename AT>
 __global__ void __launch_bounds__(kCeLongThreads) ce_loss_long_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const StageDyn& d = t.dyn[t.P - 1];
   if (d.b_mb < 0) return;
   const StageDev& sl = t.st[t.P - 1];
@@ -619,29 +628,106 @@ __global__ void __launch_bounds__(kCeLongThreads) ce_loss_long_kernel(TickArgs t
     if (tgt == c + 3) p3 -= 1.0f;
     store4<AT>(dl + c, p0 * invT, p1 * invT, p2 * invT, p3 * invT);
   }
-  ce_finish(t, d, row, mx, sum, logit_tgt);
+  ce_row_loss(t, row, mx, sum, logit_tgt);
+  ce_finish(t, d);
+}
+
+// The same for rows of up to 32 * 1024 logits (a multiple of four), with the same arithmetic in the same order.  What bounds
+// it is HBM (the logits once, their gradients once), but a block per row spends most of its life on exponentials and
+// writes while no load is in flight, and only one row fits an SM.  Here a block stays on its SM and walks rows: the
+// row moves from shared memory to registers (32 values per thread), and the next row's copies start before the first
+// exponential of this one.
+template <typename AT>
+__global__ void __launch_bounds__(kCeLongThreads, 1) ce_loss_rows_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
+  const StageDyn& d = t.dyn[t.P - 1];
+  if (d.b_mb < 0) return;
+  const StageDev& sl = t.st[t.P - 1];
+  const int V = t.n_out_last, n4 = V >> 2;
+  const uint64_t n = (uint64_t)t.T * V;
+  const float* logits = ws_at<float>(t, t.yout_off) + (uint64_t)((d.tick + 1) & 1) * n;
+  const int32_t* tgts = ws_at<int32_t>(t, t.tgt_off) + (uint64_t)(d.b_mb % (t.P + 1)) * t.T;
+  AT* grads = gin_read<AT>(t, sl, d);
+  extern __shared__ float4 rowbuf[];                         // [V / 4]
+  __shared__ float red[2][kCeLongThreads / 32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float invT = t.loss_scale / (float)t.T;
+  auto fetch = [&](int row) {
+    const float4* src = reinterpret_cast<const float4*>(logits + (uint64_t)row * V);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rowbuf);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = tid + u * kCeLongThreads;
+      if (i < n4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 16u * (uint32_t)i), "l"(src + i) : "memory");
+    }
+  };
+  if ((int)blockIdx.x < t.T) fetch(blockIdx.x);
+  for (int row = blockIdx.x; row < t.T; row += gridDim.x) {
+    const int32_t tgt = tgts[row];
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    float4 q[8];                                             // this thread copied these very values: no barrier needed to read them
+    float mx = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = tid + u * kCeLongThreads;
+      if (i < n4) {
+        q[u] = rowbuf[i];
+        mx = fmaxf(fmaxf(mx, fmaxf(q[u].x, q[u].y)), fmaxf(q[u].z, q[u].w));
+      }
+    }
+    mx = warp_max(mx);
+    if (lane == 0) red[0][warp] = mx;
+    __syncthreads();                                         // maxima visible; the row has been read (but for the target's logit)
+    mx = warp_max(red[0][lane]);
+    float logit_tgt = 0.f;
+    if (tid == 0) logit_tgt = reinterpret_cast<const float*>(rowbuf)[tgt];
+    float sum = 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (tid + u * kCeLongThreads < n4) {
+        q[u].x = ce_exp<AT>(q[u].x - mx); q[u].y = ce_exp<AT>(q[u].y - mx); q[u].z = ce_exp<AT>(q[u].z - mx); q[u].w = ce_exp<AT>(q[u].w - mx);
+        sum += q[u].x; sum += q[u].y; sum += q[u].z; sum += q[u].w;
+      }
+    sum = warp_sum(sum);
+    if (lane == 0) red[1][warp] = sum;
+    __syncthreads();                                         // sums visible; the target's logit has been read: the buffer is free
+    if (row + (int)gridDim.x < t.T) fetch(row + gridDim.x);
+    sum = 0.f;
+    for (int w = 0; w < kCeLongThreads / 32; ++w) sum += red[1][w];
+    const float rsum = 1.0f / sum;
+    AT* dl = grads + (uint64_t)row * V;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = tid + u * kCeLongThreads, c = 4 * i;
+      if (i < n4) {
+        float p0 = ce_div<AT>(q[u].x, sum, rsum), p1 = ce_div<AT>(q[u].y, sum, rsum), p2 = ce_div<AT>(q[u].z, sum, rsum), p3 = ce_div<AT>(q[u].w, sum, rsum);
+        if (tgt == c) p0 -= 1.0f;
+        if (tgt == c + 1) p1 -= 1.0f;
+        if (tgt == c + 2) p2 -= 1.0f;
+        if (tgt == c + 3) p3 -= 1.0f;
+        store4<AT>(dl + c, p0 * invT, p1 * invT, p2 * invT, p3 * invT);
+      }
+    }
+    ce_row_loss(t, row, mx, sum, logit_tgt);
+  }
+  ce_finish(t, d);
 }
 
 cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
   const int V = t.n_out_last;
   const size_t row_bytes = sizeof(float) * (size_t)V;
   if (V > 8192 && (V & 3) == 0 && row_bytes <= 200 * 1024) {
-    static bool attr_set[2] = {false, false};
-    const int which = dtype == PM_F32 ? 0 : 1;
-    if (!attr_set[which]) {
-      cudaError_t e = dtype == PM_F32
-          ? cudaFuncSetAttribute((const void*)ce_loss_long_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)
-          : cudaFuncSetAttribute((const void*)ce_loss_long_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (e != cudaSuccess) return e;
-      attr_set[which] = true;
-    }
-    if (dtype == PM_F32) ce_loss_long_kernel<float><<<t.T, kCeLongThreads, row_bytes, stream>>>(t);
-    else ce_loss_long_kernel<__nv_bfloat16><<<t.T, kCeLongThreads, row_bytes, stream>>>(t);
-    return cudaGetLastError();
+    const bool rows = V <= 32 * kCeLongThreads;              // longer rows do not fit a block's registers
+    auto* kernel = rows ? (dtype == PM_F32 ? ce_loss_rows_kernel<float> : ce_loss_rows_kernel<__nv_bfloat16>)
+                        : (dtype == PM_F32 ? ce_loss_long_kernel<float> : ce_loss_long_kernel<__nv_bfloat16>);
+    cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_bytes);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); sms = 148; }
+    return launch_pdl(kernel, dim3(rows ? std::min(sms, (int)t.T) : t.T), dim3(kCeLongThreads), row_bytes, stream, t.pdl, t);
   }
-  if (dtype == PM_F32) ce_loss_kernel<float><<<t.T, 256, 0, stream>>>(t);
-  else ce_loss_kernel<__nv_bfloat16><<<t.T, 256, 0, stream>>>(t);
-  return cudaGetLastError();
+  return launch_pdl(dtype == PM_F32 ? ce_loss_kernel<float> : ce_loss_kernel<__nv_bfloat16>, dim3(t.T), dim3(256), 0, stream, t.pdl, t);
 }
 
 // ---- pre-op backward --------------------------------------------------------------------------------------------
@@ -657,6 +743,8 @@ __device__ __forceinline__ float du_total(const AT* du, const AT* gs, uint64_t i
 //   dxhat = du_total * gain_b (gain_b = gain - gap*delta: T2);  dx = rstd * (dxhat - mean(dxhat) - xhat * mean(dxhat*xhat))
 template <typename AT>
 __global__ void __launch_bounds__(256) ln_bwd_dx_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = t.ln_ids[blockIdx.y + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -735,6 +823,8 @@ constexpr int kLnCols = 256;                         // columns per block: 8 per
 
 template <typename AT>
 __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = t.ln_ids[blockIdx.z + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -802,6 +892,8 @@ __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
 }
 
 __global__ void __launch_bounds__(256) ln_param_finish_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int p = t.ln_ids[blockIdx.y + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -826,6 +918,8 @@ __global__ void __launch_bounds__(256) ln_param_finish_kernel(TickArgs t) {
 // per-block partials in block order by ln_fused_finish_kernel.
 template <typename AT, int NP, int WPR>
 __global__ void __launch_bounds__(256, NP <= 2 ? 2 : 1) ln_bwd_fused_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int li = blockIdx.y + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -987,6 +1081,8 @@ __global__ void __launch_bounds__(256, NP <= 2 ? 2 : 1) ln_bwd_fused_kernel(Tick
 constexpr int kLnFinCols = 32, kLnFinPer = 16;
 
 __global__ void __launch_bounds__(256) ln_fused_finish_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   const int li = blockIdx.y + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -1034,9 +1130,9 @@ static cudaError_t launch_ln_fused(const TickArgs& t, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
-  ln_bwd_fused_kernel<AT, NP, WPR><<<dim3(t.ln_chunks, t.n_ln), 256, smem, stream>>>(ta);
-  if (!t.defer_finish) ln_fused_finish_kernel<<<dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), 256, 0, stream>>>(t);
-  return cudaGetLastError();
+  const cudaError_t e = launch_pdl(ln_bwd_fused_kernel<AT, NP, WPR>, dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, t.pdl, ta);
+  if (e != cudaSuccess || t.defer_finish) return e;
+  return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, t.pdl, t);
 }
 
 // Embedding gradient: dTable[v] = sqrt(d) * sum over tokens t with id[t] == v (ascending t) of du_total[t].
@@ -1106,6 +1202,8 @@ __device__ __forceinline__ void embed_gather(const int32_t* sub, int k_lo, int k
 
 template <typename AT, int CPL>
 __global__ void __launch_bounds__(256) embed_bwd_kernel(TickArgs t) {
+  pdl_trigger();
+  pdl_wait();
   constexpr int kEmbCols = 32 * CPL;
   const int p = t.embed_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
@@ -1245,9 +1343,9 @@ int pre_bwd_launches(const TickArgs& t) {
 int ln_finish_launches(const TickArgs& t) { return t.any_ln && (t.ln_fused || t.row_chunks > 1) ? 1 : 0; }
 cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream) {
   if (!t.any_ln) return cudaSuccess;
-  if (t.ln_fused) ln_fused_finish_kernel<<<dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), 256, 0, stream>>>(t);
-  else if (t.row_chunks > 1) ln_param_finish_kernel<<<dim3((t.max_ln_dim + 255) / 256, t.n_ln), 256, 0, stream>>>(t);
-  return cudaGetLastError();
+  if (t.ln_fused) return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, t.pdl, t);
+  if (t.row_chunks > 1) return launch_pdl(ln_param_finish_kernel, dim3((t.max_ln_dim + 255) / 256, t.n_ln), dim3(256), 0, stream, t.pdl, t);
+  return cudaSuccess;
 }
 
 cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
@@ -1258,14 +1356,12 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
   } else if (t.any_ln) {
     dim3 g1((t.T + 7) / 8, t.n_ln), g2((t.max_ln_dim + kLnCols - 1) / kLnCols, t.row_chunks, t.n_ln);
-    if (dtype == PM_F32) { ln_bwd_dx_kernel<float><<<g1, 256, 0, stream>>>(t); ln_bwd_param_kernel<float><<<g2, 256, 0, stream>>>(t); }
-    else { ln_bwd_dx_kernel<__nv_bfloat16><<<g1, 256, 0, stream>>>(t); ln_bwd_param_kernel<__nv_bfloat16><<<g2, 256, 0, stream>>>(t); }
-    e = cudaGetLastError();
+    e = launch_pdl(dtype == PM_F32 ? ln_bwd_dx_kernel<float> : ln_bwd_dx_kernel<__nv_bfloat16>, g1, dim3(256), 0, stream, t.pdl, t);
+    if (e == cudaSuccess) e = launch_pdl(dtype == PM_F32 ? ln_bwd_param_kernel<float> : ln_bwd_param_kernel<__nv_bfloat16>, g2, dim3(256), 0, stream, t.pdl, t);
     if (e != cudaSuccess) return e;
     if (t.row_chunks > 1 && !t.defer_finish) {
       dim3 g3((t.max_ln_dim + 255) / 256, t.n_ln);
-      ln_param_finish_kernel<<<g3, 256, 0, stream>>>(t);
-      e = cudaGetLastError();
+      e = launch_pdl(ln_param_finish_kernel, g3, dim3(256), 0, stream, t.pdl, t);
       if (e != cudaSuccess) return e;
     }
   }
@@ -1285,8 +1381,7 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
         cudaError_t ea = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (ea != cudaSuccess) return ea;
       }
-      kernel<<<g, 256, smem, stream>>>(t);
-      return cudaGetLastError();
+      return launch_pdl(kernel, g, dim3(256), smem, stream, t.pdl, t);
     };
     if (dtype == PM_F32) e = cpl == 16 ? go(embed_bwd_kernel<float, 16>) : (cpl == 8 ? go(embed_bwd_kernel<float, 8>) : go(embed_bwd_kernel<float, 4>));
     else e = cpl == 16 ? go(embed_bwd_kernel<__nv_bfloat16, 16>) : (cpl == 8 ? go(embed_bwd_kernel<__nv_bfloat16, 8>) : go(embed_bwd_kernel<__nv_bfloat16, 4>));

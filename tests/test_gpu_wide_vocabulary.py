@@ -1,0 +1,57 @@
+"""Vocabularies much larger than the microbatch: the embedding gradient that zeroes the table and sums the rows of the tokens
+that occur, and the cross-entropy that walks long rows of logits."""
+import numpy as np
+import pytest
+
+import pm_inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+# a microbatch of fewer, as many and more tokens than one pass of a warp or a block looks at (32, 256); a quarter of the
+# vocabulary and less; widths of one and several column slices, and one that leaves lanes without a column; ids all equal
+# (one row summed by eight warps), from a few values (rows of both kinds, every token repeated) and all over the table;
+# vocabularies at the ends of the long cross-entropy rows (8192 excluded, 32768, and one beyond it that takes the other kernel)
+@pytest.mark.parametrize("d_model,seq,batch,vocab,ids", [(64, 8, 4, 8196, "uniform"), (64, 8, 5, 8200, "equal"), (72, 16, 17, 9000, "few"),
+                                                         (264, 16, 16, 16384, "few"), (520, 32, 20, 32768, "uniform"), (128, 16, 8, 33000, "equal")])
+@pytest.mark.parametrize("compute", ["f32", "bf16"])
+def test_embedding_gradient_and_loss(cuda_device, compute, d_model, seq, batch, vocab, ids):
+    import torch
+    import paper_1910_05124_b200 as pm
+    if compute == "bf16":
+        vocab = (vocab + 7) // 8 * 8
+    wl = I.encoder_workload("wide", 1, d_model, {264: 6, 520: 13}.get(d_model, 2), 64, seq, batch, vocab, compute=compute, optimizer="sgdm", alpha=0.01,
+                            K=4, D=0.5, steps=1, seed=5)
+    params0 = I.init_encoder_params(wl)
+    pipe = pm.Pipeline(wl, params0, loop_order="mb_major")
+    gen = torch.Generator().manual_seed(vocab + d_model)
+    T = seq * batch
+    tok = {"uniform": torch.randint(0, vocab, (T,), generator=gen), "equal": torch.full((T,), vocab - 1),
+           "few": torch.randint(0, 12, (T,), generator=gen) * (vocab // 12)}[ids].int()
+    tgt = torch.randint(0, vocab, (T,), generator=gen).int()
+    pipe.grad.fill_(7.0)                                             # what an earlier step left in the arena
+    pipe.pm_forward(tok.cuda(), tgt.cuda())
+    pipe.pm_backward()
+    table = pipe.unpack(pipe.grad)[0][0]
+    pipe.pm_update()
+    hit = np.zeros(vocab, bool)
+    hit[tok.numpy()] = True
+    assert not table[~hit].any()                                     # rows without a token: zeros, not what was there
+    assert np.isfinite(table[hit]).all()
+    # the gradient of the table summed over its rows is sqrt(d) times the sum of du over the tokens, whatever the ids: the same
+    # network on ids spread over the table, with the embedding of the tokens it replaces, gives the same du
+    spread = torch.arange(T).int() * (vocab // T)
+    p1 = [list(st) for st in params0]
+    p1[0][0] = np.zeros_like(p1[0][0])
+    p1[0][0][spread.numpy()] = params0[0][0][tok.numpy()]
+    other = pm.Pipeline(wl, p1, loop_order="mb_major")
+    other.pm_forward(spread.cuda(), tgt.cuda())
+    other.pm_backward()
+    rows = torch.from_numpy(other.unpack(other.grad)[0][0][spread.numpy()]).double()
+    other.pm_update()
+    ref = torch.zeros(vocab, d_model, dtype=torch.float64).index_add_(0, tok.long(), rows)
+    # fp32 sums of at most T terms against float64, relative to the terms: T 2^-24; the two runs' du are the same bits
+    scale = torch.zeros(vocab, d_model, dtype=torch.float64).index_add_(0, tok.long(), rows.abs())
+    assert ((torch.from_numpy(table).double() - ref).abs() <= T * 2.0 ** -24 * scale + 1e-30).all()
+    loss = pipe.pm_get_losses(0, 1)[0]
+    assert abs(loss - other.pm_get_losses(0, 1)[0]) <= 1e-6 * loss
