@@ -626,7 +626,7 @@ def rooflines(res, peaks, steps):
         if wl.compute == "f32":
             # fp32 path: plain FFMA on the CUDA cores; peak derived from unit counts and clocks:
             # 148 SMs x 128 lanes x 2 flop x 1.965 GHz = 74.4 TFLOP/s
-            out[cls] = {"kernel": "simt_gemm_kernel (" + cls + ")", "bound": "alu", "achieved": round(tfs, 3), "peak": 74.4,
+            out[cls] = {"kernel": "f32_gemm_kernel (" + cls + ")", "bound": "alu", "achieved": round(tfs, 3), "peak": 74.4,
                         "unit": "TFLOP/s", "frac": round(tfs / 74.4, 5), "of": "derived (148 SMs x 128 FFMA lanes x 1.965 GHz)",
                         "traffic": None, "avg_ms_per_step": round(per_tick[cls], 5), "share_of_step": share,
                         "note": "46 MFLOP per step: launch-latency bound, not arithmetic bound"}

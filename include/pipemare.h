@@ -330,7 +330,8 @@ pm_status pm_selftest_wait_timeout(pm_ctx* ctx, int64_t limit_cycles);
 /* Optional timing of the tick's kernels by class, with CUDA events recorded on the context's stream around each
  * launch (up to 8192 launches between reads; later ones are not recorded).  pm_profile_read synchronises the
  * stream, writes the summed milliseconds and the number of timed launches per class (arrays of PM_PROF_CLASSES
- * entries) and clears the record. */
+ * entries) and clears the record.  The copy of the microbatch shares the schedule's launch and is timed with it
+ * (PM_PROF_SCHEDULE); PM_PROF_INGEST stays zero. */
 enum { PM_PROF_SCHEDULE = 0, PM_PROF_INGEST, PM_PROF_PRE_FWD, PM_PROF_GEMM_FWD, PM_PROF_ATTN_FWD, PM_PROF_POST_FWD,
        PM_PROF_LOSS, PM_PROF_ATTN_BWD, PM_PROF_ACT_BWD, PM_PROF_WGRAD, PM_PROF_DGRAD, PM_PROF_PRE_BWD, PM_PROF_UPDATE,
        PM_PROF_CLASSES };

@@ -1792,6 +1792,8 @@ struct UmmaPlan {
   int P = 0;
   // launches of one stage (microbatch-major order): the stage's tiles in ascending order are a slice of the identity list
   std::vector<int> h_tile_start;         // host copy of the tile starts
+  RowShape row[2][PM_MAX_LINEARS];       // launches over all stages (forward, dgrad) with few tiles: pm_umma_row.cuh
+  int row_n[2][PM_MAX_LINEARS] = {};
   std::vector<StageDev> st;              // host copy of the stages (launches of one stage with few tiles)
   const int* d_identity = nullptr;       // 0, 1, 2, ...
   int max_ctas = 148;
@@ -2064,6 +2066,8 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   plan->h_tile_start = tt.tile_start;
   plan->max_ctas = device_sms();
   plan->st = st;
+  for (int mode = 0; mode < 2; ++mode)
+    for (int l = 0; l < PM_MAX_LINEARS; ++l) plan->row[mode][l] = row_grouped_shape(t.T, st, mode, l, &plan->row_n[mode][l]);
   *out = plan;
   return PM_OK;
 }
@@ -2099,12 +2103,15 @@ cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cu
   if (t.sel_p >= 0 && mode != 2) {
     const LinDev& L = plan->st[t.sel_p].lin[lvl];
     const int N = mode == 0 ? L.n_out : L.n_in;
-    const RowShape r = mode == 0 ? row_shape(t.T, N, L.n_in, 1) : row_dgrad_shape(t.T, N, L.n_out);
+    const RowShape r = mode == 0 ? row_shape(t.T, N, L.n_in) : row_dgrad_shape(t.T, N, L.n_out);
     if (r.bn != 0)
       return mode == 0 ? row_launch<0>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
              : mode == 1 ? row_launch<1>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
                          : row_launch<2>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream);
   }
+  if (t.sel_p < 0 && mode < 2 && plan->row[mode][lvl].bn != 0)
+    return mode == 0 ? row_launch<0>(t, plan->row[0][lvl], plan->d_maps, lvl, plan->row_n[0][lvl], t.P, plan->d_status, stream)
+                     : row_launch<1>(t, plan->row[1][lvl], plan->d_maps, lvl, plan->row_n[1][lvl], t.P, plan->d_status, stream);
   int n_slots = plan->n_slots[mode][lvl];
   if (n_slots == 0) return cudaSuccess;
   int grid = plan->grid[mode][lvl];                                   // one persistent CTA per SM

@@ -1,4 +1,4 @@
-// bf16 GEMMs of launches with few output tiles: one stage of a microbatch-major network, or a few rows.
+// bf16 GEMMs of launches with few output tiles: one stage of a microbatch-major network, or all stages of a small one.
 //
 // What bounds such a launch is its own length, not a pipe: a 128 x 1024 x 1024 product is 0.3 GFLOP and 2 MB of weights, but
 // on 128-column tiles it is eight CTAs, each walking sixteen k-blocks behind a ring, and the launches of a microbatch
@@ -325,17 +325,22 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
 }
 
 // ---- host: tile width and split of the reduction -------------------------------------------------------------------
+// Up to two CTAs of 64-column tiles per SM (296 tiles): beyond that the chip is full and the larger tiles of pm_umma.cu read less.
+// Columns of 32 while those number one per SM; the reduction is split while the CTAs still fit (a 128 x 1024 x 1024 launch takes
+// 1.3 us less with four parts than with two) and a part keeps two k-blocks.
 struct RowShape { int bn = 0, split = 1; };                    // bn = 0: the launch has enough tiles for the kernels of pm_umma.cu
 
-inline RowShape row_shape(int T, int N, int K, int stages) {
+inline RowShape row_shape_of(long long t32, long long t64, int kb) {      // tiles of 32 and 64 columns, k-blocks
   RowShape r;
-  const int tm = (T + ROW_M - 1) / ROW_M, kb = (K + ROW_K - 1) / ROW_K;
-  const long long t32 = (long long)tm * ((N + 31) / 32) * stages, t64 = (long long)tm * ((N + 63) / 64) * stages;
   if (t64 > 296) return r;
   r.bn = t32 <= 148 ? 32 : 64;
   const long long base = r.bn == 32 ? t32 : t64;
   r.split = (base * 4 <= 160 && kb >= 8) ? 4 : ((base * 2 <= 296 && kb >= 4) ? 2 : 1);
   return r;
+}
+inline RowShape row_shape(int T, int N, int K) {
+  const int tm = (T + ROW_M - 1) / ROW_M;
+  return row_shape_of((long long)tm * ((N + 31) / 32), (long long)tm * ((N + 63) / 64), (K + ROW_K - 1) / ROW_K);
 }
 
 template <int MODE, int BN, int S>
@@ -362,10 +367,30 @@ static cudaError_t row_launch_t(const TickArgs& t, const CUtensorMap* maps, int 
 // 512 takes 1202 us with this kernel everywhere and 1022 without it at 4096 rows (K = 512 to 2048, 32 row tiles); at 1024
 // rows 680 with it and 702 without.
 inline RowShape row_dgrad_shape(int T, int N, int K) {
-  RowShape r = row_shape(T, N, K, 1);
+  RowShape r = row_shape(T, N, K);
   const int items = ((K + ROW_K - 1) / ROW_K + r.split - 1) / r.split * (r.bn / 32);
   if (T >= 256 && N >= 256 && items * ((T + ROW_M - 1) / ROW_M) > 200) r.bn = 0;
   return r;
+}
+
+// A launch over all stages (tick-major order): by the tiles of all of them and the shallowest reduction; `n` is the widest output.
+// (Ticks against the persistent 128-column kernels: 4 stages of width 1024 and 100 rows 94.9 -> 83.3 us, 12 x 2 Linears of 256 and
+// 200 rows 116.1 -> 109.1, 16 x 2 of 96 and 40 rows 77.8 -> 64.0, 6 stages of 512 and 512 rows 102.4 -> 94.3.)
+inline RowShape row_grouped_shape(int T, const std::vector<StageDev>& st, int mode, int lvl, int* n) {
+  const int tm = (T + ROW_M - 1) / ROW_M;
+  long long t32 = 0, t64 = 0;
+  int kb = 1 << 30;
+  *n = 0;
+  for (size_t p = 0; p < st.size(); ++p) {
+    if (lvl >= st[p].n_lin || (mode != 0 && p == 0 && lvl == 0 && st[p].pre != PRE_EMBED)) continue;
+    const LinDev& L = st[p].lin[lvl];
+    const int N = mode == 0 ? L.n_out : L.n_in, K = mode == 0 ? L.n_in : L.n_out;
+    t32 += (long long)tm * ((N + 31) / 32); t64 += (long long)tm * ((N + 63) / 64);
+    kb = std::min(kb, (K + ROW_K - 1) / ROW_K);
+    *n = std::max(*n, N);
+    if (mode != 0 && row_dgrad_shape(T, N, K).bn == 0) return RowShape{};
+  }
+  return *n > 0 ? row_shape_of(t32, t64, kb) : RowShape{};
 }
 
 template <int MODE>

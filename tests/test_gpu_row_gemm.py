@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import pm_inputs as I
+from parity_util import run_gpu_pipeline, run_oracle, compare_params
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +58,14 @@ def test_bf16_products(cuda_device, width, T, act):
         assert rel(gw, g.T @ h[i]) <= tol, (i, "weights")
         assert rel(gb, g.sum(0)) <= tol * max(1.0, float(g.norm() * np.sqrt(T) / g.sum(0).norm().clamp_min(1e-30))), (i, "bias")
         g = r16(g @ r16(W[i] - wl.tau_fwd[i // 2] * D[i]))
+
+
+# launches over all stages with few tiles: 32-column tiles unsplit, in two and in four parts, 64-column tiles, several row tiles
+@pytest.mark.parametrize("P,width,T", [(3, 40, 16), (8, 328, 72), (2, 520, 128), (4, 264, 300), (6, 512, 200)])
+def test_bf16_grouped_ticks(cuda_device, P, width, T):
+    wl = I.mlp_workload("row_ticks", P, width, 1, "relu", T, compute="bf16", optimizer="sgdm", alpha=0.01, K=4, D=0.5, steps=6, seed=11 + P)
+    params0 = I.init_stage_params(wl)
+    res = run_oracle(wl, params0, wl.steps)
+    pipe, losses, book = run_gpu_pipeline(wl, params0, wl.steps)
+    np.testing.assert_allclose(losses, np.array(res.losses), rtol=1e-3)      # the tolerances of the bf16 path up to a dozen layers
+    compare_params(pipe, res, 2e-2)
