@@ -1041,6 +1041,9 @@ static pm_status mb_backward(pm_ctx* ctx) {
       if (S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
     }
     TickArgs ta = mb_args(ctx, 2 * P, -1);
+    // the LayerNorm partial sums first: those of unfused stages (widths above 1024) lie where the column sums write theirs
+    const int n_fin = ln_finish_launches(ta);
+    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(next(ctx, ta), ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
     if (dt == PM_BF16) {
       ta.colsum_only = 1;                                       // bias gradients of all stages
       for (int l = 0; l < ctx->L.max_lin; ++l)
@@ -1048,8 +1051,6 @@ static pm_status mb_backward(pm_ctx* ctx) {
       ta.colsum_only = 0;
     }
     if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
-    const int n_fin = ln_finish_launches(ta);
-    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(next(ctx, ta), ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
     return PM_OK;
   });
   if (s != PM_OK) return s;
