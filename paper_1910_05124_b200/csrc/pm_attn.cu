@@ -114,6 +114,27 @@ __device__ __forceinline__ void zero_rows(uint8_t* tiles, int n_tiles, int S) {
   __syncthreads();
 }
 
+// Sequences shorter than the tile keep the accuracy of the CUDA-core kernels that the other lengths and head widths take: expf,
+// quotients by the row sum, and sums over keys in parts of a quarter of them.  The 128-token path takes the faster __expf
+// (an error of about 2^-22 |x|) and one reciprocal per row, in front of a rounding to bf16 either way.
+template <bool FULL> __device__ __forceinline__ float attn_exp(float x) { return FULL ? __expf(x) : expf(x); }
+// a / l with rl = 1 / l rounded: the product corrected once by its residual (Markstein 1990), half an ulp but for a rounding of
+// the correction.  A division operator for each of a thread's 64 values took 23 us in the backward kernel where this takes
+// 14.8 (64 keys, 8 blocks); an infinite product has no residual.
+template <bool FULL> __device__ __forceinline__ float attn_div(float a, float l, float rl) {
+  const float q = a * rl;
+  if (FULL) return q;
+  const float c = fmaf(fmaf(-q, l, a), rl, q);
+  return fabsf(q) <= 3.402823466e38f ? c : q;
+}
+template <bool FULL> struct KeySum {                          // sum over the keys of a row, in ascending order or as four strided parts
+  float part[FULL ? 1 : 4] = {};
+  __device__ __forceinline__ void add(int j, float v) { part[FULL ? 0 : j & 3] += v; }
+  __device__ __forceinline__ float total() const {
+    if constexpr (FULL) return part[0]; else return (part[0] + part[1]) + (part[2] + part[3]);
+  }
+};
+
 // FULL: sequences of exactly 128 tokens; otherwise S < 128 (one sequence per tile all the same: a launch is bound by the length
 // of one block's chain of products, not by their number)
 template <bool FULL>
@@ -157,7 +178,7 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
     const uint32_t lane_addr = tmem_base + ((uint32_t)(warp * 32) << 16);
     float mx = -INFINITY;
 #pragma unroll 1
-    for (int cc = 0; cc < 4; ++cc) {
+    for (int cc = 0; cc < 4 && (FULL || cc * 32 < S); ++cc) {
       uint32_t v[32];
       tmem_ld32(lane_addr + cc * 32, v);
       tmem_ld_wait();
@@ -165,17 +186,22 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
       for (int j = 0; j < 32; ++j)
         if ((FULL || cc * 32 + j < S) && (!causal || cc * 32 + j <= r)) mx = fmaxf(mx, __uint_as_float(v[j]) * scale);
     }
-    float l = 0.f;
+    KeySum<FULL> ls;
 #pragma unroll 1
     for (int cc = 0; cc < 4; ++cc) {
+      if (!FULL && cc * 32 >= S) {                           // no key: a product with zeros
+#pragma unroll
+        for (int g = 0; g < 4; ++g) put_chunk(pP, r, cc * 4 + g, make_uint4(0u, 0u, 0u, 0u));
+        continue;
+      }
       uint32_t v[32];
       tmem_ld32(lane_addr + cc * 32, v);
       tmem_ld_wait();
       float e[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        e[j] = ((FULL || cc * 32 + j < S) && (!causal || cc * 32 + j <= r)) ? __expf(__uint_as_float(v[j]) * scale - mx) : 0.f;
-        l += e[j];
+        e[j] = ((FULL || cc * 32 + j < S) && (!causal || cc * 32 + j <= r)) ? attn_exp<FULL>(__uint_as_float(v[j]) * scale - mx) : 0.f;
+        ls.add(j, e[j]);
       }
 #pragma unroll
       for (int g = 0; g < 4; ++g)
@@ -197,7 +223,7 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
       tmem_ld32(lane_addr, o0);
       tmem_ld32(lane_addr + 32, o1);
       tmem_ld_wait();
-      const float inv = 1.0f / l;
+      const float l = ls.total(), inv = 1.0f / l;
       __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(t.ring + t.st[p + 1].x_ring) + (size_t)d.f_next_xslot * ((size_t)t.T * dm) +
                            (size_t)(b * S + r) * dm + h * AT_DK;
       if (FULL || r < S)
@@ -206,7 +232,7 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
         const uint32_t* src = g < 4 ? o0 + (g & 3) * 8 : o1 + (g & 3) * 8;
         float f[8];
 #pragma unroll
-        for (int e2 = 0; e2 < 8; ++e2) f[e2] = __uint_as_float(src[e2]) * inv;
+        for (int e2 = 0; e2 < 8; ++e2) f[e2] = attn_div<FULL>(__uint_as_float(src[e2]), l, inv);
         *reinterpret_cast<uint4*>(out + g * 8) = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
       }
     }
@@ -285,25 +311,24 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
     xch[hf * AT_S + r] = mx;
     __syncthreads();
     mx = fmaxf(xch[r], xch[AT_S + r]);
-    float l = 0.f;
+    KeySum<FULL> ls;
 #pragma unroll
-    for (int j = 0; j < 64; ++j) { e[j] = __expf(e[j] - mx); l += e[j]; }
-    xch[2 * AT_S + hf * AT_S + r] = l;
+    for (int j = 0; j < 64; ++j) { e[j] = attn_exp<FULL>(e[j] - mx); ls.add(j, e[j]); }
+    xch[2 * AT_S + hf * AT_S + r] = ls.total();
     __syncthreads();
-    l = xch[2 * AT_S + r] + xch[3 * AT_S + r];
-    const float inv = 1.0f / l;
+    const float l = xch[2 * AT_S + r] + xch[3 * AT_S + r], inv = 1.0f / l;
 #pragma unroll
-    for (int j = 0; j < 64; ++j) e[j] *= inv;                // P (unrounded)
-    float D = 0.f;
+    for (int j = 0; j < 64; ++j) e[j] = attn_div<FULL>(e[j], l, inv);      // P (unrounded)
+    KeySum<FULL> dp;                                         // sum of dP * P
 #pragma unroll
     for (int cc = 0; cc < 2; ++cc) {
       uint32_t g[32];
       tmem_ld32(lane_addr + colP + cc * 32, g);
       tmem_ld_wait();
 #pragma unroll
-      for (int j = 0; j < 32; ++j) D += __uint_as_float(g[j]) * e[cc * 32 + j];
+      for (int j = 0; j < 32; ++j) dp.add(j, __uint_as_float(g[j]) * e[cc * 32 + j]);
     }
-    xch[4 * AT_S + hf * AT_S + r] = D;
+    xch[4 * AT_S + hf * AT_S + r] = dp.total();
 #pragma unroll
     for (int q = 0; q < 8; ++q)
       put_chunk(pP, r, hf * 8 + q, make_uint4(pack_bf16(e[q * 8], e[q * 8 + 1]), pack_bf16(e[q * 8 + 2], e[q * 8 + 3]),
@@ -311,7 +336,7 @@ __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
-    D = xch[4 * AT_S + r] + xch[5 * AT_S + r];
+    const float D = xch[4 * AT_S + r] + xch[5 * AT_S + r];
     const uint32_t i_mm = make_idesc_mn(128, 64, 1, 1), i_km = make_idesc_mn(128, 64, 0, 1);
     if (tid == 0) {
       tc_fence_after();
