@@ -1,5 +1,5 @@
 // Multi-head self-attention on the tensor cores (tcgen05 + TMEM + TMA), forward and backward, for
-// sequences of up to 128 tokens and heads of width 64 (bf16).  One CTA of 128 threads handles one (sequence, head):
+// sequences of 17 to 128 tokens and heads of width 64 (bf16).  One CTA of 128 threads handles one (sequence, head):
 // thread r owns query row r = TMEM lane r, so the softmax needs no cross-thread traffic.
 //
 // forward :  S = Q K^T (128x128x64)  ->  p~ = exp(S/8 - rowmax), l = sum p~  ->  O = (bf16(p~) V) / l  (128x64x128);
@@ -713,7 +713,11 @@ struct AttnPlan {
 static uint64_t attn_maps_bytes(int n_stages) { return (uint64_t)n_stages * AMAPS_PER_STAGE * sizeof(CUtensorMap); }
 uint64_t attn_workspace_bytes(int n_stages) { return 256 + attn_maps_bytes(n_stages) + ((uint64_t)n_stages * sizeof(int) + 255) / 256 * 256; }
 
-bool attn_tc_supported(int dtype, int S, int dk) { return dtype == PM_BF16 && ((S >= 1 && S <= AT_S) || S == AT2_S) && dk == AT_DK; }
+// A block multiplies 128 x 128 scores whatever the sequence's length, so sequences of up to 16 tokens keep to the CUDA cores, whose
+// work goes with the square of the length.  Forward + backward of 8 / 512 / 2048 (sequence, head) pairs in us, CUDA cores against
+// tensor cores: 16 tokens 27 / 42 / 109 and 29 / 46 / 124; 8 tokens 21 / 26 / 56 and 29 / 46 / 121; 24 tokens 37 / 65 / 187 and
+// 27 / 45 / 123.
+bool attn_tc_supported(int dtype, int S, int dk) { return dtype == PM_BF16 && ((S > 16 && S <= AT_S) || S == AT2_S) && dk == AT_DK; }
 
 pm_status attn_plan_create(AttnPlan** out, const TickArgs& t, const std::vector<StageDev>& st, void* ws_region, cudaStream_t stream, std::string& err) {
   *out = nullptr;
