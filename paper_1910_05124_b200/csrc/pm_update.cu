@@ -311,14 +311,17 @@ constexpr int kUpdThreads = 128;
 // (6.36 TB/s).  U: float4 groups per thread and array.  Two while there are many waves of blocks (one: 602 us); one for small
 // networks, where a launch is as long as a thread's chain of divisions (a tick of the 4-stage MLP 36.9 -> 34.8 us).
 
+// The stage tables and gradients come from launches that may still be running when this one starts, so they are read by plain
+// loads behind the wait: a read-only (non-coherent) load is defined for memory that nobody writes during the kernel's
+// lifetime, and the compiler may move it across the wait.
 // LP: operand-type copy of the new weights: 0 none, 1 bfloat16, 2 float (a version-ring slot of fp32 operands);
 // element e of the arenas goes to lp_base[lp_shift + e], lp_shift from the stage's table entry (0: the w_lp arena)
 template <int OPT, int LP, int U>
 __global__ void __launch_bounds__(kUpdThreads, 6)
-update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restrict__ begin64, const uint32_t* __restrict__ end64,
-              const StageDyn* __restrict__ dyn, int64_t* __restrict__ nupd, int n_stages, uint64_t total_vec4,
-              float beta1, float beta2, float eps, uint64_t first_vec4, const uint32_t* __restrict__ skip_b64, const uint32_t* __restrict__ skip_e64,
-              const float* __restrict__ gsrc, float stages_per_group) {
+update_kernel(ArenasDev a, void* lp_base, const uint32_t* begin64, const uint32_t* end64,
+              const StageDyn* dyn, int64_t* nupd, int n_stages, uint64_t total_vec4,
+              float beta1, float beta2, float eps, uint64_t first_vec4, const uint32_t* skip_b64, const uint32_t* skip_e64,
+              const float* gsrc, float stages_per_group) {
   // ranges (one per stage, in 64-element groups) that another kernel has updated already: the Linear matrices, when the
   // weight-gradient GEMM applies the update in its epilogue
   const bool skip = skip_b64 != nullptr;
@@ -331,9 +334,9 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
   int lo0 = 0, hi = n_stages - 1;
   {
     const int q = min(hi, (int)((float)g0 * stages_per_group));            // where it is if all stages have the same size
-    if (__ldg(begin64 + q) <= g0 && (q == hi || g0 < __ldg(begin64 + q + 1))) lo0 = hi = q;
+    if (begin64[q] <= g0 && (q == hi || g0 < begin64[q + 1])) lo0 = hi = q;
   }
-  while (lo0 < hi) { const int mid = (lo0 + hi + 1) >> 1; if (__ldg(begin64 + mid) <= g0) lo0 = mid; else hi = mid - 1; }
+  while (lo0 < hi) { const int mid = (lo0 + hi + 1) >> 1; if (begin64[mid] <= g0) lo0 = mid; else hi = mid - 1; }
   if (skip) {
     // the whole span of this block lies inside a skipped range (and past the stage's first group): nothing to do
     const uint32_t g1 = (uint32_t)((base + (uint64_t)kUpdThreads * U - 1) >> 4);
@@ -350,8 +353,8 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
     if (v[u] < total_vec4) {
       const uint32_t e64 = (uint32_t)(v[u] >> 4);
       int lo = lo0;
-      while (lo + 1 < n_stages && __ldg(begin64 + lo + 1) <= e64) ++lo;      // a block spans 32 groups: rarely more than one stage on
-      if (__ldg(begin64 + lo) <= e64 && e64 < __ldg(end64 + lo) && dyn[lo].active_update) {
+      while (lo + 1 < n_stages && begin64[lo + 1] <= e64) ++lo;      // a block spans 32 groups: rarely more than one stage on
+      if (begin64[lo] <= e64 && e64 < end64[lo] && dyn[lo].active_update) {
         if (skip && skip_b64[lo] <= e64 && e64 < skip_e64[lo]) {             // updated elsewhere; the stage's counter is still kept here
           if (e64 == begin64[lo] && (v[u] & 15) == 0) nupd[lo] += 1;
         } else stage[u] = lo;
@@ -411,7 +414,7 @@ update_kernel(ArenasDev a, void* __restrict__ lp_base, const uint32_t* __restric
         *reinterpret_cast<float4*>(reinterpret_cast<float*>(lp_base) + (sc[u].rc_shift + (int64_t)e)) = r;
       }
     }
-    if ((uint32_t)(v[u] >> 4) == __ldg(begin64 + stage[u]) && (v[u] & 15) == 0) nupd[stage[u]] += 1;
+    if ((uint32_t)(v[u] >> 4) == begin64[stage[u]] && (v[u] & 15) == 0) nupd[stage[u]] += 1;
   }
 }
 
@@ -439,8 +442,8 @@ cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* 
 // ---- fp32 copies of the small forward-read tensors into the version rings -------------------------------------
 // With bfloat16 operands the forward pass still reads biases and LayerNorm parameters in fp32; in microbatch-major
 // order their versions sit in a ring of their own, filled here from the master weights after every update.
-__global__ void __launch_bounds__(128) push_small_kernel(const float* __restrict__ w, const float* __restrict__ delta, char* __restrict__ ring,
-                                                         const SmallSeg* __restrict__ segs, int n_segs, const StageDyn* __restrict__ dyn, int slot_override) {
+__global__ void __launch_bounds__(128) push_small_kernel(const float* w, const float* delta, char* ring, const SmallSeg* __restrict__ segs, int n_segs,
+                                                         const StageDyn* dyn, int slot_override) {
   pdl_trigger();
   pdl_wait();
   for (int sg = blockIdx.x; sg < n_segs; sg += gridDim.x) {
