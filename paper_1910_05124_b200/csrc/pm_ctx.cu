@@ -750,11 +750,11 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
     std::string aerr;
     pm_status as = attn_plan_create(&c->attn, t, c->L.st, c->ws + L.off_attn, c->stream, aerr);
     if (as != PM_OK) { delete c; return fail(nullptr, as, aerr); }
-  } else if (L.att_blocks > 0) {
-    e = attention_set_smem_limits(L.att_S, L.att_dk, cfg->compute_dtype);
-    if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "attention shared-memory limit"); delete c; return r; }
   }
-
+  if (L.any_pre || L.att_blocks > 0 || cfg->loss == PM_LOSS_CE) {
+    e = xfmr_set_smem_limits(cfg->compute_dtype);
+    if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "shared-memory limits"); delete c; return r; }
+  }
   if (cfg->compute_dtype == PM_F32) {
     e = simt_gemm_set_limits();
     if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "GEMM shared-memory limit"); delete c; return r; }

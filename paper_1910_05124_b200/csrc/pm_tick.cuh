@@ -193,7 +193,7 @@ int ln_finish_launches(const TickArgs& t);
 cudaError_t launch_pre_fwd(const TickArgs& t, int dtype, cudaStream_t stream);        // embedding / LayerNorm forward (+ skip hand-over)
 cudaError_t launch_post_fwd(const TickArgs& t, int dtype, cudaStream_t stream, bool skip_attention);   // attention forward (SIMT), residual add
 cudaError_t launch_post_bwd(const TickArgs& t, int dtype, cudaStream_t stream);       // attention backward
-// tensor-core attention (bf16, sequences of 128, heads of 64)
+// tensor-core attention (bf16, sequences of 17 to 128 or of 256 tokens, heads of 64)
 struct AttnPlan;
 uint64_t attn_workspace_bytes(int n_stages);
 bool attn_tc_supported(int dtype, int S, int dk);
@@ -203,7 +203,9 @@ int* attn_status_word(AttnPlan* plan);
 cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream);        // LayerNorm / embedding backward
 int pre_bwd_launches(const TickArgs& t);
 size_t attention_smem_bytes(int S, int dk, int dtype);
-cudaError_t attention_set_smem_limits(int S, int dk, int dtype);
+
+// opt-in shared-memory sizes of the Transformer kernels of one operand type, on the current device
+cudaError_t xfmr_set_smem_limits(int dtype);
 
 // fp32 SIMT grouped GEMMs (PM_F32 path).  mode: 0 forward, 1 dgrad (corrected weights), 2 wgrad.
 cudaError_t simt_gemm_set_limits();

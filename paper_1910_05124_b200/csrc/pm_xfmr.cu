@@ -389,18 +389,6 @@ cudaError_t launch_post_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
                          : launch_pdl(attention_bwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 2), stream, t.pdl, t);
 }
 
-cudaError_t attention_set_smem_limits(int S, int dk, int dtype) {
-  cudaError_t e;
-  if (dtype == PM_F32) {
-    e = cudaFuncSetAttribute((const void*)attention_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_fwd_smem(S, dk, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attention_bwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_bwd_smem(S, dk, 4));
-  } else {
-    e = cudaFuncSetAttribute((const void*)attention_fwd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_fwd_smem(S, dk, 2));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)attention_bwd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_bwd_smem(S, dk, 2));
-  }
-  return e;
-}
-
 // ---- loss reduction shared by the cross-entropy kernels ----
 // per-token losses of this block's rows (ce_row_loss); the last block to arrive adds all of them in a fixed order (strided per-thread
 // partials over the first 256 threads, then a fixed tree).  Called by every thread of the block.
@@ -721,8 +709,6 @@ cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
     const bool rows = V <= 32 * kCeLongThreads;              // longer rows do not fit a block's registers
     auto* kernel = rows ? (dtype == PM_F32 ? ce_loss_rows_kernel<float> : ce_loss_rows_kernel<__nv_bfloat16>)
                         : (dtype == PM_F32 ? ce_loss_long_kernel<float> : ce_loss_long_kernel<__nv_bfloat16>);
-    cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_bytes);
-    if (e != cudaSuccess) return e;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); sms = 148; }
     return launch_pdl(kernel, dim3(rows ? std::min(sms, (int)t.T) : t.T), dim3(kCeLongThreads), row_bytes, stream, t.pdl, t);
@@ -1124,12 +1110,6 @@ static cudaError_t launch_ln_fused(const TickArgs& t, cudaStream_t stream) {
   TickArgs ta = t;
   ta.ln_stage = (t.sel_p >= 0 && stage_bytes <= 100 * 1024 && (t.max_ln_dim * sizeof(AT)) % 16 == 0) ? 1 : 0;
   if (ta.ln_stage) smem = std::max(smem, stage_bytes);
-  static size_t attr_bytes = 48 * 1024;
-  if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute((const void*)ln_bwd_fused_kernel<AT, NP, WPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_bytes = smem;
-  }
   const cudaError_t e = launch_pdl(ln_bwd_fused_kernel<AT, NP, WPR>, dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, t.pdl, ta);
   if (e != cudaSuccess || t.defer_finish) return e;
   return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, t.pdl, t);
@@ -1391,10 +1371,6 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     // the hit list, the same tokens grouped by row, and the per-warp partial sums of a shared row
     const size_t smem = 2 * sizeof(int32_t) * (size_t)t.T + sizeof(float) * 8 * 32 * (size_t)cpl;
     auto go = [&](auto kernel) -> cudaError_t {
-      if (smem + 1024 > 48 * 1024) {                         // static shared memory counts towards the default limit
-        cudaError_t ea = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (ea != cudaSuccess) return ea;
-      }
       return launch_pdl(kernel, g, dim3(256), smem, stream, t.pdl, t);
     };
     if (dtype == PM_F32) e = cpl == 16 ? go(embed_bwd_kernel<float, 16>) : (cpl == 8 ? go(embed_bwd_kernel<float, 8>) : go(embed_bwd_kernel<float, 4>));
@@ -1402,5 +1378,32 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   }
   return e;
 }
+
+// ---- shared-memory limits -----------------------------------------------------------------------------------------
+// The limit is an attribute of a kernel on a device, shared by all contexts and threads of the process: every context sets the
+// same value, the most a block can have beside the kernel's static shared memory, so that none lowers it under another.
+static cudaError_t limit_to_max(const void* kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) : e;
+}
+
+template <typename AT>
+static cudaError_t limits_of() {
+  const void* kernels[] = {(const void*)attention_fwd_kernel<AT>, (const void*)attention_bwd_kernel<AT>,
+                           (const void*)ce_loss_rows_kernel<AT>, (const void*)ce_loss_long_kernel<AT>,
+                           (const void*)ln_bwd_fused_kernel<AT, 1, 1>, (const void*)ln_bwd_fused_kernel<AT, 2, 1>, (const void*)ln_bwd_fused_kernel<AT, 2, 2>,
+                           (const void*)embed_bwd_kernel<AT, 4>, (const void*)embed_bwd_kernel<AT, 8>, (const void*)embed_bwd_kernel<AT, 16>};
+  for (const void* k : kernels) {
+    const cudaError_t e = limit_to_max(k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t xfmr_set_smem_limits(int dtype) { return dtype == PM_F32 ? limits_of<float>() : limits_of<__nv_bfloat16>(); }
 
 }  // namespace pm
