@@ -972,7 +972,7 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;
-  if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(next(ctx, ta), dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
+  if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(ta, dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
   return PM_OK;
 }
 
@@ -1043,7 +1043,7 @@ static pm_status mb_backward(pm_ctx* ctx) {
     TickArgs ta = mb_args(ctx, 2 * P, -1);
     // the LayerNorm partial sums first: those of unfused stages (widths above 1024) lie where the column sums write theirs
     const int n_fin = ln_finish_launches(ta);
-    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(next(ctx, ta), ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
+    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
     if (dt == PM_BF16) {
       ta.colsum_only = 1;                                       // bias gradients of all stages
       for (int l = 0; l < ctx->L.max_lin; ++l)
@@ -1255,7 +1255,7 @@ pm_status pm_backward(pm_ctx* ctx) {
         if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
       }
       const int n_pre = pre_bwd_launches(ctx->ta);
-      if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(next(ctx, ctx->ta), dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
+      if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(ctx->ta, dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
       return PM_OK;
     });
     if (s != PM_OK) return s;

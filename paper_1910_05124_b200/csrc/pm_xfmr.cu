@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(256) pre_fwd_kernel(TickArgs t) {
 
 cudaError_t launch_pre_fwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   dim3 grid((t.T + 7) / 8, t.n_pre);
-  return launch_pdl(dtype == PM_F32 ? pre_fwd_kernel<float> : pre_fwd_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, t.pdl, t);
+  return launch_pdl(dtype == PM_F32 ? pre_fwd_kernel<float> : pre_fwd_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, early(t, grid), t);
 }
 
 // ---- residual add: next stage's input = skip + y --------------------------------------------------------------
@@ -287,8 +287,8 @@ cudaError_t launch_post_fwd(const TickArgs& t, int dtype, cudaStream_t stream, b
   cudaError_t e = cudaSuccess;
   if (any_att) {
     dim3 grid(nblk, t.sel_p >= 0 ? 1 : t.P);
-    e = dtype == PM_F32 ? launch_pdl(attention_fwd_kernel<float>, grid, dim3(256), attn_fwd_smem(S, dk, 4), stream, t.pdl, t)
-                        : launch_pdl(attention_fwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_fwd_smem(S, dk, 2), stream, t.pdl, t);
+    e = dtype == PM_F32 ? launch_pdl(attention_fwd_kernel<float>, grid, dim3(256), attn_fwd_smem(S, dk, 4), stream, early(t, grid), t)
+                        : launch_pdl(attention_fwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_fwd_smem(S, dk, 2), stream, early(t, grid), t);
     if (e != cudaSuccess) return e;
   }
   if (any_res) {
@@ -385,8 +385,8 @@ __global__ void __launch_bounds__(256) attention_bwd_kernel(TickArgs t) {
 cudaError_t launch_post_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   if (t.att_blocks <= 0) return cudaSuccess;
   dim3 grid(t.att_blocks, t.sel_p >= 0 ? 1 : t.P);
-  return dtype == PM_F32 ? launch_pdl(attention_bwd_kernel<float>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 4), stream, t.pdl, t)
-                         : launch_pdl(attention_bwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 2), stream, t.pdl, t);
+  return dtype == PM_F32 ? launch_pdl(attention_bwd_kernel<float>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 4), stream, early(t, grid), t)
+                         : launch_pdl(attention_bwd_kernel<__nv_bfloat16>, grid, dim3(256), attn_bwd_smem(t.att_S, t.att_dk, 2), stream, early(t, grid), t);
 }
 
 // ---- loss reduction shared by the cross-entropy kernels ----
@@ -717,6 +717,11 @@ cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
 }
 
 // ---- pre-op backward --------------------------------------------------------------------------------------------
+// These launches are plain: none starts before its predecessor, the stage's dgrad, has ended (their successors may start early).
+// Blocks that become resident during a predecessor's tail crowd on the SMs that are free first and stay there; with the rows
+// of a LayerNorm backward that costs more than the launch: an update of a 2-layer encoder of width 1280 (2048 rows) takes
+// 1189 us with early launches here and 1140 without, of 4 layers of width 512 (1024 rows) 907 and 897, of the encoder of
+// 7 x 96 tokens and width 192 232 and 222.
 // du_total = du (dgrad output of the first Linear) + gradient of the skip tensor the stage emitted, if any.
 template <typename AT>
 __device__ __forceinline__ float du_total(const AT* du, const AT* gs, uint64_t i) {
@@ -730,7 +735,6 @@ __device__ __forceinline__ float du_total(const AT* du, const AT* gs, uint64_t i
 template <typename AT>
 __global__ void __launch_bounds__(256) ln_bwd_dx_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   const int p = t.ln_ids[blockIdx.y + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -810,7 +814,6 @@ constexpr int kLnCols = 256;                         // columns per block: 8 per
 template <typename AT>
 __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   const int p = t.ln_ids[blockIdx.z + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -879,7 +882,6 @@ __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
 
 __global__ void __launch_bounds__(256) ln_param_finish_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   const int p = t.ln_ids[blockIdx.y + t.ln_li0];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -905,7 +907,6 @@ __global__ void __launch_bounds__(256) ln_param_finish_kernel(TickArgs t) {
 template <typename AT, int NP, int WPR>
 __global__ void __launch_bounds__(256, NP <= 2 ? 2 : 1) ln_bwd_fused_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   const int li = blockIdx.y + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -1068,7 +1069,6 @@ constexpr int kLnFinCols = 32, kLnFinPer = 16;
 
 __global__ void __launch_bounds__(256) ln_fused_finish_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   const int li = blockIdx.y + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
@@ -1110,9 +1110,9 @@ static cudaError_t launch_ln_fused(const TickArgs& t, cudaStream_t stream) {
   TickArgs ta = t;
   ta.ln_stage = (t.sel_p >= 0 && stage_bytes <= 100 * 1024 && (t.max_ln_dim * sizeof(AT)) % 16 == 0) ? 1 : 0;
   if (ta.ln_stage) smem = std::max(smem, stage_bytes);
-  const cudaError_t e = launch_pdl(ln_bwd_fused_kernel<AT, NP, WPR>, dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, t.pdl, ta);
+  const cudaError_t e = launch_pdl(ln_bwd_fused_kernel<AT, NP, WPR>, dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, false, ta);
   if (e != cudaSuccess || t.defer_finish) return e;
-  return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, t.pdl, t);
+  return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, false, t);
 }
 
 // Embedding gradient: dTable[v] = sqrt(d) * sum over tokens t with id[t] == v (ascending t) of du_total[t].
@@ -1183,7 +1183,6 @@ __device__ __forceinline__ void embed_gather(const int32_t* sub, int k_lo, int k
 template <typename AT, int CPL>
 __global__ void __launch_bounds__(256) embed_bwd_kernel(TickArgs t) {
   pdl_trigger();
-  pdl_wait();
   constexpr int kEmbCols = 32 * CPL;
   const int p = t.embed_ids[blockIdx.y];
   const StageDyn& d = t.dyn[p];
@@ -1337,8 +1336,8 @@ int pre_bwd_launches(const TickArgs& t) {
 int ln_finish_launches(const TickArgs& t) { return t.any_ln && (t.ln_fused || t.row_chunks > 1) ? 1 : 0; }
 cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream) {
   if (!t.any_ln) return cudaSuccess;
-  if (t.ln_fused) return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, t.pdl, t);
-  if (t.row_chunks > 1) return launch_pdl(ln_param_finish_kernel, dim3((t.max_ln_dim + 255) / 256, t.n_ln), dim3(256), 0, stream, t.pdl, t);
+  if (t.ln_fused) return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, false, t);
+  if (t.row_chunks > 1) return launch_pdl(ln_param_finish_kernel, dim3((t.max_ln_dim + 255) / 256, t.n_ln), dim3(256), 0, stream, false, t);
   return cudaSuccess;
 }
 
@@ -1350,12 +1349,12 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
   } else if (t.any_ln) {
     dim3 g1((t.T + 7) / 8, t.n_ln), g2((t.max_ln_dim + kLnCols - 1) / kLnCols, t.row_chunks, t.n_ln);
-    e = launch_pdl(dtype == PM_F32 ? ln_bwd_dx_kernel<float> : ln_bwd_dx_kernel<__nv_bfloat16>, g1, dim3(256), 0, stream, t.pdl, t);
-    if (e == cudaSuccess) e = launch_pdl(dtype == PM_F32 ? ln_bwd_param_kernel<float> : ln_bwd_param_kernel<__nv_bfloat16>, g2, dim3(256), 0, stream, t.pdl, t);
+    e = launch_pdl(dtype == PM_F32 ? ln_bwd_dx_kernel<float> : ln_bwd_dx_kernel<__nv_bfloat16>, g1, dim3(256), 0, stream, false, t);
+    if (e == cudaSuccess) e = launch_pdl(dtype == PM_F32 ? ln_bwd_param_kernel<float> : ln_bwd_param_kernel<__nv_bfloat16>, g2, dim3(256), 0, stream, false, t);
     if (e != cudaSuccess) return e;
     if (t.row_chunks > 1 && !t.defer_finish) {
       dim3 g3((t.max_ln_dim + 255) / 256, t.n_ln);
-      e = launch_pdl(ln_param_finish_kernel, g3, dim3(256), 0, stream, t.pdl, t);
+      e = launch_pdl(ln_param_finish_kernel, g3, dim3(256), 0, stream, false, t);
       if (e != cudaSuccess) return e;
     }
   }
@@ -1371,7 +1370,7 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     // the hit list, the same tokens grouped by row, and the per-warp partial sums of a shared row
     const size_t smem = 2 * sizeof(int32_t) * (size_t)t.T + sizeof(float) * 8 * 32 * (size_t)cpl;
     auto go = [&](auto kernel) -> cudaError_t {
-      return launch_pdl(kernel, g, dim3(256), smem, stream, t.pdl, t);
+      return launch_pdl(kernel, g, dim3(256), smem, stream, false, t);
     };
     if (dtype == PM_F32) e = cpl == 16 ? go(embed_bwd_kernel<float, 16>) : (cpl == 8 ? go(embed_bwd_kernel<float, 8>) : go(embed_bwd_kernel<float, 4>));
     else e = cpl == 16 ? go(embed_bwd_kernel<__nv_bfloat16, 16>) : (cpl == 8 ? go(embed_bwd_kernel<__nv_bfloat16, 8>) : go(embed_bwd_kernel<__nv_bfloat16, 4>));
