@@ -927,7 +927,7 @@ static pm_status stage_forward(pm_ctx* ctx, const TickArgs& ta, int p) {
   if (sd.pre != PRE_NONE && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(next(ctx, ta), dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
   for (int l = 0; l < sd.n_lin; ++l) {
     prof_begin(ctx, PM_PROF_GEMM_FWD);
-    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), 0, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 0, l, ctx->ls);
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 0, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 0, l, ctx->ls);
     if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
   }
   const bool att = feeds_attention(sd.post);
@@ -963,12 +963,12 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     cudaError_t e;
     if (!grouped) {
       prof_begin(ctx, PM_PROF_WGRAD);
-      e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), 2, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 2, l, ctx->ls);
+      e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 2, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 2, l, ctx->ls);
       if ((s = check(ctx, e, "wgrad GEMM")) != PM_OK) return s;
     }
     if (p == 0 && l == 0 && sd.pre != PRE_EMBED) continue;          // raw network inputs need no gradient
     prof_begin(ctx, PM_PROF_DGRAD);
-    e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), 1, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
+    e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 1, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;
@@ -1007,7 +1007,7 @@ static pm_status grouped_wgrad(pm_ctx* ctx, int table, bool fused = false) {
   ta.fuse_upd = fused ? 1 : 0;
   for (int l = 0; l < ctx->L.max_lin; ++l) {
     prof_begin(ctx, PM_PROF_WGRAD);
-    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), 2, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 2, l, ctx->ls);
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 2, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 2, l, ctx->ls);
     pm_status s = check(ctx, e, "wgrad GEMM");
     if (s != PM_OK) return s;
   }
@@ -1207,7 +1207,7 @@ pm_status pm_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
       if (ctx->L.any_pre && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(next(ctx, ctx->ta), dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
       for (int l = 0; l < ctx->L.max_lin; ++l) {
         prof_begin(ctx, PM_PROF_GEMM_FWD);
-        cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), 0, l, ctx->ls)
+        cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 0, l, ctx->ls)
                                      : umma_launch(ctx->umma, next(ctx, ctx->ta), 0, l, ctx->ls);
         if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
       }
@@ -1245,12 +1245,12 @@ pm_status pm_backward(pm_ctx* ctx) {
         cudaError_t e = cudaSuccess;
         if (!ctx->L.fuse) {                                           // fused update: formed in the update phase
           prof_begin(ctx, PM_PROF_WGRAD);
-          e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), 2, l, ctx->ls)
+          e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 2, l, ctx->ls)
                            : umma_launch(ctx->umma, next(ctx, ctx->ta), 2, l, ctx->ls);
           if ((s = check(ctx, e, "wgrad GEMM")) != PM_OK) return s;
         }
         prof_begin(ctx, PM_PROF_DGRAD);
-        e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), 1, l, ctx->ls)
+        e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 1, l, ctx->ls)
                          : umma_launch(ctx->umma, next(ctx, ctx->ta), 1, l, ctx->ls);
         if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
       }

@@ -3,6 +3,8 @@
 // Every kernel is "grouped": blockIdx.z (or .y) selects the stage, the per-tick table says
 // whether that stage is active and which ring slots it touches.  Within a tick the stages
 // only read what earlier ticks left in their rings and mailboxes, so one launch covers all.
+#include <algorithm>
+
 #include "pm_tick.cuh"
 
 namespace pm {
@@ -459,7 +461,7 @@ __device__ __forceinline__ float f32_sum8(const float* p, int stride) {
 }
 
 template <int TM, int TN, int NBUF, int MODE>
-__global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int tiles_n) {
+__global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl) {
   using C = F32Cfg<TM, TN, NBUF, MODE>;
   constexpr int BM = C::BM, BN = C::BN, KC = kF32KC;
   pdl_trigger();
@@ -469,6 +471,7 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
   const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
   const int T = t.T;
   const int M = MODE == 2 ? L.n_out : T, N = MODE == 0 ? L.n_out : L.n_in, K = MODE == 0 ? L.n_in : (MODE == 1 ? L.n_out : T);
+  const unsigned tiles_n = (unsigned)(N + BN - 1) / BN;      // the grid holds the tiles of the launch's largest Linear
   const int m0 = (int)(blockIdx.x / tiles_n) * BM, n0 = (int)(blockIdx.x % tiles_n) * BN;
   if (lvl >= s.n_lin || (MODE == 0 ? d.f_mb < 0 : d.b_mb < 0) || m0 >= M || n0 >= N ||
       (MODE == 1 && p == 0 && lvl == 0 && s.pre != PRE_EMBED)) {          // raw network inputs need no gradient
@@ -633,11 +636,9 @@ __global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl, int 
 }
 
 template <int TM, int TN, int NBUF, int MODE>
-static cudaError_t launch_f32_t(const TickArgs& t, int lvl, int grid_m, cudaStream_t stream) {
+static cudaError_t launch_f32_t(const TickArgs& t, int lvl, uint64_t tiles, cudaStream_t stream) {
   using C = F32Cfg<TM, TN, NBUF, MODE>;
-  const int tiles_n = (t.max_dim + C::BN - 1) / C::BN, tiles_m = (grid_m + C::BM - 1) / C::BM;
-  dim3 grid((unsigned)tiles_m * (unsigned)tiles_n, t.sel_p >= 0 ? 1 : t.P);
-  return launch_pdl(f32_gemm_kernel<TM, TN, NBUF, MODE>, grid, dim3(256), C::kBytes, stream, t.pdl, t, lvl, tiles_n);
+  return launch_pdl(f32_gemm_kernel<TM, TN, NBUF, MODE>, dim3((unsigned)tiles, t.sel_p >= 0 ? 1 : t.P), dim3(256), C::kBytes, stream, t.pdl, t, lvl);
 }
 
 // opt-in shared-memory sizes, on the current device
@@ -650,14 +651,25 @@ cudaError_t simt_gemm_set_limits() {
   return e;
 }
 
-// 16 x 16 tiles while 32 x 32 ones would number no more than the 148 SMs: a smaller tile has a quarter of the multiplies on
-// its critical path and the chip is not full anyway.
-cudaError_t launch_simt_gemm(const TickArgs& t, int mode, int lvl, cudaStream_t stream) {
-  const int mt = mode == 2 ? t.max_dim : t.T;
-  const long long big = (long long)((t.max_dim + 31) / 32) * ((mt + 31) / 32) * (t.sel_p >= 0 ? 1 : t.P);
-  if (big <= 148)
-    return mode == 0 ? launch_f32_t<4, 2, 4, 0>(t, lvl, mt, stream) : (mode == 1 ? launch_f32_t<4, 2, 3, 1>(t, lvl, mt, stream) : launch_f32_t<4, 2, 4, 2>(t, lvl, mt, stream));
-  return mode == 0 ? launch_f32_t<8, 4, 2, 0>(t, lvl, mt, stream) : (mode == 1 ? launch_f32_t<8, 4, 2, 1>(t, lvl, mt, stream) : launch_f32_t<8, 4, 2, 2>(t, lvl, mt, stream));
+// 16 x 16 tiles while the 32 x 32 ones of all stages of the launch would number no more than the 148 SMs: a smaller tile has a
+// quarter of the multiplies on its critical path and the chip is not full anyway.
+// Tiles are counted over the launch's own Linears.  (Sized by the widest Linear of the network, the launches of a network with a
+// large vocabulary were mostly blocks without a tile: a tick of a 6-layer encoder of width 64, 64 rows and a vocabulary of
+// 8000 took 2368 us and takes 211, of a 2-layer one of width 64, 384 rows and a vocabulary of 1000 165 and 152.)
+cudaError_t launch_simt_gemm(const TickArgs& t, const std::vector<StageDev>& st, int mode, int lvl, cudaStream_t stream) {
+  uint64_t all32 = 0, most32 = 1, most16 = 1;
+  for (int p = t.sel_p >= 0 ? t.sel_p : 0; p < (t.sel_p >= 0 ? t.sel_p + 1 : t.P); ++p) {
+    if (lvl >= st[p].n_lin || (mode == 1 && p == 0 && lvl == 0 && st[p].pre != PRE_EMBED)) continue;
+    const LinDev& L = st[p].lin[lvl];
+    const uint64_t M = mode == 2 ? L.n_out : t.T, N = mode == 0 ? L.n_out : L.n_in;
+    const uint64_t n32 = ((M + 31) / 32) * ((N + 31) / 32);
+    all32 += n32;
+    most32 = std::max(most32, n32);
+    most16 = std::max(most16, ((M + 15) / 16) * ((N + 15) / 16));
+  }
+  if (all32 <= 148)
+    return mode == 0 ? launch_f32_t<4, 2, 4, 0>(t, lvl, most16, stream) : (mode == 1 ? launch_f32_t<4, 2, 3, 1>(t, lvl, most16, stream) : launch_f32_t<4, 2, 4, 2>(t, lvl, most16, stream));
+  return mode == 0 ? launch_f32_t<8, 4, 2, 0>(t, lvl, most32, stream) : (mode == 1 ? launch_f32_t<8, 4, 2, 1>(t, lvl, most32, stream) : launch_f32_t<8, 4, 2, 2>(t, lvl, most32, stream));
 }
 
 }  // namespace pm

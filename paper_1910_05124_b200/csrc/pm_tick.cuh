@@ -1,5 +1,7 @@
 // Per-tick kernel launches of the pipeline (declarations shared by the host code).
 #pragma once
+#include <vector>
+
 #include "pm_common.cuh"
 
 namespace pm {
@@ -213,6 +215,7 @@ cudaError_t xfmr_set_smem_limits(int dtype);
 
 // fp32 SIMT grouped GEMMs (PM_F32 path).  mode: 0 forward, 1 dgrad (corrected weights), 2 wgrad.
 cudaError_t simt_gemm_set_limits();
-cudaError_t launch_simt_gemm(const TickArgs& t, int mode, int lvl, cudaStream_t stream);
+// st: the host's copy of the stages.
+cudaError_t launch_simt_gemm(const TickArgs& t, const std::vector<StageDev>& st, int mode, int lvl, cudaStream_t stream);
 
 }  // namespace pm
