@@ -26,8 +26,8 @@ struct Layout {
   std::vector<StageDev> st;
   std::vector<StageSched> sched;
   std::vector<uint32_t> begin64, end64;
-  std::vector<uint32_t> skip_b64, skip_e64;   // per stage, the Linear matrix's range in 64-element groups (fused update), else empty
-  uint64_t off_skb = 0, off_ske = 0;
+  UpdParts parts;                       // fused update: what the update kernel still has to do
+  uint64_t off_parts = 0;
   int32_t fuse = 0;                     // the weight-gradient GEMM applies the update of the Linear matrices in its epilogue
   int32_t stash = 0;                    // weight stashing: every stage has tau_bkwd = tau_fwd (microbatch-major order)
   int32_t materialize = 0;              // the corrected backward weights are written by the update into a slot of the version queue
@@ -388,7 +388,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   // Fused update (pm_config.fuse_update): the weight-gradient GEMM's epilogue updates the Linear matrices, the update
   // kernel the rest of every stage (biases, LayerNorm parameters, embedding tables, padding).
   L.fuse = 0;
-  L.skip_b64.assign(P, 0); L.skip_e64.assign(P, 0);
   if (cfg->fuse_update) {
     const char* why = nullptr;
     if (cfg->compute_dtype != PM_BF16) why = "the tensor-core (PM_BF16) path";
@@ -398,11 +397,13 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
     else if (E > 1) why = "an entry period of one tick";
     if (why) { err = std::string("fuse_update is built for ") + why; return PM_ERR_UNSUPPORTED; }
     L.fuse = 1;
+    std::vector<uint32_t> skip_b(P), skip_e(P);                // the Linear matrices in 64-element groups: dimensions are multiples of 8, so whole groups
     for (int p = 0; p < P; ++p) {
       const LinDev& l0 = L.st[p].lin[0];
-      L.skip_b64[p] = (uint32_t)(l0.w_off / 64);
-      L.skip_e64[p] = (uint32_t)((l0.w_off + (uint64_t)l0.n_out * l0.n_in) / 64);     // dimensions are multiples of 8: whole groups
+      skip_b[p] = (uint32_t)(l0.w_off / 64);
+      skip_e[p] = (uint32_t)((l0.w_off + (uint64_t)l0.n_out * l0.n_in) / 64);
     }
+    L.parts = update_parts(L.begin64.data(), L.end64.data(), skip_b.data(), skip_e.data(), P);
   }
   for (int p = 0; p < P; ++p) {
     L.sched[p].next_xdepth = p + 1 < P ? L.st[p + 1].xdepth : 0;
@@ -438,8 +439,7 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   L.off_b64 = w; w = align_up(w + sizeof(uint32_t) * P, 256);
   L.off_e64 = w; w = align_up(w + sizeof(uint32_t) * P, 256);
   L.off_delays = w; w = align_up(w + sizeof(int32_t) * P, 256);
-  L.off_skb = w; w = align_up(w + sizeof(uint32_t) * P, 256);
-  L.off_ske = w; w = align_up(w + sizeof(uint32_t) * P, 256);
+  L.off_parts = w; w = align_up(w + sizeof(UpdPart) * L.parts.list.size(), 256);
   L.off_alpha = w; w = align_up(w + sizeof(double) * (cfg->alpha_by_step ? (uint64_t)cfg->alpha_len : 0), 256);
   L.off_loss = w; w = align_up(w + sizeof(float) * (uint64_t)L.loss_cap, 256);
   L.off_lossred = w; w = align_up(w + 512, 256);
@@ -669,8 +669,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   UP(L.off_sched, c->L.sched);
   UP(L.off_b64, c->L.begin64);
   UP(L.off_e64, c->L.end64);
-  UP(L.off_skb, c->L.skip_b64);
-  UP(L.off_ske, c->L.skip_e64);
+  if (!c->L.parts.list.empty()) { UP(L.off_parts, c->L.parts.list); }
   UP(L.off_ids, c->L.ids);
   if (!c->L.segs.empty()) { UP(L.off_segs, c->L.segs); }
 #undef UP
@@ -1058,6 +1057,17 @@ static pm_status mb_backward(pm_ctx* ctx) {
   return PM_OK;
 }
 
+// The update kernel over all stages: everything, or what the weight-gradient GEMM's epilogue has left.
+static cudaError_t update_all(pm_ctx* ctx, const StageDyn* dyn, const float* gsrc) {
+  const pm_config& g = ctx->cfg;
+  int64_t* nupd = (int64_t*)(ctx->ws + ctx->L.off_nupd);
+  void* lp = ctx->L.queue ? (void*)ctx->ta.ring : nullptr;
+  if (ctx->L.fuse)
+    return launch_update_parts(ctx->a, ctx->L.parts, (const UpdPart*)(ctx->ws + ctx->L.off_parts), dyn, nupd, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, early(ctx));
+  return launch_update(ctx->a, (const uint32_t*)(ctx->ws + ctx->L.off_b64), (const uint32_t*)(ctx->ws + ctx->L.off_e64), dyn, nupd, g.n_stages,
+                       ctx->L.total / 64, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, ctx->hp.lp_elem, 0, gsrc, early(ctx));
+}
+
 static pm_status mb_update(pm_ctx* ctx) {
   const int P = ctx->cfg.n_stages;
   if (ctx->n_fed % ctx->hp.n_micro != 0) {          // inside a minibatch: the gradients stay in the arena and the next microbatch adds to them
@@ -1081,11 +1091,7 @@ static pm_status mb_update(pm_ctx* ctx) {
     // fused update: the weight gradients of all stages as one launch whose epilogue updates the Linear matrices
     if (ctx->L.fuse) { pm_status fs = grouped_wgrad(ctx, 2 * P, true); if (fs != PM_OK) return fs; }
     prof_begin(ctx, PM_PROF_UPDATE);
-    cudaError_t e = launch_update(ctx->a, (const uint32_t*)(ctx->ws + ctx->L.off_b64), (const uint32_t*)(ctx->ws + ctx->L.off_e64), dyn_all,
-                                  (int64_t*)(ctx->ws + ctx->L.off_nupd), P, ctx->L.total / 64, ctx->cfg.optimizer, ctx->cfg.beta1,
-                                  ctx->cfg.beta2, ctx->cfg.eps, ctx->ls, ctx->ta.ring, ctx->hp.lp_elem, 0,
-                                  ctx->L.fuse ? (const uint32_t*)(ctx->ws + ctx->L.off_skb) : nullptr,
-                                  ctx->L.fuse ? (const uint32_t*)(ctx->ws + ctx->L.off_ske) : nullptr, gsrc, early(ctx));
+    cudaError_t e = update_all(ctx, dyn_all, gsrc);
     pm_status s = check(ctx, e, "update");
     if (s != PM_OK || ctx->L.segs.empty()) return s;
     prof_begin(ctx, PM_PROF_UPDATE);
@@ -1160,7 +1166,7 @@ static pm_status sparse_update_phase(pm_ctx* ctx) {
       cudaError_t e = launch_update(ctx->a, (const uint32_t*)(ctx->ws + ctx->L.off_b64) + p, (const uint32_t*)(ctx->ws + ctx->L.off_e64) + p,
                                     (const StageDyn*)(ctx->ws + ctx->L.off_dyn) + p, (int64_t*)(ctx->ws + ctx->L.off_nupd) + p, 1,
                                     ctx->L.end64[p], ctx->cfg.optimizer, ctx->cfg.beta1, ctx->cfg.beta2, ctx->cfg.eps, ctx->ls,
-                                    (void*)ctx->ta.ring, ctx->hp.lp_elem, ctx->L.begin64[p], nullptr, nullptr, nullptr, early(ctx));
+                                    (void*)ctx->ta.ring, ctx->hp.lp_elem, ctx->L.begin64[p], nullptr, early(ctx));
       pm_status s = check(ctx, e, "update");
       if (s != PM_OK) return s;
       if (ctx->seg_count[p] > 0) {
@@ -1286,12 +1292,7 @@ pm_status pm_update(pm_ctx* ctx) {
         if (fs != PM_OK) return fs;
       }
       prof_begin(ctx, PM_PROF_UPDATE);
-      e = launch_update(ctx->a, (const uint32_t*)(ctx->ws + ctx->L.off_b64), (const uint32_t*)(ctx->ws + ctx->L.off_e64),
-                        (const StageDyn*)(ctx->ws + ctx->L.off_dyn), (int64_t*)(ctx->ws + ctx->L.off_nupd), P,
-                        ctx->L.total / 64, ctx->cfg.optimizer, ctx->cfg.beta1, ctx->cfg.beta2, ctx->cfg.eps, ctx->ls,
-                        ctx->L.queue ? (void*)ctx->ta.ring : nullptr, ctx->hp.lp_elem, 0,
-                        ctx->L.fuse ? (const uint32_t*)(ctx->ws + ctx->L.off_skb) : nullptr,
-                        ctx->L.fuse ? (const uint32_t*)(ctx->ws + ctx->L.off_ske) : nullptr, nullptr, early(ctx));
+      e = update_all(ctx, (const StageDyn*)(ctx->ws + ctx->L.off_dyn), nullptr);
       pm_status s = check(ctx, e, "update");
       if (s != PM_OK || !ctx->L.queue || ctx->L.segs.empty()) return s;
       prof_begin(ctx, PM_PROF_UPDATE);                                 // fp32 copies of the updated stages' small tensors into their queues
@@ -1514,7 +1515,7 @@ pm_status pm_update_flat(const pm_arenas* arenas, const uint64_t* stage_offsets,
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "schedule");
   ArenasDev a{arenas->w, arenas->m, arenas->s, arenas->delta, arenas->grad, (__nv_bfloat16*)arenas->w_lp, arenas->count};
   e = launch_update(a, (const uint32_t*)(ws + off_b), (const uint32_t*)(ws + off_e), (const StageDyn*)(ws + off_dyn), (int64_t*)(ws + off_nupd), n_stages,
-                    st[n_stages - 1].end64, cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, cs, nullptr, 0, 0, nullptr, nullptr, nullptr, true);
+                    st[n_stages - 1].end64, cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, cs, nullptr, 0, 0, nullptr, true);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "update");
   return PM_OK;
 }

@@ -1,5 +1,7 @@
 // Tick scheduler and the fused multi-tensor PipeMare update (declarations).
 #pragma once
+#include <vector>
+
 #include "pm_common.cuh"
 
 namespace pm {
@@ -37,16 +39,23 @@ inline int mb_table_count(int P, int segment) { return 2 * P + 1 + (segment > 0 
 cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* end64, const StageDyn* dyn,
                           int64_t* nupd, int n_stages, uint64_t total64, int optimizer, float beta1, float beta2,
                           float eps, cudaStream_t stream, void* lp_base = nullptr, int lp_elem = 0, uint64_t first64 = 0,
-                          const uint32_t* skip_b64 = nullptr, const uint32_t* skip_e64 = nullptr, const float* gsrc = nullptr, bool pdl = false);
+                          const float* gsrc = nullptr, bool pdl = false);
 // pdl: launched as a programmatic dependent of the launch before it.
 // gsrc: where the gradients are read (element e of stage i at gsrc[dyn[i].g_shift + e]); null: the grad arena.
-// skip_b64 / skip_e64: per stage, a range of 64-element groups this launch leaves alone (device arrays, or null): the
-// Linear matrices when the weight-gradient GEMM has applied their update in its epilogue.  The stage's update
-// counter is incremented here all the same.
 // first64: the walk over the arenas starts at this 64-element group (a launch for one stage starts at that stage's slice).
 // lp_base / lp_elem: where the operand-type copy of the new weights goes: by default the bfloat16 arena a.w_lp
 // (if there is one); microbatch-major order passes the ring arena and the operand size (2 or 4 bytes), and the
 // stages' table entries give the slot (StageDyn::lp_shift).
+
+// When the weight-gradient GEMM has updated the Linear matrices in its epilogue, the parts of the stages it has left: elements in
+// groups of 64, in chunks of one block each.  The part that counts keeps the stage's update counter.
+struct UpdPart { uint32_t first_chunk, begin64, end64; int32_t stage, counts; };
+struct UpdParts { std::vector<UpdPart> list; uint32_t chunks = 0; int32_t unroll = 1; };
+// [begin64, skip_b64) and [skip_e64, end64) of every stage (host arrays)
+UpdParts update_parts(const uint32_t* begin64, const uint32_t* end64, const uint32_t* skip_b64, const uint32_t* skip_e64, int n_stages);
+// d_parts: the list on the device.  bf16 networks: lp_base is the ring arena or null (the w_lp arena).
+cudaError_t launch_update_parts(ArenasDev a, const UpdParts& p, const UpdPart* d_parts, const StageDyn* dyn, int64_t* nupd, int optimizer,
+                                float beta1, float beta2, float eps, cudaStream_t stream, void* lp_base, bool pdl);
 
 // One fp32 tensor the forward pass reads (a bias, a LayerNorm gain or bias): `count` elements (a multiple of 64,
 // padding included) at arena_off of the master weights; its versions sit at ring_off (bytes, slot 0) of the ring

@@ -112,7 +112,7 @@ pm_status pm_update_flat_static(const pm_arenas* arenas, const uint64_t* stage_o
   ArenasDev a{arenas->w, arenas->m, arenas->s, arenas->delta, arenas->grad, (__nv_bfloat16*)arenas->w_lp, arenas->count};
   e = launch_update(a, (const uint32_t*)(ws + off_b), (const uint32_t*)(ws + off_e), (const StageDyn*)(ws + off_dyn),
                     (int64_t*)(ws + off_nupd), n_stages, tab[n_stages - 1].end64, cfg->optimizer, cfg->beta1, cfg->beta2, cfg->eps, st,
-                    nullptr, 0, 0, nullptr, nullptr, nullptr, true);
+                    nullptr, 0, 0, nullptr, true);
   if (e != cudaSuccess) return fail(PM_ERR_CUDA, cudaGetErrorString(e));
   return PM_OK;
 }
