@@ -467,7 +467,7 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
     int32_t acc = 0;
     for (int p = 0; p < P; ++p) {
       L.ids.push_back(acc);
-      if (l < L.st[p].n_lin) acc += (L.st[p].lin[l].n_out + 255) / 256;
+      if (l < L.st[p].n_lin) acc += (L.st[p].lin[l].n_out + act_cols(T) - 1) / act_cols(T);
     }
     L.ids.push_back(acc);
     L.act_blocks[l] = acc;

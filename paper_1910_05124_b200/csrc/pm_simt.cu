@@ -90,11 +90,9 @@ cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
 // a column are added in warp order.  (fp32 networks: dz only, the weight-gradient GEMM sums the columns of its operand.)
 constexpr int kActWarps = 8;
 
-constexpr int kActColsV = 256;                        // columns per block: 8 per lane
+constexpr int kActColsV = kActCols;                    // columns per block: 8 per lane
 constexpr int kColsumGroup = 8;                       // row chunks per block in a launch that only sums columns
 constexpr int kStageGroup = 4;                        // ... and in a launch of one stage
-constexpr int kSmallRows = 512;                       // microbatches of up to this many rows: a block takes all rows of its columns
-constexpr int kSmallCols = 32;
 // Row chunks one block of the activation-backward launch covers; its sum is partial row (first chunk / group) of the stage.
 __host__ __device__ inline int act_chunk_group(const TickArgs& t) {
   return t.row_chunks > 1 ? (t.colsum_only ? kColsumGroup : (t.sel_p >= 0 ? kStageGroup : 1)) : 1;
@@ -212,7 +210,7 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
   }
 }
 
-// The same for microbatches of at most kSmallRows rows: a block takes 32 columns of ALL rows (eight columns per lane, eight
+// The same for microbatches of at most kActSmallRows rows: a block takes 32 columns of ALL rows (eight columns per lane, eight
 // rows per warp and step), so there are no partial sums to finish in a second launch.  What bounds these launches is the
 // number of rows a block walks one after the other and the launches themselves, not the bytes: with 256-column blocks of 32
 // rows and a finishing launch a level of the 32-stage 1024-wide MLP (128 rows) took 17.6 + 12.7 us.
@@ -220,9 +218,8 @@ template <typename AT>
 __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) {
   pdl_trigger();
   pdl_wait();
-  constexpr int kPer = kActColsV / kSmallCols;
   const int* start = t.act_start + (size_t)lvl * (t.P + 1);
-  const int blk = (int)(blockIdx.x / kPer) + t.act_first[lvl];
+  const int blk = (int)blockIdx.x + t.act_first[lvl];
   int lo = 0, hi = t.P - 1;
   if (t.sel_p >= 0) lo = hi = t.sel_p;
   while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (start[mid] <= blk) lo = mid; else hi = mid - 1; }
@@ -231,7 +228,7 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
   const StageDev& s = t.st[p];
   if (d.b_mb < 0 || lvl >= s.n_lin) return;
   const LinDev& L = s.lin[lvl];
-  const int c0 = (blk - start[p]) * kActColsV + (int)(blockIdx.x % kPer) * kSmallCols;
+  const int c0 = (blk - start[p]) * kActSmallCols;
   if (c0 >= L.n_out) return;
   const bool has_act = bwd_act(L) != PM_ACT_NONE && !t.colsum_only;
   const bool sums = sizeof(AT) == 2 && !t.dz_only;
@@ -262,7 +259,7 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
       }
   }
   if (!sums) return;
-  __shared__ float red[8][kSmallCols];
+  __shared__ float red[8][kActSmallCols];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {                             // the eight rows of the warp, in a fixed order
     sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 4));
@@ -272,7 +269,7 @@ __global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) 
   }
   __syncthreads();
   const int cc = c0 + threadIdx.x;
-  if (threadIdx.x < kSmallCols && cc < L.n_out) {
+  if (threadIdx.x < kActSmallCols && cc < L.n_out) {
     float a = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) a = __fadd_rn(a, red[w][threadIdx.x]);
@@ -360,12 +357,12 @@ __global__ void __launch_bounds__(kActColsV) bias_finish_few_kernel(TickArgs t, 
   t.a.grad[L.b_off + c] = d.accum ? __fadd_rn(t.a.grad[L.b_off + c], a) : a;
 }
 
-int actbwd_launches(const TickArgs& t, int dtype) { return (t.T <= kSmallRows || t.row_chunks == 1 || t.dz_only || dtype == PM_F32) ? 1 : 2; }
+int actbwd_launches(const TickArgs& t, int dtype) { return (t.T <= kActSmallRows || t.row_chunks == 1 || t.dz_only || dtype == PM_F32) ? 1 : 2; }
 
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream) {
   if (t.act_blocks[lvl] == 0) return cudaSuccess;
-  if (t.T <= kSmallRows)
-    return launch_pdl(dtype == PM_F32 ? actbwd_small_kernel<float> : actbwd_small_kernel<__nv_bfloat16>, dim3(t.act_blocks[lvl] * (kActColsV / kSmallCols)), dim3(256), 0, stream, t.pdl, t, lvl);
+  if (t.T <= kActSmallRows)
+    return launch_pdl(dtype == PM_F32 ? actbwd_small_kernel<float> : actbwd_small_kernel<__nv_bfloat16>, dim3(t.act_blocks[lvl]), dim3(256), 0, stream, t.pdl, t, lvl);
   const int cg = act_chunk_group(t);
   dim3 grid(t.act_blocks[lvl], (t.row_chunks + cg - 1) / cg);
   cudaError_t e;

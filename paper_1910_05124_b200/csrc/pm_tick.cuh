@@ -6,6 +6,12 @@
 
 namespace pm {
 
+// Columns of a block of the activation-backward launches.  Microbatches of up to kActSmallRows rows: a block takes all rows of
+// few columns, so the list of its blocks counts those.  (Eight blocks per 256 columns whatever the width made a tick of
+// 512 stages of width 32 80 us; the exact list 68.)
+constexpr int kActCols = 256, kActSmallRows = 512, kActSmallCols = 32;
+inline int act_cols(uint64_t T) { return T <= (uint64_t)kActSmallRows ? kActSmallCols : kActCols; }
+
 // Everything a tick kernel needs; passed by value.
 struct TickArgs {
   const StageDev* st;
@@ -27,7 +33,7 @@ struct TickArgs {
   int32_t att_S, att_dk, att_blocks;                   // attention: sequence length, head width, (sequences x heads); 0 = none
   int32_t max_vocab, max_embed_dim;
   uint64_t loss_off;      // ws: loss log [loss_cap] float
-  uint64_t lossred_off;   // ws: per-block loss partials [64] float + completion counter
+  uint64_t lossred_off;   // ws: per-block loss partials [96] float + completion counter (MSE; cross-entropy: the counter at 64)
   int64_t loss_cap;
   // stage lists of the grouped launches (device, in pipeline order): stages with a pre-op, with LayerNorm, with an
   // embedding, with a residual add; grids have one block row per list entry
@@ -35,7 +41,7 @@ struct TickArgs {
   int32_t n_pre, n_ln, n_embed, n_res;
   uint64_t lnred_off;     // ws: LayerNorm parameter-gradient partials [n_ln][ln_chunks][2*max_ln_dim] float
   int32_t ln_chunks, ln_chunk_rows, max_ln_dim;
-  // activation-backward launches: column blocks (256 columns) of Linear `lvl` over all stages, flattened;
+  // activation-backward launches: column blocks (act_cols columns) of Linear `lvl` over all stages, flattened;
   // act_start[lvl * (P + 1) + p] is the first block of stage p, act_blocks[lvl] the total
   const int32_t* act_start;
   int32_t act_blocks[PM_MAX_LINEARS];
