@@ -129,3 +129,26 @@ def test_recompute_rules(cuda_device):
     assert q(4) == q(0) and q(9) == q(0)
     # stages 1, 2 keep tau_recomp + 1 = 4, 2 corrected versions of their 64 x 64 + 64 fp32 parameters (padded to 64)
     assert q(2)[1] - q(0)[1] == (4 + 2) * (64 * 64 + 64) * 4
+
+
+# several Linears per stage: act'(z) is applied where the gradient is formed, but not across a segment's edge, and the weight
+# gradients are grouped by segment; more than 512 rows: dz alone on the way, column sums per Linear at the end
+@pytest.mark.parametrize("P,S,width,linears,T,act,compute,n_micro", [
+    (5, 2, 40, 2, 7, "gelu", "f32", 1),
+    (4, 1, 17, 3, 33, "relu", "f32", 1),
+    (6, 3, 48, 2, 9, "relu", "f32", 2),
+    (3, 2, 72, 4, 20, "gelu", "f32", 1),
+    (4, 2, 72, 2, 600, "gelu", "bf16", 1),
+    (4, 1, 264, 3, 600, "relu", "bf16", 2),
+    (3, 0, 264, 2, 700, "gelu", "bf16", 1),
+    (3, 2, 520, 2, 1100, "relu", "bf16", 1),
+])
+def test_several_linears_per_stage(cuda_device, P, S, width, linears, T, act, compute, n_micro):
+    wl = I.mlp_workload("rcl", P, width, linears, act, T, compute=compute, optimizer="sgdm", alpha=0.05 if compute == "f32" else 0.02,
+                        K=6, D=0.5, steps=4 * n_micro, seed=191005124 + 90 + P)
+    wl.tau_fwd, wl.tau_bkwd = I.pipemare_delays(P, n_micro)
+    params0 = I.init_stage_params(wl)
+    res = run_oracle(wl, params0, wl.steps, n_micro=n_micro, segment=S or None)
+    pipe, losses, _ = run_gpu_pipeline(wl, params0, wl.steps, loop_order="mb_major", n_micro=n_micro, segment=S, collect_book=False)
+    np.testing.assert_allclose(losses, np.array(res.losses), rtol=2e-5 if compute == "f32" else 1e-3)
+    compare_params(pipe, res, 1e-5 if compute == "f32" else 2e-2)
