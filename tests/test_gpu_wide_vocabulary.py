@@ -1,5 +1,5 @@
-"""Vocabularies much larger than the microbatch: the embedding gradient that zeroes the table and sums the rows of the tokens
-that occur, and the cross-entropy that walks long rows of logits."""
+"""Vocabularies much larger than the microbatch: the embedding gradient, most of whose rows have no token, and the
+cross-entropy that walks long rows of logits."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,28 @@ def test_embedding_gradient_and_loss(cuda_device, compute, d_model, seq, batch, 
     assert ((torch.from_numpy(table).double() - ref).abs() <= T * 2.0 ** -24 * scale + 1e-30).all()
     loss = pipe.pm_get_losses(0, 1)[0]
     assert abs(loss - other.pm_get_losses(0, 1)[0]) <= 1e-6 * loss
+
+
+# rows of logits that leave a thread's registers part empty and fill them, and rows too long for them; more rows than SMs (a block
+# walks several), fewer, and an odd number; the whole network in float64, with the same roundings, as the reference
+@pytest.mark.parametrize("vocab,batch", [(8200, 25), (16384, 33), (32768, 19), (32768, 40), (33000, 20)])
+@pytest.mark.parametrize("compute", ["f32", "bf16"])
+def test_cross_entropy_of_long_rows(cuda_device, compute, vocab, batch):
+    import torch
+    import paper_1910_05124_b200 as pm
+    from oracle import transformer
+    wl = I.encoder_workload("long", 1, 64, 2, 64, 9, batch, vocab, compute=compute, optimizer="sgdm", alpha=0.0, K=4, D=0.5, steps=1, seed=vocab + batch)
+    params0 = I.init_encoder_params(wl)
+    params0[-1][2] *= np.float32(3)                                  # logits of a trained network's spread: probabilities up to 1e-2
+    data = lambda t: I.token_batch(wl, 0)
+    ref_loss, ref = transformer.make_grad_fn(wl.stage_specs, data, 2, 9, vocab, compute)(0, params0, params0)
+    pipe = pm.Pipeline(wl, params0, loop_order="mb_major")
+    pipe.pm_step(*(torch.from_numpy(a.astype(np.int32)).cuda() for a in data(0)))
+    got = pipe.unpack(pipe.grad)
+    # fp32: sums of up to V terms in 64-bit against 32-bit order, sqrt(V) 2^-24; bf16: the gradient of the logits is rounded once
+    # (2^-9 at most, 2^-10 on average) and its exponentials are the hardware's
+    tol = 5e-5 if compute == "f32" else 1e-2
+    assert abs(pipe.pm_get_losses(0, 1)[0] - ref_loss) <= (1e-5 if compute == "f32" else 1e-3) * ref_loss
+    for p, stage in ((-1, got[-1]), (-2, got[-2])):
+        for j, a in enumerate(stage):
+            assert np.linalg.norm(a - ref[p][j]) <= tol * np.linalg.norm(ref[p][j]), (p, j)
