@@ -687,6 +687,28 @@ def workload_report(res, peaks, steps):
             "kernel_ms_per_step": {k: round(v, 5) for k, v in sorted(res["per_tick_ms"].items(), key=lambda kv: -kv[1])}}
 
 
+LINE_BYTES = 2500     # a reader that keeps the last few kilobytes of the output still has the whole line
+
+
+def split_line(line):
+    """The result as one short line for stdout, and everything that was measured beside it (per-kernel rooflines, other
+    workloads in full, the update sweep) as a second record, printed to stderr."""
+    long_keys = ("rooflines", "roofline_update", "gemm_all", "elementwise", "kernel_ms_per_step", "other_workloads", "variants",
+                 "update_sweep", "cpu_baseline")
+    brief = {k: v for k, v in line.items() if k not in long_keys}
+    detail = {k: v for k, v in line.items() if k in long_keys}
+    for key, label in (("other_workloads", "workload"), ("variants", "option")):
+        if line.get(key):
+            brief[key] = {str(o[label]).split(":")[0]: o.get("value", "error") for o in line[key]}
+    if "cpu_baseline" in line:
+        brief["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if k != "sample"}
+    for key in ("roofline", "repeats", "cpu_baseline", "variants", "other_workloads"):      # what can go first, should the line still be long
+        if len(json.dumps(brief)) <= LINE_BYTES:
+            break
+        detail.setdefault(key, brief.pop(key, None))
+    return brief, detail
+
+
 def run_cuda(args):
     import torch
     world, rank, local = dist_setup(args.gpus)
@@ -783,7 +805,9 @@ def run_cuda(args):
             line["cpu_baseline"] = cpu_baseline(args.workload, 2 if args.workload in ("cfg3", "cfg1") else 1)
         if not args.no_sweep:
             line["update_sweep"] = update_sweep(device, peaks["hbm"])
-    print(json.dumps(line), flush=True)
+    brief, detail = split_line(line)
+    print(json.dumps(detail), file=sys.stderr, flush=True)
+    print(json.dumps(brief), flush=True)
 
 
 # ---- the reference arm: the CPU oracle -------------------------------------------------------------
