@@ -7,6 +7,9 @@
 
 namespace pm {
 
+// SMs of a B200: the rules that choose tiles and grids were measured for it
+constexpr int kSms = 148;
+
 // Programmatic dependent launch: a kernel launched with pdl may start once every block of its predecessor has triggered (or
 // ended); pdl_wait returns when that predecessor has ended and its writes are visible, and at once in a kernel launched plainly.
 // A kernel that may be launched this way calls pdl_wait in every block before it ends, so that "its predecessor has ended"

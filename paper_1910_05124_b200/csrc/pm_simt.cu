@@ -16,8 +16,8 @@ template <typename AT> __device__ __forceinline__ AT* ws_ptr(const TickArgs& t, 
 
 // ---- MSE loss at the last stage ------------------------------------------------------------------
 // loss = mean over T*out of (y - y*)^2 ;  dy = 2 (y - y*) / (T*out), stored in the activation type.
-// Fixed summation order: each block sums a contiguous chunk (strided per-thread partials, fixed tree),
-// the last block to finish adds the per-block partials in block order.
+// Fixed summation order: each block sums a contiguous chunk (strided per-thread partials, fixed tree), the last block to
+// finish adds the per-block partials: 32 lanes every 32nd of them, then a tree over the lanes.
 constexpr int kLossBlocks = 96, kLossThreads = 256;     // partial sums and the counter share a 512-byte block of the workspace
 
 template <typename AT>
@@ -648,7 +648,7 @@ cudaError_t simt_gemm_set_limits() {
   return e;
 }
 
-// 16 x 16 tiles while the 32 x 32 ones of all stages of the launch would number no more than the 148 SMs: a smaller tile has a
+// 16 x 16 tiles while the 32 x 32 ones of all stages of the launch would number no more than the SMs: a smaller tile has a
 // quarter of the multiplies on its critical path and the chip is not full anyway.
 // Tiles are counted over the launch's own Linears.  (Sized by the widest Linear of the network, the launches of a network with a
 // large vocabulary were mostly blocks without a tile: a tick of a 6-layer encoder of width 64, 64 rows and a vocabulary of
@@ -664,7 +664,7 @@ cudaError_t launch_simt_gemm(const TickArgs& t, const std::vector<StageDev>& st,
     most32 = std::max(most32, n32);
     most16 = std::max(most16, ((M + 15) / 16) * ((N + 15) / 16));
   }
-  if (all32 <= 148)
+  if (all32 <= kSms)
     return mode == 0 ? launch_f32_t<4, 2, 4, 0>(t, lvl, most16, stream) : (mode == 1 ? launch_f32_t<4, 2, 3, 1>(t, lvl, most16, stream) : launch_f32_t<4, 2, 4, 2>(t, lvl, most16, stream));
   return mode == 0 ? launch_f32_t<8, 4, 2, 0>(t, lvl, most32, stream) : (mode == 1 ? launch_f32_t<8, 4, 2, 1>(t, lvl, most32, stream) : launch_f32_t<8, 4, 2, 2>(t, lvl, most32, stream));
 }

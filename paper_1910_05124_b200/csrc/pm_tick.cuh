@@ -191,7 +191,7 @@ template <typename AT> __device__ __forceinline__ AT* y_dest(const TickArgs& t, 
 // May this launch, of a kernel whose blocks do much between its start and its end, start early (t.pdl)?  As long as its blocks find
 // an SM each: more of them crowd on the SMs that the predecessor leaves first.  (An update of a 2-layer encoder of width 1032
 // with 384 blocks of attention on the CUDA cores: 2026 us with them early, 1942 without; with 32 blocks, 290 and 292.)
-inline bool early(const TickArgs& t, dim3 grid) { return t.pdl != 0 && grid.x * grid.y <= 148; }
+inline bool early(const TickArgs& t, dim3 grid) { return t.pdl != 0 && grid.x * grid.y <= (unsigned)kSms; }
 // MSE loss of the microbatch whose backward starts this tick, and dL/dy into the last stage's mailbox.
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream);
 // dz = dy * act'(z) and db = column sums, level `lvl` of every stage that runs backward this tick.

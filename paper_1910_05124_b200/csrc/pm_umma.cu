@@ -1797,7 +1797,7 @@ struct UmmaPlan {
   int row_n[2][PM_MAX_LINEARS] = {};
   std::vector<StageDev> st;              // host copy of the stages (launches of one stage with few tiles)
   const int* d_identity = nullptr;       // 0, 1, 2, ...
-  int max_ctas = 148;
+  int max_ctas = kSms;
 };
 
 // Tile tables of every (mode, level): the flattened tile ids per stage, and the order in which the persistent
@@ -1819,7 +1819,7 @@ static int device_sms() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
     cudaGetLastError();
-    return 148;
+    return kSms;
   }
   return sms;
 }

@@ -332,10 +332,10 @@ struct RowShape { int bn = 0, split = 1; };                    // bn = 0: the la
 
 inline RowShape row_shape_of(long long t32, long long t64, int kb) {      // tiles of 32 and 64 columns, k-blocks
   RowShape r;
-  if (t64 > 296) return r;
-  r.bn = t32 <= 148 ? 32 : 64;
+  if (t64 > 2 * kSms) return r;
+  r.bn = t32 <= kSms ? 32 : 64;
   const long long base = r.bn == 32 ? t32 : t64;
-  r.split = (base * 4 <= 160 && kb >= 8) ? 4 : ((base * 2 <= 296 && kb >= 4) ? 2 : 1);
+  r.split = (base <= 40 && kb >= 8) ? 4 : ((base <= kSms && kb >= 4) ? 2 : 1);   // CTAs: about one per SM in four parts, two in two
   return r;
 }
 inline RowShape row_shape(int T, int N, int K) {

@@ -2,10 +2,10 @@
 //
 // The update is a pure HBM stream: per parameter it reads g, w, m, delta (and s for
 // Adam) and writes w, m, delta (and s) in fp32 plus a bfloat16 copy of w: 30 bytes per
-// parameter for momentum SGD, 38 for Adam.  One launch covers every stage; the stage
-// that owns a 64-element group is found by binary search in shared memory, and that
-// stage's scalars (T1 step size, T2 decay, Adam bias corrections) come from the table
-// the scheduler wrote for this tick.
+// parameter for momentum SGD, 38 for Adam.  One launch covers every stage; a block finds
+// the stage of its first 64-element group in the table of stage bounds (by an even split's
+// guess, else by binary search), and that stage's scalars (T1 step size, T2 decay, Adam
+// bias corrections) come from the table the scheduler wrote for this tick.
 //
 // Arithmetic order (each operation rounded once in fp32, no fused multiply-add, so that
 // results can be reproduced bit for bit by any IEEE implementation):
@@ -25,8 +25,6 @@ namespace pm {
 // the one that entered at tick s-(2P-i) (microbatch = entry tick, except during a synchronous warm-up).  T1 (Eq. 2): alpha_i = alpha_base(k) / tau_i^p, p = 1 - min(k/K, 1).
 // T2: gamma_i = D^(1/(tau_fwd,i - tau_bkwd,i)).  Scalars are evaluated in double and rounded to
 // float once.
-// Per-stage state of one tick: forward microbatch a and backward microbatch b (-1: idle), `ver` updates applied to the
-// stage so far, the version `fver` its forward reads; k >= 0 activates the update with that index.
 // non-negative a modulo d, without the 64-bit division while a fits 32 bits
 __device__ __forceinline__ int32_t slot_of(int64_t a, int32_t d) {
   return ((uint64_t)a >> 32) == 0 ? (int32_t)((uint32_t)a % (uint32_t)d) : (int32_t)(a % d);
@@ -71,7 +69,9 @@ __device__ __forceinline__ DynScalars quad_scalars(const StageSched& s, const Hy
   return o;
 }
 
-// kb: the update index the microbatch in backward belongs to (one microbatch per update: itself)
+// Per-stage state of one tick: forward microbatch a and backward microbatch b (-1: idle), `ver` updates applied to the
+// stage so far, the version `fver` its forward reads; k >= 0 activates the update with that index.
+// kb: the update index the microbatch in backward belongs to (one microbatch per update: itself).
 __device__ StageDyn make_dyn(const StageSched& s, const HyperDev& hp, int64_t tick, int64_t a, int64_t b, int64_t k,
                              int64_t ver, int64_t fver, bool slots, int64_t kb) {
   StageDyn d;
@@ -419,7 +419,7 @@ update_kernel(ArenasDev a, void* lp_base, const uint32_t* begin64, const uint32_
 }
 
 // up to four waves of blocks at one float4 group per thread and array
-static bool few_chunks(uint64_t vec4) { return vec4 <= 4ull * 148 * 8 * kUpdThreads; }
+static bool few_chunks(uint64_t vec4) { return vec4 <= 4ull * kSms * 8 * kUpdThreads; }
 
 UpdParts update_parts(const uint32_t* begin64, const uint32_t* end64, const uint32_t* skip_b64, const uint32_t* skip_e64, int n_stages) {
   UpdParts p;

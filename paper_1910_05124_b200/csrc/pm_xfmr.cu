@@ -709,9 +709,7 @@ cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
     const bool rows = V <= 32 * kCeLongThreads;              // longer rows do not fit a block's registers
     auto* kernel = rows ? (dtype == PM_F32 ? ce_loss_rows_kernel<float> : ce_loss_rows_kernel<__nv_bfloat16>)
                         : (dtype == PM_F32 ? ce_loss_long_kernel<float> : ce_loss_long_kernel<__nv_bfloat16>);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); sms = 148; }
-    return launch_pdl(kernel, dim3(rows ? std::min(sms, (int)t.T) : t.T), dim3(kCeLongThreads), row_bytes, stream, t.pdl, t);
+    return launch_pdl(kernel, dim3(rows ? std::min(kSms, (int)t.T) : t.T), dim3(kCeLongThreads), row_bytes, stream, t.pdl, t);
   }
   return launch_pdl(dtype == PM_F32 ? ce_loss_kernel<float> : ce_loss_kernel<__nv_bfloat16>, dim3(t.T), dim3(256), 0, stream, t.pdl, t);
 }
@@ -1365,7 +1363,7 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     const int slices = (dm + 32 * cpl - 1) / (32 * cpl);
     int n_blk = 1;                                           // a power of two with at most kEmbRows rows per block ...
     while (n_blk * kEmbRows < t.max_vocab) n_blk <<= 1;
-    while (n_blk * slices * t.n_embed < 2 * 148 && t.max_vocab / n_blk > 32) n_blk <<= 1;   // ... and enough blocks for a small vocabulary
+    while (n_blk * slices * t.n_embed < 2 * kSms && t.max_vocab / n_blk > 32) n_blk <<= 1;   // ... and enough blocks for a small vocabulary
     dim3 g(n_blk, t.n_embed, slices);
     // the hit list, the same tokens grouped by row, and the per-warp partial sums of a shared row
     const size_t smem = 2 * sizeof(int32_t) * (size_t)t.T + sizeof(float) * 8 * 32 * (size_t)cpl;
