@@ -11,6 +11,15 @@ constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;      // bounded waits: abo
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// 16 bytes that an earlier launch of a programmatic chain wrote: an ordinary load (cached in L1, unlike ld.global.nc defined for data
+// that was written during this kernel's lifetime) which stays behind the wait; as plain C++ the compiler moves the loads of an
+// epilogue together and spills their registers.
+__device__ __forceinline__ uint4 ld_chain16(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }

@@ -208,7 +208,7 @@ __device__ __forceinline__ void epi_block(const TickArgs& t, const CUtensorMap* 
             const uint32_t w[4] = {skq[g].x, skq[g].y, skq[g].z, skq[g].w};
             // the registers just read take the NEXT block's skip values (same row, 64 columns on): their latency hides
             // behind the rest of this block instead of standing in front of the next one
-            if (next_skip) skq[g] = 8 * g < next_cols ? __ldcg(reinterpret_cast<const uint4*>(next_skip + 8 * g)) : make_uint4(0u, 0u, 0u, 0u);
+            if (next_skip) skq[g] = 8 * g < next_cols ? ld_chain16(next_skip + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const float2 sk = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
@@ -279,7 +279,8 @@ __device__ __forceinline__ void epi_block(const TickArgs& t, const CUtensorMap* 
   if (!both) es.slot ^= 1u;
 }
 
-// (Skip tensors and stashes are written by launches this one may overlap with: coherent loads, not read-only ones.)
+// (Skip tensors and stashes are written by launches this one may overlap with: ld_chain16, not read-only loads.  A lane
+// reads its row's 128 bytes in eight pieces, so they go through L1: a tick of the 6-layer encoder 1255 us, and 1259 from L2.)
 // The 64 skip-tensor values of row `row`, columns nb .. nb+63, that a residual stage's epilogue adds (zeros outside
 // the tensor and for other stages).  Issued before the accumulator is awaited, so the loads overlap the main loop.
 __device__ __forceinline__ void load_skip64(const TickArgs& t, const StageDev& s, const StageDyn& d, int N, int row, int nb, uint4 (&skq)[8]) {
@@ -287,7 +288,7 @@ __device__ __forceinline__ void load_skip64(const TickArgs& t, const StageDev& s
   const __nv_bfloat16* skrow = ws_at<__nv_bfloat16>(t, s.skip_in) + (uint64_t)d.skip_rslot * ((uint64_t)t.T * N) + (uint64_t)row * N + nb;
 #pragma unroll
   for (int g = 0; g < 8; ++g)                                       // columns are multiples of 8
-    skq[g] = (on && nb + 8 * g < N) ? __ldcg(reinterpret_cast<const uint4*>(skrow + 8 * g)) : make_uint4(0u, 0u, 0u, 0u);
+    skq[g] = (on && nb + 8 * g < N) ? ld_chain16(skrow + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
 }
 
 // dgrad epilogue of a stage whose predecessor's ReLU backward is fused here (StageDev::mask_dx): the 64 values of this
@@ -301,7 +302,7 @@ __device__ __forceinline__ uint64_t load_mask_bits64(const TickArgs& t, const St
   uint4 xq[8];
 #pragma unroll
   for (int g = 0; g < 8; ++g)
-    xq[g] = (nb + 8 * g < N) ? __ldcg(reinterpret_cast<const uint4*>(xrow + 8 * g)) : make_uint4(0u, 0u, 0u, 0u);
+    xq[g] = (nb + 8 * g < N) ? ld_chain16(xrow + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
   uint64_t mk = 0ull;
 #pragma unroll
   for (int g = 0; g < 8; ++g) {
