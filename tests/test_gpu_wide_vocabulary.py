@@ -80,3 +80,23 @@ def test_cross_entropy_of_long_rows(cuda_device, compute, vocab, batch):
     for p, stage in ((-1, got[-1]), (-2, got[-2])):
         for j, a in enumerate(stage):
             assert np.linalg.norm(a - ref[p][j]) <= tol * np.linalg.norm(ref[p][j]), (p, j)
+
+
+# the hit list of the embedding gradient grows with the microbatch: just below, at and beyond 48 KB beside the kernel's static
+# shared memory (a launch of 46 KB used to be refused)
+@pytest.mark.parametrize("batch", [224, 240, 256])
+@pytest.mark.parametrize("compute", ["f32", "bf16"])
+def test_embedding_gradient_of_long_microbatches(cuda_device, compute, batch):
+    import torch
+    import paper_1910_05124_b200 as pm
+    from oracle import transformer
+    wl = I.encoder_workload("hits", 1, 256, 4, 32, 16, batch, 40, compute=compute, optimizer="sgdm", alpha=0.0, K=4, D=0.5, steps=1, seed=batch)
+    params0 = I.init_encoder_params(wl)
+    data = lambda t: I.token_batch(wl, 0)
+    ref_loss, ref = transformer.make_grad_fn(wl.stage_specs, data, 4, 16, 40, compute)(0, params0, params0)
+    pipe = pm.Pipeline(wl, params0, loop_order="mb_major")
+    pipe.pm_step(*(torch.from_numpy(a.astype(np.int32)).cuda() for a in data(0)))
+    table = pipe.unpack(pipe.grad)[0][0]
+    assert abs(pipe.pm_get_losses(0, 1)[0] - ref_loss) <= (1e-5 if compute == "f32" else 1e-3) * ref_loss
+    # fp32: sums of a hundred tokens behind five Linears; bf16: a dozen roundings of 2^-9 in front of them
+    assert np.linalg.norm(table - ref[0][0]) <= (1e-4 if compute == "f32" else 2e-2) * np.linalg.norm(ref[0][0])
