@@ -750,10 +750,8 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
     pm_status as = attn_plan_create(&c->attn, t, c->L.st, c->ws + L.off_attn, c->stream, aerr);
     if (as != PM_OK) { delete c; return fail(nullptr, as, aerr); }
   }
-  if (L.any_pre || L.att_blocks > 0 || cfg->loss == PM_LOSS_CE) {
-    e = xfmr_set_smem_limits(cfg->compute_dtype);
-    if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "shared-memory limits"); delete c; return r; }
-  }
+  e = xfmr_set_smem_limits(t, cfg->compute_dtype, L.att_blocks > 0 && !L.att_tc);
+  if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "shared-memory limits"); delete c; return r; }
   if (cfg->compute_dtype == PM_F32) {
     e = simt_gemm_set_limits();
     if (e != cudaSuccess) { pm_status r = cuda_fail(nullptr, e, "GEMM shared-memory limit"); delete c; return r; }

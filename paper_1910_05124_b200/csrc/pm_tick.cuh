@@ -216,8 +216,8 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream);  
 int pre_bwd_launches(const TickArgs& t);
 size_t attention_smem_bytes(int S, int dk, int dtype);
 
-// opt-in shared-memory sizes of the Transformer kernels of one operand type, on the current device
-cudaError_t xfmr_set_smem_limits(int dtype);
+// opt-in shared-memory sizes of the Transformer kernels a context will launch (t: its launch arguments), on the current device
+cudaError_t xfmr_set_smem_limits(const TickArgs& t, int dtype, bool simt_attention);
 
 // fp32 SIMT grouped GEMMs (PM_F32 path).  mode: 0 forward, 1 dgrad (corrected weights), 2 wgrad.
 cudaError_t simt_gemm_set_limits();

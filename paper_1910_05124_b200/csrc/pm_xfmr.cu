@@ -702,15 +702,16 @@ __global__ void __launch_bounds__(kCeLongThreads, 1) ce_loss_rows_kernel(TickArg
   ce_finish(t, d);
 }
 
+// rows of logits that are kept in shared memory, and the kernel for them: rows too long for a block's registers take the second
+static bool ce_in_smem(int V) { return V > 8192 && (V & 3) == 0 && sizeof(float) * (size_t)V <= 200 * 1024; }
+static bool ce_in_registers(int V) { return V <= 32 * kCeLongThreads; }
+template <typename AT> static auto ce_smem_kernel(int V) { return ce_in_registers(V) ? ce_loss_rows_kernel<AT> : ce_loss_long_kernel<AT>; }
+
 cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
   const int V = t.n_out_last;
-  const size_t row_bytes = sizeof(float) * (size_t)V;
-  if (V > 8192 && (V & 3) == 0 && row_bytes <= 200 * 1024) {
-    const bool rows = V <= 32 * kCeLongThreads;              // longer rows do not fit a block's registers
-    auto* kernel = rows ? (dtype == PM_F32 ? ce_loss_rows_kernel<float> : ce_loss_rows_kernel<__nv_bfloat16>)
-                        : (dtype == PM_F32 ? ce_loss_long_kernel<float> : ce_loss_long_kernel<__nv_bfloat16>);
-    return launch_pdl(kernel, dim3(rows ? std::min(kSms, (int)t.T) : t.T), dim3(kCeLongThreads), row_bytes, stream, t.pdl, t);
-  }
+  if (ce_in_smem(V))
+    return launch_pdl(dtype == PM_F32 ? ce_smem_kernel<float>(V) : ce_smem_kernel<__nv_bfloat16>(V), dim3(ce_in_registers(V) ? std::min(kSms, (int)t.T) : t.T),
+                      dim3(kCeLongThreads), sizeof(float) * (size_t)V, stream, t.pdl, t);
   return launch_pdl(dtype == PM_F32 ? ce_loss_kernel<float> : ce_loss_kernel<__nv_bfloat16>, dim3(t.T), dim3(256), 0, stream, t.pdl, t);
 }
 
@@ -1100,15 +1101,19 @@ __global__ void __launch_bounds__(256) ln_fused_finish_kernel(TickArgs t) {
   }
 }
 
-template <typename AT, int NP, int WPR>
+// up to 256 and 512 columns a warp holds a row in one and two groups of 8 per lane, beyond that two warps share it
+template <typename AT> static auto ln_fused_kernel(int d) {
+  return d <= 256 ? ln_bwd_fused_kernel<AT, 1, 1> : (d <= 512 ? ln_bwd_fused_kernel<AT, 2, 1> : ln_bwd_fused_kernel<AT, 2, 2>);
+}
+template <typename AT>
 static cudaError_t launch_ln_fused(const TickArgs& t, cudaStream_t stream) {
-  size_t smem = (size_t)8 * 2 * NP * 256 * sizeof(float);
+  size_t smem = (size_t)8 * 2 * (t.max_ln_dim <= 256 ? 1 : 2) * 256 * sizeof(float);
   // launches of one stage stage their rows in shared memory when two such blocks fit on an SM
   const size_t stage_bytes = (size_t)3 * t.ln_chunk_rows * t.max_ln_dim * sizeof(AT);
   TickArgs ta = t;
   ta.ln_stage = (t.sel_p >= 0 && stage_bytes <= 100 * 1024 && (t.max_ln_dim * sizeof(AT)) % 16 == 0) ? 1 : 0;
   if (ta.ln_stage) smem = std::max(smem, stage_bytes);
-  const cudaError_t e = launch_pdl(ln_bwd_fused_kernel<AT, NP, WPR>, dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, false, ta);
+  const cudaError_t e = launch_pdl(ln_fused_kernel<AT>(t.max_ln_dim), dim3(t.ln_chunks, t.n_ln), dim3(256), smem, stream, false, ta);
   if (e != cudaSuccess || t.defer_finish) return e;
   return launch_pdl(ln_fused_finish_kernel, dim3((t.max_ln_dim + kLnFinCols - 1) / kLnFinCols, t.n_ln), dim3(256), 0, stream, false, t);
 }
@@ -1325,6 +1330,10 @@ __global__ void __launch_bounds__(256) embed_bwd_kernel(TickArgs t) {
   }
 }
 
+// columns per lane: wide models are cut into column slices so that a row with many tokens is spread over blocks
+static int embed_cpl(int dm) { return (dm % 16 == 0 && dm <= 512) ? 16 : (dm % 8 == 0 ? 8 : 4); }
+template <typename AT> static auto embed_kernel(int cpl) { return cpl == 16 ? embed_bwd_kernel<AT, 16> : (cpl == 8 ? embed_bwd_kernel<AT, 8> : embed_bwd_kernel<AT, 4>); }
+
 int pre_bwd_launches(const TickArgs& t) {
   const int fin = t.defer_finish ? 0 : 1;
   return (t.any_ln ? (t.ln_fused ? 1 + fin : (t.row_chunks == 1 ? 2 : 2 + fin)) : 0) + (t.any_embed ? 1 : 0);
@@ -1342,8 +1351,7 @@ cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream) {
 cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
   cudaError_t e = cudaSuccess;
   if (t.any_ln && t.ln_fused) {
-    if (dtype == PM_F32) e = t.max_ln_dim <= 256 ? launch_ln_fused<float, 1, 1>(t, stream) : (t.max_ln_dim <= 512 ? launch_ln_fused<float, 2, 1>(t, stream) : launch_ln_fused<float, 2, 2>(t, stream));
-    else e = t.max_ln_dim <= 256 ? launch_ln_fused<__nv_bfloat16, 1, 1>(t, stream) : (t.max_ln_dim <= 512 ? launch_ln_fused<__nv_bfloat16, 2, 1>(t, stream) : launch_ln_fused<__nv_bfloat16, 2, 2>(t, stream));
+    e = dtype == PM_F32 ? launch_ln_fused<float>(t, stream) : launch_ln_fused<__nv_bfloat16>(t, stream);
     if (e != cudaSuccess) return e;
   } else if (t.any_ln) {
     dim3 g1((t.T + 7) / 8, t.n_ln), g2((t.max_ln_dim + kLnCols - 1) / kLnCols, t.row_chunks, t.n_ln);
@@ -1357,9 +1365,8 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     }
   }
   if (t.any_embed) {
-    // columns per lane: wide models are cut into column slices so that a row with many tokens is spread over blocks
     const int dm = t.max_embed_dim;
-    const int cpl = (dm % 16 == 0 && dm <= 512) ? 16 : (dm % 8 == 0 ? 8 : 4);
+    const int cpl = embed_cpl(dm);
     const int slices = (dm + 32 * cpl - 1) / (32 * cpl);
     int n_blk = 1;                                           // a power of two with at most kEmbRows rows per block ...
     while (n_blk * kEmbRows < t.max_vocab) n_blk <<= 1;
@@ -1367,11 +1374,7 @@ cudaError_t launch_pre_bwd(const TickArgs& t, int dtype, cudaStream_t stream) {
     dim3 g(n_blk, t.n_embed, slices);
     // the hit list, the same tokens grouped by row, and the per-warp partial sums of a shared row
     const size_t smem = 2 * sizeof(int32_t) * (size_t)t.T + sizeof(float) * 8 * 32 * (size_t)cpl;
-    auto go = [&](auto kernel) -> cudaError_t {
-      return launch_pdl(kernel, g, dim3(256), smem, stream, false, t);
-    };
-    if (dtype == PM_F32) e = cpl == 16 ? go(embed_bwd_kernel<float, 16>) : (cpl == 8 ? go(embed_bwd_kernel<float, 8>) : go(embed_bwd_kernel<float, 4>));
-    else e = cpl == 16 ? go(embed_bwd_kernel<__nv_bfloat16, 16>) : (cpl == 8 ? go(embed_bwd_kernel<__nv_bfloat16, 8>) : go(embed_bwd_kernel<__nv_bfloat16, 4>));
+    e = launch_pdl(dtype == PM_F32 ? embed_kernel<float>(cpl) : embed_kernel<__nv_bfloat16>(cpl), g, dim3(256), smem, stream, false, t);
   }
   return e;
 }
@@ -1389,18 +1392,18 @@ static cudaError_t limit_to_max(const void* kernel) {
 }
 
 template <typename AT>
-static cudaError_t limits_of() {
-  const void* kernels[] = {(const void*)attention_fwd_kernel<AT>, (const void*)attention_bwd_kernel<AT>,
-                           (const void*)ce_loss_rows_kernel<AT>, (const void*)ce_loss_long_kernel<AT>,
-                           (const void*)ln_bwd_fused_kernel<AT, 1, 1>, (const void*)ln_bwd_fused_kernel<AT, 2, 1>, (const void*)ln_bwd_fused_kernel<AT, 2, 2>,
-                           (const void*)embed_bwd_kernel<AT, 4>, (const void*)embed_bwd_kernel<AT, 8>, (const void*)embed_bwd_kernel<AT, 16>};
-  for (const void* k : kernels) {
-    const cudaError_t e = limit_to_max(k);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+static cudaError_t limits_of(const TickArgs& t, bool simt_attention) {
+  cudaError_t e = cudaSuccess;
+  if (simt_attention) e = limit_to_max((const void*)attention_fwd_kernel<AT>);
+  if (e == cudaSuccess && simt_attention) e = limit_to_max((const void*)attention_bwd_kernel<AT>);
+  if (e == cudaSuccess && t.loss_kind == PM_LOSS_CE && ce_in_smem(t.n_out_last)) e = limit_to_max((const void*)ce_smem_kernel<AT>(t.n_out_last));
+  if (e == cudaSuccess && t.any_ln && t.ln_fused) e = limit_to_max((const void*)ln_fused_kernel<AT>(t.max_ln_dim));
+  if (e == cudaSuccess && t.any_embed) e = limit_to_max((const void*)embed_kernel<AT>(embed_cpl(t.max_embed_dim)));
+  return e;
 }
 
-cudaError_t xfmr_set_smem_limits(int dtype) { return dtype == PM_F32 ? limits_of<float>() : limits_of<__nv_bfloat16>(); }
+cudaError_t xfmr_set_smem_limits(const TickArgs& t, int dtype, bool simt_attention) {
+  return dtype == PM_F32 ? limits_of<float>(t, simt_attention) : limits_of<__nv_bfloat16>(t, simt_attention);
+}
 
 }  // namespace pm
