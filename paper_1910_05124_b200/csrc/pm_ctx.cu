@@ -708,7 +708,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   t.max_lin = L.max_lin; t.max_dim = L.max_dim;
   t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0; t.pdl = 0;
   t.res_fused = cfg->compute_dtype == PM_BF16 ? 1 : 0;
-  t.ln_li0 = 0; t.defer_finish = 0; t.colsum_only = 0; t.dz_only = 0; t.ln_stage = 0;
+  t.ln_li0 = 0; t.defer_finish = 0; t.ln_stage = 0;
   t.dgrad_split_below = 0;
   t.loss_scale = 1.0f / (float)(cfg->n_micro > 1 ? cfg->n_micro : 1);
   t.stash = (L.stash || L.materialize) ? 1 : 0;     // the backward pass reads its table entry's version slot
@@ -934,15 +934,14 @@ static pm_status stage_forward(pm_ctx* ctx, const TickArgs& ta, int p) {
   return PM_OK;
 }
 
-// does a launch of the activation backward at level l have anything to do (all stages, or stage p): the bias gradients of
-// bf16 networks are summed there, those of fp32 networks by the weight-gradient GEMM
-static bool need_actbwd(const pm_ctx* ctx, int l, int p, bool dz_only) {
-  if (!dz_only && ctx->cfg.compute_dtype == PM_BF16) return true;
+// does a launch of the activation backward at level l have anything to do (all stages, or stage p)?  (The weight-gradient GEMM sums
+// the bias gradients.)
+static bool need_actbwd(const pm_ctx* ctx, int l, int p) {
   return p >= 0 ? bwd_act(ctx->L.st[p].lin[l]) != PM_ACT_NONE : (ctx->L.act_levels >> l & 1) != 0;
 }
 
-// The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradients, the bias column sums and
-// the finishing passes are left to grouped launches over all stages (ta.dz_only and ta.defer_finish set).
+// The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradients and the finishing passes
+// are left to grouped launches over all stages (ta.defer_finish set).
 static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool grouped) {
   const int dt = ctx->cfg.compute_dtype;
   const int P = ctx->cfg.n_stages;
@@ -954,9 +953,9 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     else if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(next(ctx, ta), dt, ctx->ls), "attention backward"))) != PM_OK) return s;
   }
   for (int l = sd.n_lin - 1; l >= 0; --l) {
-    // dz = dy * act'(z) must exist before this stage's dgrad; the column sums (the bias gradient) can wait for one grouped launch
-    if (need_actbwd(ctx, l, p, grouped) &&
-        (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ta), dt, l, ctx->ls), "activation backward", actbwd_launches(ta, dt)))) != PM_OK) return s;
+    // dz = dy * act'(z) must exist before this stage's dgrad
+    if (need_actbwd(ctx, l, p) &&
+        (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ta), dt, l, ctx->ls), "activation backward"))) != PM_OK) return s;
     cudaError_t e;
     if (!grouped) {
       prof_begin(ctx, PM_PROF_WGRAD);
@@ -1032,21 +1031,14 @@ static pm_status mb_backward(pm_ctx* ctx) {
           if ((s = stage_forward(ctx, mb_args(ctx, 2 * P + 1, p), p)) != PM_OK) return s;
       for (int p = hi - 1; p >= lo; --p) {
         TickArgs ta = mb_args(ctx, 2 * P - 1 - p, p);
-        ta.dz_only = 1; ta.defer_finish = 1;    // bias and LayerNorm gradients are summed once, below
+        ta.defer_finish = 1;                    // LayerNorm gradients are summed once, below
         if ((s = stage_backward(ctx, ta, p, true)) != PM_OK) return s;
       }
       if (S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
     }
     TickArgs ta = mb_args(ctx, 2 * P, -1);
-    // the LayerNorm partial sums first: those of unfused stages (widths above 1024) lie where the column sums write theirs
     const int n_fin = ln_finish_launches(ta);
     if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
-    if (dt == PM_BF16) {
-      ta.colsum_only = 1;                                       // bias gradients of all stages
-      for (int l = 0; l < ctx->L.max_lin; ++l)
-        if ((s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ta), dt, l, ctx->ls), "bias gradient column sums", actbwd_launches(ta, dt)))) != PM_OK) return s;
-      ta.colsum_only = 0;
-    }
     if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
     return PM_OK;
   });
@@ -1244,8 +1236,8 @@ pm_status pm_backward(pm_ctx* ctx) {
       if (ctx->attn) { if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ctx->ta), false, ctx->ls), "attention backward"))) != PM_OK) return s; }
       else if (ctx->L.att_blocks > 0 && (s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(next(ctx, ctx->ta), dt, ctx->ls), "attention backward"))) != PM_OK) return s;
       for (int l = ctx->L.max_lin - 1; l >= 0; --l) {
-        if (need_actbwd(ctx, l, -1, false) &&
-            (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ctx->ta), dt, l, ctx->ls), "activation backward", actbwd_launches(ctx->ta, dt)))) != PM_OK) return s;
+        if (need_actbwd(ctx, l, -1) &&
+            (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ctx->ta), dt, l, ctx->ls), "activation backward"))) != PM_OK) return s;
         cudaError_t e = cudaSuccess;
         if (!ctx->L.fuse) {                                           // fused update: formed in the update phase
           prof_begin(ctx, PM_PROF_WGRAD);

@@ -84,63 +84,41 @@ cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
   return launch_pdl(dtype == PM_F32 ? mse_loss_kernel<float> : mse_loss_kernel<__nv_bfloat16>, dim3(kLossBlocks), dim3(kLossThreads), 0, stream, t.pdl, t);
 }
 
-// ---- activation backward + bias gradient ---------------------------------------------------------
-// dz = dy * act'(z) (stored in the activation type); db[c] = sum over rows of the stored dz.
-// A block owns 256 columns; warp w takes rows w, w + NW, ... (ascending), eight columns per lane; the per-warp partial sums of
-// a column are added in warp order.  (fp32 networks: dz only, the weight-gradient GEMM sums the columns of its operand.)
-constexpr int kActWarps = 8;
+// ---- activation backward ---------------------------------------------------------------------------
+// dz = dy * act'(z), stored in the activation type (the bias gradient, its column sums, comes from the weight-gradient GEMM).
+// A block owns 256 columns, or 32 of a microbatch of up to kActSmallRows rows; eight columns per lane, a lane has four rows in
+// flight.  Bounded by latency for short microbatches, by HBM for long ones.
 
-constexpr int kActColsV = kActCols;                    // columns per block: 8 per lane
-constexpr int kColsumGroup = 8;                       // row chunks per block in a launch that only sums columns
-constexpr int kStageGroup = 4;                        // ... and in a launch of one stage
-// Row chunks one block of the activation-backward launch covers; its sum is partial row (first chunk / group) of the stage.
-__host__ __device__ inline int act_chunk_group(const TickArgs& t) {
-  return t.row_chunks > 1 ? (t.colsum_only ? kColsumGroup : (t.sel_p >= 0 ? kStageGroup : 1)) : 1;
-}
-
-// rows r, r + NW, ... < r1 of 8 columns (NW = warps of the block): four rows are loaded before the first is used
-template <typename AT, int ACT, int NW>
-__device__ __forceinline__ void actbwd_rows(const AT* __restrict__ dy, const AT* __restrict__ z, AT* __restrict__ dz, int n_out, int c,
-                                            int r, int r1, float (&sum)[8]) {
-  for (; r + 3 * NW < r1; r += 4 * NW) {
-    float g[4][8], zz[4][8];
+// rows r, r + step, ... < r1 of 8 columns: N of them are loaded before the first is used (no branch between the loads: the
+// compiler would wait for each)
+template <typename AT, int ACT, int N>
+__device__ __forceinline__ void actbwd_rows_n(const AT* __restrict__ dy, const AT* __restrict__ z, AT* __restrict__ dz, int n_out, int c, int r, int step) {
+  float g[N][8], zz[N][8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint64_t i = (uint64_t)(r + u * NW) * n_out + c;
-      load8<AT>(dy + i, g[u]);
-      if (ACT != PM_ACT_NONE) load8<AT>(z + i, zz[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (ACT != PM_ACT_NONE) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) g[u][k] = round_as<AT>(__fmul_rn(g[u][k], act_grad(zz[u][k], ACT)));
-        store8<AT>(dz + (uint64_t)(r + u * NW) * n_out + c, g[u]);
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) sum[k] = __fadd_rn(sum[k], g[u][k]);
-    }
+  for (int u = 0; u < N; ++u) {
+    const uint64_t i = (uint64_t)(r + u * step) * n_out + c;
+    load8<AT>(dy + i, g[u]);
+    load8<AT>(z + i, zz[u]);
   }
-  for (; r < r1; r += NW) {
-    const uint64_t i = (uint64_t)r * n_out + c;
-    float g[8];
-    load8<AT>(dy + i, g);
-    if (ACT != PM_ACT_NONE) {
-      float zz[8];
-      load8<AT>(z + i, zz);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) g[k] = round_as<AT>(__fmul_rn(g[k], act_grad(zz[k], ACT)));
-      store8<AT>(dz + i, g);
-    }
+  for (int u = 0; u < N; ++u) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) sum[k] = __fadd_rn(sum[k], g[k]);
+    for (int k = 0; k < 8; ++k) g[u][k] = round_as<AT>(__fmul_rn(g[u][k], act_grad(zz[u][k], ACT)));
+    store8<AT>(dz + (uint64_t)(r + u * step) * n_out + c, g[u]);
   }
 }
+template <typename AT, int ACT>
+__device__ __forceinline__ void actbwd_rows(const AT* __restrict__ dy, const AT* __restrict__ z, AT* __restrict__ dz, int n_out, int c, int r, int step, int r1) {
+  for (; r + 3 * step < r1; r += 4 * step) actbwd_rows_n<AT, ACT, 4>(dy, z, dz, n_out, c, r, step);
+  if (r + step < r1) { actbwd_rows_n<AT, ACT, 2>(dy, z, dz, n_out, c, r, step); r += 2 * step; }
+  if (r < r1) actbwd_rows_n<AT, ACT, 1>(dy, z, dz, n_out, c, r, step);
+}
 
-// NW warps per block: 8 in a grouped launch over all stages; 16 in a launch of one stage (microbatch-major order),
-// which has fewer blocks and needs more loads in flight per block
-template <typename AT, int NW>
-__global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
+// rows a block of the launch covers: all of a short microbatch; in a launch of one stage few enough for several blocks per SM
+__host__ __device__ inline int act_block_rows(const TickArgs& t) { return t.T <= kActSmallRows ? t.T : (t.sel_p >= 0 ? 64 : 256); }
+
+template <typename AT>
+__global__ void __launch_bounds__(256) actbwd_kernel(TickArgs t, int lvl) {
   pdl_trigger();
   pdl_wait();
   const int* start = t.act_start + (size_t)lvl * (t.P + 1);
@@ -153,227 +131,36 @@ __global__ void __launch_bounds__(NW * 32) actbwd_kernel(TickArgs t, int lvl) {
   const StageDev& s = t.st[p];
   if (d.b_mb < 0 || lvl >= s.n_lin) return;
   const LinDev& L = s.lin[lvl];
-  const int c0 = (blk - start[p]) * kActColsV;
+  if (bwd_act(L) == PM_ACT_NONE) return;                    // without an activation (or with one applied upstream) dz = dy
+  const bool small = t.T <= kActSmallRows;
+  const int cols = small ? kActSmallCols : kActCols;
+  const int c0 = (blk - start[p]) * cols;
   if (c0 >= L.n_out) return;
-  // a launch that only sums columns, or a launch of one stage, gives a block several row chunks (fewer, longer-lived
-  // blocks); a block's sum is one partial row, and the finishing pass adds as many rows as the launch had blocks
-  const int cg = act_chunk_group(t);
-  const int chunk = blockIdx.y * cg;
-  const int r0 = chunk * t.chunk_rows, r1 = min(t.T, r0 + cg * t.chunk_rows);
-  if (r0 >= t.T) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = c0 + 8 * lane;
+  const int rows = act_block_rows(t), r0 = (int)blockIdx.y * rows, r1 = min(t.T, r0 + rows);
   const uint64_t n = (uint64_t)t.T * L.n_out;
-  const bool has_act = bwd_act(L) != PM_ACT_NONE && !t.colsum_only;   // without an activation (or with one applied upstream) dz = dy: nothing is stored
-  const bool sums = sizeof(AT) == 2 && !t.dz_only;
-  if (!has_act && !sums) return;
-  const AT* dy = t.colsum_only ? dz_src<AT>(t, s, d, lvl)
-                 : (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off)
-                 : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
+  const AT* dy = (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off) : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
   // the pre-activation stash, or for a ReLU without one the stashed output (same sign pattern)
-  const AT* z = !has_act ? dy
-                : !(L.flags & LF_ACT_FROM_Y) ? ring_ptr<AT>(t, L.z_ring, d.b_slot, n)
+  const AT* z = !(L.flags & LF_ACT_FROM_Y) ? ring_ptr<AT>(t, L.z_ring, d.b_slot, n)
                 : (lvl < s.n_lin - 1 ? ring_ptr<AT>(t, L.h_ring, d.b_slot, n) : ring_ptr<AT>(t, t.st[p + 1].x_ring, d.b_next_xslot, n));
   AT* dz = ws_ptr<AT>(t, L.dz_off);
-  const bool vec = (L.n_out & 7) == 0;                      // vector path needs 8-element alignment of every row
-  float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (vec) {
-    if (c < L.n_out) {
-      if (!has_act) actbwd_rows<AT, PM_ACT_NONE, NW>(dy, z, dz, L.n_out, c, r0 + warp, r1, sum);
-      else if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU, NW>(dy, z, dz, L.n_out, c, r0 + warp, r1, sum);
-      else actbwd_rows<AT, PM_ACT_GELU, NW>(dy, z, dz, L.n_out, c, r0 + warp, r1, sum);
-    }
-  } else {
-    for (int r = r0 + warp; r < r1; r += NW) {
-      const uint64_t i = (uint64_t)r * L.n_out + c;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (c + k < L.n_out) {
-          float v = has_act ? round_as<AT>(__fmul_rn(to_f<AT>(dy[i + k]), act_grad(to_f<AT>(z[i + k]), L.act))) : to_f<AT>(dy[i + k]);
-          if (has_act) dz[i + k] = from_f<AT>(v);
-          sum[k] = __fadd_rn(sum[k], v);
-        }
+  if ((L.n_out & 7) == 0) {                                 // vector path needs 8-element alignment of every row
+    const int per = cols / 8, c = c0 + 8 * (int)(threadIdx.x % per), r = r0 + (int)(threadIdx.x / per), step = 256 / per;
+    if (c >= L.n_out) return;
+    if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU>(dy, z, dz, L.n_out, c, r, step, r1);
+    else actbwd_rows<AT, PM_ACT_GELU>(dy, z, dz, L.n_out, c, r, step, r1);
+  } else {                                                  // fp32 only: bf16 Linears have widths that are multiples of 8
+    const int c1 = min(L.n_out, c0 + cols), w = c1 - c0;
+    for (int o = (int)threadIdx.x; o < w * (r1 - r0); o += 256) {
+      const uint64_t i = (uint64_t)(r0 + o / w) * L.n_out + c0 + o % w;
+      dz[i] = from_f<AT>(round_as<AT>(__fmul_rn(to_f<AT>(dy[i]), act_grad(to_f<AT>(z[i]), L.act))));
     }
   }
-  if (!sums) return;
-  __shared__ float red[NW][kActColsV];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) red[warp][8 * lane + k] = sum[k];
-  __syncthreads();
-  const int cc = c0 + threadIdx.x;
-  if (threadIdx.x < kActColsV && cc < L.n_out) {
-    float a = 0.f;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) a = __fadd_rn(a, red[w][threadIdx.x]);
-    if (t.row_chunks == 1) t.a.grad[L.b_off + cc] = d.accum ? __fadd_rn(t.a.grad[L.b_off + cc], a) : a;
-    else ws_ptr<float>(t, t.colred_off)[((uint64_t)p * t.row_chunks + blockIdx.y) * (2 * (uint64_t)t.max_dim) + cc] = a;   // partial rows are dense: one per block
-  }
 }
-
-// The same for microbatches of at most kActSmallRows rows: a block takes 32 columns of ALL rows (eight columns per lane, eight
-// rows per warp and step), so there are no partial sums to finish in a second launch.  What bounds these launches is the
-// number of rows a block walks one after the other and the launches themselves, not the bytes: with 256-column blocks of 32
-// rows and a finishing launch a level of the 32-stage 1024-wide MLP (128 rows) took 17.6 + 12.7 us.
-template <typename AT>
-__global__ void __launch_bounds__(256) actbwd_small_kernel(TickArgs t, int lvl) {
-  pdl_trigger();
-  pdl_wait();
-  const int* start = t.act_start + (size_t)lvl * (t.P + 1);
-  const int blk = (int)blockIdx.x + t.act_first[lvl];
-  int lo = 0, hi = t.P - 1;
-  if (t.sel_p >= 0) lo = hi = t.sel_p;
-  while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (start[mid] <= blk) lo = mid; else hi = mid - 1; }
-  const int p = lo;
-  const StageDyn& d = t.dyn[p];
-  const StageDev& s = t.st[p];
-  if (d.b_mb < 0 || lvl >= s.n_lin) return;
-  const LinDev& L = s.lin[lvl];
-  const int c0 = (blk - start[p]) * kActSmallCols;
-  if (c0 >= L.n_out) return;
-  const bool has_act = bwd_act(L) != PM_ACT_NONE && !t.colsum_only;
-  const bool sums = sizeof(AT) == 2 && !t.dz_only;
-  if (!has_act && !sums) return;
-  const AT* dy = t.colsum_only ? dz_src<AT>(t, s, d, lvl)
-                 : (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off)
-                 : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
-  const uint64_t n = (uint64_t)t.T * L.n_out;
-  const AT* z = !has_act ? dy
-                : !(L.flags & LF_ACT_FROM_Y) ? ring_ptr<AT>(t, L.z_ring, d.b_slot, n)
-                : (lvl < s.n_lin - 1 ? ring_ptr<AT>(t, L.h_ring, d.b_slot, n) : ring_ptr<AT>(t, t.st[p + 1].x_ring, d.b_next_xslot, n));
-  AT* dz = ws_ptr<AT>(t, L.dz_off);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if ((L.n_out & 7) == 0) {
-    const int c = c0 + 8 * (lane & 3), r = 8 * warp + (lane >> 2);
-    if (c < L.n_out) {
-      if (!has_act) actbwd_rows<AT, PM_ACT_NONE, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
-      else if (L.act == PM_ACT_RELU) actbwd_rows<AT, PM_ACT_RELU, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
-      else actbwd_rows<AT, PM_ACT_GELU, 64>(dy, z, dz, L.n_out, c, r, t.T, sum);
-    }
-  } else if (has_act) {                                     // fp32 only: bf16 Linears have widths that are multiples of 8
-    const int c = c0 + (int)(threadIdx.x & 31);
-    if (c < L.n_out)
-      for (int r = threadIdx.x >> 5; r < t.T; r += 8) {
-        const uint64_t i = (uint64_t)r * L.n_out + c;
-        dz[i] = from_f<AT>(round_as<AT>(__fmul_rn(to_f<AT>(dy[i]), act_grad(to_f<AT>(z[i]), L.act))));
-      }
-  }
-  if (!sums) return;
-  __shared__ float red[8][kActSmallCols];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {                             // the eight rows of the warp, in a fixed order
-    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 4));
-    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 8));
-    sum[k] = __fadd_rn(sum[k], __shfl_xor_sync(0xffffffffu, sum[k], 16));
-    if (lane < 4) red[warp][8 * lane + k] = sum[k];
-  }
-  __syncthreads();
-  const int cc = c0 + threadIdx.x;
-  if (threadIdx.x < kActSmallCols && cc < L.n_out) {
-    float a = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) a = __fadd_rn(a, red[w][threadIdx.x]);
-    t.a.grad[L.b_off + cc] = d.accum ? __fadd_rn(t.a.grad[L.b_off + cc], a) : a;
-  }
-}
-
-// adds the per-row-chunk partial column sums: db of Linear lvl.  A block owns 32 columns; warp w adds the partials of
-// chunks w, w + 8, ... in ascending order (all of its loads are issued before the first addition: the partials sit a
-// row of the buffer apart, so every load is a separate round trip), then the eight per-warp sums are added in warp
-// order.  The order is fixed, so the result is reproducible.
-constexpr int kFinCols = 32, kFinMaxPer = 32;            // columns per block; partials per warp held in registers at a time
-
-__global__ void __launch_bounds__(256) bias_finish_kernel(TickArgs t, int lvl) {
-  pdl_trigger();
-  pdl_wait();
-  // the grid follows the list of 256-column blocks of the activation-backward launch (kActColsV / kFinCols blocks
-  // here per entry there), so no block falls outside its Linear's columns however unequal the widths are
-  constexpr int kPer = kActColsV / kFinCols;
-  const int* __restrict__ start = t.act_start + (size_t)lvl * (t.P + 1);
-  const int blk = (int)(blockIdx.x / kPer) + t.act_first[lvl];
-  int lo = 0, hi = t.P - 1;
-  if (t.sel_p >= 0) lo = hi = t.sel_p;
-  while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (start[mid] <= blk) lo = mid; else hi = mid - 1; }
-  const int p = lo;
-  const StageDyn& d = t.dyn[p];
-  const StageDev& s = t.st[p];
-  if (d.b_mb < 0 || lvl >= s.n_lin) return;
-  const LinDev& L = s.lin[lvl];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cb = (blk - start[p]) * kActColsV + (int)(blockIdx.x % kPer) * kFinCols;
-  const int c = cb + lane;
-  if (cb >= L.n_out) return;
-  const uint64_t ps = 2 * (uint64_t)t.max_dim;
-  const float* part = ws_ptr<float>(t, t.colred_off) + (uint64_t)p * t.row_chunks * ps + (c < L.n_out ? c : 0);
-  // partial rows the activation-backward launch of this Linear wrote: one per block of that launch
-  const int cg = act_chunk_group(t);
-  const int n_rows = (t.row_chunks + cg - 1) / cg;
-  float sum = 0.f;
-  for (int k0 = warp; k0 < n_rows; k0 += 8 * kFinMaxPer) {
-    float v[kFinMaxPer];
-#pragma unroll
-    for (int u = 0; u < kFinMaxPer; ++u) { const int k = k0 + 8 * u; v[u] = k < n_rows ? part[(uint64_t)k * ps] : 0.f; }
-#pragma unroll
-    for (int u = 0; u < kFinMaxPer; ++u) if (k0 + 8 * u < n_rows) sum = __fadd_rn(sum, v[u]);
-  }
-  __shared__ float red[8][kFinCols];
-  red[warp][lane] = sum;
-  __syncthreads();
-  if (warp == 0 && c < L.n_out) {
-    float a = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) a = __fadd_rn(a, red[w][lane]);
-    t.a.grad[L.b_off + c] = d.accum ? __fadd_rn(t.a.grad[L.b_off + c], a) : a;
-  }
-}
-
-// The same for at most eight partial rows (a launch that sums the columns of up to 4096 rows): a thread adds its column's
-// partials in the same order, 256 columns per block.  (4096 rows, 45 stages: 48 us with eight warps per 32 columns,
-// whose launch is thousands of blocks with one load each.)
-constexpr int kFinFew = 8;
-__global__ void __launch_bounds__(kActColsV) bias_finish_few_kernel(TickArgs t, int lvl) {
-  pdl_trigger();
-  pdl_wait();
-  const int* __restrict__ start = t.act_start + (size_t)lvl * (t.P + 1);
-  const int blk = (int)blockIdx.x + t.act_first[lvl];
-  int lo = 0, hi = t.P - 1;
-  if (t.sel_p >= 0) lo = hi = t.sel_p;
-  while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (start[mid] <= blk) lo = mid; else hi = mid - 1; }
-  const StageDyn& d = t.dyn[lo];
-  const StageDev& s = t.st[lo];
-  if (d.b_mb < 0 || lvl >= s.n_lin) return;
-  const LinDev& L = s.lin[lvl];
-  const int c = (blk - start[lo]) * kActColsV + (int)threadIdx.x;
-  if (c >= L.n_out) return;
-  const uint64_t ps = 2 * (uint64_t)t.max_dim;
-  const float* part = ws_ptr<float>(t, t.colred_off) + (uint64_t)lo * t.row_chunks * ps + c;
-  const int cg = act_chunk_group(t), n_rows = (t.row_chunks + cg - 1) / cg;
-  float v[kFinFew];
-#pragma unroll
-  for (int k = 0; k < kFinFew; ++k) v[k] = k < n_rows ? part[(uint64_t)k * ps] : 0.f;
-  float a = 0.f;
-#pragma unroll
-  for (int k = 0; k < kFinFew; ++k) a = __fadd_rn(a, v[k]);
-  t.a.grad[L.b_off + c] = d.accum ? __fadd_rn(t.a.grad[L.b_off + c], a) : a;
-}
-
-int actbwd_launches(const TickArgs& t, int dtype) { return (t.T <= kActSmallRows || t.row_chunks == 1 || t.dz_only || dtype == PM_F32) ? 1 : 2; }
 
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream) {
   if (t.act_blocks[lvl] == 0) return cudaSuccess;
-  if (t.T <= kActSmallRows)
-    return launch_pdl(dtype == PM_F32 ? actbwd_small_kernel<float> : actbwd_small_kernel<__nv_bfloat16>, dim3(t.act_blocks[lvl]), dim3(256), 0, stream, t.pdl, t, lvl);
-  const int cg = act_chunk_group(t);
-  dim3 grid(t.act_blocks[lvl], (t.row_chunks + cg - 1) / cg);
-  cudaError_t e;
-  if (t.sel_p >= 0 && t.row_chunks > 1)
-    e = launch_pdl(dtype == PM_F32 ? actbwd_kernel<float, 16> : actbwd_kernel<__nv_bfloat16, 16>, grid, dim3(16 * 32), 0, stream, t.pdl, t, lvl);
-  else
-    e = launch_pdl(dtype == PM_F32 ? actbwd_kernel<float, kActWarps> : actbwd_kernel<__nv_bfloat16, kActWarps>, grid, dim3(kActWarps * 32), 0, stream, t.pdl, t, lvl);
-  if (e != cudaSuccess || actbwd_launches(t, dtype) == 1) return e;
-  if ((t.row_chunks + cg - 1) / cg <= kFinFew)
-    return launch_pdl(bias_finish_few_kernel, dim3(t.act_blocks[lvl]), dim3(kActColsV), 0, stream, t.pdl, t, lvl);
-  return launch_pdl(bias_finish_kernel, dim3(t.act_blocks[lvl] * (kActColsV / kFinCols)), dim3(256), 0, stream, t.pdl, t, lvl);
+  const int rows = act_block_rows(t);
+  return launch_pdl(dtype == PM_F32 ? actbwd_kernel<float> : actbwd_kernel<__nv_bfloat16>, dim3(t.act_blocks[lvl], (t.T + rows - 1) / rows), dim3(256), 0, stream, t.pdl, t, lvl);
 }
 
 // ---- fp32 SIMT grouped GEMM ------------------------------------------------------------------------

@@ -25,7 +25,7 @@ struct TickArgs {
   uint64_t tgt_off;       // ws: target ring [P+1]: [T*n_out_last] float (MSE) or [T] int32 (CE)
   uint64_t pe_off;        // ws: sinusoidal positions [seq_len][d] float (0 if no embedding stage)
   uint64_t rowloss_off;   // ws: per-token losses [T] float (cross-entropy)
-  uint64_t colred_off;    // ws: per-row-chunk partial column sums [P][row_chunks][2*max_dim] float
+  uint64_t colred_off;    // ws: per-row-chunk partial sums of unfused LayerNorm gradients [P][row_chunks][2*max_dim] float
   int32_t row_chunks;     // ceil(T / chunk_rows)
   int32_t chunk_rows;     // rows of a microbatch one block of a column reduction covers (256, or 32 for short microbatches)
   int32_t loss_kind;      // PM_LOSS_*
@@ -68,9 +68,6 @@ struct TickArgs {
                                // group (0: always two); launches of one stage need enough groups for the CTA pairs
   float loss_scale;       // factor on dL/dy: 1/N with N microbatches per update (the minibatch loss is their mean), else 1
   int32_t ln_li0;         // first entry of ln_ids a launch covers (its grid counts entries from there)
-  int32_t colsum_only;    // activation-backward launch that only sums the columns of every Linear's dz (bias gradients), all stages at
-                          // once at the end of a microbatch-major backward pass; dz was formed on the way
-  int32_t dz_only;        // ... and the launches of one stage on the way: dz, no sums
   int32_t defer_finish;   // launches of one stage leave the per-chunk partial sums of LayerNorm gradients in place;
                           // one grouped launch over all stages adds them up at the end of the backward pass
   // weight-gradient launch that applies the PipeMare update to the Linear matrices in its epilogue (bf16 tensor-core
@@ -194,9 +191,8 @@ template <typename AT> __device__ __forceinline__ AT* y_dest(const TickArgs& t, 
 inline bool early(const TickArgs& t, dim3 grid) { return t.pdl != 0 && grid.x * grid.y <= (unsigned)kSms; }
 // MSE loss of the microbatch whose backward starts this tick, and dL/dy into the last stage's mailbox.
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream);
-// dz = dy * act'(z) and db = column sums, level `lvl` of every stage that runs backward this tick.
+// dz = dy * act'(z), level `lvl` of every stage that runs backward this tick.
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream);
-int actbwd_launches(const TickArgs& t, int dtype);
 // the finishing pass that launches with defer_finish left out, grouped over all stages (LayerNorm parameter gradients)
 cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream);      // pm_xfmr.cu
 int ln_finish_launches(const TickArgs& t);

@@ -22,6 +22,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "pm_ptx.cuh"
 #include "pm_umma.cuh"
@@ -38,10 +39,13 @@ constexpr int STG_BYTES = 2 * STG_HALF_BYTES;              // w tile + delta til
 constexpr int ACC_COLS = 128, TMEM_COLS = 2 * ACC_COLS;
 constexpr int N_EPI_WARPS = 8;
 
-template <int MODE> struct Cfg {                           // MODE 0 forward, 2 wgrad, 1 dgrad against a QUEUED weight version (weight
-                                                           // stashing, tau_bkwd = tau_fwd: a plain bf16 operand; the corrected dgrad has kernels of its own)
+// MODE 0 forward, 2 wgrad, 1 dgrad against a QUEUED weight version (weight stashing, tau_bkwd = tau_fwd: a plain bf16 operand; the
+// corrected dgrad has kernels of its own).  MODE 2: four warps sum the columns of dz, the bias gradient, from the A tiles in shared
+// memory.  FUSE (MODE 2): the update is applied in the epilogue.
+template <int MODE, bool FUSE> struct Cfg {
   static constexpr int kStages = 4;                        // operand ring depth
-  static constexpr int kThreads = 32 * (2 + N_EPI_WARPS);
+  static constexpr int kSumWarps = MODE == 2 ? 4 : 0;
+  static constexpr int kThreads = 32 * (2 + kSumWarps + N_EPI_WARPS);
   static constexpr int kOutWarpBytes = 8192;               // per epilogue warp: two boxes of 32 rows x 128 B
   static constexpr int kOutBytes = N_EPI_WARPS * kOutWarpBytes;
   static constexpr int kTileBytes = kStages * STAGE_BYTES + kOutBytes;
@@ -49,7 +53,7 @@ template <int MODE> struct Cfg {                           // MODE 0 forward, 2 
 };
 
 enum { MAP_ACT_K = 0, MAP_W_K = 1, MAP_DZ_K = 2, MAP_DZ_MN = 3, MAP_ACT_MN = 4, MAP_W_F32 = 5, MAP_D_F32 = 6,
-       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_F32Q = 11, MAP_D_F32Q = 12, MAP_W_F32H = 13, MAP_D_F32H = 14, MAP_W_MN = 15, MAP_W_K32 = 16, MAPS_PER_LINEAR = 17 };
+       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_F32Q = 11, MAP_D_F32Q = 12, MAP_W_F32H = 13, MAP_D_F32H = 14, MAP_W_MN = 15, MAP_W_K32 = 16, MAP_SKIP = 17, MAPS_PER_LINEAR = 18 };
 }  // namespace pm
 #include "pm_umma_row.cuh"     // the kernel of launches with few tiles; uses the tensor maps above
 namespace pm {
@@ -60,42 +64,57 @@ __device__ __forceinline__ uint32_t make_idesc(int a_mn_major, int b_mn_major) {
          ((uint32_t)(TILE_N >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
 }
 
-// forward epilogue for 8 columns: z = bf16(acc + bias), y = bf16(act(z)); the activation is a template parameter so
-// that Linears without GELU never pay for erff
-template <int ACT>
-__device__ __forceinline__ void epi_zy8(const float (&pf)[8], uint8_t* zdst, uint8_t* ydst) {
-  float zf[8], yf[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    zf[e] = __bfloat162float(__float2bfloat16_rn(pf[e]));
-    yf[e] = ACT == PM_ACT_RELU ? fmaxf(zf[e], 0.0f) : (ACT == PM_ACT_GELU ? act_fwd(zf[e], PM_ACT_GELU) : zf[e]);
+// One epilogue warp's staging buffer: SLOTS boxes of 4 KB (32 rows of one 128-byte swizzle row), each its own TMA store.
+template <int SLOTS>
+struct EpiStage {
+  uint8_t* buf; uint32_t buf_s; int lane;
+  uint32_t bar;               // counts the skip tensor's copies into the box
+  uint32_t off = 0;           // the box written next
+  uint32_t phase = 0;         // parity of the next copy
+  bool stored = false;
+  // the box's earlier store has finished reading it
+  __device__ __forceinline__ uint8_t* begin() {
+    if (lane == 0 && stored) { if (SLOTS == 1) tma_store_wait_read(); else tma_store_wait_read_1(); }
+    __syncwarp();
+    return buf + off;
   }
-  *reinterpret_cast<uint4*>(zdst) = make_uint4(pack_bf16(zf[0], zf[1]), pack_bf16(zf[2], zf[3]), pack_bf16(zf[4], zf[5]), pack_bf16(zf[6], zf[7]));
-  *reinterpret_cast<uint4*>(ydst) = make_uint4(pack_bf16(yf[0], yf[1]), pack_bf16(yf[2], yf[3]), pack_bf16(yf[4], yf[5]), pack_bf16(yf[6], yf[7]));
-}
-
-// State of one epilogue warp's staging buffer (two slots of 4 KB) across blocks.
-struct EpiState {
-  bool stored = false;        // a TMA store of this warp may still be reading the staging buffer
-  bool prev_both = false;     // the previous block used both slots
-  uint32_t slot = 0;          // slot the next single-output block writes
+  template <class Store> __device__ __forceinline__ void end(Store store) {
+    fence_async_smem();                                           // staging writes -> visible to the TMA engine
+    __syncwarp();
+    if (lane == 0) { store(buf_s + off); tma_store_commit(); }
+    stored = true;
+    if (SLOTS == 2) off ^= 4096u;
+  }
+  // a residual stage's unit: its block of the skip tensor comes into the box in the layout the sum leaves it in
+  __device__ __forceinline__ void fetch(const CUtensorMap* map, int n, int m, int slot) {
+    begin();
+    if (lane == 0) { mbar_arrive_expect_tx(bar, 4096); tma_load_3d(buf_s + off, map, bar, n, m, slot); }
+  }
+  __device__ __forceinline__ bool fetched(volatile int* abort_flag, int* status) {
+    const bool ok = mbar_wait(bar, phase, abort_flag, status, 11);
+    phase ^= 1u;
+    return __all_sync(0xffffffffu, ok);
+  }
+  // a CTA that gives up: the copy still lands here (bounded wait)
+  __device__ __forceinline__ void drain() {
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, phase) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+  }
 };
 
-// The PipeMare update of one 32-row x 64-column block of a Linear matrix, applied to the weight gradient while it is
-// still on chip (r0, r1: the block's accumulators, lane = row).  The block goes through the warp's staging buffer
+// The PipeMare update of one 32-row x 32-column block of a Linear matrix, applied to the weight gradient while it is
+// still on chip (r: the block's accumulators, lane = row).  The block goes through the warp's staging buffer
 // once, in the layout the dW store uses, and comes back with a lane owning four consecutive columns of a row, so
 // that every access to the master weights, the moments and delta is a full 128-byte line per eight lanes.  Per
 // element the arithmetic is upd_one's, i.e. exactly what the stand-alone update kernel does with a stored gradient.
 template <int OPT>
 __device__ __forceinline__ void epi_update_block(const TickArgs& t, const StageDyn& d, const LinDev& L, int M, int N, int mrow, int nb,
-                                                 const uint32_t (&r0)[32], const uint32_t (&r1)[32], uint8_t* obuf, int lane) {
+                                                 const uint32_t (&r)[32], uint8_t* obuf, int lane) {
   const uint32_t row_off = (uint32_t)lane * 128, sw = (uint32_t)(lane & 7);
   __syncwarp();                                                   // the previous block's reads of the buffer are done
 #pragma unroll
-  for (int g = 0; g < 8; ++g) {                                   // two boxes of 32 fp32 columns, 16-byte chunks swizzled by row
-    *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) = make_uint4(r0[g * 4], r0[g * 4 + 1], r0[g * 4 + 2], r0[g * 4 + 3]);
-    *reinterpret_cast<uint4*>(obuf + 4096 + row_off + (((uint32_t)g ^ sw) << 4)) = make_uint4(r1[g * 4], r1[g * 4 + 1], r1[g * 4 + 2], r1[g * 4 + 3]);
-  }
+  for (int g = 0; g < 8; ++g)                                     // 16-byte chunks swizzled by row
+    *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) = make_uint4(r[g * 4], r[g * 4 + 1], r[g * 4 + 2], r[g * 4 + 3]);
   __syncwarp();
   UpdScalars sc;
   sc.alpha = d.alpha; sc.gamma = d.gamma; sc.omg = d.one_minus_gamma; sc.bc1 = d.bc1; sc.bc2 = d.bc2; sc.use_delta = d.use_delta;
@@ -103,20 +122,20 @@ __device__ __forceinline__ void epi_update_block(const TickArgs& t, const StageD
   const bool need_dl = sc.use_delta || sc.rc_shift >= 0;
   const float beta1 = t.upd_beta1, beta2 = t.upd_beta2, eps = t.upd_eps;
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
-  const int rr0 = lane >> 3, ch = lane & 7;                       // row within a group of four, 16-byte chunk of the 32-column box
-  constexpr int NB = 4;                                           // row groups whose loads are in flight together
+  const int rr0 = lane >> 3, ch = lane & 7;                       // row within a group of four, 16-byte chunk of the 32 columns
+  constexpr int NB = 2;                                           // row groups whose loads are in flight together
 #pragma unroll 1
-  for (int it0 = 0; it0 < 16; it0 += NB) {                        // 16 = 2 boxes x 8 groups of four rows
+  for (int it0 = 0; it0 < 8; it0 += NB) {                         // eight groups of four rows
     float4 g4[NB], w4[NB], m4[NB], s4[NB], d4[NB];
     uint64_t e[NB];
     bool on[NB];
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const int it = it0 + u, box = it >> 3, rr = (it & 7) * 4 + rr0;
-      const int row = mrow + rr, col = nb + box * 32 + ch * 4;
+      const int rr = (it0 + u) * 4 + rr0;
+      const int row = mrow + rr, col = nb + ch * 4;
       on[u] = row < M && col < N;
       e[u] = L.w_off + (uint64_t)row * (uint64_t)N + (uint64_t)col;
-      g4[u] = *reinterpret_cast<const float4*>(obuf + box * 4096 + rr * 128 + (((uint32_t)ch ^ (uint32_t)(rr & 7)) << 4));
+      g4[u] = *reinterpret_cast<const float4*>(obuf + rr * 128 + (((uint32_t)ch ^ (uint32_t)(rr & 7)) << 4));
       if (on[u]) {
         w4[u] = __ldcs(reinterpret_cast<const float4*>(t.a.w + e[u]));
         m4[u] = __ldcs(reinterpret_cast<const float4*>(t.a.m + e[u]));
@@ -152,143 +171,147 @@ __device__ __forceinline__ void epi_update_block(const TickArgs& t, const StageD
   }
 }
 
-// One epilogue block of the forward (MODE 0) or wgrad (MODE 2) GEMM: 32 rows x 64 accumulator columns held in
-// r0, r1 go through this warp's swizzled staging buffer to one or two TMA stores (full 128-byte rows; rows and
-// columns beyond the tensor are clipped).  Called by a whole warp; lane = row within the block.
-// A block with one bf16 output (a Linear without activation) fills one 4 KB slot and alternates slots, so it
-// only waits for the store issued two blocks ago; blocks with two outputs (z and y, or 64 fp32 columns) use both.
-// bias4: the bias of columns 4*l .. 4*l+3 of the warp's column range in lane l (MODE 0), fetched before the
-// accumulator was awaited; bias_lane0: the lane holding this block's first four columns.
+// What an epilogue warp needs to know of a tile's Linear, read before the accumulator is awaited: behind it every asm with a
+// memory clobber would make the compiler read the tables again.
+struct EpiTile {
+  int flags, act;             // MODE 0: LF_* and PM_ACT_* of the Linear
+  bool resid;                 // MODE 0: the stage adds its skip tensor here, from slot skip_slot of its buffer
+  int skip_slot;
+  int slot;                   // ring slot of z (MODE 0) or dx (MODE 1); MODE 2: gradients add to the arena
+  int yslot;                  // MODE 0: ring slot of y, or of the fp32 logits
+  const float* bias;          // MODE 0
+};
+
 template <int MODE>
-__device__ __forceinline__ void epi_block(const TickArgs& t, const CUtensorMap* lm, const StageDev& s, const StageDyn& d, const LinDev& L,
-                                          int p, int lvl, int N, int mrow, int nb, const uint32_t (&r0)[32], const uint32_t (&r1)[32],
-                                          uint8_t* obuf, uint32_t obuf_s, int lane, const float4 bias4, int bias_lane0, EpiState& es,
-                                          uint4 (&skq)[8], const __nv_bfloat16* next_skip = nullptr, int next_cols = 0, int yslot_pre = -1) {
-  if (MODE == 2 && t.fuse_upd) {                                  // the update is applied here; nothing is stored to the grad arena
-    if (t.upd_opt == PM_SGDM) epi_update_block<PM_SGDM>(t, d, L, L.n_out, N, mrow, nb, r0, r1, obuf, lane);
-    else epi_update_block<PM_ADAM>(t, d, L, L.n_out, N, mrow, nb, r0, r1, obuf, lane);
-    return;
-  }
-  const uint32_t row_off = (uint32_t)lane * 128;
-  const uint32_t sw = (uint32_t)(lane & 7);
-  const bool f32out = MODE == 0 && (L.flags & LF_OUT_F32) != 0;
-  const bool both = MODE == 2 || f32out || ((L.flags & LF_WRITE_Z) && (L.flags & LF_WRITE_Y));
-  if (lane == 0 && es.stored) {                                   // earlier stores must have finished reading what is overwritten
-    if (both || es.prev_both) tma_store_wait_read(); else tma_store_wait_read_1();
-  }
-  __syncwarp();
-  const uint32_t so = both ? 0u : es.slot * 4096u;                // slot of a single-output block
+__device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s, const StageDyn& d, const LinDev& L, int p, int lvl) {
+  EpiTile e{};
   if (MODE == 0) {
-    const int act = L.act;
-    // A stage that ends in a residual add writes the sum itself: out = bf16(skip + bf16(acc + b)), straight into the
-    // next stage's input (or the memory ring); the skip tensor was sent by the emitting stage skip_depth - 1 ticks ago.
-    const bool resid = s.post == POST_RESIDUAL;                     // skq: this lane's 64 skip values (see load_skip64)
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      float bb[8];
-      {
-        const int src = bias_lane0 + 2 * g;
-        bb[0] = __shfl_sync(0xffffffffu, bias4.x, src); bb[1] = __shfl_sync(0xffffffffu, bias4.y, src);
-        bb[2] = __shfl_sync(0xffffffffu, bias4.z, src); bb[3] = __shfl_sync(0xffffffffu, bias4.w, src);
-        bb[4] = __shfl_sync(0xffffffffu, bias4.x, src + 1); bb[5] = __shfl_sync(0xffffffffu, bias4.y, src + 1);
-        bb[6] = __shfl_sync(0xffffffffu, bias4.z, src + 1); bb[7] = __shfl_sync(0xffffffffu, bias4.w, src + 1);
-      }
-      float pf[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) pf[e] = __fadd_rn(__uint_as_float(g < 4 ? r0[(g & 3) * 8 + e] : r1[(g & 3) * 8 + e]), bb[e]);
-      if (f32out) {
-        // fp32 logits: two 32-column boxes per warp, eight 16-byte chunks per row each
-        uint8_t* box = obuf + (g >> 2) * 4096;
-        *reinterpret_cast<float4*>(box + row_off + ((((uint32_t)(g & 3) * 2) ^ sw) << 4)) = make_float4(pf[0], pf[1], pf[2], pf[3]);
-        *reinterpret_cast<float4*>(box + row_off + ((((uint32_t)(g & 3) * 2 + 1) ^ sw) << 4)) = make_float4(pf[4], pf[5], pf[6], pf[7]);
-      } else {
-        const uint32_t off = row_off + (((uint32_t)g ^ sw) << 4);
-        if (!both) {                                                // one output: no activation (z = y = bf16(acc + b)), or a ReLU whose z is not kept
-          if (resid) {
-            const uint32_t w[4] = {skq[g].x, skq[g].y, skq[g].z, skq[g].w};
-            // the registers just read take the NEXT block's skip values (same row, 64 columns on): their latency hides
-            // behind the rest of this block instead of standing in front of the next one
-            if (next_skip) skq[g] = 8 * g < next_cols ? ld_chain16(next_skip + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 sk = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
-              pf[2 * e] = __fadd_rn(sk.x, __bfloat162float(__float2bfloat16_rn(pf[2 * e])));
-              pf[2 * e + 1] = __fadd_rn(sk.y, __bfloat162float(__float2bfloat16_rn(pf[2 * e + 1])));
-            }
-          }
-          if (act == PM_ACT_RELU) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) pf[e] = fmaxf(pf[e], 0.0f);   // bf16(max(x, 0)) = max(bf16(x), 0)
-          }
-          *reinterpret_cast<uint4*>(obuf + so + off) = make_uint4(pack_bf16(pf[0], pf[1]), pack_bf16(pf[2], pf[3]), pack_bf16(pf[4], pf[5]), pack_bf16(pf[6], pf[7]));
-        }
-        else if (act == PM_ACT_NONE) epi_zy8<PM_ACT_NONE>(pf, obuf + off, obuf + 4096 + off);
-        else if (act == PM_ACT_RELU) epi_zy8<PM_ACT_RELU>(pf, obuf + off, obuf + 4096 + off);
-        else epi_zy8<PM_ACT_GELU>(pf, obuf + off, obuf + 4096 + off);
-      }
-    }
+    e.flags = L.flags; e.act = L.act;
+    e.resid = s.post == POST_RESIDUAL && !((L.flags & LF_WRITE_Z) && (L.flags & LF_WRITE_Y));
+    e.skip_slot = d.skip_rslot;
+    e.slot = d.f_slot;
+    e.yslot = lvl < s.n_lin - 1 ? d.f_slot : (s.emit_memory ? (int)(d.f_mb % t.mem_depth) : (p < t.P - 1 ? d.f_next_xslot : (int)(d.tick & 1)));
+    e.bias = fwd_small<__nv_bfloat16>(t, s, d, L.b_off, L.b_soff);
   } else if (MODE == 1) {
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {                                 // dx: one bf16 output, 64 columns per row
-      float f[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(g < 4 ? r0[(g & 3) * 8 + e] : r1[(g & 3) * 8 + e]);
-      *reinterpret_cast<uint4*>(obuf + so + row_off + (((uint32_t)g ^ sw) << 4)) =
-          make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-    }
+    e.slot = (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0;
   } else {
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {                                 // two boxes of 32 fp32 columns
-      *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) = make_uint4(r0[g * 4], r0[g * 4 + 1], r0[g * 4 + 2], r0[g * 4 + 3]);
-      *reinterpret_cast<uint4*>(obuf + 4096 + row_off + (((uint32_t)g ^ sw) << 4)) = make_uint4(r1[g * 4], r1[g * 4 + 1], r1[g * 4 + 2], r1[g * 4 + 3]);
-    }
+    e.slot = d.accum;
   }
-  fence_async_smem();                                             // staging writes -> visible to the TMA engine
-  __syncwarp();
-  if (lane == 0) {
-    if (MODE == 0) {
-      // (the caller may have formed the slot before it waited for the accumulator: it is the same for every block of a tile)
-      const int yslot = yslot_pre >= 0 ? yslot_pre : (lvl < s.n_lin - 1 ? d.f_slot
-                        : (s.emit_memory ? (int)(d.f_mb % t.mem_depth) : (p < t.P - 1 ? d.f_next_xslot : (int)(d.tick & 1))));
-      if (f32out) {
-        tma_store_3d(lm + MAP_Y_OUT, obuf_s, nb, mrow, (int)(d.tick & 1));
-        if (nb + 32 < N) tma_store_3d(lm + MAP_Y_OUT, obuf_s + 4096, nb + 32, mrow, (int)(d.tick & 1));
-      } else if (!both) {
-        if (L.flags & LF_WRITE_Z) tma_store_3d(lm + MAP_Z_OUT, obuf_s + so, nb, mrow, d.f_slot);
-        else if (L.flags & LF_WRITE_Y) tma_store_3d(lm + MAP_Y_OUT, obuf_s + so, nb, mrow, yslot);
-      } else {
-        tma_store_3d(lm + MAP_Z_OUT, obuf_s, nb, mrow, d.f_slot);
-        tma_store_3d(lm + MAP_Y_OUT, obuf_s + 4096, nb, mrow, yslot);
-      }
-    } else if (MODE == 1) {
-      // to the previous stage's gradient mailbox, or this stage's own scratch when a pre-op stands before the Linear
-      tma_store_3d(lm + MAP_DX_OUT, obuf_s + so, nb, mrow, (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0);
-    } else {
-      if (d.accum) {                                                // a later microbatch of the minibatch: dW adds to the arena
-        tma_reduce_add_2d(lm + MAP_DW_OUT, obuf_s, nb, mrow);
-        if (nb + 32 < N) tma_reduce_add_2d(lm + MAP_DW_OUT, obuf_s + 4096, nb + 32, mrow);
-      } else {
-        tma_store_2d(lm + MAP_DW_OUT, obuf_s, nb, mrow);
-        if (nb + 32 < N) tma_store_2d(lm + MAP_DW_OUT, obuf_s + 4096, nb + 32, mrow);
-      }
-    }
-    tma_store_commit();
-  }
-  es.stored = true;
-  es.prev_both = both;
-  if (!both) es.slot ^= 1u;
+  return e;
 }
 
-// (Skip tensors and stashes are written by launches this one may overlap with: ld_chain16, not read-only loads.  A lane
-// reads its row's 128 bytes in eight pieces, so they go through L1: a tick of the 6-layer encoder 1255 us, and 1259 from L2.)
-// The 64 skip-tensor values of row `row`, columns nb .. nb+63, that a residual stage's epilogue adds (zeros outside
-// the tensor and for other stages).  Issued before the accumulator is awaited, so the loads overlap the main loop.
-__device__ __forceinline__ void load_skip64(const TickArgs& t, const StageDev& s, const StageDyn& d, int N, int row, int nb, uint4 (&skq)[8]) {
-  const bool on = s.post == POST_RESIDUAL && row < t.T;
-  const __nv_bfloat16* skrow = ws_at<__nv_bfloat16>(t, s.skip_in) + (uint64_t)d.skip_rslot * ((uint64_t)t.T * N) + (uint64_t)row * N + nb;
+// One epilogue unit: 32 rows x 64 columns of the accumulator at tensor-memory address `taddr`, read 32 columns at a time
+// and passed through this warp's swizzled staging boxes to TMA stores (full 128-byte rows; rows and columns beyond the
+// tensor are clipped).  Called by a whole warp; lane = row within the block.  `release` is called once the accumulator has
+// been read.  A residual stage's skip values wait in the box (EpiStage::fetch).
+// What bounds it is the number of instructions: a tile of 128 x 256 per CTA is sixteen units on four schedulers, and the tensor core
+// takes 4096 cycles for it at a reduction of 512.  Hence two columns per instruction everywhere (a bf16 sum of two bf16 values
+// rounded once is what the fp32 sum rounds to: at most 16 binary digits apart the fp32 sum is exact, further apart neither
+// reaches a tie), and one branch per half on what the Linear does.
+// bias: that of columns 2 l and 2 l + 1 in lane l.  (With one column per instruction the
+// forward of the 6-layer encoder's tick took 194 us, 164 now; reading the skip values row by row into registers 172.)
+template <int MODE, bool FUSE, int SLOTS, class Release>
+__device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* lm, const StageDyn& d, const LinDev& L, const EpiTile& et,
+                                         int M, int N, int mrow, int nb, uint32_t taddr, EpiStage<SLOTS>& es,
+                                         const float2 bias, Release release) {
+  const int lane = es.lane;
+  const uint32_t row_off = (uint32_t)lane * 128, sw = (uint32_t)(lane & 7);
+  uint32_t r[32];
+  auto load_half = [&](int h) {
+    tmem_ld32(taddr + 32 * h, r);
+    tmem_ld_wait();
+    if (h == 1) release();
+  };
+  if (mrow >= M || nb >= N) { release(); return; }                // nothing of this unit lies in the tensor
+  auto bias4 = [&](int h, int g) {
+    const int src = 16 * h + 2 * g;
+    return make_float4(__shfl_sync(0xffffffffu, bias.x, src), __shfl_sync(0xffffffffu, bias.y, src),
+                       __shfl_sync(0xffffffffu, bias.x, src + 1), __shfl_sync(0xffffffffu, bias.y, src + 1));
+  };
+  auto pair = [&](int i, float bx, float by) {                    // two columns of the half in r, with the bias
+    const float2 v = make_float2(__uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+    return MODE == 0 ? add_f32x2(v, make_float2(bx, by)) : v;
+  };
+  if (MODE == 2 || (MODE == 0 && (et.flags & LF_OUT_F32))) {      // two boxes of 32 fp32 columns
+#pragma unroll (FUSE ? 2 : 1)
+    for (int h = 0; h < 2; ++h) {
+      load_half(h);
+      if (MODE == 2 && FUSE) {                                    // the update is applied here; nothing is stored to the grad arena
+        if (t.upd_opt == PM_SGDM) epi_update_block<PM_SGDM>(t, d, L, M, N, mrow, nb + 32 * h, r, es.buf, lane);
+        else epi_update_block<PM_ADAM>(t, d, L, M, N, mrow, nb + 32 * h, r, es.buf, lane);
+        continue;
+      }
+      uint8_t* box = es.begin();
 #pragma unroll
-  for (int g = 0; g < 8; ++g)                                       // columns are multiples of 8
-    skq[g] = (on && nb + 8 * g < N) ? ld_chain16(skrow + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
+      for (int g = 0; g < 8; ++g) {
+        const float4 b = MODE == 0 ? bias4(h, g) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float2 v0 = pair(4 * g, b.x, b.y), v1 = pair(4 * g + 2, b.z, b.w);
+        *reinterpret_cast<float4*>(box + row_off + (((uint32_t)g ^ sw) << 4)) = make_float4(v0.x, v0.y, v1.x, v1.y);
+      }
+      es.end([&](uint32_t src) {
+        if (nb + 32 * h >= N) return;
+        if (MODE == 0) tma_store_3d(lm + MAP_Y_OUT, src, nb + 32 * h, mrow, et.yslot);
+        else if (et.slot) tma_reduce_add_2d(lm + MAP_DW_OUT, src, nb + 32 * h, mrow);   // a later microbatch of the minibatch: dW adds to the arena
+        else tma_store_2d(lm + MAP_DW_OUT, src, nb + 32 * h, mrow);
+      });
+    }
+    return;
+  }
+  const bool both = MODE == 0 && (et.flags & LF_WRITE_Z) && (et.flags & LF_WRITE_Y);   // z, then y = act(z) from the staged z
+  // A stage that ends in a residual add writes the sum itself: out = bf16(skip + bf16(acc + b)), straight into the
+  // next stage's input (or the memory ring); the skip tensor was sent by the emitting stage skip_depth - 1 ticks ago.
+  enum { PLAIN, RELU, RESIDUAL };
+  uint8_t* box = nullptr;
+  auto half = [&](int h, auto kind) {
+    constexpr int KIND = decltype(kind)::value;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const float4 b0 = MODE == 0 ? bias4(h, 2 * g) : make_float4(0.f, 0.f, 0.f, 0.f), b1 = MODE == 0 ? bias4(h, 2 * g + 1) : b0;
+      const float2 v0 = pair(8 * g, b0.x, b0.y), v1 = pair(8 * g + 2, b0.z, b0.w), v2 = pair(8 * g + 4, b1.x, b1.y), v3 = pair(8 * g + 6, b1.z, b1.w);
+      uint4 o = make_uint4(pack_bf16(v0.x, v0.y), pack_bf16(v1.x, v1.y), pack_bf16(v2.x, v2.y), pack_bf16(v3.x, v3.y));
+      if (KIND == RELU) o = make_uint4(relu_bf16x2(o.x), relu_bf16x2(o.y), relu_bf16x2(o.z), relu_bf16x2(o.w));   // bf16(max(x, 0)) = max(bf16(x), 0)
+      if (KIND == RESIDUAL) {
+        const uint4 k = *reinterpret_cast<const uint4*>(box + row_off + (((uint32_t)(4 * h + g) ^ sw) << 4));
+        o = make_uint4(add_bf16x2(k.x, o.x), add_bf16x2(k.y, o.y), add_bf16x2(k.z, o.z), add_bf16x2(k.w, o.w));
+      }
+      *reinterpret_cast<uint4*>(box + row_off + (((uint32_t)(4 * h + g) ^ sw) << 4)) = o;
+    }
+  };
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    load_half(h);
+    if (h == 0) box = MODE == 0 && et.resid ? es.buf + es.off : es.begin();
+    if (MODE == 0 && et.resid) half(h, std::integral_constant<int, RESIDUAL>());
+    else if (MODE == 0 && et.act == PM_ACT_RELU && !both) half(h, std::integral_constant<int, RELU>());
+    else half(h, std::integral_constant<int, PLAIN>());
+  }
+  es.end([&](uint32_t src) {
+    // dx: to the previous stage's gradient mailbox, or this stage's own scratch when a pre-op stands before the Linear
+    if (MODE == 1) tma_store_3d(lm + MAP_DX_OUT, src, nb, mrow, et.slot);
+    else if (et.flags & LF_WRITE_Z) tma_store_3d(lm + MAP_Z_OUT, src, nb, mrow, et.slot);
+    else if (et.flags & LF_WRITE_Y) tma_store_3d(lm + MAP_Y_OUT, src, nb, mrow, et.yslot);
+  });
+  if (!both) return;
+  uint8_t* ybox = es.begin();                                     // one slot: z's own box, which its store has read by now
+  auto write_y = [&](auto a) {
+    constexpr int ACT = decltype(a)::value;
+#pragma unroll 1
+    for (int g = 0; g < 8; ++g) {
+      const uint32_t off = row_off + (((uint32_t)g ^ sw) << 4);
+      const uint4 z = *reinterpret_cast<const uint4*>(box + off);
+      uint32_t o[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&o[e]));
+        if (ACT != PM_ACT_NONE) o[e] = pack_bf16(act_fwd(f.x, ACT), act_fwd(f.y, ACT));
+      }
+      *reinterpret_cast<uint4*>(ybox + off) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  };
+  if (et.act == PM_ACT_GELU) write_y(std::integral_constant<int, PM_ACT_GELU>());
+  else if (et.act == PM_ACT_RELU) write_y(std::integral_constant<int, PM_ACT_RELU>());
+  else write_y(std::integral_constant<int, PM_ACT_NONE>());
+  es.end([&](uint32_t src) { tma_store_3d(lm + MAP_Y_OUT, src, nb, mrow, et.yslot); });
 }
 
 // dgrad epilogue of a stage whose predecessor's ReLU backward is fused here (StageDev::mask_dx): the 64 values of this
@@ -324,38 +347,65 @@ __device__ __forceinline__ void apply_mask8(float (&f)[8], uint32_t bits) {
   for (int e = 0; e < 8; ++e) if (!((bits >> e) & 1u)) f[e] = 0.0f;
 }
 
-// bias of columns n .. n+3 (zero beyond the tensor); n is a multiple of four
-__device__ __forceinline__ float4 load_bias4(const float* bias, int n, int N) {
-  return n < N ? __ldg(reinterpret_cast<const float4*>(bias + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
 // ---- tile walk ---------------------------------------------------------------------------------------
 // tile_start[p] .. tile_start[p+1] are the flattened tile ids of stage p for this (mode, level).
-struct Tile { int p, m0, n0, M, N, K, n_kb; bool valid; };
 // the tile a CTA's slot holds: from the launch's order list, or, in a launch of one stage (its tiles in ascending
 // order), from the launch arguments alone, so that no role starts with a chain of dependent global loads
 __device__ __forceinline__ int tile_at(const TickArgs& t, const int* __restrict__ order, int slot) {
   return t.sel_p >= 0 ? t.sel_tile0 + slot : order[slot];
 }
 
-template <int MODE>
-__device__ __forceinline__ Tile decode_tile(const TickArgs& t, const int* __restrict__ tile_start, int lvl, int tile) {
-  Tile r;
-  const int lo = t.sel_p >= 0 ? t.sel_p : tile_start[t.P + 1 + tile];                           // the stage of this tile: table behind the P + 1 starts
-  r.p = lo;
-  const StageDyn& d = t.dyn[lo];
-  const StageDev& s = t.st[lo];
-  r.valid = lvl < s.n_lin && (MODE == 0 ? d.f_mb >= 0 : d.b_mb >= 0) && !(MODE == 1 && lo == 0 && lvl == 0 && s.pre != PRE_EMBED);
-  const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
-  if (MODE == 0) { r.M = t.T; r.N = L.n_out; r.K = L.n_in; }
-  else if (MODE == 1) { r.M = t.T; r.N = L.n_in; r.K = L.n_out; }
-  else { r.M = L.n_out; r.N = L.n_in; r.K = t.T; }
-  const int tiles_n = (r.N + TILE_N - 1) / TILE_N;
-  const int local = tile - (t.sel_p >= 0 ? t.sel_tile0 : tile_start[lo]);
-  r.m0 = (local / tiles_n) * TILE_M;
-  r.n0 = (local % tiles_n) * TILE_N;
-  r.n_kb = (r.K + TILE_K - 1) / TILE_K;
+// A tile as one lane decodes it.  sa, sb: ring slots of the operands.
+struct Tile { int p, m0, n0, n_kb, sa, sb; };                         // p < 0: the slot holds no tile, or one of an idle stage
+
+// TS: rows and columns of a tile
+template <int MODE, int TS>
+__device__ __forceinline__ Tile decode_tile(const TickArgs& t, const int* __restrict__ tile_start, const int* __restrict__ order, int n_slots, int lvl, int slot) {
+  Tile r{-1, 0, 0, 0, 0, 0};
+  if (slot >= n_slots) return r;
+  const int tile = tile_at(t, order, slot);
+  if (tile < 0) return r;
+  const int p = t.sel_p >= 0 ? t.sel_p : tile_start[t.P + 1 + tile];                            // the stage of this tile: table behind the P + 1 starts
+  const StageDyn& d = t.dyn[p];
+  const StageDev& s = t.st[p];
+  if (lvl >= s.n_lin || (MODE == 0 ? d.f_mb < 0 : d.b_mb < 0) || (MODE == 1 && p == 0 && lvl == 0 && s.pre != PRE_EMBED)) return r;
+  const LinDev& L = s.lin[lvl];
+  const int N = MODE == 0 ? L.n_out : L.n_in, K = MODE == 0 ? L.n_in : (MODE == 1 ? L.n_out : t.T);
+  const int tiles_n = (N + TS - 1) / TS, local = tile - (t.sel_p >= 0 ? t.sel_tile0 : tile_start[p]);
+  r.p = p;
+  r.m0 = local / tiles_n * TS;
+  r.n0 = local % tiles_n * TS;
+  r.n_kb = (K + TILE_K - 1) / TILE_K;
+  const bool own_input = lvl == 0 && s.pre == PRE_NONE;
+  // dz operand: the dz scratch, or (no activation) the incoming gradient itself, which for the last Linear of a stage without
+  // attention is the rotating mailbox slot written during the previous tick
+  if (MODE != 0) r.sa = (bwd_act(L) == PM_ACT_NONE && lvl == s.n_lin - 1 && !feeds_attention(s.post)) ? dz_mailbox_slot(t, s, d) : 0;
+  else r.sa = own_input ? d.f_xslot : d.f_slot;
+  r.sb = MODE == 2 ? (own_input ? d.b_xslot : d.b_slot) : d.f_vslot;   // wgrad: the input's slot; else the weight version
   return r;
+}
+
+// A role's walk over its CTA's tiles.  The tables that say what a tile is are four dependent loads deep, several microseconds of
+// an idle tensor core when every role reads them between two tiles (a tick's forward of the 6-layer encoder, eight k-blocks per
+// tile: 205 us, 194 with this walk).  So the lanes of a warp decode 32 tiles at a time, each its own, and hand them round.
+// `body` runs warp-wide and returns (the same in all lanes) whether to go on.  `mine`: the first 32, decoded before the launch
+// waited for its predecessor.
+template <class Decode, class Body>
+__device__ __forceinline__ void walk_tiles(Tile mine, int first, int step, int n_slots, int lane, Decode decode, Body body) {
+  for (int s0 = first;;) {
+    uint32_t todo = __ballot_sync(0xffffffffu, mine.p >= 0);
+    while (todo) {
+      const int j = __ffs(todo) - 1;
+      todo &= todo - 1;
+      Tile tl;
+      tl.p = __shfl_sync(0xffffffffu, mine.p, j); tl.m0 = __shfl_sync(0xffffffffu, mine.m0, j); tl.n0 = __shfl_sync(0xffffffffu, mine.n0, j);
+      tl.n_kb = __shfl_sync(0xffffffffu, mine.n_kb, j); tl.sa = __shfl_sync(0xffffffffu, mine.sa, j); tl.sb = __shfl_sync(0xffffffffu, mine.sb, j);
+      if (!body(tl)) return;
+    }
+    s0 += 32 * step;
+    if (s0 >= n_slots) return;
+    mine = decode(s0 + lane * step);
+  }
 }
 
 struct Ring {                       // position in a ring of mbarrier-guarded slots
@@ -363,11 +413,76 @@ struct Ring {                       // position in a ring of mbarrier-guarded sl
   __device__ __forceinline__ void advance(int n) { if (++idx == n) { idx = 0; phase ^= 1u; } }
 };
 
+// ---- bias gradient: column sums of dz in the weight-gradient kernels -----------------------------------
+// The A operand of the weight gradient is dz itself, so db needs no pass of its own: in the tiles of the first column the
+// tensor core's release of an operand slot goes to four summing warps first, which take the slot's 64 rows of dz to registers,
+// hand it to the producer and add.  Warp w owns the columns 32 w .. 32 w + 31 of the CTA's 128: lane = (16-byte chunk of eight
+// columns, row group); the two row groups of a quarter-warp differ in bit 2, which the swizzle turns into distinct banks.  Eight
+// rows are added pairwise, then to the running sum of their row group, the eight row groups pairwise at the end.
+// What it replaced: launches that read dz again, 92 + 15 us of a tick of the 6-layer encoder (57 now, for the activations alone), 121 us of
+// an update of the encoder-decoder of 2 + 2 layers of width 1024; the weight gradients themselves 148 -> 146 and 532 -> 493 us, the
+// sums costing them less than the elected-lane loops gave.  (Releasing the slot only after the additions: 166 us.)
+__device__ __forceinline__ void colsum_add8(const uint4 (&q)[8], float (&acc)[8]) {
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    float lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t x = w == 0 ? q[j].x : w == 1 ? q[j].y : w == 2 ? q[j].z : q[j].w;
+      lo[j] = __uint_as_float(x << 16); hi[j] = __uint_as_float(x & 0xFFFF0000u);
+    }
+    auto sum8 = [](const float (&v)[8]) {
+      return __fadd_rn(__fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3])), __fadd_rn(__fadd_rn(v[4], v[5]), __fadd_rn(v[6], v[7])));
+    };
+    acc[2 * w] = __fadd_rn(acc[2 * w], sum8(lo));
+    acc[2 * w + 1] = __fadd_rn(acc[2 * w + 1], sum8(hi));
+  }
+}
+// the lanes of a column chunk meet; lanes 0..3 write eight columns each
+__device__ __forceinline__ void colsum_store(const TickArgs& t, const StageDyn& d, const LinDev& L, int m, int lane, float (&acc)[8]) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    acc[e] = __fadd_rn(acc[e], __shfl_xor_sync(0xffffffffu, acc[e], 4));
+    acc[e] = __fadd_rn(acc[e], __shfl_xor_sync(0xffffffffu, acc[e], 8));
+    acc[e] = __fadd_rn(acc[e], __shfl_xor_sync(0xffffffffu, acc[e], 16));
+  }
+  if (lane < 4 && m < L.n_out) {                                  // widths are multiples of 8
+    float* db = t.a.grad + L.b_off + m;
+    if (d.accum) { float o[8]; load8<float>(db, o);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] = __fadd_rn(o[e], acc[e]); }
+    store8<float>(db, acc);
+  }
+}
+// One summing warp's part of a tile.  `done` completes when the MMAs have read a slot of a summed tile (phases: the parity of
+// each slot's next completion), the arrival on `empty` hands the slot back.
+template <int NS>
+__device__ __forceinline__ void colsum_tile(const TickArgs& t, int lvl, const Tile& tl, int row0, int sw, int lane, int& idx, uint32_t& phases, bool& ok,
+                                            const uint8_t* tiles_ptr, uint32_t bar_done, uint32_t bar_empty, volatile int* abort_flag, int* status) {
+  if (tl.n0 != 0) { idx = (idx + tl.n_kb) % NS; return; }
+  const int r = lane >> 2, chunk = 4 * sw + (lane & 3), row = ((r & 1) << 2) | (r >> 1);
+  const uint32_t off = (uint32_t)(chunk >> 3) * (A_BYTES / 2) + (uint32_t)row * 128 + (uint32_t)(((chunk & 7) ^ row) << 4);   // rows row + 8 j: the same swizzle
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int kb = 0; kb < tl.n_kb; ++kb) {
+    const bool ready = mbar_wait(bar_done + 8 * idx, (phases >> idx) & 1u, abort_flag, status, 9);
+    ok = __all_sync(0xffffffffu, ready) && ok;                    // a CTA that gives up: the warps still meet at every k-block
+    phases ^= 1u << idx;
+    uint4 q[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) q[j] = *reinterpret_cast<const uint4*>(tiles_ptr + idx * STAGE_BYTES + off + j * 1024);
+    asm volatile("bar.sync 1, 128;" ::: "memory");                // the four summing warps have read the slot
+    if (ok && sw == 0 && lane == 0) mbar_arrive(bar_empty + 8 * idx);
+    colsum_add8(q, acc);
+    if (++idx == NS) idx = 0;
+  }
+  if (ok) colsum_store(t, t.dyn[tl.p], t.st[tl.p].lin[lvl], tl.m0 + row0 + 8 * chunk, lane, acc);
+}
+
 // ---- the kernel --------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1)
+template <int MODE, bool FUSE>
+__global__ void __launch_bounds__(Cfg<MODE, FUSE>::kThreads, 1)
 umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ tile_start, const int* __restrict__ order, int n_slots, int lvl, int* status) {
-  using C = Cfg<MODE>;
+  using C = Cfg<MODE, FUSE>;
   constexpr int NS = C::kStages;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -376,16 +491,17 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
   const uint32_t outs = tiles + NS * STAGE_BYTES;                     // epilogue staging for TMA stores
   uint8_t* outs_ptr = tiles_ptr + NS * STAGE_BYTES;
   const uint32_t bars = tiles + C::kTileBytes;
-  // barrier block: full[NS] empty[NS] tfull[2] tempty[2], then tmem base word and abort flag
-  const uint32_t bar_full = bars, bar_empty = bar_full + 8 * NS, bar_tfull = bar_empty + 8 * NS, bar_tempty = bar_tfull + 16;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tiles_ptr + C::kTileBytes + 8 * (2 * NS + 4));
+  // barrier block: full[NS] empty[NS] done[NS] tfull[2] tempty[2] skip[one per epilogue warp], then tmem base word and abort flag
+  const uint32_t bar_full = bars, bar_empty = bar_full + 8 * NS, bar_done = bar_empty + 8 * NS, bar_tfull = bar_done + 8 * NS, bar_tempty = bar_tfull + 16, bar_skip = bar_tempty + 16;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tiles_ptr + C::kTileBytes + 8 * (3 * NS + 4 + N_EPI_WARPS));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NS; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
+    for (int i = 0; i < NS; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); mbar_init(bar_done + 8 * i, 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull + 8 * i, 1); mbar_init(bar_tempty + 8 * i, N_EPI_WARPS); }
+    for (int i = 0; i < N_EPI_WARPS; ++i) mbar_init(bar_skip + 8 * i, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -394,6 +510,9 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
     tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
     tmem_relinquish();
   }
+  const int first = (int)blockIdx.x, step = (int)gridDim.x;
+  auto decode = [&](int slot) { return decode_tile<MODE, TILE_N>(t, tile_start, order, n_slots, lvl, slot); };
+  const Tile mine = decode(first + lane * step);                      // tables no launch of the phase writes
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -403,137 +522,115 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      Ring op{0, 0};
-      int issued_op = 0;
-      bool ok = true;
-      for (int slot = blockIdx.x; slot < n_slots && ok; slot += gridDim.x) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const Tile tl = decode_tile<MODE>(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        const StageDyn& d = t.dyn[tl.p];
-        const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-        // dz operand: the dz scratch, or (no activation) the incoming gradient itself, which for the last Linear of a
-        // stage without attention is the rotating mailbox slot written during the previous tick
-        const StageDev& sd_ = t.st[tl.p];
-        const int dz_slot = (bwd_act(sd_.lin[lvl]) == PM_ACT_NONE && lvl == sd_.n_lin - 1 && !feeds_attention(sd_.post)) ? dz_mailbox_slot(t, sd_, d) : 0;
-        if (MODE == 0) { tma_prefetch_desc(lm + MAP_ACT_K); tma_prefetch_desc(lm + MAP_W_K); }
-        else if (MODE == 1) { tma_prefetch_desc(lm + MAP_DZ_K); tma_prefetch_desc(lm + MAP_W_MN); }
-        else { tma_prefetch_desc(lm + MAP_DZ_MN); tma_prefetch_desc(lm + MAP_ACT_MN); }
-        for (int kb = 0; kb < tl.n_kb; ++kb) {
-          const int k0 = kb * TILE_K;
-          if (!mbar_wait(bar_empty + 8 * op.idx, op.phase ^ 1, abort_flag, status, 1)) { ok = false; break; }
-          const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES, fb = bar_full + 8 * op.idx;
+    Ring op{0, 0};
+    int issued_op = 0;
+    walk_tiles(mine, first, step, n_slots, lane, decode, [&](const Tile& tl) {
+      const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
+      for (int kb = 0; kb < tl.n_kb; ++kb) {
+        const int k0 = kb * TILE_K;
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * op.idx, op.phase ^ 1, abort_flag, status, 1))) return false;
+        const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES, fb = bar_full + 8 * op.idx;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(fb, A_BYTES + B_BYTES);
           if (MODE == 0) {
-            mbar_arrive_expect_tx(fb, A_BYTES + B_BYTES);
-            tma_load_3d(sa, lm + MAP_ACT_K, fb, k0, tl.m0, (lvl == 0 && t.st[tl.p].pre == PRE_NONE) ? d.f_xslot : d.f_slot);
-            tma_load_3d(sb, lm + MAP_W_K, fb, k0, tl.n0, d.f_vslot);
+            tma_load_3d(sa, lm + MAP_ACT_K, fb, k0, tl.m0, tl.sa);
+            tma_load_3d(sb, lm + MAP_W_K, fb, k0, tl.n0, tl.sb);
           } else if (MODE == 1) {
-            // dx = dz W_v: dz K-major, the queued version v of the weights (the one the microbatch's forward read) as the
-            // MN-major operand, two 64-column runs
-            mbar_arrive_expect_tx(fb, A_BYTES + B_BYTES);
-            tma_load_3d(sa, lm + MAP_DZ_K, fb, k0, tl.m0, dz_slot);
-            tma_load_3d(sb, lm + MAP_W_MN, fb, tl.n0, k0, d.f_vslot);
-            tma_load_3d(sb + B_BYTES / 2, lm + MAP_W_MN, fb, tl.n0 + 64, k0, d.f_vslot);
+            // dx = dz W: dz K-major, the weights as the MN-major operand, two 64-column runs
+            tma_load_3d(sa, lm + MAP_DZ_K, fb, k0, tl.m0, tl.sa);
+            tma_load_3d(sb, lm + MAP_W_MN, fb, tl.n0, k0, tl.sb);
+            tma_load_3d(sb + B_BYTES / 2, lm + MAP_W_MN, fb, tl.n0 + 64, k0, tl.sb);
           } else {
-            mbar_arrive_expect_tx(fb, A_BYTES + B_BYTES);
-            const int slot = (lvl == 0 && t.st[tl.p].pre == PRE_NONE) ? d.b_xslot : d.b_slot;
-            tma_load_3d(sa, lm + MAP_DZ_MN, fb, tl.m0, k0, dz_slot);
-            tma_load_3d(sa + A_BYTES / 2, lm + MAP_DZ_MN, fb, tl.m0 + 64, k0, dz_slot);
-            tma_load_3d(sb, lm + MAP_ACT_MN, fb, tl.n0, k0, slot);
-            tma_load_3d(sb + B_BYTES / 2, lm + MAP_ACT_MN, fb, tl.n0 + 64, k0, slot);
+            tma_load_3d(sa, lm + MAP_DZ_MN, fb, tl.m0, k0, tl.sa);
+            tma_load_3d(sa + A_BYTES / 2, lm + MAP_DZ_MN, fb, tl.m0 + 64, k0, tl.sa);
+            tma_load_3d(sb, lm + MAP_ACT_MN, fb, tl.n0, k0, tl.sb);
+            tma_load_3d(sb + B_BYTES / 2, lm + MAP_ACT_MN, fb, tl.n0 + 64, k0, tl.sb);
           }
-          op.advance(NS); ++issued_op;
         }
+        __syncwarp();
+        op.advance(NS); ++issued_op;
       }
-      if (*abort_flag) {
-        // copies already issued still land in this CTA's shared memory: wait for them (bounded) before leaving
-        for (int back = 1; back <= NS && back <= issued_op; ++back) {
-          const int it = issued_op - back;
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar_full + 8 * (it % NS), (uint32_t)(it / NS) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
+      return true;
+    });
+    if (lane == 0 && *abort_flag) {
+      // copies already issued still land in this CTA's shared memory: wait for them (bounded) before leaving
+      for (int back = 1; back <= NS && back <= issued_op; ++back) {
+        const int it = issued_op - back;
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_full + 8 * (it % NS), (uint32_t)(it / NS) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc(MODE == 2, MODE != 0);
-      // K-major: 16 elements = 32 bytes along the swizzled row.  MN-major: 16 k-rows of 128 bytes.
-      const uint64_t dba = MODE == 2 ? desc_base(A_BYTES / 2, 1024) : desc_base(16, 1024);
-      const uint64_t dbb = MODE == 0 ? desc_base(16, 1024) : desc_base(B_BYTES / 2, 1024);
-      const uint32_t ka = MODE == 2 ? 2048 : 32, kb_ = MODE == 0 ? 32 : 2048;
-      Ring op{0, 0}, acc{0, 0};
-      bool ok = true;
-      for (int slot = blockIdx.x; slot < n_slots && ok; slot += gridDim.x) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const Tile tl = decode_tile<MODE>(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        if (!mbar_wait(bar_tempty + 8 * acc.idx, acc.phase ^ 1, abort_flag, status, 6)) { ok = false; break; }
+    const uint32_t idesc = make_idesc(MODE == 2, MODE != 0);
+    // K-major: 16 elements = 32 bytes along the swizzled row.  MN-major: 16 k-rows of 128 bytes.
+    const uint64_t dba = MODE == 2 ? desc_base(A_BYTES / 2, 1024) : desc_base(16, 1024);
+    const uint64_t dbb = MODE == 0 ? desc_base(16, 1024) : desc_base(B_BYTES / 2, 1024);
+    const uint32_t ka = MODE == 2 ? 2048 : 32, kb_ = MODE == 0 ? 32 : 2048;
+    Ring op{0, 0}, acc{0, 0};
+    walk_tiles(mine, first, step, n_slots, lane, decode, [&](const Tile& tl) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_tempty + 8 * acc.idx, acc.phase ^ 1, abort_flag, status, 6))) return false;
+      tc_fence_after();
+      const uint32_t tmem_acc = tmem_base + (uint32_t)(acc.idx * ACC_COLS);
+      // a slot is free once these MMAs have read it (first column of a weight gradient: by way of the summing warps)
+      const uint32_t release = C::kSumWarps && tl.n0 == 0 ? bar_done : bar_empty;
+      for (int kb = 0; kb < tl.n_kb; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * op.idx, op.phase, abort_flag, status, 2))) return false;
         tc_fence_after();
-        const uint32_t tmem_acc = tmem_base + (uint32_t)(acc.idx * ACC_COLS);
-        for (int kb = 0; kb < tl.n_kb; ++kb) {
-          if (!mbar_wait(bar_full + 8 * op.idx, op.phase, abort_flag, status, 2)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+        const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+        if (elect_one()) {
 #pragma unroll
           for (int k16 = 0; k16 < TILE_K / 16; ++k16)
             tc_mma_bf16(tmem_acc, desc_at(dba, sa + k16 * ka), desc_at(dbb, sb + k16 * kb_), idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-          tc_commit(bar_empty + 8 * op.idx);      // frees the operand slot once these MMAs have read it
-          op.advance(NS);
+          tc_commit(release + 8 * op.idx);
+          if (kb == tl.n_kb - 1) tc_commit(bar_tfull + 8 * acc.idx);   // accumulator complete
         }
-        if (ok) tc_commit(bar_tfull + 8 * acc.idx);   // accumulator complete
-        acc.advance(2);
+        __syncwarp();
+        op.advance(NS);
       }
-    }
+      acc.advance(2);
+      return true;
+    });
+  } else if (warp < 2 + C::kSumWarps) {
+    // ---------------- bias gradient: column sums of dz ----------------
+    int idx = 0;
+    uint32_t phases = 0;
+    bool ok = true;
+    walk_tiles(mine, first, step, n_slots, lane, decode, [&](const Tile& tl) {
+      colsum_tile<NS>(t, lvl, tl, 0, warp - 2, lane, idx, phases, ok, tiles_ptr, bar_done, bar_empty, abort_flag, status);
+      return true;
+    });
   } else {
     // ---------------- epilogue: 8 warps, warp%4 = TMEM lane group, two warps per group split the columns ----------------
-    // Each warp drains a 32-row x 64-column block, writes it into its own swizzled staging buffer and lets
-    // the TMA engine store it (full 128-byte rows; rows and columns beyond the tensor are clipped).
     const int q = warp & 3;
-    const int ew = warp - 2;                                          // 0..7
+    const int ew = warp - 2 - C::kSumWarps;                           // 0..7
     const int half = ew >> 2;                                         // 0: columns 0..63, 1: columns 64..127
-    uint8_t* obuf = outs_ptr + ew * C::kOutWarpBytes;
-    const uint32_t obuf_s = outs + ew * C::kOutWarpBytes;
-    const uint32_t row_off = (uint32_t)lane * 128;
-    const uint32_t sw = (uint32_t)(lane & 7);
+    EpiStage<2> es{outs_ptr + ew * C::kOutWarpBytes, outs + ew * C::kOutWarpBytes, lane, bar_skip + 8 * ew};
     Ring acc{0, 0};
-    bool ok = true;
-    EpiState es;
-    for (int slot = blockIdx.x; slot < n_slots && ok; slot += gridDim.x) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const Tile tl = decode_tile<MODE>(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
+    walk_tiles(mine, first, step, n_slots, lane, decode, [&](const Tile& tl) {
       const StageDyn& d = t.dyn[tl.p];
       const StageDev& s = t.st[tl.p];
       const LinDev& L = s.lin[lvl];
       const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-      const int mrow = tl.m0 + q * 32;                                // first row of this warp's block
-      const int nb = tl.n0 + half * 64;
-      // bias of this warp's 64 columns, four per lane in lanes 0..15, on its way while the accumulator completes
-      const float4 bias4 = (MODE == 0 && lane < 16) ? load_bias4(fwd_small<__nv_bfloat16>(t, s, d, L.b_off, L.b_soff), nb + 4 * lane, tl.N) : make_float4(0.f, 0.f, 0.f, 0.f);
-      uint4 skq[8];
-      if (MODE == 0) load_skip64(t, s, d, tl.N, mrow + lane, nb, skq);
-      bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 4);
-      ready = __all_sync(0xffffffffu, ready);                         // tcgen05.ld needs the whole warp
-      if (!ready) { ok = false; break; }
+      const int M = MODE == 2 ? L.n_out : t.T, N = MODE == 0 ? L.n_out : L.n_in;
+      const int mrow = tl.m0 + q * 32, nb = tl.n0 + half * 64;        // this warp's block
+      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl);
+      const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
+      const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
+      if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
+      const bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 4);
+      bool go = __all_sync(0xffffffffu, ready);                       // tcgen05.ld needs the whole warp
+      if (fetch && go) go = es.fetched(abort_flag, status);
+      if (!go) { if (fetch) es.drain(); return false; }
       tc_fence_after();
-      uint32_t r0[32], r1[32];
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64);
-      tmem_ld32(taddr, r0);
-      tmem_ld32(taddr + 32, r1);
-      tmem_ld_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tempty + 8 * acc.idx);           // the accumulator buffer may be overwritten now
-      __syncwarp();
+      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias, [&] {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tempty + 8 * acc.idx);         // the accumulator buffer may be overwritten now
+      });
       acc.advance(2);
-      if (mrow >= tl.M || nb >= tl.N) continue;                       // nothing of this block is inside the tensor
-      epi_block<MODE>(t, lm, s, d, L, tl.p, lvl, tl.N, mrow, nb, r0, r1, obuf, obuf_s, lane, bias4, 0, es, skq);
-    }
+      return true;
+    });
     if (lane == 0 && es.stored) tma_store_wait_all();                    // global writes complete before the CTA retires
   }
   tc_fence_before();
@@ -546,46 +643,31 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
 }
 
 // ---- CTA-pair GEMM: 256 x 256 output tiles ---------------------------------------------------------------
-// The same forward / wgrad products on tiles of 256 x 256 computed by two CTAs of a cluster with one
+// The same products on tiles of 256 x 256 computed by two CTAs of a cluster with one
 // tcgen05.mma.cta_group::2 per 16 k-columns.  Each CTA loads its 128 rows of A and its 128 of the 256
 // columns of B, so a CTA ingests 32 KB per 128x256x64 product: half the shared-memory fill per FLOP of the
 // single-CTA kernel, whose tensor pipe waits on that fill.  Roles per CTA: warp 0 = TMA producer (loads
 // land in its own shared memory and are counted on the leader's `full` barrier), warp 1 = TMEM owner and,
-// in the leader (cluster rank 0), MMA issuer; eight epilogue warps drain the CTA's own 128 accumulator
-// rows (two warps per lane group, 128 columns each, in two blocks of 64).  tcgen05.commit arrives on the
+// in the leader (cluster rank 0), MMA issuer; sixteen epilogue warps drain the CTA's own 128 accumulator
+// rows (four warps per lane group, 64 columns each).  tcgen05.commit arrives on the
 // `empty` / `tfull` barriers of both CTAs; the epilogue warps of both arrive on the leader's `tempty`.
 // Used when every GEMM of the launch has at least 256 rows and columns; smaller shapes keep the kernel above.
 constexpr int P2_TILE = 256;
 constexpr int P2_STAGES = 5;
 constexpr int P2_ACC_COLS = 256;                                      // two accumulators fill the 512 TMEM columns
-constexpr int P2_THREADS = 32 * (2 + N_EPI_WARPS);
-constexpr int P2_TILE_BYTES = P2_STAGES * STAGE_BYTES + N_EPI_WARPS * 8192;
+constexpr int P2_TILE_BYTES = P2_STAGES * STAGE_BYTES + 16 * 4096;
 constexpr int P2_SMEM_BYTES = P2_TILE_BYTES + 1024 + 512;
+template <int MODE, bool FUSE> struct P2Cfg {
+  static constexpr int kSumWarps = Cfg<MODE, FUSE>::kSumWarps;
+  static constexpr int kEpiWarps = FUSE ? 8 : 16;        // those with more registers per thread
+  static constexpr int kUnits = 16 / kEpiWarps;                       // 32 x 64 blocks of the CTA's accumulator per warp
+  static constexpr int kThreads = 32 * (2 + kSumWarps + kEpiWarps);
+};
 
-template <int MODE>
-__device__ __forceinline__ Tile decode_pair_tile(const TickArgs& t, const int* __restrict__ tile_start, int lvl, int tile) {
-  Tile r;
-  const int lo = t.sel_p >= 0 ? t.sel_p : tile_start[t.P + 1 + tile];                           // the stage of this tile: table behind the P + 1 starts
-  r.p = lo;
-  const StageDyn& d = t.dyn[lo];
-  const StageDev& s = t.st[lo];
-  r.valid = lvl < s.n_lin && (MODE == 0 ? d.f_mb >= 0 : d.b_mb >= 0) && !(MODE == 1 && lo == 0 && lvl == 0 && s.pre != PRE_EMBED);
-  const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
-  if (MODE == 0) { r.M = t.T; r.N = L.n_out; r.K = L.n_in; }
-  else if (MODE == 1) { r.M = t.T; r.N = L.n_in; r.K = L.n_out; }
-  else { r.M = L.n_out; r.N = L.n_in; r.K = t.T; }
-  const int tiles_n = (r.N + P2_TILE - 1) / P2_TILE;
-  const int local = tile - (t.sel_p >= 0 ? t.sel_tile0 : tile_start[lo]);
-  r.m0 = (local / tiles_n) * P2_TILE;
-  r.n0 = (local % tiles_n) * P2_TILE;
-  r.n_kb = (r.K + TILE_K - 1) / TILE_K;
-  return r;
-}
-
-template <int MODE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P2_THREADS, 1)
+template <int MODE, bool FUSE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P2Cfg<MODE, FUSE>::kThreads, 1)
 umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ tile_start, const int* __restrict__ order, int n_slots, int lvl, int* status) {
-  constexpr int NS = P2_STAGES;
+  constexpr int NS = P2_STAGES, SUM = P2Cfg<MODE, FUSE>::kSumWarps, UNITS = P2Cfg<MODE, FUSE>::kUnits;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;                      // same offset in both CTAs of the pair
@@ -593,9 +675,9 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
   const uint32_t outs = tiles + NS * STAGE_BYTES;
   uint8_t* outs_ptr = tiles_ptr + NS * STAGE_BYTES;
   const uint32_t bars = tiles + P2_TILE_BYTES;
-  // barrier block: full[NS] (used in the leader) empty[NS] tfull[2] tempty[2] (leader), tmem base word, abort flag
-  const uint32_t bar_full = bars, bar_empty = bar_full + 8 * NS, bar_tfull = bar_empty + 8 * NS, bar_tempty = bar_tfull + 16;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tiles_ptr + P2_TILE_BYTES + 8 * (2 * NS + 4));
+  // barrier block: full[NS] (used in the leader) empty[NS] done[NS] tfull[2] tempty[2] (leader) skip[one per epilogue warp], tmem base word, abort flag
+  const uint32_t bar_full = bars, bar_empty = bar_full + 8 * NS, bar_done = bar_empty + 8 * NS, bar_tfull = bar_done + 8 * NS, bar_tempty = bar_tfull + 16, bar_skip = bar_tempty + 16;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tiles_ptr + P2_TILE_BYTES + 8 * (3 * NS + 4 + 16));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -603,8 +685,9 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NS; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull + 8 * i, 1); mbar_init(bar_tempty + 8 * i, 2 * N_EPI_WARPS); }
+    for (int i = 0; i < NS; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); mbar_init(bar_done + 8 * i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull + 8 * i, 1); mbar_init(bar_tempty + 8 * i, 2 * P2Cfg<MODE, FUSE>::kEpiWarps); }
+    for (int i = 0; i < P2Cfg<MODE, FUSE>::kEpiWarps; ++i) mbar_init(bar_skip + 8 * i, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -613,6 +696,8 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
     tmem_alloc_pair(smem_u32(tmem_slot), 2 * P2_ACC_COLS);
     tmem_relinquish_pair();
   }
+  auto decode = [&](int slot) { return decode_tile<MODE, P2_TILE>(t, tile_start, order, n_slots, lvl, slot); };
+  const Tile mine = decode(pair + lane * n_pairs);                    // tables no launch of the phase writes
   tc_fence_before();
   cluster_sync_all();                                                 // barriers of both CTAs are initialised
   tc_fence_after();
@@ -622,148 +707,122 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
-      Ring op{0, 0};
-      int issued_op = 0;
-      bool ok = true;
-      for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const Tile tl = decode_pair_tile<MODE>(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        const StageDyn& d = t.dyn[tl.p];
-        const StageDev& sd_ = t.st[tl.p];
-        const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-        const int dz_slot = (bwd_act(sd_.lin[lvl]) == PM_ACT_NONE && lvl == sd_.n_lin - 1 && !feeds_attention(sd_.post)) ? dz_mailbox_slot(t, sd_, d) : 0;
-        if (MODE == 0) { tma_prefetch_desc(lm + MAP_ACT_K); tma_prefetch_desc(lm + MAP_W_K); }
-        else if (MODE == 1) { tma_prefetch_desc(lm + MAP_DZ_K); tma_prefetch_desc(lm + MAP_W_MN); }
-        else { tma_prefetch_desc(lm + MAP_DZ_MN); tma_prefetch_desc(lm + MAP_ACT_MN); }
-        const int ma = tl.m0 + rank * TILE_M, nbh = tl.n0 + rank * TILE_N;   // this CTA's rows of A and of B
-        // ring slots of the operands: read here, once per tile (the k-block loop is the critical path of the kernel and
-        // every wait in it makes the compiler re-read what lives in memory)
-        const int aslot = (lvl == 0 && sd_.pre == PRE_NONE) ? d.f_xslot : d.f_slot;
-        const int xslot = (lvl == 0 && sd_.pre == PRE_NONE) ? d.b_xslot : d.b_slot;
-        const int vslot = d.f_vslot;                                  // weight version the forward reads
-        const int n_kb = tl.n_kb;
-        for (int kb = 0; kb < n_kb; ++kb) {
-          const int k0 = kb * TILE_K;
-          if (!mbar_wait(bar_empty + 8 * op.idx, op.phase ^ 1, abort_flag, status, 31)) { ok = false; break; }
-          const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+    Ring op{0, 0};
+    int issued_op = 0;
+    const uint32_t leader_full = mapa_shared(bar_full, 0);
+    walk_tiles(mine, pair, n_pairs, n_slots, lane, decode, [&](const Tile& tl) {
+      const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
+      const int ma = tl.m0 + rank * TILE_M, nbh = tl.n0 + rank * TILE_N;   // this CTA's rows of A and of B
+      for (int kb = 0; kb < tl.n_kb; ++kb) {
+        const int k0 = kb * TILE_K;
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * op.idx, op.phase ^ 1, abort_flag, status, 31))) return false;
+        const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+        const uint32_t fb = leader_full + 8 * op.idx;
+        if (elect_one()) {
           if (rank == 0) mbar_arrive_expect_tx(bar_full + 8 * op.idx, 2 * (A_BYTES + B_BYTES));   // the bytes of both CTAs
-          const uint32_t fb = mapa_shared(bar_full + 8 * op.idx, 0);
           if (MODE == 0) {
-            tma_load_3d_pair(sa, lm + MAP_ACT_K, fb, k0, ma, aslot);
-            tma_load_3d_pair(sb, lm + MAP_W_K, fb, k0, nbh, vslot);
+            tma_load_3d_pair(sa, lm + MAP_ACT_K, fb, k0, ma, tl.sa);
+            tma_load_3d_pair(sb, lm + MAP_W_K, fb, k0, nbh, tl.sb);
           } else if (MODE == 1) {
-            tma_load_3d_pair(sa, lm + MAP_DZ_K, fb, k0, ma, dz_slot);
-            tma_load_3d_pair(sb, lm + MAP_W_MN, fb, nbh, k0, vslot);
-            tma_load_3d_pair(sb + B_BYTES / 2, lm + MAP_W_MN, fb, nbh + 64, k0, vslot);
+            tma_load_3d_pair(sa, lm + MAP_DZ_K, fb, k0, ma, tl.sa);
+            tma_load_3d_pair(sb, lm + MAP_W_MN, fb, nbh, k0, tl.sb);
+            tma_load_3d_pair(sb + B_BYTES / 2, lm + MAP_W_MN, fb, nbh + 64, k0, tl.sb);
           } else {
-            tma_load_3d_pair(sa, lm + MAP_DZ_MN, fb, ma, k0, dz_slot);
-            tma_load_3d_pair(sa + A_BYTES / 2, lm + MAP_DZ_MN, fb, ma + 64, k0, dz_slot);
-            tma_load_3d_pair(sb, lm + MAP_ACT_MN, fb, nbh, k0, xslot);
-            tma_load_3d_pair(sb + B_BYTES / 2, lm + MAP_ACT_MN, fb, nbh + 64, k0, xslot);
-          }
-          op.advance(NS); ++issued_op;
-        }
-      }
-      if (*abort_flag) {
-        // copies already issued still land in this CTA's shared memory: give them time (bounded) before leaving
-        if (rank == 0) {
-          for (int back = 1; back <= NS && back <= issued_op; ++back) {
-            const int it = issued_op - back;
-            const long long t0 = clock64();
-            while (!mbar_try_wait(bar_full + 8 * (it % NS), (uint32_t)(it / NS) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+            tma_load_3d_pair(sa, lm + MAP_DZ_MN, fb, ma, k0, tl.sa);
+            tma_load_3d_pair(sa + A_BYTES / 2, lm + MAP_DZ_MN, fb, ma + 64, k0, tl.sa);
+            tma_load_3d_pair(sb, lm + MAP_ACT_MN, fb, nbh, k0, tl.sb);
+            tma_load_3d_pair(sb + B_BYTES / 2, lm + MAP_ACT_MN, fb, nbh + 64, k0, tl.sb);
           }
         }
-        // rank 1's copies are counted on the same barriers of the leader (the expected bytes are those of both CTAs), and
-        // no CTA of the pair leaves before the cluster barrier at the end of the kernel, which the leader reaches only
-        // after these waits: rank 1 needs no wait of its own
+        __syncwarp();
+        op.advance(NS); ++issued_op;
       }
-    }
+      return true;
+    });
+    // Copies already issued still land here: give them time (bounded) before leaving.  Rank 1's copies are counted on the same
+    // barriers of the leader (the expected bytes are those of both CTAs), and no CTA of the pair leaves before the cluster
+    // barrier at the end of the kernel, which the leader reaches only after these waits: rank 1 needs no wait of its own.
+    if (lane == 0 && *abort_flag && rank == 0)
+      for (int back = 1; back <= NS && back <= issued_op; ++back) {
+        const int it = issued_op - back;
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_full + 8 * (it % NS), (uint32_t)(it / NS) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+      }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc = make_idesc_mn(P2_TILE, P2_TILE, MODE == 2, MODE != 0);
-      const uint64_t dba = MODE == 2 ? desc_base(A_BYTES / 2, 1024) : desc_base(16, 1024);
-      const uint64_t dbb = MODE == 0 ? desc_base(16, 1024) : desc_base(B_BYTES / 2, 1024);
-      const uint32_t ka = MODE == 2 ? 2048 : 32, kb_ = MODE == 0 ? 32 : 2048;
-      Ring op{0, 0}, acc{0, 0};
-      bool ok = true;
-      for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const Tile tl = decode_pair_tile<MODE>(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        if (!mbar_wait(bar_tempty + 8 * acc.idx, acc.phase ^ 1, abort_flag, status, 36)) { ok = false; break; }
+    const uint32_t idesc = make_idesc_mn(P2_TILE, P2_TILE, MODE == 2, MODE != 0);
+    const uint64_t dba = MODE == 2 ? desc_base(A_BYTES / 2, 1024) : desc_base(16, 1024);
+    const uint64_t dbb = MODE == 0 ? desc_base(16, 1024) : desc_base(B_BYTES / 2, 1024);
+    const uint32_t ka = MODE == 2 ? 2048 : 32, kb_ = MODE == 0 ? 32 : 2048;
+    Ring op{0, 0}, acc{0, 0};
+    if (rank == 0) walk_tiles(mine, pair, n_pairs, n_slots, lane, decode, [&](const Tile& tl) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_tempty + 8 * acc.idx, acc.phase ^ 1, abort_flag, status, 36))) return false;
+      tc_fence_after();
+      const uint32_t tmem_acc = tmem_base + (uint32_t)(acc.idx * P2_ACC_COLS);
+      // a slot is free in both CTAs once these MMAs have read it (first column of a weight gradient: by way of the summing warps)
+      const uint32_t release = SUM && tl.n0 == 0 ? bar_done : bar_empty;
+      for (int kb = 0; kb < tl.n_kb; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * op.idx, op.phase, abort_flag, status, 32))) return false;
         tc_fence_after();
-        const uint32_t tmem_acc = tmem_base + (uint32_t)(acc.idx * P2_ACC_COLS);
-        for (int kb = 0; kb < tl.n_kb; ++kb) {
-          if (!mbar_wait(bar_full + 8 * op.idx, op.phase, abort_flag, status, 32)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+        const uint32_t sa = tiles + op.idx * STAGE_BYTES, sb = sa + A_BYTES;
+        if (elect_one()) {
 #pragma unroll
           for (int k16 = 0; k16 < TILE_K / 16; ++k16)
             tc_mma_bf16_pair(tmem_acc, desc_at(dba, sa + k16 * ka), desc_at(dbb, sb + k16 * kb_), idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-          tc_commit_pair(bar_empty + 8 * op.idx, 3);                  // frees the operand slot in both CTAs
-          op.advance(NS);
+          tc_commit_pair(release + 8 * op.idx, 3);
+          if (kb == tl.n_kb - 1) tc_commit_pair(bar_tfull + 8 * acc.idx, 3);   // accumulator complete, both CTAs
         }
-        if (ok) tc_commit_pair(bar_tfull + 8 * acc.idx, 3);           // accumulator complete, both CTAs
-        acc.advance(2);
+        __syncwarp();
+        op.advance(NS);
       }
-    }
-  } else {
-    // ---------------- epilogue: 8 warps per CTA, warp%4 = TMEM lane group, two warps per group split the 256 columns ----------------
-    const int q = warp & 3;
-    const int ew = warp - 2;                                          // 0..7
-    const int half = ew >> 2;                                         // 0: columns 0..127, 1: columns 128..255
-    uint8_t* obuf = outs_ptr + ew * 8192;
-    const uint32_t obuf_s = outs + ew * 8192;
-    Ring acc{0, 0};
+      acc.advance(2);
+      return true;
+    });
+  } else if (warp < 2 + SUM) {
+    // ---------------- bias gradient: column sums of this CTA's rows of the A tile ----------------
+    int idx = 0;
+    uint32_t phases = 0;
     bool ok = true;
-    EpiState es;
-    for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const Tile tl = decode_pair_tile<MODE>(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
+    walk_tiles(mine, pair, n_pairs, n_slots, lane, decode, [&](const Tile& tl) {
+      colsum_tile<NS>(t, lvl, tl, rank * TILE_M, warp - 2, lane, idx, phases, ok, tiles_ptr, bar_done, bar_empty, abort_flag, status);
+      return true;
+    });
+  } else {
+    // ---------------- epilogue: 16 warps per CTA (fused update: 8), warp%4 = TMEM lane group, the warps of a group split the 256 columns ----------------
+    const int q = warp & 3;
+    const int ew = warp - 2 - SUM;
+    const int part = (ew >> 2) * UNITS;                               // first of this warp's blocks of 64 columns
+    const uint32_t leader_tempty = mapa_shared(bar_tempty, 0);
+    EpiStage<1> es{outs_ptr + ew * 4096, outs + ew * 4096, lane, bar_skip + 8 * ew};
+    Ring acc{0, 0};
+    walk_tiles(mine, pair, n_pairs, n_slots, lane, decode, [&](const Tile& tl) {
       const StageDyn& d = t.dyn[tl.p];
       const StageDev& s = t.st[tl.p];
       const LinDev& L = s.lin[lvl];
       const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-      const int mrow = tl.m0 + rank * TILE_M + q * 32;                // first row of this warp's blocks
-      // bias of this warp's 128 columns, four per lane, on its way while the accumulator completes
-      const float4 bias4 = MODE == 0 ? load_bias4(fwd_small<__nv_bfloat16>(t, s, d, L.b_off, L.b_soff), tl.n0 + half * 128 + 4 * lane, tl.N) : make_float4(0.f, 0.f, 0.f, 0.f);
-      uint4 skq[8];                                                   // skip values of the 64-column block in hand (residual stages)
-      if (MODE == 0) load_skip64(t, s, d, tl.N, mrow + lane, tl.n0 + half * 128, skq);
-      // ring slot of the forward output, formed while the accumulator completes (the elected lane needs it for its stores)
-      const int yslot_pre = MODE != 0 ? -1 : (lvl < s.n_lin - 1 ? d.f_slot
-                            : (s.emit_memory ? (int)(d.f_mb % t.mem_depth) : (tl.p < t.P - 1 ? d.f_next_xslot : (int)(d.tick & 1))));
-      bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 34);
-      ready = __all_sync(0xffffffffu, ready);                         // tcgen05.ld needs the whole warp
-      if (!ready) { ok = false; break; }
+      const int M = MODE == 2 ? L.n_out : t.T, N = MODE == 0 ? L.n_out : L.n_in;
+      const int mrow = tl.m0 + rank * TILE_M + q * 32, nb = tl.n0 + part * 64;   // this warp's (first) block
+      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl);
+      const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
+      const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
+      if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
+      const bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 34);
+      bool go = __all_sync(0xffffffffu, ready);                       // tcgen05.ld needs the whole warp
+      if (fetch && go) go = es.fetched(abort_flag, status);
+      if (!go) { if (fetch) es.drain(); return false; }
       tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        const int nb = tl.n0 + half * 128 + c * 64;
-        uint32_t r0[32], r1[32];
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + half * 128 + c * 64);
-        tmem_ld32(taddr, r0);
-        tmem_ld32(taddr + 32, r1);
-        tmem_ld_wait();
-        if (c == 1) tc_fence_before();
-        __syncwarp();
-        if (c == 1 && lane == 0) mbar_arrive_cluster(mapa_shared(bar_tempty + 8 * acc.idx, 0));   // this warp has read its part of the accumulator
-        __syncwarp();
-        if (mrow >= tl.M || nb >= tl.N) continue;                     // nothing of this block is inside the tensor
-        // a residual stage: block 0 refills the skip registers with block 1's values as it consumes them
-        const __nv_bfloat16* nxt = nullptr;
-        if (MODE == 0 && c == 0 && s.post == POST_RESIDUAL && mrow + lane < t.T && nb + 64 < tl.N)
-          nxt = ws_at<__nv_bfloat16>(t, s.skip_in) + (uint64_t)d.skip_rslot * ((uint64_t)t.T * tl.N) + (uint64_t)(mrow + lane) * tl.N + nb + 64;
-        epi_block<MODE>(t, lm, s, d, L, tl.p, lvl, tl.N, mrow, nb, r0, r1, obuf, obuf_s, lane, bias4, c * 16, es, skq, nxt, tl.N - (nb + 64), yslot_pre);
+      for (int u = 0; u < UNITS; ++u) {                               // (MODE 0: one)
+        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias, [&] {
+          if (u != UNITS - 1) return;
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc.idx);   // this warp has read its part of the accumulator
+        });
       }
       acc.advance(2);
-    }
+      return true;
+    });
     if (lane == 0 && es.stored) tma_store_wait_all();                    // global writes complete before the CTA retires
   }
   tc_fence_before();
@@ -2013,6 +2072,10 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
           uint64_t yd[3] = {n_out, T, yslots};
           okm = okm && encode(fn, m + MAP_Y_OUT, 1, ybase, 3, yd, zs, box_bf, err);
         }
+        if (s.post == POST_RESIDUAL && l == s.n_lin - 1) {
+          uint64_t sd[3] = {n_out, T, (uint64_t)s.skip_depth};
+          okm = okm && encode(fn, m + MAP_SKIP, 1, t.ws + s.skip_in, 3, sd, zs, box_bf, err);
+        }
         if (!(p == 0 && l == 0 && s.pre != PRE_EMBED)) {
           const bool to_prev = l == 0 && s.pre == PRE_NONE;
           char* xbase = to_prev ? t.ws + st[p - 1].gin : t.ws + (l > 0 ? s.lin[l - 1].dy_off : s.dh);
@@ -2047,13 +2110,15 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   if (e == cudaSuccess) e = cudaMemsetAsync(region, 0, 256, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) { err = std::string("tensor map upload: ") + cudaGetErrorString(e); delete plan; return PM_ERR_CUDA; }
-  e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<0>::kSmemBytes);
+  e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<0, false>::kSmemBytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::kSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::kSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2, false>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2, true>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1, false>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DP_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D1_SMEM_BYTES);
   if (e == cudaSuccess) e = row_set_limits<0>();
@@ -2143,16 +2208,18 @@ cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cu
     return launch_pdl(kernel, dim3(grid), dim3(threads), smem, stream, t.pdl, ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
   };
   if (plan->pair[mode][lvl]) {
-    if (mode == 0) return go(umma_pair_gemm_kernel<0>, P2_THREADS, P2_SMEM_BYTES);
+    if (mode == 0) return go(umma_pair_gemm_kernel<0, false>, P2Cfg<0, false>::kThreads, P2_SMEM_BYTES);
     if (mode == 1) return go(umma_dgrad_pair_kernel, DP_THREADS, DP_SMEM_BYTES);
     if (mode == 3) return go(umma_dgrad_pair128_kernel, D1_THREADS, D1_SMEM_BYTES);
-    if (mode == 4) return go(umma_pair_gemm_kernel<1>, P2_THREADS, P2_SMEM_BYTES);
-    return go(umma_pair_gemm_kernel<2>, P2_THREADS, P2_SMEM_BYTES);
+    if (mode == 4) return go(umma_pair_gemm_kernel<1, false>, P2Cfg<1, false>::kThreads, P2_SMEM_BYTES);
+    if (t.fuse_upd) return go(umma_pair_gemm_kernel<2, true>, P2Cfg<2, true>::kThreads, P2_SMEM_BYTES);
+    return go(umma_pair_gemm_kernel<2, false>, P2Cfg<2, false>::kThreads, P2_SMEM_BYTES);
   }
-  if (mode == 0) return go(umma_gemm_kernel<0>, Cfg<0>::kThreads, Cfg<0>::kSmemBytes);
+  if (mode == 0) return go(umma_gemm_kernel<0, false>, Cfg<0, false>::kThreads, Cfg<0, false>::kSmemBytes);
   if (mode == 1) return go(umma_dgrad_kernel, DG_THREADS, DG_SMEM_BYTES);
-  if (mode == 4) return go(umma_gemm_kernel<1>, Cfg<1>::kThreads, Cfg<1>::kSmemBytes);
-  return go(umma_gemm_kernel<2>, Cfg<2>::kThreads, Cfg<2>::kSmemBytes);
+  if (mode == 4) return go(umma_gemm_kernel<1, false>, Cfg<1, false>::kThreads, Cfg<1, false>::kSmemBytes);
+  if (t.fuse_upd) return go(umma_gemm_kernel<2, true>, Cfg<2, true>::kThreads, Cfg<2, true>::kSmemBytes);
+  return go(umma_gemm_kernel<2, false>, Cfg<2, false>::kThreads, Cfg<2, false>::kSmemBytes);
 }
 
 }  // namespace pm
