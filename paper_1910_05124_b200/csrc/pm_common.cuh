@@ -49,6 +49,7 @@ struct LinDev {
   uint32_t _pad;
   uint64_t dz_off;            // ws: dz = dy * act'(z) [T*n_out] (a Linear whose backward applies its activation itself)
   uint64_t dy_off;            // ws: gradient w.r.t. this Linear's output [T*n_out] (a Linear inside a stage)
+  uint64_t wc_off;            // ws: bf16(w - gap*delta) [n_out*n_in], formed at the start of the backward phase (0: the dgrad forms it itself)
 };
 
 // Static description of one stage (device copy).  A stage is [pre-op] Linear{1..4} [post-op]:

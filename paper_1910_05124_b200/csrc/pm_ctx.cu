@@ -480,7 +480,14 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   L.off_lnred = w; w = align_up(w + (uint64_t)L.n_ln * L.ln_chunks * 2 * L.max_ln_dim * 4, 256);
   L.off_tgt = w; w = align_up(w + (uint64_t)(P + 1) * T * (ce ? 4 : (uint64_t)L.n_out_last * 4), 256);
   L.off_yout = w; w = align_up(w + 2 * T * L.n_out_last * (ce ? 4 : esz), 256);
-  L.off_umma = w; w = align_up(w + (cfg->compute_dtype == PM_BF16 ? umma_workspace_bytes((int)T, L.st, 0) : 0), 256);
+  if (cfg->compute_dtype == PM_BF16 && !L.stash && !L.materialize)
+    for (int p = 0; p < P; ++p)
+      for (int l = 0; l < L.st[p].n_lin; ++l)
+        if (umma_corr_weights((int)T, L.st, p, l, mb || E > 1, !mb)) {
+          LinDev& ld = L.st[p].lin[l];
+          ld.wc_off = w; w = align_up(w + (uint64_t)ld.n_in * ld.n_out * 2, 256);
+        }
+  L.off_umma = w; w = align_up(w + (cfg->compute_dtype == PM_BF16 ? umma_workspace_bytes((int)T, L.st) : 0), 256);
   L.off_attn = w; w = align_up(w + (L.att_tc ? attn_workspace_bytes(P) : 0), 256);
   L.off_gmem = w; w = align_up(w + (uint64_t)L.gmem_depth * T * L.mem_dim * esz, 256);
   for (int p = 0; p < P; ++p) {
@@ -709,7 +716,6 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0; t.pdl = 0;
   t.res_fused = cfg->compute_dtype == PM_BF16 ? 1 : 0;
   t.ln_li0 = 0; t.defer_finish = 0; t.ln_stage = 0;
-  t.dgrad_split_below = 0;
   t.loss_scale = 1.0f / (float)(cfg->n_micro > 1 ? cfg->n_micro : 1);
   t.stash = (L.stash || L.materialize) ? 1 : 0;     // the backward pass reads its table entry's version slot
   t.fuse_upd = 0; t.upd_opt = cfg->optimizer; t.upd_beta1 = cfg->beta1; t.upd_beta2 = cfg->beta2; t.upd_eps = cfg->eps;
@@ -940,6 +946,12 @@ static bool need_actbwd(const pm_ctx* ctx, int l, int p) {
   return p >= 0 ? bwd_act(ctx->L.st[p].lin[l]) != PM_ACT_NONE : (ctx->L.act_levels >> l & 1) != 0;
 }
 
+// The corrected weights of the stages that dgrad launches read them for (ta.sel_p >= 0: that stage's).
+static pm_status corr_weights(pm_ctx* ctx, const TickArgs& ta) {
+  if (!ctx->umma || umma_corr_blocks(ctx->umma, ta.sel_p) == 0) return PM_OK;
+  return TIMED(PM_PROF_DGRAD, check(ctx, umma_corr_launch(ctx->umma, next(ctx, ta), ctx->ls), "corrected weights"));
+}
+
 // The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradients and the finishing passes
 // are left to grouped launches over all stages (ta.defer_finish set).
 static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool grouped) {
@@ -947,6 +959,7 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
   const int P = ctx->cfg.n_stages;
   const StageDev& sd = ctx->L.st[p];
   pm_status s;
+  if (!grouped && (s = corr_weights(ctx, ta)) != PM_OK) return s;
   if (p == P - 1 && (s = TIMED(PM_PROF_LOSS, check(ctx, launch_loss(next(ctx, ta), dt, ctx->ls), "loss"))) != PM_OK) return s;
   if (feeds_attention(sd.post)) {
     if (ctx->attn) { if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ta), false, ctx->ls), "attention backward"))) != PM_OK) return s; }
@@ -964,7 +977,7 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     }
     if (p == 0 && l == 0 && sd.pre != PRE_EMBED) continue;          // raw network inputs need no gradient
     prof_begin(ctx, PM_PROF_DGRAD);
-    e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 1, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), (ctx->L.stash || ctx->L.materialize) ? 4 : 1, l, ctx->ls);
+    e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ta), ctx->L.st, 1, l, ctx->ls) : umma_launch(ctx->umma, next(ctx, ta), 1, l, ctx->ls);
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;
@@ -1024,6 +1037,7 @@ static pm_status mb_backward(pm_ctx* ctx) {
   const int n_seg = S > 0 ? (P + S - 1) / S : 1;
   pm_status s = run_phase(ctx, ctx->g_bwd, [&]() -> pm_status {
     pm_status s;
+    if ((s = corr_weights(ctx, mb_args(ctx, 2 * P, -1))) != PM_OK) return s;
     for (int k = n_seg - 1; k >= 0; --k) {
       const int lo = S > 0 ? k * S : 0, hi = S > 0 ? std::min(P, lo + S) : P;
       if (S > 0 && k < n_seg - 1)
@@ -1232,6 +1246,7 @@ pm_status pm_backward(pm_ctx* ctx) {
   } else if (any) {
     s = run_phase(ctx, ctx->g_bwd, [&]() -> pm_status {
       pm_status s;
+      if ((s = corr_weights(ctx, ctx->ta)) != PM_OK) return s;
       if ((s = TIMED(PM_PROF_LOSS, check(ctx, launch_loss(next(ctx, ctx->ta), dt, ctx->ls), "loss"))) != PM_OK) return s;
       if (ctx->attn) { if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ctx->ta), false, ctx->ls), "attention backward"))) != PM_OK) return s; }
       else if (ctx->L.att_blocks > 0 && (s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(next(ctx, ctx->ta), dt, ctx->ls), "attention backward"))) != PM_OK) return s;

@@ -9,14 +9,13 @@
 //
 //   mode 0 forward  D[T,out]  = x[T,in] * W[out,in]^T      A K-major (TMA), B K-major (TMA, bf16 shadow)
 //                   z = bf16(D + b) -> ring,  y = bf16(act(z)) -> next consumer
-//   mode 1 dgrad    D[T,in]   = dz[T,out] * Wc[out,in]     A K-major (TMA); the fp32 master weights and the
-//                   T2 accumulator delta arrive by TMA in a staging ring, four transform warps turn them
-//                   into the MN-major bf16 operand bf16(w - gap*delta) (Section 3.2): the corrected
-//                   weights exist only in shared memory
+//   mode 1 dgrad    D[T,in]   = dz[T,out] * Wc[out,in]     A K-major (TMA), B MN-major (TMA): a queued version of the weights, or
+//                   the T2-corrected weights bf16(w - gap*delta) (Section 3.2).  Where a launch has fewer than 256 rows or columns,
+//                   umma_dgrad_kernel forms those itself from the fp32 master weights and the accumulator delta
 //   mode 2 wgrad    D[out,in] = dz[T,out]^T * x[T,in]      A MN-major (TMA), B MN-major (TMA), fp32 out
 //
-// Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer + TMEM owner, (mode 1: warps 2..5 = operand
-// transform,) last eight warps = epilogue (two per TMEM lane group, each taking 64 of the 128 columns).
+// Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer + TMEM owner, (mode 2: warps 2..5 = column sums,) last eight warps =
+// epilogue (two per TMEM lane group, each taking 64 of the 128 columns).
 // Every wait on an mbarrier is bounded; on expiry the CTA records a code in a status word, stops
 // issuing work, waits (bounded) for its copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
@@ -53,7 +52,7 @@ template <int MODE, bool FUSE> struct Cfg {
 };
 
 enum { MAP_ACT_K = 0, MAP_W_K = 1, MAP_DZ_K = 2, MAP_DZ_MN = 3, MAP_ACT_MN = 4, MAP_W_F32 = 5, MAP_D_F32 = 6,
-       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_F32Q = 11, MAP_D_F32Q = 12, MAP_W_F32H = 13, MAP_D_F32H = 14, MAP_W_MN = 15, MAP_W_K32 = 16, MAP_SKIP = 17, MAPS_PER_LINEAR = 18 };
+       MAP_Z_OUT = 7, MAP_Y_OUT = 8, MAP_DX_OUT = 9, MAP_DW_OUT = 10, MAP_W_MN = 11, MAP_W_K32 = 12, MAP_SKIP = 13, MAPS_PER_LINEAR = 14 };
 }  // namespace pm
 #include "pm_umma_row.cuh"     // the kernel of launches with few tiles; uses the tensor maps above
 namespace pm {
@@ -381,7 +380,8 @@ __device__ __forceinline__ Tile decode_tile(const TickArgs& t, const int* __rest
   // attention is the rotating mailbox slot written during the previous tick
   if (MODE != 0) r.sa = (bwd_act(L) == PM_ACT_NONE && lvl == s.n_lin - 1 && !feeds_attention(s.post)) ? dz_mailbox_slot(t, s, d) : 0;
   else r.sa = own_input ? d.f_xslot : d.f_slot;
-  r.sb = MODE == 2 ? (own_input ? d.b_xslot : d.b_slot) : d.f_vslot;   // wgrad: the input's slot; else the weight version
+  // wgrad: the input's slot; else the weight version, or the corrected weights
+  r.sb = MODE == 2 ? (own_input ? d.b_xslot : d.b_slot) : (MODE == 1 && L.wc_off ? 0 : d.f_vslot);
   return r;
 }
 
@@ -1122,715 +1122,48 @@ umma_dgrad_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* _
   }
 }
 
-// ---- dgrad on CTA pairs ------------------------------------------------------------------------------------
-// The same product and the same on-the-fly correction on tiles of 256 rows x 256 columns per CTA pair
-// (tcgen05.mma.cta_group::2, M = 256, N = 256: the width at which the tensor pipe runs at its full rate; an MMA
-// costs at least ~84 cycles whatever its width, so 128-column tiles cap it at 77 %).  Each CTA stages the fp32 w
-// and delta of ITS 128 columns in slabs of 32 k-rows (2 x 16 KB per slab, three slabs in flight), converts them to
-// bf16(w - gap*delta) in its own shared memory, and loads its 128 rows of dz.  Up to two 256-row tiles share one
-// converted tile (then the two 256-column accumulators fill the tensor memory and the epilogue drains the first
-// while the MMAs of the second finish; the next group's MMAs start on an accumulator as soon as it is drained);
-// a Linear with few tiles takes one row tile per group and alternates between the two accumulators.
-// Barriers: staging (sfull / sempty) is local to a CTA; the converted tile (bfull) and the dz tiles (afull) are
-// counted in the leader, which issues the MMAs; tcgen05.commit releases slots (bempty, aempty) and publishes
-// accumulators (tfull) in both CTAs; the epilogue warps of both arrive on the leader's tempty.
-constexpr int DP_TILE_M = 256, DP_TILE_N = 256, DP_HALF_N = 128;
-constexpr int DP_MG = 2;                                   // 256-row tiles per converted tile (at most)
-constexpr int DP_SLAB_K = 32;                              // k-rows per fp32 staging slab
-constexpr int DP_NG = 3, DP_NB = 2, DP_NA = 4;             // fp32 slab ring, converted ring, dz ring (two k-blocks of dz in flight)
-constexpr int DP_STG_HALF = DP_SLAB_K * DP_HALF_N * 4;     // one fp32 [32 x 128] slab: 16 KB
-constexpr int DP_STG_BYTES = 2 * DP_STG_HALF;              // w slab + delta slab
-constexpr int DP_B_BYTES = TILE_K * DP_HALF_N * 2;         // converted [64 k x 128 n] bf16: 16 KB (two 64-column runs of 8 KB)
-constexpr int DP_ACC_COLS = DP_TILE_N;                     // 256 columns per accumulator; two fill the tensor memory
-constexpr int DP_XF_WARPS = 8, DP_EPI_WARPS = 8;
-constexpr int DP_THREADS = 32 * (3 + DP_XF_WARPS + DP_EPI_WARPS);   // staging producer, MMA issuer, transform, epilogue, dz producer
-constexpr int DP_TILE_BYTES = DP_NG * DP_STG_BYTES + DP_NB * DP_B_BYTES + DP_NA * A_BYTES + DP_EPI_WARPS * 4096;
-constexpr int DP_SMEM_BYTES = DP_TILE_BYTES + 1024 + 512;
-static_assert(DP_SMEM_BYTES <= 227 * 1024, "pair dgrad kernel: shared memory");
+// ---- the corrected weights as an operand ------------------------------------------------------------------
+// Launches of many rows (CTA pairs) read the T2-corrected weights bf16(w - gap*delta) from a scratch copy that this kernel forms at
+// the start of the backward phase, so that their dgrad is the plain GEMM above.  Forming them inside the GEMM costs every group of
+// row tiles the fp32 stream (8 B per weight through L2 and shared memory) and the conversion again, and their staging left room
+// for 1.5 k-blocks of latency: an update of the encoder-decoder of 4 + 4 layers of width 1024 spent 1700 us in such a dgrad, and spends
+// 222 here (6.9 TB/s) and 1005 in the plain one; a tick of the 6-layer encoder 215, and 35 + 142.  With fewer rows the stream is read
+// once either way and umma_dgrad_kernel stays.
+// One block per entry of the list: up to 8192 consecutive weights of one Linear.  Bound by HBM (10 B per weight).
+struct CorrBlock { uint32_t src64, dst64, n64; int32_t stage; };      // in groups of 64 elements; dst64 from the workspace's start
+constexpr int CORR_THREADS = 256, CORR_GROUPS = 4;                    // groups of eight elements per thread
+constexpr uint32_t CORR_N64 = CORR_THREADS * CORR_GROUPS * 8 / 64;
 
-// Row tiles per group for a Linear with these dimensions: two, unless that leaves fewer than `split_below` groups
-// (a launch that covers one stage only must still bring a tile group for most CTA pairs).
-__host__ __device__ inline int dgrad_pair_mg(int T, int n_in, int split_below) {
-  const int tiles_n = (n_in + DP_TILE_N - 1) / DP_TILE_N, tiles_m = (T + DP_TILE_M - 1) / DP_TILE_M;
-  return (((tiles_m + DP_MG - 1) / DP_MG) * tiles_n < split_below) ? 1 : DP_MG;
-}
-
-__device__ __forceinline__ DgTile decode_dgrad_pair(const TickArgs& t, const int* __restrict__ tile_start, int lvl, int tile) {
-  DgTile r;
-  const int lo = t.sel_p >= 0 ? t.sel_p : tile_start[t.P + 1 + tile];                           // the stage of this tile: table behind the P + 1 starts
-  r.p = lo;
-  const StageDyn& d = t.dyn[lo];
-  const StageDev& s = t.st[lo];
-  r.valid = lvl < s.n_lin && d.b_mb >= 0 && !(lo == 0 && lvl == 0 && s.pre != PRE_EMBED);
-  const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
-  r.M = t.T; r.N = L.n_in; r.K = L.n_out;
-  const int mgr = dgrad_pair_mg(r.M, r.N, t.dgrad_split_below);
-  const int tiles_n = (r.N + DP_TILE_N - 1) / DP_TILE_N;
-  const int tiles_m = (r.M + DP_TILE_M - 1) / DP_TILE_M;
-  const int local = tile - (t.sel_p >= 0 ? t.sel_tile0 : tile_start[lo]);
-  const int mg = local / tiles_n;
-  r.m0 = mg * mgr * DP_TILE_M;
-  r.n0 = (local % tiles_n) * DP_TILE_N;
-  r.n_m = min(mgr, tiles_m - mg * mgr);
-  r.n_kb = (r.K + TILE_K - 1) / TILE_K;
-  return r;
-}
-
-// Which accumulator (0 | 1: tensor-memory columns 0..255 | 256..511) a row tile of a group uses, and how often each
-// has been used so far (the barrier phases follow from the counts).  The MMA issuer and the epilogue warps walk the
-// same tile sequence and keep identical copies.
-struct DpAcc {
-  uint32_t uses[2];
-  int next1;                                                         // accumulator of the next single-row-tile group
-  __device__ __forceinline__ int buf(int mi, int n_m) const { return n_m == 2 ? mi : next1; }
-  __device__ __forceinline__ void done_group(int n_m) { if (n_m == 2) { ++uses[0]; ++uses[1]; } else { ++uses[next1]; next1 ^= 1; } }
-};
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(DP_THREADS, 1)
-umma_dgrad_pair_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ tile_start, const int* __restrict__ order, int n_slots, int lvl, int* status) {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* base_ptr = smem_raw + (base - raw);
-  const uint32_t stg = base;                                          // [DP_NG][w 16 KB | delta 16 KB] fp32 slabs of 32 k-rows x 128 columns
-  const uint32_t sB = stg + DP_NG * DP_STG_BYTES;                     // [DP_NB][16 KB] converted operand (this CTA's 128 columns, 64 k-rows)
-  const uint32_t sA = sB + DP_NB * DP_B_BYTES;                        // [DP_NA][16 KB] dz tiles (this CTA's 128 rows, 64 k-columns)
-  const uint32_t sO = sA + DP_NA * A_BYTES;                           // [8][4 KB] epilogue staging
-  uint8_t* stg_ptr = base_ptr;
-  uint8_t* sB_ptr = base_ptr + DP_NG * DP_STG_BYTES;
-  uint8_t* sO_ptr = sB_ptr + DP_NB * DP_B_BYTES + DP_NA * A_BYTES;
-  const uint32_t bars = base + DP_TILE_BYTES;
-  const uint32_t bar_sfull = bars, bar_sempty = bar_sfull + 8 * DP_NG, bar_bfull = bar_sempty + 8 * DP_NG,
-                 bar_bempty = bar_bfull + 8 * DP_NB, bar_afull = bar_bempty + 8 * DP_NB, bar_aempty = bar_afull + 8 * DP_NA,
-                 bar_tfull = bar_aempty + 8 * DP_NA, bar_tempty = bar_tfull + 16;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + DP_TILE_BYTES + 8 * (2 * DP_NG + 2 * DP_NB + 2 * DP_NA + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = (int)cluster_ctarank();                            // 0 = leader
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < DP_NG; ++i) { mbar_init(bar_sfull + 8 * i, 1); mbar_init(bar_sempty + 8 * i, DP_XF_WARPS); }
-    for (int i = 0; i < DP_NB; ++i) { mbar_init(bar_bfull + 8 * i, 2 * 2 * DP_XF_WARPS); mbar_init(bar_bempty + 8 * i, 1); }   // two slabs x two CTAs x eight warps
-    for (int i = 0; i < DP_NA; ++i) { mbar_init(bar_afull + 8 * i, 1); mbar_init(bar_aempty + 8 * i, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull + 8 * i, 1); mbar_init(bar_tempty + 8 * i, 2 * DP_EPI_WARPS); }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    __syncwarp();
-    tmem_alloc_pair(smem_u32(tmem_slot), 2 * DP_ACC_COLS);
-    tmem_relinquish_pair();
-  }
-  tc_fence_before();
-  cluster_sync_all();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
+__global__ void __launch_bounds__(CORR_THREADS) corr_weights_kernel(TickArgs t, const CorrBlock* __restrict__ list) {
+  pdl_trigger();
   pdl_wait();
-
-  // Two producer threads, each with its own cursor over the same (tile, k-block) sequence: warp 0 feeds the fp32
-  // slab ring (w, delta), the last warp the dz ring.  Everything that is fixed for a tile is read once when the
-  // cursor reaches the tile; the loops hold nothing but barrier waits and copies.
-  struct Cursor { int tile, kb; DgTile tl; bool done; const CUtensorMap* lm; bool corr; int dz_slot; };
-  auto seek = [&](Cursor& c) {
-    for (; c.tile < n_slots; c.tile += n_pairs) {
-      const int tile = tile_at(t, order, c.tile);
-      if (tile < 0) continue;
-      c.tl = decode_dgrad_pair(t, tile_start, lvl, tile);
-      if (c.tl.valid) {
-        const StageDyn& d = t.dyn[c.tl.p];
-        const StageDev& sd_ = t.st[c.tl.p];
-        c.lm = maps + ((size_t)c.tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-        c.corr = d.use_delta != 0;
-        c.dz_slot = (bwd_act(sd_.lin[lvl]) == PM_ACT_NONE && lvl == sd_.n_lin - 1 && !feeds_attention(sd_.post)) ? dz_mailbox_slot(t, sd_, d) : 0;
-        c.kb = 0; c.done = false;
-        return;
-      }
-    }
-    c.done = true;
-  };
-  auto step = [&](Cursor& c) { if (++c.kb >= c.tl.n_kb) { c.tile += n_pairs; seek(c); } };
-
-  if (warp == 0) {
-    // ---------------- TMA producer of the fp32 slab ring (both CTAs): two slabs of 32 k-rows per k-block ----------------
-    if (lane == 0) {
-      Cursor cs{pair, 0, DgTile{}, false, nullptr, false, 0};
-      seek(cs);
-      Ring sg{0, 0};
-      int issued_sg = 0;
-      bool ok = true;
-      while (!cs.done && ok) {
-        const int ncol = cs.tl.n0 + rank * DP_HALF_N;
-        for (int h = 0; h < TILE_K / DP_SLAB_K; ++h) {
-          if (!mbar_wait(bar_sempty + 8 * sg.idx, sg.phase ^ 1, abort_flag, status, 41)) { ok = false; break; }
-          const uint32_t sw = stg + sg.idx * DP_STG_BYTES, fb = bar_sfull + 8 * sg.idx;
-          mbar_arrive_expect_tx(fb, cs.corr ? DP_STG_BYTES : DP_STG_HALF);
-          tma_load_2d(sw, cs.lm + MAP_W_F32Q, fb, ncol, cs.kb * TILE_K + h * DP_SLAB_K);
-          if (cs.corr) tma_load_2d(sw + DP_STG_HALF, cs.lm + MAP_D_F32Q, fb, ncol, cs.kb * TILE_K + h * DP_SLAB_K);
-          sg.advance(DP_NG); ++issued_sg;
-        }
-        step(cs);
-      }
-      if (*abort_flag) {                                              // copies already issued still land here: wait (bounded)
-        for (int back = 1; back <= DP_NG && back <= issued_sg; ++back) {
-          const int it = issued_sg - back;
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar_sfull + 8 * (it % DP_NG), (uint32_t)(it / DP_NG) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
-      }
-    }
-  } else if (warp == 2 + DP_XF_WARPS + DP_EPI_WARPS) {
-    // ---------------- TMA producer of the dz ring (both CTAs) ----------------
-    if (lane == 0) {
-      Cursor ca{pair, 0, DgTile{}, false, nullptr, false, 0};
-      seek(ca);
-      Ring ar{0, 0};
-      int issued_a = 0;
-      bool ok = true;
-      while (!ca.done && ok) {
-        for (int mi = 0; mi < ca.tl.n_m; ++mi) {
-          if (!mbar_wait(bar_aempty + 8 * ar.idx, ar.phase ^ 1, abort_flag, status, 42)) { ok = false; break; }
-          if (rank == 0) mbar_arrive_expect_tx(bar_afull + 8 * ar.idx, 2 * A_BYTES);       // the rows of both CTAs
-          tma_load_3d_pair(sA + ar.idx * A_BYTES, ca.lm + MAP_DZ_K, mapa_shared(bar_afull + 8 * ar.idx, 0),
-                           ca.kb * TILE_K, ca.tl.m0 + mi * DP_TILE_M + rank * TILE_M, ca.dz_slot);
-          ar.advance(DP_NA); ++issued_a;
-        }
-        step(ca);
-      }
-      if (*abort_flag) {
-        if (rank == 0) {
-          for (int back = 1; back <= DP_NA && back <= issued_a; ++back) {
-            const int it = issued_a - back;
-            const long long t0 = clock64();
-            while (!mbar_try_wait(bar_afull + 8 * (it % DP_NA), (uint32_t)(it / DP_NA) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-          }
-        }
-        // rank 1's copies are counted on the same barriers of the leader (the expected bytes are those of both CTAs), and
-        // no CTA of the pair leaves before the cluster barrier at the end of the kernel, which the leader reaches only
-        // after these waits: rank 1 needs no wait of its own
-      }
-    }
+  const CorrBlock b = list[blockIdx.x];
+  const StageDyn& d = t.dyn[b.stage];
+  if (d.b_mb < 0) return;
+  const bool corr = d.use_delta != 0;
+  const float gapf = (float)t.st[b.stage].gap;
+  const float* w = t.a.w + (uint64_t)b.src64 * 64;
+  const float* dl = t.a.delta + (uint64_t)b.src64 * 64;
+  __nv_bfloat16* out = ws_at<__nv_bfloat16>(t, (uint64_t)b.dst64 * 128);
+  const uint32_t n8 = b.n64 * 8;
+  float4 w0[CORR_GROUPS], w1[CORR_GROUPS], d0[CORR_GROUPS], d1[CORR_GROUPS];
+#pragma unroll
+  for (int u = 0; u < CORR_GROUPS; ++u) {
+    const uint32_t i = min(threadIdx.x + u * CORR_THREADS, n8 - 1);     // (beyond the end: the last group again, not stored)
+    w0[u] = __ldcs(reinterpret_cast<const float4*>(w) + 2 * i); w1[u] = __ldcs(reinterpret_cast<const float4*>(w) + 2 * i + 1);
+    if (corr) { d0[u] = __ldcs(reinterpret_cast<const float4*>(dl) + 2 * i); d1[u] = __ldcs(reinterpret_cast<const float4*>(dl) + 2 * i + 1); }
   }
-  else if (warp == 1) {
-    // ---------------- MMA issuer (leader CTA only) ----------------
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc = make_idesc_mn(DP_TILE_M, DP_TILE_N, 0, 1);
-      const uint64_t dba = desc_base(16, 1024), dbb = desc_base(DP_B_BYTES / 2, 1024);   // B: two 64-column runs per CTA, 8 KB apart
-      Ring br{0, 0}, ar{0, 0};
-      DpAcc acc{{0u, 0u}, 0};
-      bool ok = true;
-      for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const DgTile tl = decode_dgrad_pair(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        const int n_m = tl.n_m, n_kb = tl.n_kb;
-        for (int kb = 0; kb < n_kb && ok; ++kb) {
-          if (!mbar_wait(bar_bfull + 8 * br.idx, br.phase, abort_flag, status, 44)) { ok = false; break; }
-          const uint32_t sb = sB + br.idx * DP_B_BYTES;
-          uint32_t sa[DP_MG], abar[DP_MG];
-          for (int mi = 0; mi < n_m; ++mi) {
-            if (!mbar_wait(bar_afull + 8 * ar.idx, ar.phase, abort_flag, status, 45)) { ok = false; break; }
-            sa[mi] = sA + ar.idx * A_BYTES;
-            abar[mi] = bar_aempty + 8 * ar.idx;
-            ar.advance(DP_NA);
-          }
-          if (!ok) break;
-          tc_fence_after();
-          // one row tile after the other: the first k-block of a group waits for each accumulator to be drained just
-          // before its first product, and the last k-block publishes the first accumulator while the products of
-          // the second are still running
-          for (int mi = 0; mi < n_m && ok; ++mi) {
-            const int b = acc.buf(mi, n_m);
-            if (kb == 0) {
-              if (!mbar_wait(bar_tempty + 8 * b, (acc.uses[b] & 1u) ^ 1u, abort_flag, status, 43)) { ok = false; break; }
-              tc_fence_after();
-            }
-            const uint32_t tmem_acc = tmem_base + (uint32_t)(b * DP_ACC_COLS);
 #pragma unroll
-            for (int k16 = 0; k16 < TILE_K / 16; ++k16)
-              tc_mma_bf16_pair(tmem_acc, desc_at(dba, sa[mi] + k16 * 32), desc_at(dbb, sb + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-            tc_commit_pair(abar[mi], 3);                              // this dz tile may be overwritten in both CTAs
-            if (kb == n_kb - 1) tc_commit_pair(bar_tfull + 8 * b, 3);  // accumulator complete, both CTAs
-          }
-          if (ok) tc_commit_pair(bar_bempty + 8 * br.idx, 3);
-          br.advance(DP_NB);
-        }
-        acc.done_group(n_m);
-      }
+  for (int u = 0; u < CORR_GROUPS; ++u) {
+    const uint32_t i = threadIdx.x + u * CORR_THREADS;
+    if (i >= n8) break;
+    float v[8] = {w0[u].x, w0[u].y, w0[u].z, w0[u].w, w1[u].x, w1[u].y, w1[u].z, w1[u].w};
+    if (corr) {
+      const float dd[8] = {d0[u].x, d0[u].y, d0[u].z, d0[u].w, d1[u].x, d1[u].y, d1[u].z, d1[u].w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = __fsub_rn(v[e], __fmul_rn(gapf, dd[e]));   // w - (tau_fwd - tau_bkwd) * delta
     }
-  } else if (warp < 2 + DP_XF_WARPS) {
-    // ---------------- operand transform (both CTAs): fp32 w, delta [32 k][128 n] -> bf16(w - gap*delta), MN-major ----------------
-    // thread: four consecutive columns (c4) of rows rbase + 8 j; reads are contiguous float4, stores 8 bytes into the swizzled atom.
-    // Two slabs (k-rows 0..31 and 32..63) fill one converted tile.
-    const int tt = threadIdx.x - 64;                                  // 0..255
-    const int c4 = tt & 31, rbase = tt >> 5;                          // 0..31 (four columns each), 0..7
-    const int run = c4 >> 4, cc = (c4 & 15);                          // 64-column run of the tile, position inside it (units of four columns)
-    const uint32_t leader_bfull = mapa_shared(bar_bfull, 0);
-    Ring br{0, 0}, sg{0, 0};
-    bool ok = true;
-    for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const DgTile tl = decode_dgrad_pair(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
-      const float gapf = (float)t.st[tl.p].gap;
-      const bool corr = t.dyn[tl.p].use_delta != 0;
-      for (int kb = 0; kb < tl.n_kb && ok; ++kb) {
-        for (int h = 0; h < TILE_K / DP_SLAB_K; ++h) {
-          bool go = mbar_wait(bar_sfull + 8 * sg.idx, sg.phase, abort_flag, status, 46);
-          if (h == 0) go = go && mbar_wait(bar_bempty + 8 * br.idx, br.phase ^ 1, abort_flag, status, 47);
-          go = __all_sync(0xffffffffu, go);
-          if (!go) { ok = false; break; }
-          const uint8_t* src = stg_ptr + sg.idx * DP_STG_BYTES;
-          uint8_t* dst = sB_ptr + br.idx * DP_B_BYTES + run * (DP_B_BYTES / 2);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int rs = rbase + 8 * j;                             // row of the slab
-            const int r = h * DP_SLAB_K + rs;                         // k-row of the tile
-            const float4 w = *reinterpret_cast<const float4*>(src + rs * (DP_HALF_N * 4) + c4 * 16);
-            float v[4] = {w.x, w.y, w.z, w.w};
-            if (corr) {
-              const float4 dl = *reinterpret_cast<const float4*>(src + DP_STG_HALF + rs * (DP_HALF_N * 4) + c4 * 16);
-              v[0] = __fsub_rn(v[0], __fmul_rn(gapf, dl.x)); v[1] = __fsub_rn(v[1], __fmul_rn(gapf, dl.y));   // w - (tau_fwd - tau_bkwd) * delta
-              v[2] = __fsub_rn(v[2], __fmul_rn(gapf, dl.z)); v[3] = __fsub_rn(v[3], __fmul_rn(gapf, dl.w));
-            }
-            const uint32_t off = (uint32_t)(r >> 3) * 1024 + (uint32_t)(r & 7) * 128 + ((((uint32_t)cc >> 1) ^ (uint32_t)(r & 7)) << 4) + ((uint32_t)cc & 1) * 8;
-            *reinterpret_cast<uint2*>(dst + off) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
-          }
-          fence_async_smem();
-          __syncwarp();
-          if (lane == 0) { mbar_arrive_cluster(leader_bfull + 8 * br.idx); mbar_arrive(bar_sempty + 8 * sg.idx); }
-          sg.advance(DP_NG);
-        }
-        br.advance(DP_NB);
-      }
-    }
-  }
-  else {
-    // ---------------- epilogue (both CTAs): 8 warps, warp%4 = TMEM lane group, two warps per group split the 256 columns ----------------
-    const int q = warp & 3;
-    const int ew = warp - 2 - DP_XF_WARPS;                            // 0..7
-    const int half = ew >> 2;                                         // 0: columns 0..127 of the tile, 1: columns 128..255
-    uint8_t* obuf = sO_ptr + ew * 4096;
-    const uint32_t obuf_s = sO + ew * 4096;
-    const uint32_t row_off = (uint32_t)lane * 128, sw = (uint32_t)(lane & 7);
-    const uint32_t leader_tempty = mapa_shared(bar_tempty, 0);
-    DpAcc acc{{0u, 0u}, 0};
-    bool ok = true, stored = false;
-    for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const DgTile tl = decode_dgrad_pair(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
-      const StageDyn& d = t.dyn[tl.p];
-      const StageDev& s = t.st[tl.p];
-      const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-      const int dslot = (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0;
-      const bool masked = lvl == 0 && s.mask_dx != 0;              // the previous stage's ReLU backward is applied here
-#pragma unroll 1
-      for (int mi = 0; mi < tl.n_m && ok; ++mi) {
-        const int b = acc.buf(mi, tl.n_m);
-        bool ready = mbar_wait(bar_tfull + 8 * b, acc.uses[b] & 1u, abort_flag, status, 48);
-        ready = __all_sync(0xffffffffu, ready);
-        if (!ready) { ok = false; break; }
-        tc_fence_after();
-        const int mrow = tl.m0 + mi * DP_TILE_M + rank * TILE_M + q * 32;
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-          const int nb = tl.n0 + half * 128 + c * 64;
-          uint32_t r0[32], r1[32];
-          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * DP_ACC_COLS + half * 128 + c * 64);
-          const uint64_t mk = masked ? load_mask_bits64(t, s, d, tl.N, mrow + lane, nb) : ~0ull;
-          tmem_ld32(taddr, r0);
-          tmem_ld32(taddr + 32, r1);
-          tmem_ld_wait();
-          if (c == 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * b);   // this warp has read its part of this accumulator
-          }
-          if (mrow >= tl.M || nb >= tl.N) continue;
-          if (lane == 0 && stored) tma_store_wait_read();
-          __syncwarp();
-#pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            float f[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(g < 4 ? r0[(g & 3) * 8 + e] : r1[(g & 3) * 8 + e]);
-            if (masked) apply_mask8(f, (uint32_t)(mk >> (8 * g)) & 0xFFu);
-            *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) =
-                make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-          }
-          fence_async_smem();
-          __syncwarp();
-          if (lane == 0) { tma_store_3d(lm + MAP_DX_OUT, obuf_s, nb, mrow, dslot); tma_store_commit(); }
-          stored = true;
-        }
-      }
-      acc.done_group(tl.n_m);
-    }
-    if (lane == 0 && stored) tma_store_wait_all();
-  }
-  tc_fence_before();
-  cluster_sync_all();                                                 // no barrier or shared memory of a CTA is touched after this
-  if (warp == 1) {
-    __syncwarp();
-    tc_fence_after();
-    tmem_dealloc_pair(tmem_base, 2 * DP_ACC_COLS);
-  }
-}
-
-// ---- dgrad on CTA pairs, 128-column tiles ----------------------------------------------------------------------
-// Used where a launch covers ONE stage whose input is narrow (microbatch-major order): with 256-column tiles such a
-// Linear has too few tile groups for the CTA pairs, and a single row tile per group doubles the fp32 traffic per
-// FLOP beyond what L2 delivers.  Here a tile is half as wide, so twice as many groups exist.
-// The same product and the same on-the-fly correction on tiles of 256 rows x 128 columns per CTA pair
-// (tcgen05.mma.cta_group::2, M = 256, N = 128).  Each CTA stages the fp32 w and delta of ITS 64 columns
-// (2 x 16 KB per k-block), converts them to bf16(w - gap*delta) in its own shared memory, and loads its 128
-// rows of dz; two 256-row tiles share one converted tile, so a CTA ingests 64 KB per 2 x (128x128x64) of its
-// own products, as the single-CTA kernel does, but the accumulators (2 x 128 columns) are double-buffered and
-// the eight epilogue warps drain one group while the next is computed.  Barriers: staging (sfull / sempty)
-// is local to a CTA; the converted tile (bfull) and the dz tiles (afull) are counted in the leader, which
-// issues the MMAs; tcgen05.commit releases slots (bempty, aempty) and publishes accumulators (tfull) in both
-// CTAs; the epilogue warps of both arrive on the leader's tempty.
-constexpr int D1_TILE_M = 256, D1_TILE_N = 128, D1_HALF_N = 64;
-constexpr int D1_MG = 2;                                   // 256-row tiles per converted tile
-constexpr int D1_PF = 4;                                   // k-blocks of fp32 w and delta asked of L2 ahead of the staging ring
-constexpr int D1_NG = 2, D1_NB = 2, D1_NA = 7;             // fp32 staging ring, converted ring, dz ring (3.5 k-blocks of dz in flight)
-constexpr int D1_STG_HALF = TILE_K * D1_HALF_N * 4;        // one fp32 [64 x 64] tile: 16 KB
-constexpr int D1_STG_BYTES = 2 * D1_STG_HALF;
-constexpr int D1_B_BYTES = TILE_K * D1_HALF_N * 2;         // converted [64 k x 64 n] bf16: 8 KB
-constexpr int D1_ACC_COLS = D1_MG * D1_TILE_N;             // 256 columns per accumulator buffer
-constexpr int D1_XF_WARPS = 8, D1_EPI_WARPS = 8;
-constexpr int D1_THREADS = 32 * (4 + D1_XF_WARPS + D1_EPI_WARPS);   // staging producer, MMA issuer, transform, epilogue, dz producer, second MMA issuer
-constexpr int D1_TILE_BYTES = D1_NG * D1_STG_BYTES + D1_NB * D1_B_BYTES + D1_NA * A_BYTES + D1_EPI_WARPS * 4096;
-constexpr int D1_SMEM_BYTES = D1_TILE_BYTES + 1024 + 512;
-
-__device__ __forceinline__ DgTile decode_dgrad_pair128(const TickArgs& t, const int* __restrict__ tile_start, int lvl, int tile) {
-  DgTile r;
-  const int lo = t.sel_p >= 0 ? t.sel_p : tile_start[t.P + 1 + tile];                           // the stage of this tile: table behind the P + 1 starts
-  r.p = lo;
-  const StageDyn& d = t.dyn[lo];
-  const StageDev& s = t.st[lo];
-  r.valid = lvl < s.n_lin && d.b_mb >= 0 && !(lo == 0 && lvl == 0 && s.pre != PRE_EMBED);
-  const LinDev& L = s.lin[lvl < s.n_lin ? lvl : 0];
-  r.M = t.T; r.N = L.n_in; r.K = L.n_out;
-  const int tiles_n = (r.N + D1_TILE_N - 1) / D1_TILE_N;
-  const int tiles_m = (r.M + D1_TILE_M - 1) / D1_TILE_M;
-  const int local = tile - (t.sel_p >= 0 ? t.sel_tile0 : tile_start[lo]);
-  const int mg = local / tiles_n;
-  r.m0 = mg * D1_MG * D1_TILE_M;
-  r.n0 = (local % tiles_n) * D1_TILE_N;
-  r.n_m = min(D1_MG, tiles_m - mg * D1_MG);
-  r.n_kb = (r.K + TILE_K - 1) / TILE_K;
-  return r;
-}
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D1_THREADS, 1)
-umma_dgrad_pair128_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ tile_start, const int* __restrict__ order, int n_slots, int lvl, int* status) {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* base_ptr = smem_raw + (base - raw);
-  const uint32_t stg = base;                                          // [D1_NG][w 16 KB | delta 16 KB]
-  const uint32_t sB = stg + D1_NG * D1_STG_BYTES;                     // [D1_NB][8 KB] converted operand (this CTA's 64 columns)
-  const uint32_t sA = sB + D1_NB * D1_B_BYTES;                        // [D1_NA][16 KB] dz tiles (this CTA's 128 rows)
-  const uint32_t sO = sA + D1_NA * A_BYTES;                           // [8][4 KB] epilogue staging
-  uint8_t* stg_ptr = base_ptr;
-  uint8_t* sB_ptr = base_ptr + D1_NG * D1_STG_BYTES;
-  uint8_t* sO_ptr = sB_ptr + D1_NB * D1_B_BYTES + D1_NA * A_BYTES;
-  const uint32_t bars = base + D1_TILE_BYTES;
-  const uint32_t bar_sfull = bars, bar_sempty = bar_sfull + 8 * D1_NG, bar_bfull = bar_sempty + 8 * D1_NG,
-                 bar_bempty = bar_bfull + 8 * D1_NB, bar_afull = bar_bempty + 8 * D1_NB, bar_aempty = bar_afull + 8 * D1_NA,
-                 bar_tfull = bar_aempty + 8 * D1_NA, bar_tempty = bar_tfull + 16;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + D1_TILE_BYTES + 8 * (2 * D1_NG + 2 * D1_NB + 2 * D1_NA + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = (int)cluster_ctarank();                            // 0 = leader
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < D1_NG; ++i) { mbar_init(bar_sfull + 8 * i, 1); mbar_init(bar_sempty + 8 * i, D1_XF_WARPS); }
-    for (int i = 0; i < D1_NB; ++i) { mbar_init(bar_bfull + 8 * i, 2 * D1_XF_WARPS); mbar_init(bar_bempty + 8 * i, D1_MG); }   // released by both MMA issuers
-    for (int i = 0; i < D1_NA; ++i) { mbar_init(bar_afull + 8 * i, 1); mbar_init(bar_aempty + 8 * i, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull + 8 * i, D1_MG); mbar_init(bar_tempty + 8 * i, 2 * D1_EPI_WARPS); }   // published by both MMA issuers
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    __syncwarp();
-    tmem_alloc_pair(smem_u32(tmem_slot), 2 * D1_ACC_COLS);
-    tmem_relinquish_pair();
-  }
-  tc_fence_before();
-  cluster_sync_all();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  pdl_trigger();                                                      // behind the tensor-memory allocation: a successor's must not come first
-  pdl_wait();
-
-  // Two producer threads, each with its own cursor over the same (tile, k-block) sequence: warp 0 feeds the fp32
-  // staging ring (w, delta), the last warp the dz ring.  Their k-block loops are the critical path of the kernel
-  // (a handful of extra loads in them cost 3 %), so everything that is fixed for a tile is read once when the
-  // cursor reaches the tile and the loops hold nothing but barrier waits and copies.
-  struct Cursor { int tile, kb; DgTile tl; bool done; const CUtensorMap* lm; bool corr; int dz_slot; };
-  auto seek = [&](Cursor& c) {
-    for (; c.tile < n_slots; c.tile += n_pairs) {
-      const int tile = tile_at(t, order, c.tile);
-      if (tile < 0) continue;
-      c.tl = decode_dgrad_pair128(t, tile_start, lvl, tile);
-      if (c.tl.valid) {
-        const StageDyn& d = t.dyn[c.tl.p];
-        const StageDev& sd_ = t.st[c.tl.p];
-        c.lm = maps + ((size_t)c.tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-        c.corr = d.use_delta != 0;
-        c.dz_slot = (bwd_act(sd_.lin[lvl]) == PM_ACT_NONE && lvl == sd_.n_lin - 1 && !feeds_attention(sd_.post)) ? dz_mailbox_slot(t, sd_, d) : 0;
-        c.kb = 0; c.done = false;
-        return;
-      }
-    }
-    c.done = true;
-  };
-  auto step = [&](Cursor& c) { if (++c.kb >= c.tl.n_kb) { c.tile += n_pairs; seek(c); } };
-
-  if (warp == 0) {
-    // ---------------- TMA producer of the fp32 staging ring (both CTAs) ----------------
-    if (lane == 0) {
-      Cursor cs{pair, 0, DgTile{}, false, nullptr, false, 0};
-      seek(cs);
-      Cursor cp = cs;                                                 // runs D1_PF k-blocks ahead and asks L2 for them
-      auto prefetch = [&]() {
-        if (cp.done) return;
-        if (cp.tl.m0 == 0) {                                          // the pairs of one row group ask for all: the others run beside them
-          tma_prefetch_2d(cp.lm + MAP_W_F32H, cp.tl.n0 + rank * D1_HALF_N, cp.kb * TILE_K);
-          if (cp.corr) tma_prefetch_2d(cp.lm + MAP_D_F32H, cp.tl.n0 + rank * D1_HALF_N, cp.kb * TILE_K);
-        }
-        step(cp);
-      };
-      for (int i = 0; i < D1_NG; ++i) step(cp);                       // the first D1_NG k-blocks are loaded at once
-      for (int i = 0; i < D1_PF; ++i) prefetch();
-      Ring sg{0, 0};
-      int issued_sg = 0;
-      while (!cs.done) {
-        prefetch();
-        if (!mbar_wait(bar_sempty + 8 * sg.idx, sg.phase ^ 1, abort_flag, status, 41)) break;
-        const uint32_t sw = stg + sg.idx * D1_STG_BYTES, fb = bar_sfull + 8 * sg.idx;
-        mbar_arrive_expect_tx(fb, cs.corr ? D1_STG_BYTES : D1_STG_HALF);
-        tma_load_2d(sw, cs.lm + MAP_W_F32H, fb, cs.tl.n0 + rank * D1_HALF_N, cs.kb * TILE_K);
-        if (cs.corr) tma_load_2d(sw + D1_STG_HALF, cs.lm + MAP_D_F32H, fb, cs.tl.n0 + rank * D1_HALF_N, cs.kb * TILE_K);
-        sg.advance(D1_NG); ++issued_sg;
-        step(cs);
-      }
-      if (*abort_flag) {                                              // copies already issued still land here: wait (bounded)
-        for (int back = 1; back <= D1_NG && back <= issued_sg; ++back) {
-          const int it = issued_sg - back;
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar_sfull + 8 * (it % D1_NG), (uint32_t)(it / D1_NG) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-        }
-      }
-    }
-  } else if (warp == 2 + D1_XF_WARPS + D1_EPI_WARPS) {
-    // ---------------- TMA producer of the dz ring (both CTAs) ----------------
-    if (lane == 0) {
-      Cursor ca{pair, 0, DgTile{}, false, nullptr, false, 0};
-      seek(ca);
-      Ring ar{0, 0};
-      int issued_a = 0;
-      bool ok = true;
-      while (!ca.done && ok) {
-        for (int mi = 0; mi < ca.tl.n_m; ++mi) {
-          if (!mbar_wait(bar_aempty + 8 * ar.idx, ar.phase ^ 1, abort_flag, status, 42)) { ok = false; break; }
-          if (rank == 0) mbar_arrive_expect_tx(bar_afull + 8 * ar.idx, 2 * A_BYTES);       // the rows of both CTAs
-          tma_load_3d_pair(sA + ar.idx * A_BYTES, ca.lm + MAP_DZ_K, mapa_shared(bar_afull + 8 * ar.idx, 0),
-                           ca.kb * TILE_K, ca.tl.m0 + mi * D1_TILE_M + rank * TILE_M, ca.dz_slot);
-          ar.advance(D1_NA); ++issued_a;
-        }
-        step(ca);
-      }
-      if (*abort_flag) {
-        if (rank == 0) {
-          for (int back = 1; back <= D1_NA && back <= issued_a; ++back) {
-            const int it = issued_a - back;
-            const long long t0 = clock64();
-            while (!mbar_try_wait(bar_afull + 8 * (it % D1_NA), (uint32_t)(it / D1_NA) & 1u) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-          }
-        }
-        // rank 1's copies are counted on the same barriers of the leader (the expected bytes are those of both CTAs), and
-        // no CTA of the pair leaves before the cluster barrier at the end of the kernel, which the leader reaches only
-        // after these waits: rank 1 needs no wait of its own
-      }
-    }
-  } else if (warp == 1 || warp == 3 + D1_XF_WARPS + D1_EPI_WARPS) {
-    // ---------------- MMA issuers (leader CTA only): one thread per row tile of a group ----------------
-    // Issuing an MMA, its commits and the barrier polls in front of them cost the issuing thread about 1400 cycles per
-    // k-block of two row tiles, of which the tensor pipe works 512: one thread cannot keep the pipe busy.  The two row tiles
-    // of a group have accumulators of their own, so their MMAs need no order between them: thread `me` waits for the
-    // shared converted tile and for ITS dz tile, issues its four MMAs and commits its dz slot; both threads commit the
-    // converted slot and the accumulator buffer (those barriers count two arrivals).
-    if (lane == 0 && rank == 0) {
-      const int me = warp == 1 ? 0 : 1;
-      const uint32_t idesc = make_idesc_mn(D1_TILE_M, D1_TILE_N, 0, 1);
-      const uint64_t dba = desc_base(16, 1024), dbb = desc_base(D1_B_BYTES, 1024);   // B: one 64-column run per CTA
-      Ring br{0, 0}, ar{0, 0}, acc{0, 0};
-      bool ok = true;
-      for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-        const int tile = tile_at(t, order, slot);
-        if (tile < 0) continue;
-        const DgTile tl = decode_dgrad_pair128(t, tile_start, lvl, tile);
-        if (!tl.valid) continue;
-        if (!mbar_wait(bar_tempty + 8 * acc.idx, acc.phase ^ 1, abort_flag, status, 43)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t tmem_acc = tmem_base + (uint32_t)(acc.idx * D1_ACC_COLS + me * D1_TILE_N);
-        const bool mine = me < tl.n_m;                               // a group at the end of the rows may hold one tile only
-        for (int kb = 0; kb < tl.n_kb && ok; ++kb) {
-          if (!mbar_wait(bar_bfull + 8 * br.idx, br.phase, abort_flag, status, 44)) { ok = false; break; }
-          const uint32_t sb = sB + br.idx * D1_B_BYTES;
-          // the dz slots of this k-block sit in ring order, row tile 0 first; this thread's is the me-th
-          Ring mr = ar;
-          if (me == 1) mr.advance(D1_NA);
-          for (int mi = 0; mi < tl.n_m; ++mi) ar.advance(D1_NA);
-          if (mine) {
-            if (!mbar_wait(bar_afull + 8 * mr.idx, mr.phase, abort_flag, status, 45)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t sa = sA + mr.idx * A_BYTES;
-#pragma unroll
-            for (int k16 = 0; k16 < TILE_K / 16; ++k16)
-              tc_mma_bf16_pair(tmem_acc, desc_at(dba, sa + k16 * 32), desc_at(dbb, sb + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-            tc_commit_pair(bar_aempty + 8 * mr.idx, 3);
-          }
-          tc_commit_pair(bar_bempty + 8 * br.idx, 3);                 // with no MMA of this thread outstanding it arrives at once
-          br.advance(D1_NB);
-        }
-        if (ok) tc_commit_pair(bar_tfull + 8 * acc.idx, 3);
-        acc.advance(2);
-      }
-    }
-  } else if (warp < 2 + D1_XF_WARPS) {
-    // ---------------- operand transform (both CTAs): fp32 w, delta [64 k][64 n] -> bf16(w - gap*delta), MN-major ----------------
-    // thread: four consecutive columns (c4) of rows r0 + 16 j; reads are contiguous float4, stores 8 bytes into the swizzled atom
-    const int tt = threadIdx.x - 64;                                  // 0..255
-    const int c4 = tt & 15, rbase = tt >> 4;                          // 0..15, 0..15
-    const uint32_t leader_bfull = mapa_shared(bar_bfull, 0);
-    Ring br{0, 0}, sg{0, 0};
-    bool ok = true;
-    for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const DgTile tl = decode_dgrad_pair128(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
-      const float gapf = (float)t.st[tl.p].gap;
-      const bool corr = t.dyn[tl.p].use_delta != 0;
-      for (int kb = 0; kb < tl.n_kb; ++kb) {
-        bool go = mbar_wait(bar_sfull + 8 * sg.idx, sg.phase, abort_flag, status, 46);
-        go = __all_sync(0xffffffffu, go);
-        if (!go) { ok = false; break; }
-        // the staged fp32 values go to registers and the staging slot back to its producer at once: the wait for a free
-        // converted slot and the stores into it are then off the slot's round trip (copy latency + this read)
-        const uint8_t* src = stg_ptr + sg.idx * D1_STG_BYTES;
-        float4 w[4], dl[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int r = rbase + 16 * j;                               // k-row
-          w[j] = *reinterpret_cast<const float4*>(src + r * (D1_HALF_N * 4) + c4 * 16);
-          if (corr) dl[j] = *reinterpret_cast<const float4*>(src + D1_STG_HALF + r * (D1_HALF_N * 4) + c4 * 16);
-        }
-        uint2 o[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float v[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
-          if (corr) {
-            v[0] = __fsub_rn(v[0], __fmul_rn(gapf, dl[j].x)); v[1] = __fsub_rn(v[1], __fmul_rn(gapf, dl[j].y));   // w - (tau_fwd - tau_bkwd) * delta
-            v[2] = __fsub_rn(v[2], __fmul_rn(gapf, dl[j].z)); v[3] = __fsub_rn(v[3], __fmul_rn(gapf, dl[j].w));
-          }
-          o[j] = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
-        }
-        __syncwarp();                                                 // every lane's values have arrived (they were used above)
-        if (lane == 0) mbar_arrive(bar_sempty + 8 * sg.idx);
-        go = mbar_wait(bar_bempty + 8 * br.idx, br.phase ^ 1, abort_flag, status, 47);
-        go = __all_sync(0xffffffffu, go);
-        if (!go) { ok = false; break; }
-        uint8_t* dst = sB_ptr + br.idx * D1_B_BYTES;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int r = rbase + 16 * j;
-          const uint32_t off = (uint32_t)(r >> 3) * 1024 + (uint32_t)(r & 7) * 128 + ((((uint32_t)c4 >> 1) ^ (uint32_t)(r & 7)) << 4) + ((uint32_t)c4 & 1) * 8;
-          *reinterpret_cast<uint2*>(dst + off) = o[j];
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(leader_bfull + 8 * br.idx);
-        br.advance(D1_NB); sg.advance(D1_NG);
-      }
-    }
-  } else {
-    // ---------------- epilogue (both CTAs): 8 warps, warp%4 = TMEM lane group, two warps per group split the 128 columns ----------------
-    const int q = warp & 3;
-    const int ew = warp - 2 - D1_XF_WARPS;                            // 0..7
-    const int half = ew >> 2;
-    uint8_t* obuf = sO_ptr + ew * 4096;
-    const uint32_t obuf_s = sO + ew * 4096;
-    const uint32_t row_off = (uint32_t)lane * 128, sw = (uint32_t)(lane & 7);
-    const uint32_t leader_tempty = mapa_shared(bar_tempty, 0);
-    Ring acc{0, 0};
-    bool ok = true, stored = false;
-    for (int slot = pair; slot < n_slots && ok; slot += n_pairs) {
-      const int tile = tile_at(t, order, slot);
-      if (tile < 0) continue;
-      const DgTile tl = decode_dgrad_pair128(t, tile_start, lvl, tile);
-      if (!tl.valid) continue;
-      const StageDyn& d = t.dyn[tl.p];
-      const StageDev& s = t.st[tl.p];
-      const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
-      bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 48);
-      ready = __all_sync(0xffffffffu, ready);
-      if (!ready) { ok = false; break; }
-      tc_fence_after();
-      const int dslot = (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0;
-      const bool masked = lvl == 0 && s.mask_dx != 0;              // the previous stage's ReLU backward is applied here
-      const int nb = tl.n0 + half * 64;
-#pragma unroll 1
-      for (int mi = 0; mi < tl.n_m; ++mi) {
-        const int mrow = tl.m0 + mi * D1_TILE_M + rank * TILE_M + q * 32;
-        uint32_t r0[32], r1[32];
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * D1_ACC_COLS + mi * D1_TILE_N + half * 64);
-        const uint64_t mk = masked ? load_mask_bits64(t, s, d, tl.N, mrow + lane, nb) : ~0ull;
-        tmem_ld32(taddr, r0);
-        tmem_ld32(taddr + 32, r1);
-        tmem_ld_wait();
-        if (mi == tl.n_m - 1) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * acc.idx);   // this warp has read its part of both accumulators
-        }
-        if (mrow >= tl.M || nb >= tl.N) continue;
-        if (lane == 0 && stored) tma_store_wait_read();
-        __syncwarp();
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-          float f[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(g < 4 ? r0[(g & 3) * 8 + e] : r1[(g & 3) * 8 + e]);
-          if (masked) apply_mask8(f, (uint32_t)(mk >> (8 * g)) & 0xFFu);
-          *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) =
-              make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) { tma_store_3d(lm + MAP_DX_OUT, obuf_s, nb, mrow, dslot); tma_store_commit(); }
-        stored = true;
-      }
-      acc.advance(2);
-    }
-    if (lane == 0 && stored) tma_store_wait_all();
-  }
-  tc_fence_before();
-  cluster_sync_all();                                                 // no barrier or shared memory of a CTA is touched after this
-  if (warp == 1) {
-    __syncwarp();
-    tc_fence_after();
-    tmem_dealloc_pair(tmem_base, 2 * D1_ACC_COLS);
+    store8<__nv_bfloat16>(out + (uint64_t)i * 8, v);
   }
 }
 
@@ -1843,13 +1176,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 struct UmmaPlan {
   const CUtensorMap* d_maps = nullptr;
   const int* d_tile_start = nullptr;     // per (mode, level) at ts_off: [P+1] starts, then the stage of each tile
-  size_t ts_off[5][PM_MAX_LINEARS] = {};
+  size_t ts_off[4][PM_MAX_LINEARS] = {};
   const int* d_orders = nullptr;         // concatenated order arrays
   int* d_status = nullptr;
-  int n_slots[5][PM_MAX_LINEARS] = {};
-  int grid[5][PM_MAX_LINEARS] = {};
-  bool pair[5][PM_MAX_LINEARS] = {};     // launch uses the CTA-pair kernel (256 x 256 tiles)
-  size_t order_off[5][PM_MAX_LINEARS] = {};
+  int n_slots[4][PM_MAX_LINEARS] = {};
+  int grid[4][PM_MAX_LINEARS] = {};
+  bool pair[4][PM_MAX_LINEARS] = {};     // launch uses the CTA-pair kernel (256 x 256 tiles)
+  size_t order_off[4][PM_MAX_LINEARS] = {};
   int P = 0;
   // launches of one stage (microbatch-major order): the stage's tiles in ascending order are a slice of the identity list
   std::vector<int> h_tile_start;         // host copy of the tile starts
@@ -1857,6 +1190,8 @@ struct UmmaPlan {
   int row_n[2][PM_MAX_LINEARS] = {};
   std::vector<StageDev> st;              // host copy of the stages (launches of one stage with few tiles)
   const int* d_identity = nullptr;       // 0, 1, 2, ...
+  const CorrBlock* d_corr = nullptr;     // blocks of the corrected weights, and each stage's first
+  std::vector<uint32_t> corr_first;
   int max_ctas = kSms;
 };
 
@@ -1866,12 +1201,12 @@ struct UmmaPlan {
 // projection next to d_model-sized layers) does not leave most SMs idle.  Unused slots hold -1.
 struct TileTables {
   std::vector<int> tile_start;           // per (mode, level): [P+1] starts, then the stage of each tile
-  size_t ts_off[5][PM_MAX_LINEARS] = {};
+  size_t ts_off[4][PM_MAX_LINEARS] = {};
   std::vector<int> orders;
-  int n_slots[5][PM_MAX_LINEARS] = {};
-  int grid[5][PM_MAX_LINEARS] = {};
-  bool pair[5][PM_MAX_LINEARS] = {};
-  size_t order_off[5][PM_MAX_LINEARS] = {};
+  int n_slots[4][PM_MAX_LINEARS] = {};
+  int grid[4][PM_MAX_LINEARS] = {};
+  bool pair[4][PM_MAX_LINEARS] = {};
+  size_t order_off[4][PM_MAX_LINEARS] = {};
   int max_tiles = 0;                     // most tiles of any (mode, level)
 };
 
@@ -1890,44 +1225,49 @@ static bool pair_kernels_allowed() {
   return !(v && v[0] == '0');
 }
 
-static TileTables build_tile_tables(int T, const std::vector<StageDev>& st, int sms, int dgrad_split_below) {
+// Launches of a level whose GEMMs all have at least 256 rows and columns run on CTA pairs.
+static bool level_on_pairs(int T, const std::vector<StageDev>& st, int mode, int l) {
+  int n = 0;
+  for (size_t p = 0; p < st.size(); ++p)
+    if (l < st[p].n_lin) {
+      const LinDev& L = st[p].lin[l];
+      if ((mode == 2 ? L.n_out : T) < P2_TILE || (mode == 0 ? L.n_out : L.n_in) < P2_TILE) return false;
+      if ((mode == 0 || mode == 2) || p > 0 || l > 0 || st[p].pre == PRE_EMBED) ++n;   // the first Linear of the network has no input gradient
+    }
+  return n > 0 && pair_kernels_allowed();
+}
+
+// Does the dgrad of Linear l of stage p read the corrected weights from scratch?  one_stage: in launches of its stage alone; grouped: in
+// launches over all stages.
+bool umma_corr_weights(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped) {
+  if (l >= st[p].n_lin || (p == 0 && l == 0 && st[p].pre != PRE_EMBED) || device_sms() < 2 || !level_on_pairs(T, st, 3, l)) return false;
+  int n;
+  return (one_stage && row_dgrad_shape(T, st[p].lin[l].n_in, st[p].lin[l].n_out).bn == 0) || (grouped && row_grouped_shape(T, st, 1, l, &n).bn == 0);
+}
+
+static TileTables build_tile_tables(int T, const std::vector<StageDev>& st, int sms) {
   const int P = (int)st.size();
-  const bool allow_pair = pair_kernels_allowed();
   TileTables tt;
   auto cdiv = [](int a, int b) { return (a + b - 1) / b; };
-  for (int mode = 0; mode < 5; ++mode)                      // 3: dgrad once more, on 128-column pair tiles (launches of one narrow stage);
-                                                            // 4: dgrad as a plain GEMM against a queued weight version (weight stashing)
+  for (int mode = 0; mode < 4; ++mode)                      // 1: dgrad on the kernel that forms the corrected operand; 3: as a plain GEMM
     for (int l = 0; l < PM_MAX_LINEARS; ++l) {
       // block of this (mode, level): P + 1 tile starts, then the stage of every tile (one load instead of a search)
       tt.ts_off[mode][l] = tt.tile_start.size();
       std::vector<int> ts_block((size_t)P + 1, 0);
       int* ts = ts_block.data();
       std::vector<std::pair<long long, int>> work;          // (weight, tile id)
-      // forward and wgrad launches whose GEMMs all have at least 256 rows and columns run on CTA pairs
-      bool pair = allow_pair && sms >= 2;
-      int n_lin_here = 0;
-      for (int p = 0; p < P && pair; ++p)
-        if (l < st[p].n_lin) {
-          const LinDev& L = st[p].lin[l];
-          ++n_lin_here;
-          if ((mode == 2 ? L.n_out : T) < P2_TILE || (mode == 0 ? L.n_out : L.n_in) < P2_TILE) pair = false;
-          if ((mode == 1 || mode == 3 || mode == 4) && p == 0 && l == 0 && st[p].pre != PRE_EMBED) --n_lin_here;   // the first Linear of the network has no input gradient
-        }
-      pair = pair && n_lin_here > 0;
+      const bool pair = mode != 1 && sms >= 2 && level_on_pairs(T, st, mode, l);
       tt.pair[mode][l] = pair;
-      if (mode == 3 && !pair) { tt.n_slots[mode][l] = 0; tt.grid[mode][l] = 0; tt.order_off[mode][l] = tt.orders.size();
-                                tt.tile_start.insert(tt.tile_start.end(), (size_t)P + 1, 0); continue; }
-      const bool dg = mode == 1 || mode == 3;
-      const int tile_m = pair ? P2_TILE : TILE_M, tile_n = pair ? (mode == 1 ? DP_TILE_N : (mode == 3 ? D1_TILE_N : P2_TILE)) : TILE_N;
-      const int mg_rows_fixed = pair ? (mode == 3 ? D1_MG : DP_MG) : DG_MG;   // dgrad: row tiles sharing one converted weight tile
+      const bool dg = mode == 1;
+      const int tile_m = pair ? P2_TILE : TILE_M, tile_n = tile_m;
+      const int mg_rows = DG_MG;                            // mode 1: row tiles sharing one converted weight tile
       int acc = 0;
       for (int p = 0; p < P; ++p) {
         ts[p] = acc;
         if (l < st[p].n_lin) {
           const LinDev& L = st[p].lin[l];
-          const int M = mode == 2 ? L.n_out : T, N = mode == 0 ? L.n_out : L.n_in, K = mode == 0 ? L.n_in : ((dg || mode == 4) ? L.n_out : T);
+          const int M = mode == 2 ? L.n_out : T, N = mode == 0 ? L.n_out : L.n_in, K = mode == 0 ? L.n_in : (mode == 2 ? T : L.n_out);
           const int tm = cdiv(M, tile_m), tn = cdiv(N, tile_n), n_kb = cdiv(K, TILE_K);
-          const int mg_rows = (pair && mode == 1) ? dgrad_pair_mg(T, L.n_in, dgrad_split_below) : mg_rows_fixed;
           const int groups = dg ? cdiv(tm, mg_rows) : tm;
           for (int g = 0; g < groups; ++g) {
             const int n_m = dg ? std::min(mg_rows, tm - g * mg_rows) : 1;
@@ -1964,12 +1304,30 @@ static TileTables build_tile_tables(int T, const std::vector<StageDev>& st, int 
   return tt;
 }
 
+// the blocks of corr_weights_kernel, stage by stage; first: per stage its first block, and the total
+static std::vector<CorrBlock> corr_list(const std::vector<StageDev>& st, std::vector<uint32_t>* first) {
+  std::vector<CorrBlock> out;
+  for (size_t p = 0; p < st.size(); ++p) {
+    if (first) first->push_back((uint32_t)out.size());
+    for (int l = 0; l < st[p].n_lin; ++l) {
+      const LinDev& L = st[p].lin[l];
+      if (!L.wc_off) continue;
+      const uint32_t n64 = (uint32_t)((uint64_t)L.n_in * L.n_out / 64);          // dimensions are multiples of 8
+      for (uint32_t o = 0; o < n64; o += CORR_N64)
+        out.push_back(CorrBlock{(uint32_t)(L.w_off / 64) + o, (uint32_t)(L.wc_off / 128) + o, std::min(CORR_N64, n64 - o), (int32_t)p});
+    }
+  }
+  if (first) first->push_back((uint32_t)out.size());
+  return out;
+}
+
 static uint64_t maps_bytes(int P) { return (uint64_t)P * PM_MAX_LINEARS * MAPS_PER_LINEAR * sizeof(CUtensorMap); }
 static uint64_t ints_bytes(size_t n) { return ((uint64_t)n * sizeof(int) + 255) / 256 * 256; }
 
-uint64_t umma_workspace_bytes(int T, const std::vector<StageDev>& st, int dgrad_split_below) {
-  const TileTables tt = build_tile_tables(T, st, device_sms(), dgrad_split_below);
-  return 256 + maps_bytes((int)st.size()) + ints_bytes(tt.tile_start.size()) + ints_bytes(tt.orders.size()) + ints_bytes((size_t)tt.max_tiles);
+uint64_t umma_workspace_bytes(int T, const std::vector<StageDev>& st) {
+  const TileTables tt = build_tile_tables(T, st, device_sms());
+  return 256 + maps_bytes((int)st.size()) + ints_bytes(tt.tile_start.size()) + ints_bytes(tt.orders.size()) + ints_bytes((size_t)tt.max_tiles) +
+         corr_list(st, nullptr).size() * sizeof(CorrBlock);
 }
 
 static bool encode(EncodeTiledFn fn, CUtensorMap* m, int kind, void* base, int rank, const uint64_t* dims,
@@ -2029,17 +1387,12 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
           okm = okm && encode(fn, m + MAP_W_K, 0, wbase, 3, dims3, strides3, box3, err);
           uint32_t box32[3] = {TILE_K, 32, 1};                          // 32 columns of an output tile (launches with few tiles)
           okm = okm && encode(fn, m + MAP_W_K32, 0, wbase, 3, dims3, strides3, box32, err);
-          uint32_t box3mn[3] = {64, TILE_K, 1};                         // the same copies as an MN-major operand (dgrad against a queued version)
+          uint32_t box3mn[3] = {64, TILE_K, 1};                         // the same copies as an MN-major operand (dgrad against a queued version),
+          if (L.wc_off) { wbase = (void*)(t.ws + L.wc_off); dims3[2] = 1; strides3[1] = n_in * n_out * 2; }   // or the corrected weights
           okm = okm && encode(fn, m + MAP_W_MN, 0, wbase, 3, dims3, strides3, box3mn, err);
         }
         okm = okm && encode(fn, m + MAP_W_F32, 3, (void*)(t.a.w + L.w_off), 2, dims, strides4, box4, err);
         okm = okm && encode(fn, m + MAP_D_F32, 3, (void*)(t.a.delta + L.w_off), 2, dims, strides4, box4, err);
-        uint32_t box4q[2] = {DP_HALF_N, DP_SLAB_K};                     // CTA-pair dgrad: slabs of 32 k-rows x 128 columns per CTA
-        okm = okm && encode(fn, m + MAP_W_F32Q, 3, (void*)(t.a.w + L.w_off), 2, dims, strides4, box4q, err);
-        okm = okm && encode(fn, m + MAP_D_F32Q, 3, (void*)(t.a.delta + L.w_off), 2, dims, strides4, box4q, err);
-        uint32_t box4h[2] = {64, TILE_K};                               // 128-column pair dgrad: 64 columns per CTA
-        okm = okm && encode(fn, m + MAP_W_F32H, 3, (void*)(t.a.w + L.w_off), 2, dims, strides4, box4h, err);
-        okm = okm && encode(fn, m + MAP_D_F32H, 3, (void*)(t.a.delta + L.w_off), 2, dims, strides4, box4h, err);
       }
       {
         // dz operand (same rule as dz_src): dz scratch | gradient inside the stage | attention's dy | rotating incoming-gradient mailbox
@@ -2088,8 +1441,8 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
       if (!okm) { delete plan; return PM_ERR_CUDA; }
     }
   }
-  const TileTables tt = build_tile_tables(t.T, st, device_sms(), t.dgrad_split_below);
-  for (int mode = 0; mode < 5; ++mode)
+  const TileTables tt = build_tile_tables(t.T, st, device_sms());
+  for (int mode = 0; mode < 4; ++mode)
     for (int l = 0; l < PM_MAX_LINEARS; ++l) {
       plan->n_slots[mode][l] = tt.n_slots[mode][l];
       plan->grid[mode][l] = tt.grid[mode][l];
@@ -2107,6 +1460,9 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   std::vector<int> identity((size_t)tt.max_tiles);
   for (int i = 0; i < tt.max_tiles; ++i) identity[(size_t)i] = i;
   if (e == cudaSuccess && tt.max_tiles > 0) e = cudaMemcpyAsync(id_dev, identity.data(), identity.size() * sizeof(int), cudaMemcpyHostToDevice, stream);
+  char* corr_dev = id_dev + ints_bytes(identity.size());
+  const std::vector<CorrBlock> corr = corr_list(st, &plan->corr_first);
+  if (e == cudaSuccess && !corr.empty()) e = cudaMemcpyAsync(corr_dev, corr.data(), corr.size() * sizeof(CorrBlock), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(region, 0, 256, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) { err = std::string("tensor map upload: ") + cudaGetErrorString(e); delete plan; return PM_ERR_CUDA; }
@@ -2119,8 +1475,6 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_pair_gemm_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P2_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DP_SMEM_BYTES);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)umma_dgrad_pair128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D1_SMEM_BYTES);
   if (e == cudaSuccess) e = row_set_limits<0>();
   if (e == cudaSuccess) e = row_set_limits<1>();
   if (e == cudaSuccess) e = row_set_limits<2>();
@@ -2130,6 +1484,7 @@ pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<
   plan->d_tile_start = (const int*)ts_dev;
   plan->d_orders = (const int*)ord_dev;
   plan->d_identity = (const int*)id_dev;
+  plan->d_corr = (const CorrBlock*)corr_dev;
   plan->h_tile_start = tt.tile_start;
   plan->max_ctas = device_sms();
   plan->st = st;
@@ -2166,31 +1521,36 @@ int* umma_status_word(UmmaPlan* plan) { return plan ? plan->d_status : nullptr; 
 
 bool umma_row_dgrad(int T, const LinDev& L) { return row_dgrad_shape(T, L.n_in, L.n_out).bn != 0; }
 
+int umma_corr_blocks(const UmmaPlan* plan, int p) { return (int)(p >= 0 ? plan->corr_first[p + 1] - plan->corr_first[p] : plan->corr_first.back()); }
+
+cudaError_t umma_corr_launch(UmmaPlan* plan, const TickArgs& t, cudaStream_t stream) {
+  const int n = umma_corr_blocks(plan, t.sel_p);
+  if (n == 0) return cudaSuccess;
+  return launch_pdl(corr_weights_kernel, dim3((unsigned)n), dim3(CORR_THREADS), 0, stream, t.pdl, t, plan->d_corr + (t.sel_p >= 0 ? plan->corr_first[t.sel_p] : 0));
+}
+
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream) {
+  const bool queued = mode == 1 && t.stash;                           // dgrad against a queued version of the weights
   if (t.sel_p >= 0 && mode != 2) {
     const LinDev& L = plan->st[t.sel_p].lin[lvl];
     const int N = mode == 0 ? L.n_out : L.n_in;
     const RowShape r = mode == 0 ? row_shape(t.T, N, L.n_in) : row_dgrad_shape(t.T, N, L.n_out);
     if (r.bn != 0)
       return mode == 0 ? row_launch<0>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
-             : mode == 1 ? row_launch<1>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
-                         : row_launch<2>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream);
+             : !queued ? row_launch<1>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream)
+                       : row_launch<2>(t, r, plan->d_maps, lvl, N, 1, plan->d_status, stream);
   }
-  if (t.sel_p < 0 && mode < 2 && plan->row[mode][lvl].bn != 0)
+  if (t.sel_p < 0 && mode < 2 && !queued && plan->row[mode][lvl].bn != 0)
     return mode == 0 ? row_launch<0>(t, plan->row[0][lvl], plan->d_maps, lvl, plan->row_n[0][lvl], t.P, plan->d_status, stream)
                      : row_launch<1>(t, plan->row[1][lvl], plan->d_maps, lvl, plan->row_n[1][lvl], t.P, plan->d_status, stream);
+  if (mode == 1 && (queued || plan->pair[3][lvl])) mode = 3;          // a plain GEMM: a queued version, or the corrected weights in scratch
   int n_slots = plan->n_slots[mode][lvl];
   if (n_slots == 0) return cudaSuccess;
   int grid = plan->grid[mode][lvl];                                   // one persistent CTA per SM
   const int* ts = plan->d_tile_start + plan->ts_off[mode][lvl];
   const int* ord = plan->d_orders + plan->order_off[mode][lvl];
+  const bool pair = plan->pair[mode][lvl];
   int tile0 = 0;
-  bool narrow = false;                                                // dgrad of one narrow stage: 128-column tiles
-  if (t.sel_p >= 0 && mode == 1 && plan->pair[1][lvl] && plan->pair[3][lvl]) {
-    const int* h1 = plan->h_tile_start.data() + plan->ts_off[1][lvl];
-    narrow = h1[t.sel_p + 1] - h1[t.sel_p] < 64;                      // too few 256-column tile groups for the CTA pairs
-    if (narrow) { mode = 3; ts = plan->d_tile_start + plan->ts_off[3][lvl]; }
-  }
   if (t.sel_p >= 0) {                                                 // the tiles of one stage, in ascending order
     const int* hts = plan->h_tile_start.data() + plan->ts_off[mode][lvl];
     const int first = hts[t.sel_p];
@@ -2198,26 +1558,23 @@ cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cu
     if (n_slots == 0) return cudaSuccess;
     ord = plan->d_identity + first;
     tile0 = first;
-    const bool pr = plan->pair[mode][lvl];
-    const int G = std::max(1, std::min(n_slots, pr ? plan->max_ctas / 2 : plan->max_ctas));
-    grid = pr ? 2 * G : G;
+    const int G = std::max(1, std::min(n_slots, pair ? plan->max_ctas / 2 : plan->max_ctas));
+    grid = pair ? 2 * G : G;
   }
   TickArgs ta = t;
   ta.sel_tile0 = tile0;
   auto go = [&](auto kernel, int threads, int smem) {
     return launch_pdl(kernel, dim3(grid), dim3(threads), smem, stream, t.pdl, ta, plan->d_maps, ts, ord, n_slots, lvl, plan->d_status);
   };
-  if (plan->pair[mode][lvl]) {
+  if (pair) {
     if (mode == 0) return go(umma_pair_gemm_kernel<0, false>, P2Cfg<0, false>::kThreads, P2_SMEM_BYTES);
-    if (mode == 1) return go(umma_dgrad_pair_kernel, DP_THREADS, DP_SMEM_BYTES);
-    if (mode == 3) return go(umma_dgrad_pair128_kernel, D1_THREADS, D1_SMEM_BYTES);
-    if (mode == 4) return go(umma_pair_gemm_kernel<1, false>, P2Cfg<1, false>::kThreads, P2_SMEM_BYTES);
+    if (mode == 3) return go(umma_pair_gemm_kernel<1, false>, P2Cfg<1, false>::kThreads, P2_SMEM_BYTES);
     if (t.fuse_upd) return go(umma_pair_gemm_kernel<2, true>, P2Cfg<2, true>::kThreads, P2_SMEM_BYTES);
     return go(umma_pair_gemm_kernel<2, false>, P2Cfg<2, false>::kThreads, P2_SMEM_BYTES);
   }
   if (mode == 0) return go(umma_gemm_kernel<0, false>, Cfg<0, false>::kThreads, Cfg<0, false>::kSmemBytes);
   if (mode == 1) return go(umma_dgrad_kernel, DG_THREADS, DG_SMEM_BYTES);
-  if (mode == 4) return go(umma_gemm_kernel<1, false>, Cfg<1, false>::kThreads, Cfg<1, false>::kSmemBytes);
+  if (mode == 3) return go(umma_gemm_kernel<1, false>, Cfg<1, false>::kThreads, Cfg<1, false>::kSmemBytes);
   if (t.fuse_upd) return go(umma_gemm_kernel<2, true>, Cfg<2, true>::kThreads, Cfg<2, true>::kSmemBytes);
   return go(umma_gemm_kernel<2, false>, Cfg<2, false>::kThreads, Cfg<2, false>::kSmemBytes);
 }

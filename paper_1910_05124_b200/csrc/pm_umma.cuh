@@ -8,9 +8,8 @@ namespace pm {
 
 struct UmmaPlan;   // tensor maps and launch geometry, built once per context
 
-// Bytes of caller workspace the plan needs (status word + tensor maps).
-// dgrad_split_below: see TickArgs::dgrad_split_below (the plan must be created with the same value).
-uint64_t umma_workspace_bytes(int T, const std::vector<StageDev>& st, int dgrad_split_below);
+// Bytes of caller workspace the plan needs (status word, tensor maps, tile tables).
+uint64_t umma_workspace_bytes(int T, const std::vector<StageDev>& st);
 // ws_region: device memory of at least umma_workspace_bytes(T, stages), 256-byte aligned.  Synchronises `stream`.
 pm_status umma_plan_create(UmmaPlan** out, const TickArgs& t, const std::vector<StageDev>& st, void* ws_region,
                            cudaStream_t stream, std::string& err);
@@ -23,7 +22,13 @@ cudaError_t umma_wait_timeout_probe(UmmaPlan* plan, long long limit_cycles, int*
 cudaError_t umma_clear_status(UmmaPlan* plan, cudaStream_t stream);
 // does the dgrad of this Linear, launched for its stage alone, run on the kernel for few tiles (pm_umma_row.cuh)?
 bool umma_row_dgrad(int T, const LinDev& L);
-// mode: 0 forward, 1 dgrad (corrected weights formed in the operand-load path), 2 wgrad.
+// Does the dgrad of Linear l of stage p read the corrected weights from scratch (LinDev::wc_off)?  one_stage / grouped: the context
+// launches it for its stage alone / for all stages together.
+bool umma_corr_weights(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped);
+// Forms them, for the stages in backward (t.sel_p >= 0: that one); umma_corr_blocks: blocks of that launch (p < 0: all stages).
+int umma_corr_blocks(const UmmaPlan* plan, int p);
+cudaError_t umma_corr_launch(UmmaPlan* plan, const TickArgs& t, cudaStream_t stream);
+// mode: 0 forward, 1 dgrad (corrected weights, or with t.stash the queued version), 2 wgrad.
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream);
 
 }  // namespace pm
