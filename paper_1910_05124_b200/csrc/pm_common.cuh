@@ -50,6 +50,10 @@ struct LinDev {
   uint64_t dz_off;            // ws: dz = dy * act'(z) [T*n_out] (a Linear whose backward applies its activation itself)
   uint64_t dy_off;            // ws: gradient w.r.t. this Linear's output [T*n_out] (a Linear inside a stage)
   uint64_t wc_off;            // ws: bf16(w - gap*delta) [n_out*n_in], formed at the start of the backward phase (0: the dgrad forms it itself)
+  // A ReLU whose backward is applied where its gradient is produced by a plain GEMM: one bit per element, y > 0, at ring offset
+  // mask_out of the Linear with the ReLU = mask_in of the Linear that takes y as its input (0: none); slots as that input's, each
+  // ceil(T / 32) x ceil(n / 64) blocks of 32 rows x 64 columns, eight bytes per row: bit i of word h is column 32 h + 2 i, bit 16 + i the next
+  uint64_t mask_out, mask_in;
 };
 
 // Static description of one stage (device copy).  A stage is [pre-op] Linear{1..4} [post-op]:
@@ -73,8 +77,6 @@ struct StageDev {
   int32_t mem_first;          // from_memory stage that runs its backward first (the last one): it stores, the others add
   int32_t ids_stream;         // embedding: which input stream (0, 1)
   int32_t ids_depth;          // embedding: slots of ids_ring, slot = microbatch % ids_depth
-  int32_t mask_dx;            // the gradient this stage's first Linear sends to the previous stage is masked with (own input > 0):
-                              // the previous stage ends in a ReLU whose backward is fused here (LF_DZ_FUSED)
   int32_t vdepth;             // weight versions the forward pass can reach: 1 (the live weights, tick-major) or tau_f + 1
   uint32_t small_count;       // fp32 elements of a slot of s_ring (biases, LayerNorm gain and bias), a multiple of 64
   uint32_t g_soff, beta_soff; // offsets of LayerNorm gain / bias inside a slot of s_ring

@@ -303,17 +303,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       if ((ld.act != PM_ACT_NONE && !(ld.flags & LF_ACT_FROM_Y)) || to_attention) ld.flags |= LF_WRITE_Z;
       if (!to_attention && !logits) ld.flags |= LF_WRITE_Y;
       if (logits) ld.flags |= LF_OUT_F32;
-      // The ReLU's backward can be applied by the next stage's dgrad epilogue when that stage takes y as its plain input
-      // (tensor-core path).  Off unless PM_RELU_FUSE=1 is in the environment: the mask costs the dgrad epilogue, which is on
-      // that kernel's critical path (single-buffered accumulators), more than the separate pass costs (measured: config 4
-      // dgrad 0.215 -> 0.290 ms per tick against 0.014 ms saved in the activation-backward pass).
-      const char* fuse_env = getenv("PM_RELU_FUSE");
-      const bool fuse_ok = fuse_env && fuse_env[0] == '1';
-      // (never with weight stashing, whose plain dgrad epilogue applies no mask: a stage with tau_bkwd = tau_fwd > 0)
-      if (fuse_ok && cfg->compute_dtype == PM_BF16 && last && (ld.flags & LF_ACT_FROM_Y) && next_takes_y &&
-          stages[p + 1].ops[0].kind == PM_OP_LINEAR && !(sd.tau_fwd > 0 && sd.tau_bkwd == sd.tau_fwd) &&
-          !(stages[p + 1].tau_fwd > 0 && stages[p + 1].tau_bkwd == stages[p + 1].tau_fwd))
-        ld.flags |= LF_DZ_FUSED;
       // fp32 networks: the gradient of a Linear's output is multiplied by act'(z) where it is formed (the next Linear's dgrad,
       // the MSE loss), which saves a launch per Linear.  Not across a recompute segment's edge: there the z of the earlier
       // stage is formed again only after the later stage's dgrad has run.
@@ -328,9 +317,7 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
         if (nx) { nl.n_in = nx->n_in; nl.n_out = nx->n_out; }
         if (nx ? umma_row_dgrad((int)T, nl) : (last && p == P - 1 && !ce && s.post == POST_NONE)) ld.flags |= LF_DZ_FUSED;
       }
-      if (bwd_act(ld) != PM_ACT_NONE) L.act_levels |= 1 << l;
     }
-    if (p > 0 && (L.st[p - 1].lin[L.st[p - 1].n_lin - 1].flags & LF_DZ_FUSED)) s.mask_dx = 1;
     // ---- rings
     if (s.pre != PRE_EMBED) { s.x_ring = ring; ring = align_up(ring + (uint64_t)s.xdepth * T * s.d_in * esz, 256); }
     if (s.pre != PRE_NONE) { s.u_ring = ring; ring = align_up(ring + (uint64_t)s.depth * T * s.d_in * esz, 256); }
@@ -405,6 +392,25 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
     }
     L.parts = update_parts(L.begin64.data(), L.end64.data(), skip_b.data(), skip_e.data(), P);
   }
+  // bf16 ReLUs whose gradient comes from a plain GEMM on the kernels for many tiles: that GEMM's epilogue applies the mask, one bit per
+  // element that the forward left.  (A launch of its own read y and dy again: 57 us of a tick of the 6-layer encoder; fetching y in
+  // the epilogue instead put its latency between the accumulator and the store.)  Not across a recompute segment's edge.
+  if (cfg->compute_dtype == PM_BF16)
+    for (int p = 0; p < P; ++p)
+      for (int l = 0; l < L.st[p].n_lin; ++l) {
+        StageDev& s = L.st[p];
+        const bool last = l == s.n_lin - 1;
+        if (s.lin[l].act != PM_ACT_RELU || !(s.lin[l].flags & LF_ACT_FROM_Y) || (s.lin[l].flags & LF_DZ_FUSED)) continue;
+        const int pc = last ? p + 1 : p, lc = last ? 0 : l + 1;      // the Linear that takes y as its input
+        if (pc >= P || (last && (L.st[pc].pre != PRE_NONE || (S > 0 && pc % S == 0)))) continue;
+        if (!umma_fwd_plain((int)T, L.st, p, l, queue, !mb) || !umma_dgrad_plain((int)T, L.st, pc, lc, queue, !mb, L.stash || L.materialize)) continue;
+        s.lin[l].flags |= LF_DZ_FUSED;
+        s.lin[l].mask_out = L.st[pc].lin[lc].mask_in = ring;
+        const uint64_t slots = lc == 0 ? L.st[pc].xdepth : L.st[pc].depth;
+        ring = align_up(ring + slots * ((T + 31) / 32) * (((uint64_t)s.lin[l].n_out + 63) / 64) * 256, 256);
+      }
+  for (int p = 0; p < P; ++p)
+    for (int l = 0; l < L.st[p].n_lin; ++l) if (bwd_act(L.st[p].lin[l]) != PM_ACT_NONE) L.act_levels |= 1 << l;
   for (int p = 0; p < P; ++p) {
     L.sched[p].next_xdepth = p + 1 < P ? L.st[p + 1].xdepth : 0;
     L.sched[p].gin_depth = L.st[p].gin_depth;

@@ -176,6 +176,20 @@ __device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
   asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
+// 0xFFFF in the halves that are > 0
+__device__ __forceinline__ uint32_t positive_bf16x2(uint32_t v) {
+  __nv_bfloat162 x, zero = __floats2bfloat162_rn(0.f, 0.f);
+  *reinterpret_cast<uint32_t*>(&x) = v;
+  return __hgt2_mask(x, zero);
+}
+// v times 1 or 0: bits 15 and 31 of `m` say which for the two halves
+__device__ __forceinline__ uint32_t mask_bf16x2(uint32_t v, uint32_t m) {
+  uint32_t one, r;
+  asm("prmt.b32 %0, %1, %1, 0xBB99;" : "=r"(one) : "r"(m));          // the sign bits over their halves
+  one &= 0x3F803F80u;
+  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(one));
+  return r;
+}
 
 // The same descriptor split into its address-independent part and the start address, so that issuing loops add
 // only the address: desc = desc_base(leading, stride) + (saddr >> 4)   (valid while saddr < 256 KB).

@@ -179,10 +179,17 @@ struct EpiTile {
   int slot;                   // ring slot of z (MODE 0) or dx (MODE 1); MODE 2: gradients add to the arena
   int yslot;                  // MODE 0: ring slot of y, or of the fp32 logits
   const float* bias;          // MODE 0
+  uint2* mask;                // the mask bits a ReLU writes (MODE 0) or the gradient of its output reads (MODE 1); null: none
 };
 
+// this lane's eight bytes of the mask bits of a block of 32 rows x 64 columns (row0 a multiple of 32, n a multiple of 64)
+__device__ __forceinline__ uint2* mask_at(const TickArgs& t, uint64_t ring_off, int slot, int N, int row0, int n, int lane) {
+  const uint64_t cb = (uint64_t)(N + 63) / 64, rb = (uint64_t)(t.T + 31) / 32;
+  return reinterpret_cast<uint2*>(t.ring + ring_off) + (((uint64_t)slot * rb + row0 / 32) * cb + n / 64) * 32 + lane;
+}
+
 template <int MODE>
-__device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s, const StageDyn& d, const LinDev& L, int p, int lvl) {
+__device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s, const StageDyn& d, const LinDev& L, int p, int lvl, int mrow, int nb, int lane) {
   EpiTile e{};
   if (MODE == 0) {
     e.flags = L.flags; e.act = L.act;
@@ -191,8 +198,10 @@ __device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s
     e.slot = d.f_slot;
     e.yslot = lvl < s.n_lin - 1 ? d.f_slot : (s.emit_memory ? (int)(d.f_mb % t.mem_depth) : (p < t.P - 1 ? d.f_next_xslot : (int)(d.tick & 1)));
     e.bias = fwd_small<__nv_bfloat16>(t, s, d, L.b_off, L.b_soff);
+    if (L.mask_out) e.mask = mask_at(t, L.mask_out, e.yslot, L.n_out, mrow, nb, lane);
   } else if (MODE == 1) {
     e.slot = (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0;
+    if (L.mask_in) e.mask = mask_at(t, L.mask_in, (lvl == 0 && s.pre == PRE_NONE) ? d.b_xslot : d.b_slot, L.n_in, mrow, nb, lane);
   } else {
     e.slot = d.accum;
   }
@@ -207,12 +216,12 @@ __device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s
 // takes 4096 cycles for it at a reduction of 512.  Hence two columns per instruction everywhere (a bf16 sum of two bf16 values
 // rounded once is what the fp32 sum rounds to: at most 16 binary digits apart the fp32 sum is exact, further apart neither
 // reaches a tie), and one branch per half on what the Linear does.
-// bias: that of columns 2 l and 2 l + 1 in lane l.  (With one column per instruction the
+// bias: that of columns 2 l and 2 l + 1 in lane l.  mask: this row's mask bits where a ReLU's backward is applied (MODE 1).  (With one column per instruction the
 // forward of the 6-layer encoder's tick took 194 us, 164 now; reading the skip values row by row into registers 172.)
 template <int MODE, bool FUSE, int SLOTS, class Release>
 __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* lm, const StageDyn& d, const LinDev& L, const EpiTile& et,
                                          int M, int N, int mrow, int nb, uint32_t taddr, EpiStage<SLOTS>& es,
-                                         const float2 bias, Release release) {
+                                         const float2 bias, const uint2 mask, Release release) {
   const int lane = es.lane;
   const uint32_t row_off = (uint32_t)lane * 128, sw = (uint32_t)(lane & 7);
   uint32_t r[32];
@@ -259,7 +268,8 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
   const bool both = MODE == 0 && (et.flags & LF_WRITE_Z) && (et.flags & LF_WRITE_Y);   // z, then y = act(z) from the staged z
   // A stage that ends in a residual add writes the sum itself: out = bf16(skip + bf16(acc + b)), straight into the
   // next stage's input (or the memory ring); the skip tensor was sent by the emitting stage skip_depth - 1 ticks ago.
-  enum { PLAIN, RELU, RESIDUAL };
+  enum { PLAIN, RELU, RESIDUAL, MASKED };
+  uint2 bits = make_uint2(0u, 0u);                                // the mask bits a ReLU leaves
   uint8_t* box = nullptr;
   auto half = [&](int h, auto kind) {
     constexpr int KIND = decltype(kind)::value;
@@ -269,6 +279,17 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
       const float2 v0 = pair(8 * g, b0.x, b0.y), v1 = pair(8 * g + 2, b0.z, b0.w), v2 = pair(8 * g + 4, b1.x, b1.y), v3 = pair(8 * g + 6, b1.z, b1.w);
       uint4 o = make_uint4(pack_bf16(v0.x, v0.y), pack_bf16(v1.x, v1.y), pack_bf16(v2.x, v2.y), pack_bf16(v3.x, v3.y));
       if (KIND == RELU) o = make_uint4(relu_bf16x2(o.x), relu_bf16x2(o.y), relu_bf16x2(o.z), relu_bf16x2(o.w));   // bf16(max(x, 0)) = max(bf16(x), 0)
+      if (KIND == RELU) {
+        const uint32_t w[4] = {o.x, o.y, o.z, o.w};
+        uint32_t m = 0u;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) m |= positive_bf16x2(w[e]) & (0x00010001u << (4 * g + e));
+        if (h == 0) bits.x |= m; else bits.y |= m;
+      }
+      if (KIND == MASKED) {                                         // dz = bf16(dx) * (1 or 0)
+        const uint32_t m = h == 0 ? mask.x : mask.y;
+        o = make_uint4(mask_bf16x2(o.x, m << (15 - 4 * g)), mask_bf16x2(o.y, m << (14 - 4 * g)), mask_bf16x2(o.z, m << (13 - 4 * g)), mask_bf16x2(o.w, m << (12 - 4 * g)));
+      }
       if (KIND == RESIDUAL) {
         const uint4 k = *reinterpret_cast<const uint4*>(box + row_off + (((uint32_t)(4 * h + g) ^ sw) << 4));
         o = make_uint4(add_bf16x2(k.x, o.x), add_bf16x2(k.y, o.y), add_bf16x2(k.z, o.z), add_bf16x2(k.w, o.w));
@@ -282,8 +303,10 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
     if (h == 0) box = MODE == 0 && et.resid ? es.buf + es.off : es.begin();
     if (MODE == 0 && et.resid) half(h, std::integral_constant<int, RESIDUAL>());
     else if (MODE == 0 && et.act == PM_ACT_RELU && !both) half(h, std::integral_constant<int, RELU>());
+    else if (MODE == 1 && et.mask) half(h, std::integral_constant<int, MASKED>());
     else half(h, std::integral_constant<int, PLAIN>());
   }
+  if (MODE == 0 && et.mask) *et.mask = bits;
   es.end([&](uint32_t src) {
     // dx: to the previous stage's gradient mailbox, or this stage's own scratch when a pre-op stands before the Linear
     if (MODE == 1) tma_store_3d(lm + MAP_DX_OUT, src, nb, mrow, et.slot);
@@ -311,39 +334,6 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
   else if (et.act == PM_ACT_RELU) write_y(std::integral_constant<int, PM_ACT_RELU>());
   else write_y(std::integral_constant<int, PM_ACT_NONE>());
   es.end([&](uint32_t src) { tma_store_3d(lm + MAP_Y_OUT, src, nb, mrow, et.yslot); });
-}
-
-// dgrad epilogue of a stage whose predecessor's ReLU backward is fused here (StageDev::mask_dx): the 64 values of this
-// stage's own stashed input x (row `row`, columns nb .. nb+63, the slot of the microbatch in backward) whose sign
-// decides which entries of dx survive: dz_prev = dx where x > 0 (x = ReLU(z_prev) > 0 exactly where z_prev > 0), else 0.
-__device__ __forceinline__ uint64_t load_mask_bits64(const TickArgs& t, const StageDev& s, const StageDyn& d, int N, int row, int nb) {
-  // Bit i is set where x[row, nb + i] > 0.  The 64 values are compressed to bits BEFORE the accumulator is read from
-  // tensor memory, so that they never share the register file with it (the kernel runs at 96 registers per thread).
-  if (row >= t.T) return 0ull;
-  const __nv_bfloat16* xrow = ring_at<__nv_bfloat16>(t, s.x_ring, d.b_xslot, (uint64_t)t.T * N) + (uint64_t)row * N + nb;
-  uint4 xq[8];
-#pragma unroll
-  for (int g = 0; g < 8; ++g)
-    xq[g] = (nb + 8 * g < N) ? ld_chain16(xrow + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
-  uint64_t mk = 0ull;
-#pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    const uint32_t w[4] = {xq[g].x, xq[g].y, xq[g].z, xq[g].w};
-    uint32_t bits = 0u;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t lo = w[e] & 0xFFFFu, hi = w[e] >> 16;
-      bits |= (uint32_t)(!(lo & 0x8000u) && (lo & 0x7FFFu) != 0u) << (2 * e);
-      bits |= (uint32_t)(!(hi & 0x8000u) && (hi & 0x7FFFu) != 0u) << (2 * e + 1);
-    }
-    mk |= (uint64_t)bits << (8 * g);
-  }
-  return mk;
-}
-// zeroes f[e] where bit e of `bits` is clear
-__device__ __forceinline__ void apply_mask8(float (&f)[8], uint32_t bits) {
-#pragma unroll
-  for (int e = 0; e < 8; ++e) if (!((bits >> e) & 1u)) f[e] = 0.0f;
 }
 
 // ---- tile walk ---------------------------------------------------------------------------------------
@@ -614,7 +604,9 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
       const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
       const int M = MODE == 2 ? L.n_out : t.T, N = MODE == 0 ? L.n_out : L.n_in;
       const int mrow = tl.m0 + q * 32, nb = tl.n0 + half * 64;        // this warp's block
-      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl);
+      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl, mrow, nb, lane);
+      // (written by the forward phase, which this launch's predecessors ended: read behind the wait)
+      const uint2 mask = MODE == 1 && et.mask && mrow < M && nb < N ? *et.mask : make_uint2(0u, 0u);
       const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
       const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
       if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
@@ -623,7 +615,7 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
       if (fetch && go) go = es.fetched(abort_flag, status);
       if (!go) { if (fetch) es.drain(); return false; }
       tc_fence_after();
-      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias, [&] {
+      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias, mask, [&] {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8 * acc.idx);         // the accumulator buffer may be overwritten now
@@ -802,7 +794,9 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
       const CUtensorMap* lm = maps + ((size_t)tl.p * PM_MAX_LINEARS + lvl) * MAPS_PER_LINEAR;
       const int M = MODE == 2 ? L.n_out : t.T, N = MODE == 0 ? L.n_out : L.n_in;
       const int mrow = tl.m0 + rank * TILE_M + q * 32, nb = tl.n0 + part * 64;   // this warp's (first) block
-      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl);
+      const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl, mrow, nb, lane);
+      // (written by the forward phase, which this launch's predecessors ended: read behind the wait)
+      const uint2 mask = MODE == 1 && et.mask && mrow < M && nb < N ? *et.mask : make_uint2(0u, 0u);
       const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
       const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
       if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
@@ -813,7 +807,7 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
       tc_fence_after();
 #pragma unroll 1
       for (int u = 0; u < UNITS; ++u) {                               // (MODE 0: one)
-        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias, [&] {
+        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias, mask, [&] {
           if (u != UNITS - 1) return;
           tc_fence_before();
           __syncwarp();
@@ -1076,7 +1070,6 @@ umma_dgrad_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* _
       if (!ready) { ok = false; break; }
       tc_fence_after();
       const int dslot = (lvl == 0 && s.pre == PRE_NONE) ? d.prev_wslot : 0;
-      const bool masked = lvl == 0 && s.mask_dx != 0;              // the previous stage's ReLU backward is applied here
       for (int mi = 0; mi < tl.n_m; ++mi) {
         const int mrow = tl.m0 + mi * TILE_M + q * 32;
 #pragma unroll 1
@@ -1084,7 +1077,6 @@ umma_dgrad_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* _
           const int nb = tl.n0 + half * 64;
           uint32_t r0[32], r1[32];
           const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(mi * ACC_COLS + half * 64);
-          const uint64_t mk = masked ? load_mask_bits64(t, s, d, tl.N, mrow + lane, nb) : ~0ull;
           tmem_ld32(taddr, r0);
           tmem_ld32(taddr + 32, r1);
           tmem_ld_wait();
@@ -1096,7 +1088,6 @@ umma_dgrad_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* _
             float f[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(g < 4 ? r0[(g & 3) * 8 + e] : r1[(g & 3) * 8 + e]);
-            if (masked) apply_mask8(f, (uint32_t)(mk >> (8 * g)) & 0xFFu);
             *reinterpret_cast<uint4*>(obuf + row_off + (((uint32_t)g ^ sw) << 4)) =
                 make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
           }
@@ -1243,6 +1234,18 @@ bool umma_corr_weights(int T, const std::vector<StageDev>& st, int p, int l, boo
   if (l >= st[p].n_lin || (p == 0 && l == 0 && st[p].pre != PRE_EMBED) || device_sms() < 2 || !level_on_pairs(T, st, 3, l)) return false;
   int n;
   return (one_stage && row_dgrad_shape(T, st[p].lin[l].n_in, st[p].lin[l].n_out).bn == 0) || (grouped && row_grouped_shape(T, st, 1, l, &n).bn == 0);
+}
+
+// Do the forward of Linear l of stage p / its dgrad run on the kernels above in every launch the context makes (queued: against a
+// queued version of the weights)?
+bool umma_fwd_plain(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped) {
+  int n;
+  return (!one_stage || row_shape(T, st[p].lin[l].n_out, st[p].lin[l].n_in).bn == 0) && (!grouped || row_grouped_shape(T, st, 0, l, &n).bn == 0);
+}
+bool umma_dgrad_plain(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped, bool queued) {
+  if (!queued && (device_sms() < 2 || !level_on_pairs(T, st, 3, l))) return false;
+  int n;
+  return (!one_stage || row_dgrad_shape(T, st[p].lin[l].n_in, st[p].lin[l].n_out).bn == 0) && (!grouped || row_grouped_shape(T, st, 1, l, &n).bn == 0);
 }
 
 static TileTables build_tile_tables(int T, const std::vector<StageDev>& st, int sms) {

@@ -28,6 +28,10 @@ bool umma_corr_weights(int T, const std::vector<StageDev>& st, int p, int l, boo
 // Forms them, for the stages in backward (t.sel_p >= 0: that one); umma_corr_blocks: blocks of that launch (p < 0: all stages).
 int umma_corr_blocks(const UmmaPlan* plan, int p);
 cudaError_t umma_corr_launch(UmmaPlan* plan, const TickArgs& t, cudaStream_t stream);
+// Does the forward / the dgrad of Linear l of stage p run on the kernels for many tiles, whose epilogues write and apply ReLU mask bits
+// (LinDev::mask_out), in every launch?  queued: the dgrad reads a queued version of the weights.
+bool umma_fwd_plain(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped);
+bool umma_dgrad_plain(int T, const std::vector<StageDev>& st, int p, int l, bool one_stage, bool grouped, bool queued);
 // mode: 0 forward, 1 dgrad (corrected weights, or with t.stash the queued version), 2 wgrad.
 cudaError_t umma_launch(UmmaPlan* plan, const TickArgs& t, int mode, int lvl, cudaStream_t stream);
 
