@@ -540,6 +540,7 @@ struct pm_ctx {
   // phase on plain launches.
   struct PhaseGraph { cudaGraphExec_t exec = nullptr; int eager_runs = 0; uint64_t launches = 0; bool failed = false; };
   PhaseGraph g_fwd, g_bwd, g_upd;
+  PhaseGraph g_step, g_part;            // pm_step: the three phases as one graph; the first two alone (inside a minibatch)
   // Tick-major order with an entry period E > 1 ("sparse ticks"): a tick's launches cover only the stages whose turn it
   // is (those at distance = tick mod E from a microbatch's entry), one graph per phase and residue; the forward stages
   // run on a stream of their own, next to the backward and update of the same tick (see sparse_forward).
@@ -552,14 +553,22 @@ struct pm_ctx {
   bool graphs = true;
   cudaStream_t cap_stream = nullptr;
   bool chained = false;                 // a launch of the running phase body precedes: the next may be a programmatic dependent of it
-  cudaStream_t ls = nullptr;            // the stream the phase bodies launch on: `stream`, or `cap_stream` while capturing
+  cudaStream_t ls = nullptr;            // the stream the phase bodies launch on: `stream`, or while capturing `cap_stream` or a side stream
+  // launches of a tick that need nothing of each other become parallel branches of the captured graph: side streams that fork from the
+  // capture stream and join it again (only during a capture; plain launches run one after the other)
+  static constexpr int kSides = 3;
+  cudaStream_t side[kSides] = {};
+  cudaEvent_t side_ev = nullptr;
+  bool capturing = false, side_used[kSides] = {};
   ~pm_ctx() {
-    for (PhaseGraph* g : {&g_fwd, &g_bwd, &g_upd}) if (g->exec) cudaGraphExecDestroy(g->exec);
+    for (PhaseGraph* g : {&g_fwd, &g_bwd, &g_upd, &g_step, &g_part}) if (g->exec) cudaGraphExecDestroy(g->exec);
     for (auto* v : {&gs_fwd, &gs_bwd, &gs_upd}) for (auto& g : *v) if (g.exec) cudaGraphExecDestroy(g.exec);
     if (fwd_stream) cudaStreamDestroy(fwd_stream);
     if (ev_sched) cudaEventDestroy(ev_sched);
     if (ev_fwd) cudaEventDestroy(ev_fwd);
     if (cap_stream) cudaStreamDestroy(cap_stream);
+    for (auto st : side) if (st) cudaStreamDestroy(st);
+    if (side_ev) cudaEventDestroy(side_ev);
   }
   // optional per-kernel-class timing with CUDA events on the context's stream
   bool prof_on = false;
@@ -671,6 +680,11 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   c->ls = c->stream;
   { const char* v = getenv("PM_CUDA_GRAPHS"); c->graphs = !(v && v[0] == '0'); }
   if (c->graphs && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); c->cap_stream = nullptr; }
+  if (c->cap_stream) {
+    bool ok = cudaEventCreateWithFlags(&c->side_ev, cudaEventDisableTiming) == cudaSuccess;
+    for (auto& st : c->side) ok = ok && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); if (c->side_ev) cudaEventDestroy(c->side_ev); c->side_ev = nullptr; }
+  }
   c->ws = (char*)workspace;
   const int P = cfg->n_stages;
   c->a = ArenasDev{arenas->w, arenas->m, arenas->s, arenas->delta, arenas->grad, (__nv_bfloat16*)arenas->w_lp, arenas->count};
@@ -846,7 +860,10 @@ static pm_status run_phase(pm_ctx* ctx, pm_ctx::PhaseGraph& g, const std::functi
   const uint64_t l0 = ctx->launches;
   if (cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) { cudaGetLastError(); g.failed = true; return body(); }
   ctx->ls = ctx->cap_stream;
+  ctx->capturing = true;
+  for (bool& u : ctx->side_used) u = false;
   const pm_status sb = body();
+  ctx->capturing = false;
   ctx->ls = run_on;
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &graph);
@@ -864,6 +881,28 @@ static pm_status run_phase(pm_ctx* ctx, pm_ctx::PhaseGraph& g, const std::functi
   }
   e = cudaGraphLaunch(g.exec, run_on);
   return e == cudaSuccess ? PM_OK : cuda_fail(ctx, e, "graph launch");
+}
+
+// Runs `body` as branch i of the graph being captured: behind what the current stream has launched so far, beside what it launches
+// from here to rejoin(i).  Outside a capture it runs in line.
+static pm_status branch(pm_ctx* ctx, int i, const std::function<pm_status()>& body) {
+  if (!ctx->capturing || !ctx->side_ev) return body();
+  const cudaStream_t from = ctx->ls;
+  cudaError_t e = cudaEventRecord(ctx->side_ev, from);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side[i], ctx->side_ev, 0);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "graph branch");
+  ctx->side_used[i] = true;
+  ctx->ls = ctx->side[i];
+  const pm_status s = body();
+  ctx->ls = from;
+  return s;
+}
+static pm_status rejoin(pm_ctx* ctx, int i) {
+  if (!ctx->capturing || !ctx->side_used[i]) return PM_OK;
+  ctx->side_used[i] = false;
+  cudaError_t e = cudaEventRecord(ctx->side_ev, ctx->side[i]);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->ls, ctx->side_ev, 0);
+  return e == cudaSuccess ? PM_OK : cuda_fail(ctx, e, "graph branch");
 }
 
 // is a microbatch in flight at any of the stages whose distance from the entry tick lies in [lo, hi]?
@@ -991,26 +1030,22 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
   return PM_OK;
 }
 
-static pm_status mb_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
+// Takes a microbatch in: the schedule tables and the inputs.
+static pm_status mb_begin(pm_ctx* ctx, const void* inputs, const void* targets) {
   if (!inputs || !targets) return fail(ctx, PM_ERR_INVALID_ARG, "microbatch-major order takes a microbatch at every step (there is nothing to drain)");
-  const int dt = ctx->cfg.compute_dtype;
-  const int P = ctx->cfg.n_stages;
   const int64_t mb = ctx->n_fed;
-  pm_status s;
   const bool stoch = ctx->L.stochastic > 0;
-  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn),
+  const pm_status s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn),
                                                       ctx->hp, 0, 0, true, stoch ? (const int32_t*)(ctx->ws + ctx->L.off_delays) : nullptr,
-                                                      (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, dt, inputs, targets, mb, ctx->stream), "schedule and ingest"));
-  if (s != PM_OK) return s;
-  s = run_phase(ctx, ctx->g_fwd, [&]() -> pm_status {
-    pm_status s;
-    for (int p = 0; p < P; ++p)
-      if ((s = stage_forward(ctx, mb_args(ctx, p, p), p)) != PM_OK) return s;
-    return PM_OK;
-  });
-  if (s != PM_OK) return s;
-  ctx->n_fed = mb + 1;
-  ctx->phase = 1;
+                                                      (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, ctx->cfg.compute_dtype, inputs, targets, mb, ctx->stream), "schedule and ingest"));
+  if (s == PM_OK) ctx->n_fed = mb + 1;
+  return s;
+}
+
+static pm_status mb_forward_body(pm_ctx* ctx) {
+  pm_status s;
+  for (int p = 0; p < ctx->cfg.n_stages; ++p)
+    if ((s = stage_forward(ctx, mb_args(ctx, p, p), p)) != PM_OK) return s;
   return PM_OK;
 }
 
@@ -1029,8 +1064,7 @@ static pm_status grouped_wgrad(pm_ctx* ctx, int table, bool fused = false) {
   return PM_OK;
 }
 
-static pm_status mb_backward(pm_ctx* ctx) {
-  const int dt = ctx->cfg.compute_dtype;
+static pm_status mb_backward_body(pm_ctx* ctx) {
   const int P = ctx->cfg.n_stages;
   // Nothing overwrites a Linear's dz before the end of the backward chain, so the weight gradients of all stages run as
   // ONE grouped launch per Linear of a stage (the tick schedule's launches, which fill the GPU).
@@ -1041,29 +1075,24 @@ static pm_status mb_backward(pm_ctx* ctx) {
   // recomputed, because that recomputation overwrites the input of this segment's first stage.
   const int S = ctx->L.segment;
   const int n_seg = S > 0 ? (P + S - 1) / S : 1;
-  pm_status s = run_phase(ctx, ctx->g_bwd, [&]() -> pm_status {
-    pm_status s;
-    if ((s = corr_weights(ctx, mb_args(ctx, 2 * P, -1))) != PM_OK) return s;
-    for (int k = n_seg - 1; k >= 0; --k) {
-      const int lo = S > 0 ? k * S : 0, hi = S > 0 ? std::min(P, lo + S) : P;
-      if (S > 0 && k < n_seg - 1)
-        for (int p = lo; p < hi; ++p)
-          if ((s = stage_forward(ctx, mb_args(ctx, 2 * P + 1, p), p)) != PM_OK) return s;
-      for (int p = hi - 1; p >= lo; --p) {
-        TickArgs ta = mb_args(ctx, 2 * P - 1 - p, p);
-        ta.defer_finish = 1;                    // LayerNorm gradients are summed once, below
-        if ((s = stage_backward(ctx, ta, p, true)) != PM_OK) return s;
-      }
-      if (S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
+  pm_status s;
+  if ((s = corr_weights(ctx, mb_args(ctx, 2 * P, -1))) != PM_OK) return s;
+  for (int k = n_seg - 1; k >= 0; --k) {
+    const int lo = S > 0 ? k * S : 0, hi = S > 0 ? std::min(P, lo + S) : P;
+    if (S > 0 && k < n_seg - 1)
+      for (int p = lo; p < hi; ++p)
+        if ((s = stage_forward(ctx, mb_args(ctx, 2 * P + 1, p), p)) != PM_OK) return s;
+    for (int p = hi - 1; p >= lo; --p) {
+      TickArgs ta = mb_args(ctx, 2 * P - 1 - p, p);
+      ta.defer_finish = 1;                    // LayerNorm gradients are summed once, below
+      if ((s = stage_backward(ctx, ta, p, true)) != PM_OK) return s;
     }
-    TickArgs ta = mb_args(ctx, 2 * P, -1);
-    const int n_fin = ln_finish_launches(ta);
-    if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
-    if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
-    return PM_OK;
-  });
-  if (s != PM_OK) return s;
-  ctx->phase = 2;
+    if (S > 0 && (s = grouped_wgrad(ctx, 2 * P + 2 + k)) != PM_OK) return s;
+  }
+  TickArgs ta = mb_args(ctx, 2 * P, -1);
+  const int n_fin = ln_finish_launches(ta);
+  if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
+  if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
   return PM_OK;
 }
 
@@ -1078,14 +1107,25 @@ static cudaError_t update_all(pm_ctx* ctx, const StageDyn* dyn, const float* gsr
                        ctx->L.total / 64, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, ctx->hp.lp_elem, 0, gsrc, early(ctx));
 }
 
-static pm_status mb_update(pm_ctx* ctx) {
+// Inside a minibatch the gradients stay in the arena and the next microbatch adds to them.
+static bool mb_updates(const pm_ctx* ctx) { return ctx->n_fed % ctx->hp.n_micro == 0; }
+
+static pm_status mb_update_body(pm_ctx* ctx, const float* gsrc) {
   const int P = ctx->cfg.n_stages;
-  if (ctx->n_fed % ctx->hp.n_micro != 0) {          // inside a minibatch: the gradients stay in the arena and the next microbatch adds to them
-    ctx->tick += 1;
-    ctx->phase = 0;
-    return PM_OK;
-  }
   const StageDyn* dyn_all = (const StageDyn*)(ctx->ws + ctx->L.off_dyn) + (size_t)2 * P * P;
+  // fused update: the weight gradients of all stages as one launch whose epilogue updates the Linear matrices
+  if (ctx->L.fuse) { pm_status fs = grouped_wgrad(ctx, 2 * P, true); if (fs != PM_OK) return fs; }
+  prof_begin(ctx, PM_PROF_UPDATE);
+  cudaError_t e = update_all(ctx, dyn_all, gsrc);
+  pm_status s = check(ctx, e, "update");
+  if (s != PM_OK || ctx->L.segs.empty()) return s;
+  prof_begin(ctx, PM_PROF_UPDATE);
+  e = launch_push_small(ctx->a.w, ctx->a.delta, ctx->ta.ring, (const SmallSeg*)(ctx->ws + ctx->L.off_segs), (int)ctx->L.segs.size(), dyn_all, -1, ctx->ls, early(ctx));
+  return check(ctx, e, "weight-version push");
+}
+
+static pm_status mb_update(pm_ctx* ctx) {
+  if (!mb_updates(ctx)) return PM_OK;
   const float* gsrc = nullptr;
   if (ctx->L.stochastic > 0) {
     // stochastic delays (Appendix E): this microbatch's gradients join the ring of the last tau_max + 1; every stage's update
@@ -1097,21 +1137,7 @@ static pm_status mb_update(pm_ctx* ctx) {
     if (ce != cudaSuccess) return cuda_fail(ctx, ce, "gradient ring copy");
     gsrc = gq;
   }
-  pm_status s = run_phase(ctx, ctx->g_upd, [&]() -> pm_status {
-    // fused update: the weight gradients of all stages as one launch whose epilogue updates the Linear matrices
-    if (ctx->L.fuse) { pm_status fs = grouped_wgrad(ctx, 2 * P, true); if (fs != PM_OK) return fs; }
-    prof_begin(ctx, PM_PROF_UPDATE);
-    cudaError_t e = update_all(ctx, dyn_all, gsrc);
-    pm_status s = check(ctx, e, "update");
-    if (s != PM_OK || ctx->L.segs.empty()) return s;
-    prof_begin(ctx, PM_PROF_UPDATE);
-    e = launch_push_small(ctx->a.w, ctx->a.delta, ctx->ta.ring, (const SmallSeg*)(ctx->ws + ctx->L.off_segs), (int)ctx->L.segs.size(), dyn_all, -1, ctx->ls, early(ctx));
-    return check(ctx, e, "weight-version push");
-  });
-  if (s != PM_OK) return s;
-  ctx->tick += 1;
-  ctx->phase = 0;
-  return PM_OK;
+  return run_phase(ctx, ctx->g_upd, [&]() { return mb_update_body(ctx, gsrc); });
 }
 
 // ---- sparse ticks (tick-major order with an entry period E > 1) ----------------------------------------------------
@@ -1191,136 +1217,165 @@ static pm_status sparse_update_phase(pm_ctx* ctx) {
   });
 }
 
-pm_status pm_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
-  if (!ctx) return fail(nullptr, PM_ERR_INVALID_ARG, "null context");
-  if (ctx->phase != 0) return fail(ctx, PM_ERR_STATE, "pm_forward called out of order (expected pm_backward or pm_update)");
-  if (ctx->L.mb) return mb_forward(ctx, inputs, targets);
+// ---- a tick's launches over all stages --------------------------------------------------------------------------
+static pm_status tick_forward_body(pm_ctx* ctx) {
+  const int dt = ctx->cfg.compute_dtype;
+  pm_status s;
+  if (ctx->L.any_pre && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(next(ctx, ctx->ta), dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
+  for (int l = 0; l < ctx->L.max_lin; ++l) {
+    prof_begin(ctx, PM_PROF_GEMM_FWD);
+    cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 0, l, ctx->ls)
+                                 : umma_launch(ctx->umma, next(ctx, ctx->ta), 0, l, ctx->ls);
+    if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
+  }
+  if (ctx->attn && (s = TIMED(PM_PROF_ATTN_FWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ctx->ta), true, ctx->ls), "attention forward"))) != PM_OK) return s;
+  const int n_post = ((ctx->L.att_blocks > 0 && !ctx->attn) ? 1 : 0) + ((ctx->L.any_residual && !ctx->ta.res_fused) ? 1 : 0);
+  if (n_post && (s = TIMED(PM_PROF_POST_FWD, check(ctx, launch_post_fwd(next(ctx, ctx->ta), dt, ctx->ls, ctx->attn != nullptr), "attention / residual forward", n_post))) != PM_OK) return s;
+  return PM_OK;
+}
+
+// Within a tick a stage reads only what earlier ticks left in its rings and mailboxes, so the attention backward needs nothing of
+// the loss (which feeds the last stage), a weight gradient nothing of the input gradients, the embedding gradient nothing of the
+// LayerNorms: branches of the graph.  (One graph per tick and these branches: small encoder-decoder 80 -> 46 us, ragged 8-stage MLP
+// 62 -> 43, 32-stage MLP of width 1024 600 -> 585, 6-layer encoder 1083 -> 1030; one graph without them 75, 55, 598.)
+static pm_status tick_backward_body(pm_ctx* ctx) {
+  const int dt = ctx->cfg.compute_dtype;
+  pm_status s;
+  if (ctx->L.att_blocks > 0 && (s = branch(ctx, 1, [&]() {
+        return TIMED(PM_PROF_ATTN_BWD, check(ctx, ctx->attn ? attn_tc_launch(ctx->attn, next(ctx, ctx->ta), false, ctx->ls) : launch_post_bwd(next(ctx, ctx->ta), dt, ctx->ls), "attention backward"));
+      })) != PM_OK) return s;
+  if ((s = corr_weights(ctx, ctx->ta)) != PM_OK) return s;
+  if ((s = TIMED(PM_PROF_LOSS, check(ctx, launch_loss(next(ctx, ctx->ta), dt, ctx->ls), "loss"))) != PM_OK) return s;
+  if ((s = rejoin(ctx, 1)) != PM_OK) return s;
+  for (int l = ctx->L.max_lin - 1; l >= 0; --l) {
+    if (need_actbwd(ctx, l, -1) &&
+        (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ctx->ta), dt, l, ctx->ls), "activation backward"))) != PM_OK) return s;
+    if (!ctx->L.fuse && (s = branch(ctx, 1, [&]() {               // fused update: formed in the update phase
+          prof_begin(ctx, PM_PROF_WGRAD);
+          const cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 2, l, ctx->ls)
+                                             : umma_launch(ctx->umma, next(ctx, ctx->ta), 2, l, ctx->ls);
+          return check(ctx, e, "wgrad GEMM");
+        })) != PM_OK) return s;
+    prof_begin(ctx, PM_PROF_DGRAD);
+    const cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 1, l, ctx->ls)
+                                       : umma_launch(ctx->umma, next(ctx, ctx->ta), 1, l, ctx->ls);
+    if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
+  }
+  TickArgs ta = ctx->ta;
+  auto pre_bwd = [&]() {
+    const int n = pre_bwd_launches(ta);
+    return n ? TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(ta, dt, ctx->ls), "LayerNorm / embedding backward", n)) : PM_OK;
+  };
+  ta.any_ln = 0;
+  if ((s = branch(ctx, 2, pre_bwd)) != PM_OK) return s;
+  ta.any_ln = ctx->ta.any_ln; ta.any_embed = 0;
+  if ((s = pre_bwd()) != PM_OK) return s;
+  for (int i = 1; i <= 2; ++i) if ((s = rejoin(ctx, i)) != PM_OK) return s;
+  return PM_OK;
+}
+
+static pm_status tick_update_body(pm_ctx* ctx) {
+  cudaError_t e;
+  if (ctx->L.fuse) {
+    // the weight gradients of the stages in backward, with the update of their Linear matrices in the epilogue
+    TickArgs ta = ctx->ta;
+    ta.fuse_upd = 1;
+    prof_begin(ctx, PM_PROF_WGRAD);
+    e = umma_launch(ctx->umma, next(ctx, ta), 2, 0, ctx->ls);
+    pm_status fs = check(ctx, e, "wgrad GEMM with fused update");
+    if (fs != PM_OK) return fs;
+  }
+  prof_begin(ctx, PM_PROF_UPDATE);
+  e = update_all(ctx, (const StageDyn*)(ctx->ws + ctx->L.off_dyn), nullptr);
+  pm_status s = check(ctx, e, "update");
+  if (s != PM_OK || !ctx->L.queue || ctx->L.segs.empty()) return s;
+  prof_begin(ctx, PM_PROF_UPDATE);                                 // fp32 copies of the updated stages' small tensors into their queues
+  e = launch_push_small(ctx->a.w, ctx->a.delta, ctx->ta.ring, (const SmallSeg*)(ctx->ws + ctx->L.off_segs), (int)ctx->L.segs.size(),
+                        (const StageDyn*)(ctx->ws + ctx->L.off_dyn), -1, ctx->ls, early(ctx));
+  return check(ctx, e, "weight-version push");
+}
+
+// Takes the tick's microbatch in (or none): the schedule table and the inputs.
+static pm_status tick_begin(pm_ctx* ctx, const void* inputs, const void* targets) {
   if ((inputs == nullptr) != (targets == nullptr)) return fail(ctx, PM_ERR_INVALID_ARG, "inputs and targets must both be given or both be NULL");
   if (inputs && ctx->draining) return fail(ctx, PM_ERR_STATE, "microbatches must be fed on consecutive ticks; the pipeline is already draining");
   const int64_t mb = mb_at_tick(ctx->tick, ctx->hp.warm, ctx->hp.period, ctx->hp.entry_period);   // the microbatch that may enter now, or -1
   if (inputs && mb < 0) return fail(ctx, PM_ERR_STATE, ctx->hp.entry_period > 1 ? "a microbatch enters every entry_period ticks; this tick takes none"
                                                                                : "during the synchronous warm-up a microbatch enters every 2 * n_stages ticks; this tick takes none");
-  const int dt = ctx->cfg.compute_dtype;
-  pm_status s;
   if (inputs) ctx->n_fed = mb + 1; else if (mb >= 0) ctx->draining = true;   // an empty tick between two warm-up microbatches ends nothing
   if (ctx->fwd_pending) {                          // sparse ticks: the previous tick's forward still reads the schedule table
     cudaError_t ew = cudaStreamWaitEvent(ctx->stream, ctx->ev_fwd, 0);
     if (ew != cudaSuccess) return cuda_fail(ctx, ew, "forward stream");
     ctx->fwd_pending = false;
   }
-  s = TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn), ctx->hp, ctx->tick, ctx->n_fed, false, nullptr,
-                                                      (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, dt, inputs, targets, mb, ctx->stream), "schedule and ingest"));
-  if (s != PM_OK) return s;
-  if (sparse_ticks(ctx)) {
-    if (any_stage_active(ctx, 0, ctx->cfg.n_stages - 1) && (s = sparse_forward_phase(ctx)) != PM_OK) return s;
-    ctx->phase = 1;
-    return PM_OK;
-  }
-  // forward of every stage whose microbatch exists
-  if (any_stage_active(ctx, 0, ctx->cfg.n_stages - 1)) {
-    s = run_phase(ctx, ctx->g_fwd, [&]() -> pm_status {
-      pm_status s;
-      if (ctx->L.any_pre && (s = TIMED(PM_PROF_PRE_FWD, check(ctx, launch_pre_fwd(next(ctx, ctx->ta), dt, ctx->ls), "embedding / LayerNorm forward"))) != PM_OK) return s;
-      for (int l = 0; l < ctx->L.max_lin; ++l) {
-        prof_begin(ctx, PM_PROF_GEMM_FWD);
-        cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 0, l, ctx->ls)
-                                     : umma_launch(ctx->umma, next(ctx, ctx->ta), 0, l, ctx->ls);
-        if ((s = check(ctx, e, "forward GEMM")) != PM_OK) return s;
-      }
-      if (ctx->attn && (s = TIMED(PM_PROF_ATTN_FWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ctx->ta), true, ctx->ls), "attention forward"))) != PM_OK) return s;
-      const int n_post = ((ctx->L.att_blocks > 0 && !ctx->attn) ? 1 : 0) + ((ctx->L.any_residual && !ctx->ta.res_fused) ? 1 : 0);
-      if (n_post && (s = TIMED(PM_PROF_POST_FWD, check(ctx, launch_post_fwd(next(ctx, ctx->ta), dt, ctx->ls, ctx->attn != nullptr), "attention / residual forward", n_post))) != PM_OK) return s;
-      return PM_OK;
-    });
-    if (s != PM_OK) return s;
-  }
-  ctx->phase = 1;
-  return PM_OK;
+  return TIMED(PM_PROF_SCHEDULE, check(ctx, launch_begin((const StageSched*)(ctx->ws + ctx->L.off_sched), (StageDyn*)(ctx->ws + ctx->L.off_dyn), ctx->hp, ctx->tick, ctx->n_fed, false, nullptr,
+                                                         (const int64_t*)(ctx->ws + ctx->L.off_nupd), ctx->ta, ctx->cfg.compute_dtype, inputs, targets, mb, ctx->stream), "schedule and ingest"));
+}
+
+// forward of every stage whose microbatch exists / any backward this tick?  (Stage P runs the microbatch that entered P ticks ago, stage
+// 1 the one from 2P-1 ticks ago.)  In microbatch-major order always.
+static bool forward_active(const pm_ctx* ctx) { return ctx->L.mb || any_stage_active(ctx, 0, ctx->cfg.n_stages - 1); }
+static bool backward_active(const pm_ctx* ctx) { return ctx->L.mb || any_stage_active(ctx, ctx->cfg.n_stages, 2 * ctx->cfg.n_stages - 1); }
+static pm_status forward_body(pm_ctx* ctx) { return ctx->L.mb ? mb_forward_body(ctx) : tick_forward_body(ctx); }
+static pm_status backward_body(pm_ctx* ctx) { return ctx->L.mb ? mb_backward_body(ctx) : tick_backward_body(ctx); }
+
+static pm_status run_forward(pm_ctx* ctx) {
+  pm_status s = PM_OK;
+  if (forward_active(ctx)) s = sparse_ticks(ctx) ? sparse_forward_phase(ctx) : run_phase(ctx, ctx->g_fwd, [&]() { return forward_body(ctx); });
+  if (s == PM_OK) ctx->phase = 1;
+  return s;
+}
+
+pm_status pm_forward(pm_ctx* ctx, const void* inputs, const void* targets) {
+  if (!ctx) return fail(nullptr, PM_ERR_INVALID_ARG, "null context");
+  if (ctx->phase != 0) return fail(ctx, PM_ERR_STATE, "pm_forward called out of order (expected pm_backward or pm_update)");
+  const pm_status s = ctx->L.mb ? mb_begin(ctx, inputs, targets) : tick_begin(ctx, inputs, targets);
+  return s == PM_OK ? run_forward(ctx) : s;
 }
 
 pm_status pm_backward(pm_ctx* ctx) {
   if (!ctx) return fail(nullptr, PM_ERR_INVALID_ARG, "null context");
   if (ctx->phase != 1) return fail(ctx, PM_ERR_STATE, "pm_backward must follow pm_forward");
-  if (ctx->L.mb) return mb_backward(ctx);
-  const int dt = ctx->cfg.compute_dtype;
-  const int P = ctx->cfg.n_stages;
-  pm_status s;
-  // any backward this tick?  stage P runs the microbatch that entered P ticks ago, stage 1 the one from 2P-1 ticks ago
-  const bool any = any_stage_active(ctx, P, 2 * P - 1);
-  if (any && sparse_ticks(ctx)) {
-    if ((s = sparse_backward_phase(ctx)) != PM_OK) return s;
-  } else if (any) {
-    s = run_phase(ctx, ctx->g_bwd, [&]() -> pm_status {
-      pm_status s;
-      if ((s = corr_weights(ctx, ctx->ta)) != PM_OK) return s;
-      if ((s = TIMED(PM_PROF_LOSS, check(ctx, launch_loss(next(ctx, ctx->ta), dt, ctx->ls), "loss"))) != PM_OK) return s;
-      if (ctx->attn) { if ((s = TIMED(PM_PROF_ATTN_BWD, check(ctx, attn_tc_launch(ctx->attn, next(ctx, ctx->ta), false, ctx->ls), "attention backward"))) != PM_OK) return s; }
-      else if (ctx->L.att_blocks > 0 && (s = TIMED(PM_PROF_ATTN_BWD, check(ctx, launch_post_bwd(next(ctx, ctx->ta), dt, ctx->ls), "attention backward"))) != PM_OK) return s;
-      for (int l = ctx->L.max_lin - 1; l >= 0; --l) {
-        if (need_actbwd(ctx, l, -1) &&
-            (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ctx->ta), dt, l, ctx->ls), "activation backward"))) != PM_OK) return s;
-        cudaError_t e = cudaSuccess;
-        if (!ctx->L.fuse) {                                           // fused update: formed in the update phase
-          prof_begin(ctx, PM_PROF_WGRAD);
-          e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 2, l, ctx->ls)
-                           : umma_launch(ctx->umma, next(ctx, ctx->ta), 2, l, ctx->ls);
-          if ((s = check(ctx, e, "wgrad GEMM")) != PM_OK) return s;
-        }
-        prof_begin(ctx, PM_PROF_DGRAD);
-        e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 1, l, ctx->ls)
-                         : umma_launch(ctx->umma, next(ctx, ctx->ta), 1, l, ctx->ls);
-        if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
-      }
-      const int n_pre = pre_bwd_launches(ctx->ta);
-      if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(ctx->ta, dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
-      return PM_OK;
-    });
-    if (s != PM_OK) return s;
-  }
-  ctx->phase = 2;
-  return PM_OK;
+  pm_status s = PM_OK;
+  if (backward_active(ctx)) s = sparse_ticks(ctx) ? sparse_backward_phase(ctx) : run_phase(ctx, ctx->g_bwd, [&]() { return backward_body(ctx); });
+  if (s == PM_OK) ctx->phase = 2;
+  return s;
 }
 
 pm_status pm_update(pm_ctx* ctx) {
   if (!ctx) return fail(nullptr, PM_ERR_INVALID_ARG, "null context");
   if (ctx->phase != 2) return fail(ctx, PM_ERR_STATE, "pm_update must follow pm_backward");
-  if (ctx->L.mb) return mb_update(ctx);
-  const int P = ctx->cfg.n_stages;
-  const bool any = any_stage_active(ctx, P, 2 * P - 1);
-  if (any && sparse_ticks(ctx)) {
-    pm_status s = sparse_update_phase(ctx);
-    if (s != PM_OK) return s;
-  } else if (any) {
-    pm_status s = run_phase(ctx, ctx->g_upd, [&]() -> pm_status {
-      cudaError_t e;
-      if (ctx->L.fuse) {
-        // the weight gradients of the stages in backward, with the update of their Linear matrices in the epilogue
-        TickArgs ta = ctx->ta;
-        ta.fuse_upd = 1;
-        prof_begin(ctx, PM_PROF_WGRAD);
-        e = umma_launch(ctx->umma, next(ctx, ta), 2, 0, ctx->ls);
-        pm_status fs = check(ctx, e, "wgrad GEMM with fused update");
-        if (fs != PM_OK) return fs;
-      }
-      prof_begin(ctx, PM_PROF_UPDATE);
-      e = update_all(ctx, (const StageDyn*)(ctx->ws + ctx->L.off_dyn), nullptr);
-      pm_status s = check(ctx, e, "update");
-      if (s != PM_OK || !ctx->L.queue || ctx->L.segs.empty()) return s;
-      prof_begin(ctx, PM_PROF_UPDATE);                                 // fp32 copies of the updated stages' small tensors into their queues
-      e = launch_push_small(ctx->a.w, ctx->a.delta, ctx->ta.ring, (const SmallSeg*)(ctx->ws + ctx->L.off_segs), (int)ctx->L.segs.size(),
-                            (const StageDyn*)(ctx->ws + ctx->L.off_dyn), -1, ctx->ls, early(ctx));
-      return check(ctx, e, "weight-version push");
-    });
-    if (s != PM_OK) return s;
-  }
+  pm_status s = PM_OK;
+  if (ctx->L.mb) s = mb_update(ctx);
+  else if (backward_active(ctx)) s = sparse_ticks(ctx) ? sparse_update_phase(ctx) : run_phase(ctx, ctx->g_upd, [&]() { return tick_update_body(ctx); });
+  if (s != PM_OK) return s;
   ctx->tick += 1;
   ctx->phase = 0;
   return PM_OK;
 }
 
+// The three phases in one call.  Where all of them run, they are one graph: between two graphs the GPU is idle for about 3 us, a tenth
+// of a small network's tick.
 pm_status pm_step(pm_ctx* ctx, const void* inputs, const void* targets) {
-  pm_status s = pm_forward(ctx, inputs, targets);
+  if (!ctx) return fail(nullptr, PM_ERR_INVALID_ARG, "null context");
+  if (ctx->phase != 0) return fail(ctx, PM_ERR_STATE, "pm_forward called out of order (expected pm_backward or pm_update)");
+  pm_status s = ctx->L.mb ? mb_begin(ctx, inputs, targets) : tick_begin(ctx, inputs, targets);
   if (s != PM_OK) return s;
+  if (forward_active(ctx) && backward_active(ctx) && !sparse_ticks(ctx) && ctx->L.stochastic == 0 && ctx->graphs && !ctx->prof_on) {
+    const bool upd = !ctx->L.mb || mb_updates(ctx);
+    s = run_phase(ctx, upd ? ctx->g_step : ctx->g_part, [&]() {
+      // a tick's forward and backward are branches, too: the rings keep their slots apart
+      pm_status s = ctx->L.mb ? forward_body(ctx) : branch(ctx, 0, [&]() { return forward_body(ctx); });
+      if (s == PM_OK) s = backward_body(ctx);
+      if (s == PM_OK) s = rejoin(ctx, 0);
+      if (s == PM_OK && upd) s = ctx->L.mb ? mb_update_body(ctx, nullptr) : tick_update_body(ctx);
+      return s;
+    });
+    if (s != PM_OK) { ctx->phase = 1; return s; }
+    ctx->tick += 1;
+    return PM_OK;
+  }
+  if ((s = run_forward(ctx)) != PM_OK) return s;
   if ((s = pm_backward(ctx)) != PM_OK) return s;
   return pm_update(ctx);
 }
