@@ -245,7 +245,7 @@ __device__ __forceinline__ float f32_sum8(const float* p, int stride) {
 }
 
 template <int TM, int TN, int NBUF, int MODE>
-__global__ void __launch_bounds__(256) f32_gemm_kernel(TickArgs t, int lvl) {
+__global__ void __launch_bounds__(256, 2) f32_gemm_kernel(TickArgs t, int lvl) {
   using C = F32Cfg<TM, TN, NBUF, MODE>;
   constexpr int BM = C::BM, BN = C::BN, KC = kF32KC;
   pdl_trigger();
@@ -425,12 +425,15 @@ static cudaError_t launch_f32_t(const TickArgs& t, int lvl, uint64_t tiles, cuda
   return launch_pdl(f32_gemm_kernel<TM, TN, NBUF, MODE>, dim3((unsigned)tiles, t.sel_p >= 0 ? 1 : t.P), dim3(256), C::kBytes, stream, t.pdl, t, lvl);
 }
 
+// The instances: small tiles with one chunk per warp in flight, two, or the most that leave two blocks on an SM; large tiles with one or two.
+#define PM_F32_INSTANCES(X) X(4, 2, 1, 0) X(4, 2, 2, 0) X(4, 2, 4, 0) X(4, 2, 1, 1) X(4, 2, 2, 1) X(4, 2, 3, 1) X(4, 2, 1, 2) X(4, 2, 2, 2) X(4, 2, 4, 2) \
+                            X(8, 4, 1, 0) X(8, 4, 2, 0) X(8, 4, 1, 1) X(8, 4, 2, 1) X(8, 4, 1, 2) X(8, 4, 2, 2)
+
 // opt-in shared-memory sizes, on the current device
 cudaError_t simt_gemm_set_limits() {
   cudaError_t e = cudaSuccess;
-#define PM_F32_LIMIT(TM, TN, NB, MODE) if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)f32_gemm_kernel<TM, TN, NB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Cfg<TM, TN, NB, MODE>::kBytes)
-  PM_F32_LIMIT(4, 2, 4, 0); PM_F32_LIMIT(4, 2, 3, 1); PM_F32_LIMIT(4, 2, 4, 2);
-  PM_F32_LIMIT(8, 4, 2, 0); PM_F32_LIMIT(8, 4, 2, 1); PM_F32_LIMIT(8, 4, 2, 2);
+#define PM_F32_LIMIT(TM, TN, NB, MODE) if (e == cudaSuccess) e = cudaFuncSetAttribute((const void*)f32_gemm_kernel<TM, TN, NB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Cfg<TM, TN, NB, MODE>::kBytes);
+  PM_F32_INSTANCES(PM_F32_LIMIT)
 #undef PM_F32_LIMIT
   return e;
 }
@@ -440,20 +443,29 @@ cudaError_t simt_gemm_set_limits() {
 // Tiles are counted over the launch's own Linears.  (Sized by the widest Linear of the network, the launches of a network with a
 // large vocabulary were mostly blocks without a tile: a tick of a 6-layer encoder of width 64, 64 rows and a vocabulary of
 // 8000 took 2368 us and takes 211, of a 2-layer one of width 64, 384 rows and a vocabulary of 1000 165 and 152.)
+// A warp has at most as many chunks of the reduction in flight as it owns (one in eight): a panel it never fills is shared memory
+// that the blocks of the launches beside it could use.  (A tick of the 4-stage MLP, whose forward, input and weight gradients run side
+// by side, 33.0 -> 31.9 us.)
 cudaError_t launch_simt_gemm(const TickArgs& t, const std::vector<StageDev>& st, int mode, int lvl, cudaStream_t stream) {
   uint64_t all32 = 0, most32 = 1, most16 = 1;
+  int chunks = 1;                                          // of the deepest reduction, per warp
   for (int p = t.sel_p >= 0 ? t.sel_p : 0; p < (t.sel_p >= 0 ? t.sel_p + 1 : t.P); ++p) {
     if (lvl >= st[p].n_lin || (mode == 1 && p == 0 && lvl == 0 && st[p].pre != PRE_EMBED)) continue;
     const LinDev& L = st[p].lin[lvl];
     const uint64_t M = mode == 2 ? L.n_out : t.T, N = mode == 0 ? L.n_out : L.n_in;
+    const int K = mode == 2 ? t.T : (mode == 0 ? L.n_in : L.n_out);
     const uint64_t n32 = ((M + 31) / 32) * ((N + 31) / 32);
     all32 += n32;
     most32 = std::max(most32, n32);
     most16 = std::max(most16, ((M + 15) / 16) * ((N + 15) / 16));
+    chunks = std::max(chunks, (K + 8 * kF32KC - 1) / (8 * kF32KC));
   }
-  if (all32 <= kSms)
-    return mode == 0 ? launch_f32_t<4, 2, 4, 0>(t, lvl, most16, stream) : (mode == 1 ? launch_f32_t<4, 2, 3, 1>(t, lvl, most16, stream) : launch_f32_t<4, 2, 4, 2>(t, lvl, most16, stream));
-  return mode == 0 ? launch_f32_t<8, 4, 2, 0>(t, lvl, most32, stream) : (mode == 1 ? launch_f32_t<8, 4, 2, 1>(t, lvl, most32, stream) : launch_f32_t<8, 4, 2, 2>(t, lvl, most32, stream));
+  const bool small = all32 <= kSms;
+  const int tm = small ? 4 : 8, nb = chunks <= 2 ? chunks : (small ? (mode == 1 ? 3 : 4) : 2);
+#define PM_F32_LAUNCH(TM, TN, NB, MODE) if (tm == TM && nb == NB && mode == MODE) return launch_f32_t<TM, TN, NB, MODE>(t, lvl, small ? most16 : most32, stream);
+  PM_F32_INSTANCES(PM_F32_LAUNCH)
+#undef PM_F32_LAUNCH
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace pm
