@@ -902,6 +902,7 @@ static pm_status rejoin(pm_ctx* ctx, int i) {
   ctx->side_used[i] = false;
   cudaError_t e = cudaEventRecord(ctx->side_ev, ctx->side[i]);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->ls, ctx->side_ev, 0);
+  ctx->chained = false;                 // the next launch follows two others: a plain one
   return e == cudaSuccess ? PM_OK : cuda_fail(ctx, e, "graph branch");
 }
 
@@ -1103,8 +1104,10 @@ static cudaError_t update_all(pm_ctx* ctx, const StageDyn* dyn, const float* gsr
   void* lp = ctx->L.queue ? (void*)ctx->ta.ring : nullptr;
   if (ctx->L.fuse)
     return launch_update_parts(ctx->a, ctx->L.parts, (const UpdPart*)(ctx->ws + ctx->L.off_parts), dyn, nupd, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, early(ctx));
+  // (a long update does not start early: its first blocks would sit beside the weight gradients instead of walking the arenas in order;
+  // 67 M parameters, SGD-m: 383 us early, 307 behind them)
   return launch_update(ctx->a, (const uint32_t*)(ctx->ws + ctx->L.off_b64), (const uint32_t*)(ctx->ws + ctx->L.off_e64), dyn, nupd, g.n_stages,
-                       ctx->L.total / 64, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, ctx->hp.lp_elem, 0, gsrc, early(ctx));
+                       ctx->L.total / 64, g.optimizer, g.beta1, g.beta2, g.eps, ctx->ls, lp, ctx->hp.lp_elem, 0, gsrc, early(ctx) && update_is_short(ctx->L.total / 64));
 }
 
 // Inside a minibatch the gradients stay in the arena and the next microbatch adds to them.

@@ -437,6 +437,8 @@ UpdParts update_parts(const uint32_t* begin64, const uint32_t* end64, const uint
   return p;
 }
 
+bool update_is_short(uint64_t groups64) { return few_chunks(groups64 * 16); }
+
 cudaError_t launch_update(ArenasDev a, const uint32_t* begin64, const uint32_t* end64, const StageDyn* dyn,
                           int64_t* nupd, int n_stages, uint64_t total64, int optimizer, float beta1, float beta2,
                           float eps, cudaStream_t stream, void* lp_base, int lp_elem, uint64_t first64, const float* gsrc, bool pdl) {

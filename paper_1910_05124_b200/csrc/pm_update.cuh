@@ -28,6 +28,8 @@ struct TickArgs;
 // delays (stochastic delay model only, else null): the step's per-stage delays.  nupd: the stages' update counters.
 cudaError_t launch_begin(const StageSched* sched, StageDyn* dyn, HyperDev hp, int64_t tick, int64_t n_fed, bool mb_order, const int32_t* delays,
                          const int64_t* nupd, const TickArgs& t, int dtype, const void* inputs, const void* targets, int64_t mb, cudaStream_t stream);
+// Is the update of that many groups of 64 elements a few waves of blocks?
+bool update_is_short(uint64_t groups64);
 // Stand-alone update: bounds, scalars of update index k and zeroed counters of hp.n_stages stages into device tables.
 struct FlatStage { uint32_t begin64, end64; int32_t tau_f, gap; };
 template <int N> struct FlatTable { uint32_t begin64[N], end64[N]; int32_t tau_f[N], gap[N]; };
