@@ -560,6 +560,9 @@ struct pm_ctx {
   cudaStream_t side[kSides] = {};
   cudaEvent_t side_ev = nullptr;
   bool capturing = false, side_used[kSides] = {};
+  // what pm_get_losses reads back in one go: page-locked host memory [kReport losses | two status words]
+  static constexpr int kReport = 1024;
+  float* report = nullptr;
   ~pm_ctx() {
     for (PhaseGraph* g : {&g_fwd, &g_bwd, &g_upd, &g_step, &g_part}) if (g->exec) cudaGraphExecDestroy(g->exec);
     for (auto* v : {&gs_fwd, &gs_bwd, &gs_upd}) for (auto& g : *v) if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -568,6 +571,7 @@ struct pm_ctx {
     if (ev_fwd) cudaEventDestroy(ev_fwd);
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (auto st : side) if (st) cudaStreamDestroy(st);
+    if (report) cudaFreeHost(report);
     if (side_ev) cudaEventDestroy(side_ev);
   }
   // optional per-kernel-class timing with CUDA events on the context's stream
@@ -1383,6 +1387,9 @@ pm_status pm_step(pm_ctx* ctx, const void* inputs, const void* targets) {
   return pm_update(ctx);
 }
 
+static pm_status status_error(pm_ctx* ctx, int code) {
+  return fail(ctx, PM_ERR_TIMEOUT, "a bounded device-side wait expired in a tensor-core kernel (role code " + std::to_string(code) + ")");
+}
 // After a synchronisation: did any CTA give up on a bounded wait?
 static pm_status check_device_status(pm_ctx* ctx) {
   int* words[2] = {umma_status_word(ctx->umma), attn_status_word(ctx->attn)};
@@ -1391,7 +1398,7 @@ static pm_status check_device_status(pm_ctx* ctx) {
     int code = 0;
     cudaError_t e = cudaMemcpy(&code, w, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "status read-back");
-    if (code != 0) return fail(ctx, PM_ERR_TIMEOUT, "a bounded device-side wait expired in a tensor-core kernel (role code " + std::to_string(code) + ")");
+    if (code != 0) return status_error(ctx, code);
   }
   return PM_OK;
 }
@@ -1456,12 +1463,25 @@ pm_status pm_get_losses(pm_ctx* ctx, float* host_out, int64_t first_mb, int64_t 
   const int64_t done = ctx->L.mb ? ctx->n_fed - (ctx->phase == 1 ? 1 : 0) : std::min<int64_t>(ctx->n_fed, entered);
   if (first_mb + n > done) return fail(ctx, PM_ERR_INVALID_ARG, "loss of a microbatch that has not finished was requested");
   if (done - first_mb > ctx->L.loss_cap) return fail(ctx, PM_ERR_INVALID_ARG, "requested losses have left the device log");
-  cudaError_t e = cudaStreamSynchronize(ctx->stream);
-  if (e == cudaSuccess && ctx->fwd_stream) e = cudaStreamSynchronize(ctx->fwd_stream);
-  for (int64_t i = 0; i < n && e == cudaSuccess; ++i)
-    e = cudaMemcpy(host_out + i, ctx->ws + ctx->L.off_loss + sizeof(float) * ((first_mb + i) % ctx->L.loss_cap), sizeof(float), cudaMemcpyDeviceToHost);
+  // One kernel gathers the losses and the status words into page-locked host memory, behind the steps so far: a copy of its own for
+  // each of them is a round trip of about 9 us with the GPU idle.  (A logged update of the ragged 2-layer encoder 266 -> 235 us, of the
+  // 6-stage fp32 MLP 273 -> 232.)
+  cudaError_t e = cudaSuccess;
+  if (ctx->fwd_stream) e = cudaStreamSynchronize(ctx->fwd_stream);
+  if (e == cudaSuccess && !ctx->report) e = cudaHostAlloc((void**)&ctx->report, (pm_ctx::kReport + 2) * sizeof(float), cudaHostAllocMapped);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "loss read-back");
-  if (pm_status ds = check_device_status(ctx)) return ds;
+  for (int64_t i = 0; i < n || i == 0; i += pm_ctx::kReport) {      // n = 0: the status words
+    const int m = (int)std::min<int64_t>(n - i, pm_ctx::kReport);
+    e = launch_report((const float*)(ctx->ws + ctx->L.off_loss), first_mb + i, m, ctx->L.loss_cap, umma_status_word(ctx->umma), attn_status_word(ctx->attn), ctx->report, pm_ctx::kReport, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "loss read-back");
+    std::memcpy(host_out + i, ctx->report, sizeof(float) * (size_t)m);
+    for (int w = 0; w < 2; ++w) {
+      int code;
+      std::memcpy(&code, ctx->report + pm_ctx::kReport + w, sizeof(int));
+      if (code != 0) return status_error(ctx, code);
+    }
+  }
   return PM_OK;
 }
 

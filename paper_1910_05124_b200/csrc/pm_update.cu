@@ -267,6 +267,21 @@ cudaError_t launch_begin(const StageSched* sched, StageDyn* dyn, HyperDev hp, in
   return cudaGetLastError();
 }
 
+// ---- read-back ------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) report_kernel(const float* log, int64_t first, int n, int64_t cap, const int* status0, const int* status1, float* host, int words) {
+  for (int i = (int)threadIdx.x; i < n; i += 128) host[i] = log[(first + i) % cap];
+  if (threadIdx.x < 2) {
+    const int* w = threadIdx.x == 0 ? status0 : status1;
+    reinterpret_cast<int*>(host)[words + threadIdx.x] = w ? *w : 0;
+  }
+  __threadfence_system();
+}
+
+cudaError_t launch_report(const float* log, int64_t first, int n, int64_t cap, const int* status0, const int* status1, float* host, int words, cudaStream_t stream) {
+  report_kernel<<<1, 128, 0, stream>>>(log, first, n, cap, status0, status1, host, words);
+  return cudaGetLastError();
+}
+
 // ---- stand-alone update: stage tables ------------------------------------------------------------------------
 // The caller's stage split comes as a kernel argument (no copy from pageable host memory in front of the launch); the kernel
 // writes the bounds, the scalars of update index k and zeroed counters into the workspace.

@@ -30,6 +30,9 @@ cudaError_t launch_begin(const StageSched* sched, StageDyn* dyn, HyperDev hp, in
                          const int64_t* nupd, const TickArgs& t, int dtype, const void* inputs, const void* targets, int64_t mb, cudaStream_t stream);
 // Is the update of that many groups of 64 elements a few waves of blocks?
 bool update_is_short(uint64_t groups64);
+// Losses of microbatches first .. first + n - 1 from the log (a ring of `cap`) and up to two status words (null: 0) into host memory the
+// device can write: host[0 .. n) and host[words], host[words + 1].
+cudaError_t launch_report(const float* log, int64_t first, int n, int64_t cap, const int* status0, const int* status1, float* host, int words, cudaStream_t stream);
 // Stand-alone update: bounds, scalars of update index k and zeroed counters of hp.n_stages stages into device tables.
 struct FlatStage { uint32_t begin64, end64; int32_t tau_f, gap; };
 template <int N> struct FlatTable { uint32_t begin64[N], end64[N]; int32_t tau_f[N], gap[N]; };
