@@ -607,7 +607,8 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
       const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl, mrow, nb, lane);
       // (written by the forward phase, which this launch's predecessors ended: read behind the wait)
       const uint2 mask = MODE == 1 && et.mask && mrow < M && nb < N ? *et.mask : make_uint2(0u, 0u);
-      const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
+      const float* bias = et.bias;
+      const float2 bias2 = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
       const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
       if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
       const bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 4);
@@ -615,7 +616,7 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
       if (fetch && go) go = es.fetched(abort_flag, status);
       if (!go) { if (fetch) es.drain(); return false; }
       tc_fence_after();
-      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias, mask, [&] {
+      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias2, mask, [&] {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8 * acc.idx);         // the accumulator buffer may be overwritten now
@@ -797,7 +798,8 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
       const EpiTile et = epi_tile<MODE>(t, s, d, L, tl.p, lvl, mrow, nb, lane);
       // (written by the forward phase, which this launch's predecessors ended: read behind the wait)
       const uint2 mask = MODE == 1 && et.mask && mrow < M && nb < N ? *et.mask : make_uint2(0u, 0u);
-      const float2 bias = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(et.bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
+      const float* bias = et.bias;
+      const float2 bias2 = MODE == 0 && nb + 2 * lane < N ? __ldg(reinterpret_cast<const float2*>(bias + nb + 2 * lane)) : make_float2(0.f, 0.f);
       const bool fetch = MODE == 0 && et.resid && mrow < M && nb < N;
       if (fetch) es.fetch(lm + MAP_SKIP, nb, mrow, et.skip_slot);
       const bool ready = mbar_wait(bar_tfull + 8 * acc.idx, acc.phase, abort_flag, status, 34);
@@ -807,7 +809,7 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
       tc_fence_after();
 #pragma unroll 1
       for (int u = 0; u < UNITS; ++u) {                               // (MODE 0: one)
-        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias, mask, [&] {
+        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias2, mask, [&] {
           if (u != UNITS - 1) return;
           tc_fence_before();
           __syncwarp();
@@ -1125,7 +1127,7 @@ struct CorrBlock { uint32_t src64, dst64, n64; int32_t stage; };      // in grou
 constexpr int CORR_THREADS = 256, CORR_GROUPS = 4;                    // groups of eight elements per thread
 constexpr uint32_t CORR_N64 = CORR_THREADS * CORR_GROUPS * 8 / 64;
 
-__global__ void __launch_bounds__(CORR_THREADS) corr_weights_kernel(TickArgs t, const CorrBlock* __restrict__ list) {
+__global__ void __launch_bounds__(CORR_THREADS) corr_weights_kernel(TickArgs t, const CorrBlock* list) {
   pdl_trigger();
   pdl_wait();
   const CorrBlock b = list[blockIdx.x];
