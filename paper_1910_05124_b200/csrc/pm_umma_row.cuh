@@ -160,21 +160,22 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) umma_row_kernel(TickArgs t, co
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc_mn(ROW_M, BN, 0, 0);
-      const uint64_t base = desc_base(16, 1024);
-      bool ok = true;
-      for (int i = 0; i < n_kb; ++i) {
-        const int st = i % NS;
-        if (!mbar_wait(bar_full + 8 * st, (uint32_t)(i / NS) & 1u, abort_flag, status, 62)) { ok = false; break; }
-        tc_fence_after();
+    const uint32_t idesc = make_idesc_mn(ROW_M, BN, 0, 0);
+    const uint64_t base = desc_base(16, 1024);
+    for (int i = 0; i < n_kb; ++i) {
+      const int st = i % NS;
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * st, (uint32_t)(i / NS) & 1u, abort_flag, status, 62))) break;
+      tc_fence_after();
+      if (elect_one()) {
 #pragma unroll
         for (int k16 = 0; k16 < ROW_K / 16; ++k16)
           tc_mma_bf16(tmem, desc_at(base, tiles + st * C::kA + k16 * 32), desc_at(base, sB + st * C::kB + k16 * 32), idesc, (i > 0 || k16 > 0) ? 1u : 0u);
         tc_commit(bar_empty + 8 * st);
+        if (i == n_kb - 1) tc_commit(bar_acc);
       }
-      if (ok) tc_commit(bar_acc);
+      __syncwarp();
     }
+    if (n_kb == 0 && lane == 0) tc_commit(bar_acc);
   } else {
     const int w = warp - 2;
     if (MODE != 0) {
