@@ -753,6 +753,8 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
     const int32_t* ids = (const int32_t*)(c->ws + L.off_ids);
     t.pre_ids = ids; t.ln_ids = ids + P; t.embed_ids = ids + 2 * P; t.res_ids = ids + 3 * P;
     t.n_pre = L.n_pre; t.n_ln = L.n_ln; t.n_embed = L.n_embed; t.n_res = L.n_res;
+    t.pre_dim = L.n_pre > 0 ? L.st[L.ids[0]].d_in : 0;
+    for (int i = 0; i < L.n_pre; ++i) if (L.st[L.ids[i]].d_in != t.pre_dim) t.pre_dim = 0;
     t.lnred_off = L.off_lnred; t.ln_chunks = L.ln_chunks; t.ln_chunk_rows = L.ln_chunk_rows; t.max_ln_dim = L.max_ln_dim;
     t.ln_fused = L.ln_fused;
     t.act_start = ids + 4 * P;
@@ -1031,7 +1033,7 @@ static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool gro
     if ((s = check(ctx, e, "dgrad GEMM")) != PM_OK) return s;
   }
   const int n_pre = sd.pre != PRE_NONE ? pre_bwd_launches(ta) : 0;
-  if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(ta, dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
+  if (n_pre && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_pre_bwd(next(ctx, ta), dt, ctx->ls), "LayerNorm / embedding backward", n_pre))) != PM_OK) return s;
   return PM_OK;
 }
 

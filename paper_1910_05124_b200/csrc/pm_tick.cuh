@@ -39,6 +39,7 @@ struct TickArgs {
   // embedding, with a residual add; grids have one block row per list entry
   const int32_t* pre_ids; const int32_t* ln_ids; const int32_t* embed_ids; const int32_t* res_ids;
   int32_t n_pre, n_ln, n_embed, n_res;
+  int32_t pre_dim;        // width of every pre-op, if they share one (else 0)
   uint64_t lnred_off;     // ws: LayerNorm parameter-gradient partials [n_ln][ln_chunks][2*max_ln_dim] float
   int32_t ln_chunks, ln_chunk_rows, max_ln_dim;
   // activation-backward launches: column blocks (act_cols columns) of Linear `lvl` over all stages, flattened;
