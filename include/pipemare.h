@@ -183,9 +183,9 @@ typedef struct {
                                     further slots of the stage's version queue (counted by pm_query_bytes). */
   int32_t fuse_update;           /* 1: the weight-gradient GEMM of a Linear applies the update of its matrix in its epilogue,
                                     while dW is still on chip (same arithmetic per element, bit for bit; dW of Linear matrices
-                                    is then NOT written to arenas.grad).  The weight-gradient GEMMs move from pm_backward to
-                                    pm_update, whose update kernel covers the remaining parameters (biases, LayerNorm
-                                    parameters, embedding tables).  Needs PM_BF16, one Linear per stage, n_micro <= 1,
+                                    is then NOT written to arenas.grad).  The weight-gradient GEMMs, and with them the bias
+                                    gradients they sum, move from pm_backward to pm_update, whose update kernel covers the
+                                    remaining parameters (biases, LayerNorm parameters, embedding tables).  Needs PM_BF16, one Linear per stage, n_micro <= 1,
                                     entry_period <= 1 and recompute_segment = 0, else PM_ERR_UNSUPPORTED.  0: off. */
   int32_t stochastic_tau_max;    /* > 0: the stage-wise stochastic delay model of Appendix E instead of the pipeline's fixed delays:
                                       w_{i,t+1} = w_{i,t} - alpha [grad f_{t-tau_i}(w_{t-tau_i})]_i,   tau_i drawn per step and stage.
@@ -198,8 +198,9 @@ typedef struct {
                                     pm_stage_desc.tau_fwd is the delay T1 divides by (the mean of the stage's distribution),
                                     tau_bkwd must be 0 and T2 has nothing to correct.  Needs PM_MB_MAJOR, n_micro <= 1,
                                     recompute_segment = 0, fuse_update = 0, else PM_ERR_UNSUPPORTED.  0: off. */
-  int32_t materialize_backward;  /* 0 (default): the T2-corrected backward weights w - tau delta exist only inside the dgrad
-                                    kernel, formed while the operand is loaded; no second copy of the weights is kept.
+  int32_t materialize_backward;  /* 0 (default): the T2-corrected backward weights w - tau delta are formed in the backward pass
+                                    that reads them, while the dgrad operand is loaded or (bfloat16, many rows) into the
+                                    workspace at its start; no second copy of the weights is kept from call to call.
                                     1: the update that produces version v also writes bf16(w_v - tau delta_v) (fp32 with
                                     PM_F32) into one more slot of the stage's version queue, and the backward pass of the next
                                     step reads that copy: dgrad becomes a plain GEMM.  The same bits in every result (the
