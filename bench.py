@@ -597,7 +597,7 @@ def measure(args, workload, world, rank, local, device, sampler=None, with_e2e=T
 
 GEMM_KERNELS = {"gemm_fwd": "umma_pair_gemm_kernel<0> / umma_gemm_kernel<0> (forward GEMMs)",
                 "wgrad": "umma_pair_gemm_kernel<2> / umma_gemm_kernel<2> (wgrad GEMMs)",
-                "dgrad": "umma_dgrad_pair_kernel / umma_dgrad_kernel (dgrad GEMMs, weights corrected while loading)"}
+                "dgrad": "corr_weights_kernel + umma_pair_gemm_kernel<1>, or umma_dgrad_kernel (dgrad GEMMs and the corrected weights they read)"}
 
 
 def rooflines(res, peaks, steps):
@@ -637,7 +637,7 @@ def rooflines(res, peaks, steps):
             kname = "umma_pair_gemm_kernel<1> / umma_gemm_kernel<1> (dgrad as a plain GEMM against a queued operand copy)"
         ratio, note = NCU_TRAFFIC[cls + "_ratio"], "DRAM bytes per launch, scaled from the ncu capture of the 2-layer cut of cfg4 by algorithmic bytes"
         if cls == "dgrad" and res.get("order") == "mb_major" and not res.get("plain_dgrad") and wl.kind == "encoder":
-            kname = "umma_dgrad_pair128_kernel / umma_dgrad_pair_kernel (dgrad of one stage per launch, weights corrected while loading)"
+            kname = "corr_weights_kernel + umma_pair_gemm_kernel<1> (dgrad of one stage per launch and the corrected weights it reads)"
             ratio, note = NCU_TRAFFIC["dgrad_one_stage_ratio"], "DRAM bytes per launch, scaled from the ncu capture of one-stage launches on config 5's widths (1 + 1 layers) by algorithmic bytes"
         out[cls] = {"kernel": kname, "bound": "tensor", "achieved": round(tfs, 1), "peak": tf_peak, "unit": "TFLOP/s",
                     "frac": round(tfs / tf_peak, 4), "of": f"{peaks['kind']} ({tf_kind} bf16 matmul; the median SM clock of the timed region decides)",
