@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "pm_copy_parity.cuh"
 #include "pm_ptx.cuh"
 #include "pm_umma.cuh"
 #include "pm_update_math.cuh"
@@ -69,7 +70,7 @@ struct EpiStage {
   uint8_t* buf; uint32_t buf_s; int lane;
   uint32_t bar;               // counts the skip tensor's copies into the box
   uint32_t off = 0;           // the box written next
-  uint32_t phase = 0;         // parity of the next copy
+  CopyParity copy{};          // of those copies
   bool stored = false;
   // the box's earlier store has finished reading it
   __device__ __forceinline__ uint8_t* begin() {
@@ -90,14 +91,12 @@ struct EpiStage {
     if (lane == 0) { mbar_arrive_expect_tx(bar, 4096); tma_load_3d(buf_s + off, map, bar, n, m, slot); }
   }
   __device__ __forceinline__ bool fetched(volatile int* abort_flag, int* status) {
-    const bool ok = mbar_wait(bar, phase, abort_flag, status, 11);
-    phase ^= 1u;
-    return __all_sync(0xffffffffu, ok);
+    return copy.await([&](uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, 11)) != 0; });
   }
   // a CTA that gives up: the copy still lands here (bounded wait)
   __device__ __forceinline__ void drain() {
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, phase) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+    copy.drain([&](uint32_t parity) { return mbar_try_wait(bar, parity); }, [&] { return clock64() - t0 < WAIT_LIMIT_CYCLES; });
   }
 };
 
