@@ -173,7 +173,7 @@ __device__ __forceinline__ void epi_update_block(const TickArgs& t, const StageD
 // memory clobber would make the compiler read the tables again.
 struct EpiTile {
   int flags, act;             // MODE 0: LF_* and PM_ACT_* of the Linear
-  bool resid;                 // MODE 0: the stage adds its skip tensor here, from slot skip_slot of its buffer
+  bool resid;                 // MODE 0: the stage adds its skip tensor to z here, from slot skip_slot of its buffer
   int skip_slot;
   int slot;                   // ring slot of z (MODE 0) or dx (MODE 1); MODE 2: gradients add to the arena
   int yslot;                  // MODE 0: ring slot of y, or of the fp32 logits
@@ -218,7 +218,7 @@ __device__ __forceinline__ EpiTile epi_tile(const TickArgs& t, const StageDev& s
 // bias: that of columns 2 l and 2 l + 1 in lane l.  mask: this row's mask bits where a ReLU's backward is applied (MODE 1).  (With one column per instruction the
 // forward of the 6-layer encoder's tick took 194 us, 164 now; reading the skip values row by row into registers 172.)
 template <int MODE, bool FUSE, int SLOTS, class Release>
-__device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* lm, const StageDyn& d, const LinDev& L, const EpiTile& et,
+__device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* lm, const StageDev& s, const StageDyn& d, const LinDev& L, const EpiTile& et,
                                          int M, int N, int mrow, int nb, uint32_t taddr, EpiStage<SLOTS>& es,
                                          const float2 bias, const uint2 mask, Release release) {
   const int lane = es.lane;
@@ -313,6 +313,9 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
     else if (et.flags & LF_WRITE_Y) tma_store_3d(lm + MAP_Y_OUT, src, nb, mrow, et.yslot);
   });
   if (!both) return;
+  // With an activation in front of a residual add the skip tensor joins y: out = bf16(skip + y).  (Read plainly, a row per lane: the
+  // box holds z, and none of the networks this library's configurations describe has such a stage.)
+  const __nv_bfloat16* skip = s.post == POST_RESIDUAL && mrow + lane < M ? ws_at<__nv_bfloat16>(t, s.skip_in) + ((uint64_t)et.skip_slot * M + mrow + lane) * N + nb : nullptr;
   uint8_t* ybox = es.begin();                                     // one slot: z's own box, which its store has read by now
   auto write_y = [&](auto a) {
     constexpr int ACT = decltype(a)::value;
@@ -325,6 +328,10 @@ __device__ __forceinline__ void epi_unit(const TickArgs& t, const CUtensorMap* l
       for (int e = 0; e < 4; ++e) {
         const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&o[e]));
         if (ACT != PM_ACT_NONE) o[e] = pack_bf16(act_fwd(f.x, ACT), act_fwd(f.y, ACT));
+      }
+      if (skip && nb + 8 * g < N) {                                 // widths are multiples of 8
+        const uint4 k = ld_chain16(skip + 8 * g);
+        o[0] = add_bf16x2(k.x, o[0]); o[1] = add_bf16x2(k.y, o[1]); o[2] = add_bf16x2(k.z, o[2]); o[3] = add_bf16x2(k.w, o[3]);
       }
       *reinterpret_cast<uint4*>(ybox + off) = make_uint4(o[0], o[1], o[2], o[3]);
     }
@@ -615,7 +622,7 @@ umma_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __
       if (fetch && go) go = es.fetched(abort_flag, status);
       if (!go) { if (fetch) es.drain(); return false; }
       tc_fence_after();
-      epi_unit<MODE, FUSE, 2>(t, lm, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias2, mask, [&] {
+      epi_unit<MODE, FUSE, 2>(t, lm, s, d, L, et, M, N, mrow, nb, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * ACC_COLS + half * 64), es, bias2, mask, [&] {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8 * acc.idx);         // the accumulator buffer may be overwritten now
@@ -808,7 +815,7 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
       tc_fence_after();
 #pragma unroll 1
       for (int u = 0; u < UNITS; ++u) {                               // (MODE 0: one)
-        epi_unit<MODE, FUSE, 1>(t, lm, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias2, mask, [&] {
+        epi_unit<MODE, FUSE, 1>(t, lm, s, d, L, et, M, N, mrow, nb + 64 * u, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc.idx * P2_ACC_COLS + (part + u) * 64), es, bias2, mask, [&] {
           if (u != UNITS - 1) return;
           tc_fence_before();
           __syncwarp();
