@@ -183,9 +183,9 @@ typedef struct {
                                     further slots of the stage's version queue (counted by pm_query_bytes). */
   int32_t fuse_update;           /* 1: the weight-gradient GEMM of a Linear applies the update of its matrix in its epilogue,
                                     while dW is still on chip (same arithmetic per element, bit for bit; dW of Linear matrices
-                                    is then NOT written to arenas.grad).  The weight-gradient GEMMs, and with them the bias
-                                    gradients they sum, move from pm_backward to pm_update, whose update kernel covers the
-                                    remaining parameters (biases, LayerNorm parameters, embedding tables).  Needs PM_BF16, one Linear per stage, n_micro <= 1,
+                                    is then NOT written to arenas.grad).  The weight-gradient GEMMs move from pm_backward to
+                                    pm_update, whose update kernel covers the remaining parameters (biases, LayerNorm
+                                    parameters, embedding tables).  Needs PM_BF16, one Linear per stage, n_micro <= 1,
                                     entry_period <= 1 and recompute_segment = 0, else PM_ERR_UNSUPPORTED.  0: off. */
   int32_t stochastic_tau_max;    /* > 0: the stage-wise stochastic delay model of Appendix E instead of the pipeline's fixed delays:
                                       w_{i,t+1} = w_{i,t} - alpha [grad f_{t-tau_i}(w_{t-tau_i})]_i,   tau_i drawn per step and stage.

@@ -1004,6 +1004,11 @@ static pm_status corr_weights(pm_ctx* ctx, const TickArgs& ta) {
   return TIMED(PM_PROF_DGRAD, check(ctx, umma_corr_launch(ctx->umma, next(ctx, ta), ctx->ls), "corrected weights"));
 }
 
+// The bias gradients of a network with a fused update: what the weight gradients' launch would have summed.
+static pm_status bias_grad(pm_ctx* ctx, const TickArgs& ta, int l) {
+  return TIMED(PM_PROF_ACT_BWD, check(ctx, launch_bias_grad(next(ctx, ta), l, ctx->ls), "bias gradients"));
+}
+
 // The launches of ONE stage's backward pass (ta restricted to it).  grouped: the weight gradients and the finishing passes
 // are left to grouped launches over all stages (ta.defer_finish set).
 static pm_status stage_backward(pm_ctx* ctx, const TickArgs& ta, int p, bool grouped) {
@@ -1099,8 +1104,8 @@ static pm_status mb_backward_body(pm_ctx* ctx) {
   TickArgs ta = mb_args(ctx, 2 * P, -1);
   const int n_fin = ln_finish_launches(ta);
   if (n_fin && (s = TIMED(PM_PROF_PRE_BWD, check(ctx, launch_ln_finish(ta, ctx->ls), "LayerNorm gradient sums", n_fin))) != PM_OK) return s;
-  if (S == 0 && !ctx->L.fuse && (s = grouped_wgrad(ctx, 2 * P)) != PM_OK) return s;   // fused update: formed in the update phase
-  return PM_OK;
+  if (ctx->L.fuse) return bias_grad(ctx, ta, 0);              // (one Linear per stage; the weight gradients are formed in the update phase)
+  return S == 0 ? grouped_wgrad(ctx, 2 * P) : PM_OK;
 }
 
 // The update kernel over all stages: everything, or what the weight-gradient GEMM's epilogue has left.
@@ -1259,7 +1264,8 @@ static pm_status tick_backward_body(pm_ctx* ctx) {
   for (int l = ctx->L.max_lin - 1; l >= 0; --l) {
     if (need_actbwd(ctx, l, -1) &&
         (s = TIMED(PM_PROF_ACT_BWD, check(ctx, launch_actbwd(next(ctx, ctx->ta), dt, l, ctx->ls), "activation backward"))) != PM_OK) return s;
-    if (!ctx->L.fuse && (s = branch(ctx, 1, [&]() {               // fused update: formed in the update phase
+    if ((s = branch(ctx, 1, [&]() {
+          if (ctx->L.fuse) return bias_grad(ctx, ctx->ta, l);       // fused update: the weight gradients are formed in the update phase
           prof_begin(ctx, PM_PROF_WGRAD);
           const cudaError_t e = dt == PM_F32 ? launch_simt_gemm(next(ctx, ctx->ta), ctx->L.st, 2, l, ctx->ls)
                                              : umma_launch(ctx->umma, next(ctx, ctx->ta), 2, l, ctx->ls);

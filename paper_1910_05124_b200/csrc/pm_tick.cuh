@@ -192,6 +192,8 @@ inline bool early(const TickArgs& t, dim3 grid) { return t.pdl != 0 && grid.x * 
 cudaError_t launch_loss(const TickArgs& t, int dtype, cudaStream_t stream);
 // dz = dy * act'(z), level `lvl` of every stage that runs backward this tick.
 cudaError_t launch_actbwd(const TickArgs& t, int dtype, int lvl, cudaStream_t stream);
+// db = column sums of dz, level `lvl` of every stage that runs backward (bf16 with a fused update; else the weight-gradient GEMM sums them)
+cudaError_t launch_bias_grad(const TickArgs& t, int lvl, cudaStream_t stream);
 // the finishing pass that launches with defer_finish left out, grouped over all stages (LayerNorm parameter gradients)
 cudaError_t launch_ln_finish(const TickArgs& t, cudaStream_t stream);      // pm_xfmr.cu
 int ln_finish_launches(const TickArgs& t);

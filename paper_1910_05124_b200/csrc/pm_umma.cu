@@ -41,10 +41,10 @@ constexpr int N_EPI_WARPS = 8;
 
 // MODE 0 forward, 2 wgrad, 1 dgrad against a QUEUED weight version (weight stashing, tau_bkwd = tau_fwd: a plain bf16 operand; the
 // corrected dgrad has kernels of its own).  MODE 2: four warps sum the columns of dz, the bias gradient, from the A tiles in shared
-// memory.  FUSE (MODE 2): the update is applied in the epilogue.
+// memory.  FUSE (MODE 2): the update is applied in the epilogue; the bias gradients belong to the backward phase (bias_grad_kernel).
 template <int MODE, bool FUSE> struct Cfg {
   static constexpr int kStages = 4;                        // operand ring depth
-  static constexpr int kSumWarps = MODE == 2 ? 4 : 0;
+  static constexpr int kSumWarps = MODE == 2 && !FUSE ? 4 : 0;
   static constexpr int kThreads = 32 * (2 + kSumWarps + N_EPI_WARPS);
   static constexpr int kOutWarpBytes = 8192;               // per epilogue warp: two boxes of 32 rows x 128 B
   static constexpr int kOutBytes = N_EPI_WARPS * kOutWarpBytes;
