@@ -114,8 +114,13 @@ __device__ __forceinline__ void actbwd_rows(const AT* __restrict__ dy, const AT*
   if (r < r1) actbwd_rows_n<AT, ACT, 1>(dy, z, dz, n_out, c, r, step);
 }
 
-// rows a block of the launch covers: all of a short microbatch; in a launch of one stage few enough for several blocks per SM
-__host__ __device__ inline int act_block_rows(const TickArgs& t) { return t.T <= kActSmallRows ? t.T : (t.sel_p >= 0 ? 64 : 256); }
+// rows a block of the launch covers: all of a short microbatch; in a launch of one stage few enough for several blocks per SM; more where
+// the grid's second dimension, at most 65535, would not reach the last row
+__host__ __device__ inline int act_block_rows(const TickArgs& t) {
+  int rows = t.T <= kActSmallRows ? t.T : (t.sel_p >= 0 ? 64 : 256);
+  while (((int64_t)t.T + rows - 1) / rows > 65535) rows *= 2;
+  return rows;
+}
 
 template <typename AT>
 __global__ void __launch_bounds__(256) actbwd_kernel(TickArgs t, int lvl) {
@@ -136,7 +141,7 @@ __global__ void __launch_bounds__(256) actbwd_kernel(TickArgs t, int lvl) {
   const int cols = small ? kActSmallCols : kActCols;
   const int c0 = (blk - start[p]) * cols;
   if (c0 >= L.n_out) return;
-  const int rows = act_block_rows(t), r0 = (int)blockIdx.y * rows, r1 = min(t.T, r0 + rows);
+  const int rows = act_block_rows(t), r0 = (int)blockIdx.y * rows, r1 = r0 + min(t.T - r0, rows);
   const uint64_t n = (uint64_t)t.T * L.n_out;
   const AT* dy = (lvl < s.n_lin - 1) ? ws_ptr<AT>(t, L.dy_off) : (feeds_attention(s.post) ? ws_ptr<AT>(t, s.dy) : gin_read<AT>(t, s, d));
   // the pre-activation stash, or for a ReLU without one the stashed output (same sign pattern)
