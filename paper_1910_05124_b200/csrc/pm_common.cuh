@@ -63,7 +63,6 @@ struct StageDev {
   int32_t n_lin;
   int32_t depth;              // slots of the stash rings = tau_f + 1
   int32_t xdepth;             // slots of the main-input ring = tau_f + 2 (it doubles as the forward mailbox)
-  int32_t max_dim;
   int32_t pre, post;
   int32_t n_heads, seq_len, vocab;
   int32_t d_in;               // width of the main input (= width of u, the first Linear's input)

@@ -48,7 +48,7 @@ struct Layout {
   int32_t any_pre = 0, any_ln = 0, any_embed = 0, any_residual = 0, att_S = 0, att_dk = 0, att_blocks = 0, max_vocab = 0;
   int32_t pe_seq = 0, pe_d = 0;
   int64_t loss_cap = 0;
-  int32_t max_lin = 0, max_dim = 0, n_in_first = 0, n_out_last = 0;
+  int32_t max_lin = 0, n_in_first = 0, n_out_last = 0;
   int32_t act_levels = 0;               // bit l: some stage's Linear l applies its activation's derivative in its own backward
   // microbatch-major order
   bool mb = false;
@@ -217,8 +217,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       idx = 1;
     }
     const int pre_width = idx == 1 ? sd.ops[0].n_out : -1;
-    s.max_dim = 0;
-    int max_out = 0, max_in = 0;
     while (idx < sd.n_ops && sd.ops[idx].kind == PM_OP_LINEAR) {
       if (s.n_lin == PM_MAX_LINEARS) { stage_err(p, "too many Linear ops"); return PM_ERR_INVALID_ARG; }
       const pm_op_desc& op = sd.ops[idx];
@@ -228,7 +226,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       ld.n_in = op.n_in; ld.n_out = op.n_out; ld.act = op.act;
       offsets(idx, &ld.w_off, &ld.b_off);
       if (s.n_lin > 0 && op.n_in != s.lin[s.n_lin - 1].n_out) { stage_err(p, "Linear n_in does not match the previous n_out"); return PM_ERR_SHAPE; }
-      max_out = std::max(max_out, op.n_out); max_in = std::max(max_in, op.n_in);
       ++s.n_lin; ++idx;
     }
     if (s.n_lin < 1) { stage_err(p, "a stage needs at least one LINEAR"); return PM_ERR_INVALID_ARG; }
@@ -268,7 +265,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       if (L.mem_stage < 0 || L.mem_dim != s.lin[0].n_in) { stage_err(p, "no memory of this width was emitted before this stage"); return PM_ERR_UNSUPPORTED; }
       L.last_mem_reader = p;
     }
-    s.max_dim = std::max(std::max(max_in, max_out), s.d_in);
     // ---- chaining
     if (p > 0) {
       const StageDev& q = L.st[p - 1];
@@ -350,7 +346,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
       }
     }
     L.max_lin = std::max(L.max_lin, s.n_lin);
-    L.max_dim = std::max(L.max_dim, s.max_dim);
     if (s.pre != PRE_NONE) L.any_pre = 1;
     if (s.pre == PRE_LN) L.any_ln = 1;
     if (s.pre == PRE_EMBED) { L.any_embed = 1; L.max_vocab = std::max(L.max_vocab, s.vocab); }
@@ -454,7 +449,6 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   // microbatch-major order, whose grids cover a single stage
   L.chunk_rows = T > 512 ? (mb ? 64 : 256) : 32;
   L.row_chunks = (int32_t)((T + L.chunk_rows - 1) / L.chunk_rows);
-  L.off_colred = w; w = align_up(w + (L.row_chunks > 1 ? (uint64_t)P * L.row_chunks * 2 * L.max_dim * 4 : 0), 256);
   L.off_pe = w; w = align_up(w + (uint64_t)L.pe_seq * L.pe_d * 4, 256);
   L.ids.assign((size_t)4 * P, 0);
   L.pre_idx.assign(P, -1); L.ln_idx.assign(P, -1); L.embed_idx.assign(P, -1); L.res_idx.assign(P, -1);
@@ -483,6 +477,7 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   if (L.mem_stage >= 0 && !L.ln_fused) { err = "stages that read the memory need LayerNorm widths that are multiples of 8 and at most 1024"; return PM_ERR_UNSUPPORTED; }
   L.ln_chunk_rows = mb ? 16 : 64;
   L.ln_chunks = (int32_t)((T + L.ln_chunk_rows - 1) / L.ln_chunk_rows);
+  L.off_colred = w; w = align_up(w + (!L.ln_fused && L.row_chunks > 1 ? (uint64_t)L.n_ln * L.row_chunks * 2 * L.max_ln_dim * 4 : 0), 256);
   L.off_lnred = w; w = align_up(w + (uint64_t)L.n_ln * L.ln_chunks * 2 * L.max_ln_dim * 4, 256);
   L.off_tgt = w; w = align_up(w + (uint64_t)(P + 1) * T * (ce ? 4 : (uint64_t)L.n_out_last * 4), 256);
   L.off_yout = w; w = align_up(w + 2 * T * L.n_out_last * (ce ? 4 : esz), 256);
@@ -736,7 +731,7 @@ pm_status pm_init_stages(pm_ctx** out, const pm_config* cfg, const pm_stage_desc
   t.a = c->a; t.ring = (char*)ring; t.ws = c->ws; t.T = cfg->microbatch; t.P = P;
   t.n_in_first = L.n_in_first; t.n_out_last = L.n_out_last;
   t.yout_off = L.off_yout; t.tgt_off = L.off_tgt; t.loss_off = L.off_loss; t.loss_cap = L.loss_cap; t.lossred_off = L.off_lossred;
-  t.max_lin = L.max_lin; t.max_dim = L.max_dim;
+  t.max_lin = L.max_lin;
   t.mb_major = L.queue ? 1 : 0; t.sel_p = -1; t.sel_tile0 = 0; t.pdl = 0;
   t.res_fused = cfg->compute_dtype == PM_BF16 ? 1 : 0;
   t.ln_li0 = 0; t.defer_finish = 0; t.ln_stage = 0;

@@ -25,7 +25,7 @@ struct TickArgs {
   uint64_t tgt_off;       // ws: target ring [P+1]: [T*n_out_last] float (MSE) or [T] int32 (CE)
   uint64_t pe_off;        // ws: sinusoidal positions [seq_len][d] float (0 if no embedding stage)
   uint64_t rowloss_off;   // ws: per-token losses [T] float (cross-entropy)
-  uint64_t colred_off;    // ws: per-row-chunk partial sums of unfused LayerNorm gradients [P][row_chunks][2*max_dim] float
+  uint64_t colred_off;    // ws: per-row-chunk partial sums of unfused LayerNorm gradients [n_ln][row_chunks][2*max_ln_dim] float
   int32_t row_chunks;     // ceil(T / chunk_rows)
   int32_t chunk_rows;     // rows of a microbatch one block of a column reduction covers (256, or 32 for short microbatches)
   int32_t loss_kind;      // PM_LOSS_*
@@ -53,7 +53,6 @@ struct TickArgs {
   int32_t mem_depth, gmem_depth, mem_dim, n_streams;
   int32_t second_embed_stage;   // the stage that embeds the second token stream (when n_streams == 2)
   int32_t max_lin;        // largest n_lin over stages
-  int32_t max_dim;        // largest n_in / n_out over stages
   // microbatch-major order: the forward pass reads its weights from the stages' version rings
   int32_t mb_major;
   // launches restricted to one stage (microbatch-major order runs the stages one after the other): kernels that take

@@ -833,7 +833,7 @@ constexpr int kLnCols = 256;                         // columns per block: 8 per
 template <typename AT>
 __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
   pdl_trigger();
-  const int p = t.ln_ids[blockIdx.z + t.ln_li0];
+  const int li = blockIdx.z + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
   if (d.b_mb < 0 || s.pre != PRE_LN) return;
@@ -892,26 +892,26 @@ __global__ void __launch_bounds__(256) ln_bwd_param_kernel(TickArgs t) {
       t.a.grad[s.g_off + cc] = d.accum ? __fadd_rn(t.a.grad[s.g_off + cc], a) : a;
       t.a.grad[s.beta_off + cc] = d.accum ? __fadd_rn(t.a.grad[s.beta_off + cc], b2) : b2;
     } else {
-      float* part = ws_at<float>(t, t.colred_off) + ((uint64_t)p * t.row_chunks + chunk) * (2 * (uint64_t)t.max_dim);
+      float* part = ws_at<float>(t, t.colred_off) + ((uint64_t)li * t.row_chunks + chunk) * (2 * (uint64_t)t.max_ln_dim);
       part[cc] = a;
-      part[t.max_dim + cc] = b2;
+      part[t.max_ln_dim + cc] = b2;
     }
   }
 }
 
 __global__ void __launch_bounds__(256) ln_param_finish_kernel(TickArgs t) {
   pdl_trigger();
-  const int p = t.ln_ids[blockIdx.y + t.ln_li0];
+  const int li = blockIdx.y + t.ln_li0, p = t.ln_ids[li];
   const StageDyn& d = t.dyn[p];
   const StageDev& s = t.st[p];
   if (d.b_mb < 0 || s.pre != PRE_LN) return;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= s.d_in) return;
-  const float* part = ws_at<float>(t, t.colred_off) + (uint64_t)p * t.row_chunks * (2 * (uint64_t)t.max_dim);
+  const float* part = ws_at<float>(t, t.colred_off) + (uint64_t)li * t.row_chunks * (2 * (uint64_t)t.max_ln_dim);
   float a = 0.f, b2 = 0.f;
   for (int k = 0; k < t.row_chunks; ++k) {
-    a = __fadd_rn(a, part[(uint64_t)k * 2 * t.max_dim + c]);
-    b2 = __fadd_rn(b2, part[(uint64_t)k * 2 * t.max_dim + t.max_dim + c]);
+    a = __fadd_rn(a, part[(uint64_t)k * 2 * t.max_ln_dim + c]);
+    b2 = __fadd_rn(b2, part[(uint64_t)k * 2 * t.max_ln_dim + t.max_ln_dim + c]);
   }
   t.a.grad[s.g_off + c] = d.accum ? __fadd_rn(t.a.grad[s.g_off + c], a) : a;
   t.a.grad[s.beta_off + c] = d.accum ? __fadd_rn(t.a.grad[s.beta_off + c], b2) : b2;
