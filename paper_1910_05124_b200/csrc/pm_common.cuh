@@ -98,7 +98,7 @@ struct StageDev {
   uint64_t stat_ring;         // ring: LayerNorm mean, rstd [depth][T*2] float
   uint64_t ids_ring;          // ring: token ids [depth][T] int32 (embedding stage)
   uint64_t skip_in;           // ws: incoming skip tensor [2][T*n_out] (residual stage), slot = tick parity of its writer
-  uint64_t ytmp;              // ws: Linear output awaiting the residual add [T*n_out]
+  uint64_t ytmp;              // ws, fp32 networks: Linear output awaiting the residual add [T*n_out]
   uint64_t gin;               // ws: incoming gradient w.r.t. the main output [3][T*d_out_main], slot = writer's tick % 3
   uint64_t dy;                // ws: gradient w.r.t. the Linear output when a post-op produces it [T*n_out] (attention)
   uint64_t dh;                // ws: gradient w.r.t. the pre-op's output u [T*d_in] (stages with a pre-op)

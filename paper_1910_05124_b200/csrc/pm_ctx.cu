@@ -497,7 +497,7 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
     s.gin = w; w = align_up(w + (uint64_t)s.gin_depth * T * s.d_out_main * esz, 256);
     if (s.post == POST_RESIDUAL) {
       s.skip_in = w; w = align_up(w + (uint64_t)s.skip_depth * T * n_out_last * esz, 256);
-      s.ytmp = w; w = align_up(w + T * n_out_last * esz, 256);
+      if (esz == 4) { s.ytmp = w; w = align_up(w + T * n_out_last * esz, 256); }   // (bf16: the forward GEMM adds the skip tensor itself)
     }
     if (s.post == POST_ATTENTION || s.post == POST_CROSS_ATTENTION) { s.dy = w; w = align_up(w + T * n_out_last * esz, 256); }
     // every Linear keeps its dz until the grouped weight-gradient launches at the end of a backward pass

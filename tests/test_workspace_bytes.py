@@ -29,3 +29,13 @@ def test_a_layer_costs_no_vocabulary(built_lib, order, compute, seq):
     wide, narrow = need[2, 8264] - need[1, 8264], need[2, 264] - need[1, 264]
     assert abs(wide - narrow) < 1 << 18, (wide, narrow)
 
+
+# A bf16 residual stage's GEMM adds the skip tensor itself: nothing waits for a launch that does.  What a layer keeps, in tensors of
+# T x d bf16: attention stage 3 (gradient of q, k, v) + 3 mailbox slots + 1 (gradient of the LayerNorm's output); projection 3 mailbox slots +
+# 2 of the skip tensor; hidden stage, 4 d wide, 4 x 3 mailbox slots + 4 (dz) + 1; output stage 3 + 2.  Tables and partial sums are less than one.
+def test_residual_stages_keep_no_sum_waiting(built_lib):
+    T, d, need = 4096, 64, {}
+    for layers in (1, 2):
+        wl = I.encoder_workload("ws", layers, d, 1, 4 * d, 128, 32, 264, compute="bf16", optimizer="adam", alpha=1e-3, K=4, D=0.1, steps=1, seed=1)
+        need[layers] = workspace(wl, "tick_major")
+    assert 34 <= (need[2] - need[1]) / (T * d * 2) < 35
