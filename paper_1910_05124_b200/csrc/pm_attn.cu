@@ -248,7 +248,6 @@ __global__ void __launch_bounds__(128, 4) attn_fwd_tc_kernel(TickArgs t, const C
 // dQ at 64..127, dK at 128..191.
 constexpr int AT_BWD_THREADS = 256;
 constexpr int AT_BWD_TILES = 5;
-constexpr int AT_XCH_BYTES = 3 * 2 * AT_S * 4;
 
 template <bool FULL>
 __global__ void __launch_bounds__(AT_BWD_THREADS, 2) attn_bwd_tc_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const int* __restrict__ stage_ids, int* status) {
