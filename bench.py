@@ -409,10 +409,18 @@ def gemm_flops(wl):
     return {"gemm_fwd": full, "wgrad": full, "dgrad": dgrad}
 
 
-def gemm_bytes(wl):
+def corrected_in_scratch(wl):
+    """Do this workload's dgrads read the corrected weights from a copy formed at the start of the backward phase?"""
+    dims = [d for st in ([wl.stage_specs] if wl.kind == "encoder" else wl.stages) for sp in st for d in (sp.n_in, sp.n_out)]
+    return wl.microbatch >= 256 and min(dims) >= 256
+
+
+def gemm_bytes(wl, plain_dgrad=False, fused=False):
     """Algorithmic HBM bytes of one tick per GEMM class on the bf16 path: every operand read once, every result
-    written once (bf16 activations, fp32 weights / discrepancy / gradient, fp32 logits under cross-entropy)."""
+    written once (bf16 activations, fp32 weights / discrepancy / gradient, fp32 logits under cross-entropy).
+    plain_dgrad: dgrad reads a queued bf16 copy; fused: the weight gradients' launch updates the matrices."""
     T = wl.microbatch
+    grad_b = 4.0 if not fused else (34.0 if wl.optimizer == "adam" else 26.0)
     if wl.kind == "encoder":
         lin = [(sp.n_in, sp.n_out, sp.act) for sp in wl.stage_specs]
         gaps = [f - b for f, b in zip(wl.tau_fwd, wl.tau_bkwd)]
@@ -427,25 +435,26 @@ def gemm_bytes(wl):
         # z stash and activation y; a ReLU that is not the very last Linear stashes only y
         out_b = 4 if (last and logits_f32) else 2 * (2 if (act == "gelu" or (act == "relu" and last)) else 1)
         fwd += 2.0 * T * a + 2.0 * a * b + out_b * T * b
-        wgrad += 2.0 * T * a + 2.0 * T * b + 4.0 * a * b
+        wgrad += 2.0 * T * a + 2.0 * T * b + grad_b * a * b
         if j > 0 or wl.kind == "encoder":
-            dgrad += 2.0 * T * b + (8.0 if (wl.t2 and gap > 0) else 4.0) * a * b + 2.0 * T * a
+            w_b = 8.0 if (wl.t2 and gap > 0) else 4.0                              # fp32 w and delta
+            w_b = 2.0 if plain_dgrad else w_b + (4.0 if corrected_in_scratch(wl) else 0.0)   # the bf16 copy written and read
+            dgrad += 2.0 * T * b + w_b * a * b + 2.0 * T * a
     return {"gemm_fwd": fwd, "wgrad": wgrad, "dgrad": dgrad}
 
 
 # DRAM traffic per launch from ncu captures summarised under profiles/ (bytes); scaled to the benchmark workload by
 # the stated unit counts because the full-size workloads hold more device memory than a multi-pass capture may.
 NCU_TRAFFIC = {
-    # GEMM kernels: measured DRAM bytes / algorithmic bytes on the 2-layer cut of cfg4
-    # (profiles/gemm_and_attention_kernels_cfg4_2layer_cut.md); every operand crosses HBM once, so traffic grows
-    # with the algorithmic bytes of the launch
-    "gemm_fwd_ratio": (84.2 + 149.1) / (83.9 + 209.7),
-    "wgrad_ratio": (211.1 + 24.9) / (205.5 + 42.0),
-    "dgrad_ratio": (231.8 + 29.2) / (226.5 + 33.6),
-    # dgrad launched one stage at a time on config 5's widths (profiles/narrow_dgrad_and_ln_backward_cfg5_1+1_layers.md):
-    # six launches read 776.4 MB and wrote 16.7 MB of DRAM against 826.2 MB of dz, fp32 w and delta, and dx (the
-    # dx of a launch is still in L2 when it ends)
-    "dgrad_one_stage_ratio": (776.4 + 16.7) / 826.2,
+    # GEMM kernels: measured DRAM bytes / algorithmic bytes (profiles/pair_gemms_and_corrected_weights.md); every operand crosses
+    # HBM once and part of what a launch writes is still in L2 when it ends, so traffic grows with the algorithmic bytes.
+    # Grouped launches, 2-layer cut of cfg4; dgrad: corrected weights and the GEMM that reads them
+    "gemm_fwd_ratio": (101.5 + 151.3) / (83.9 + 209.7),
+    "wgrad_ratio": (211.5 + 22.7) / (205.5 + 42.0),
+    "dgrad_ratio": (83.9 + 3.5 + 165.9 + 20.1) / (83.9 + 21.0 + 21.0 + 142.6 + 33.6),
+    # launches of one stage on config 5's widths (1 + 1 layers): the corrected weights of all stages and three dgrads, and the latter alone
+    "dgrad_one_stage_ratio": (571.8 + 392.5) / (621.5 + 436.8),
+    "plain_dgrad_one_stage_ratio": 392.5 / 436.8,
     # fused update: 2.941 GB at 100 M parameters, momentum SGD (profiles/update_kernel_100M_params.md); pure streaming,
     # so it is scaled by the algorithmic bytes of the launch (30 B/param there; 38 B/param with Adam's second moment)
     "update_bytes_per_param": 29.41,
@@ -470,7 +479,7 @@ def elementwise_bytes(wl):
             out["pre_bwd"] += T * d * e * (1 + (1 if emits else 0)) + 4.0 * wl.vocab * d   # du (+ skip gradient); whole fp32 table gradient
         if sp.post == "residual":
             out["post_fwd"] += 3.0 * T * sp.n_out * e                          # skip + y -> next input
-        out["act_bwd"] += T * sp.n_out * e * (3 if sp.act != "none" else 1)     # dy (column sums); with an activation also the mask source and dz
+        out["act_bwd"] += T * sp.n_out * e                                     # fused update: dz, for the bias gradients (else no launch)
     V = wl.stage_specs[-1].n_out
     out["loss"] = T * V * (4 + e)                                              # fp32 logits in, gradient out
     return out
@@ -608,7 +617,8 @@ def rooflines(res, peaks, steps):
     hbm_peak = peaks["hbm"]
     out = {}
     upd_ms = per_tick.get("update", 0.0)
-    alg_bytes = BYTES_PER_PARAM[wl.optimizer] * res["n_params"]
+    own = res["n_params"] - (sum(sp.n_in * sp.n_out for st in ([wl.stage_specs] if wl.kind == "encoder" else wl.stages) for sp in st) if res["fused"] else 0)
+    alg_bytes = BYTES_PER_PARAM[wl.optimizer] * own                     # fused update: the matrices are updated elsewhere
     upd_launches = max(res["prof"].get("update", (0, 1))[1] / steps, 1)
     upd_gbs = alg_bytes / (upd_ms * 1e-3) / 1e9 if upd_ms > 0 else 0.0
     out["update"] = {"kernel": "update_kernel (fused PipeMare update)", "bound": "hbm", "achieved": round(upd_gbs, 1),
@@ -633,19 +643,25 @@ def rooflines(res, peaks, steps):
             continue
         launches = res["prof"][cls][1] / steps
         kname = GEMM_KERNELS[cls]
-        if cls == "dgrad" and res.get("plain_dgrad"):
+        plain, fused, one_stage = bool(res.get("plain_dgrad")), bool(res["fused"]), res.get("order") == "mb_major" and wl.kind == "encoder"
+        bytes_ = gemm_bytes(wl, plain, fused)[cls]
+        if cls == "dgrad" and plain:
             kname = "umma_pair_gemm_kernel<1> / umma_gemm_kernel<1> (dgrad as a plain GEMM against a queued operand copy)"
         ratio, note = NCU_TRAFFIC[cls + "_ratio"], "DRAM bytes per launch, scaled from the ncu capture of the 2-layer cut of cfg4 by algorithmic bytes"
-        if cls == "dgrad" and res.get("order") == "mb_major" and not res.get("plain_dgrad") and wl.kind == "encoder":
-            kname = "corr_weights_kernel + umma_pair_gemm_kernel<1> (dgrad of one stage per launch and the corrected weights it reads)"
-            ratio, note = NCU_TRAFFIC["dgrad_one_stage_ratio"], "DRAM bytes per launch, scaled from the ncu capture of one-stage launches on config 5's widths (1 + 1 layers) by algorithmic bytes"
+        if cls == "dgrad" and one_stage:
+            if not plain:
+                kname = "corr_weights_kernel + umma_pair_gemm_kernel<1> (dgrad of one stage per launch and the corrected weights it reads)"
+            ratio = NCU_TRAFFIC["plain_dgrad_one_stage_ratio" if plain else "dgrad_one_stage_ratio"]
+            note = "DRAM bytes per launch, scaled from the ncu capture of one-stage launches on config 5's widths (1 + 1 layers) by algorithmic bytes"
+        elif (cls == "dgrad" and (plain or not corrected_in_scratch(wl))) or (cls == "wgrad" and fused):
+            ratio, note = None, "no capture of these launches"
         out[cls] = {"kernel": kname, "bound": "tensor", "achieved": round(tfs, 1), "peak": tf_peak, "unit": "TFLOP/s",
                     "frac": round(tfs / tf_peak, 4), "of": f"{peaks['kind']} ({tf_kind} bf16 matmul; the median SM clock of the timed region decides)",
                     "frac_of_burst": round(tfs / peaks["tf_burst"], 4), "frac_of_sustained": round(tfs / peaks["tf_sustained"], 4),
                     "frac_of_nominal_2250TFs": round(tfs / 2250.0, 4),
-                    "traffic": int(ratio * gemm_bytes(wl)[cls] / launches),
+                    "traffic": int(ratio * bytes_ / launches) if ratio else None,
                     "traffic_note": note,
-                    "algorithmic_bytes_per_step": gemm_bytes(wl)[cls], "algorithmic_flops_per_step": flops[cls],
+                    "algorithmic_bytes_per_step": bytes_, "algorithmic_flops_per_step": flops[cls],
                     "launches_per_step": launches, "avg_ms_per_step": round(per_tick[cls], 5), "share_of_step": share}
     dominant = max(out, key=lambda k: out[k].get("share_of_step") or 0.0)
     return out, dominant
@@ -795,7 +811,7 @@ def run_cuda(args):
             line["variants"] = [{
                 "option": "materialize_backward",
                 "what": "the update writes bf16(w - tau delta) into one more slot of the version queue and dgrad reads it as a plain "
-                        "operand; every result has the same bits as the headline run, which forms the corrected weights inside dgrad",
+                        "operand; every result has the same bits as the headline run, which forms the corrected weights in every backward pass",
                 "value": round(variant["units"] / (variant["t_ms"] * 1e-3), 2), "unit": UNIT,
                 "ms_per_step": round(variant["t_ms"] / steps, 5), "best_ms_per_step": round(min(variant["times"]) / steps, 5),
                 "ring_bytes": variant["ring_bytes"], "clocks": variant["clocks"], "rooflines": vrep["rooflines"],

@@ -445,8 +445,8 @@ pm_status build_layout(const pm_config* cfg, const pm_stage_desc* stages, Layout
   L.off_loss = w; w = align_up(w + sizeof(float) * (uint64_t)L.loss_cap, 256);
   L.off_lossred = w; w = align_up(w + 512, 256);
   L.off_rowloss = w; w = align_up(w + (ce ? T * 4 : 0), 256);
-  // short microbatches: more, smaller blocks (the reductions are latency-bound); so do the one-stage launches of
-  // microbatch-major order, whose grids cover a single stage
+  // rows per block of an unfused LayerNorm's parameter gradients: short microbatches take more, smaller blocks (the reductions are
+  // latency-bound), and so do the one-stage launches of microbatch-major order, whose grids cover a single stage
   L.chunk_rows = T > 512 ? (mb ? 64 : 256) : 32;
   L.row_chunks = (int32_t)((T + L.chunk_rows - 1) / L.chunk_rows);
   L.off_pe = w; w = align_up(w + (uint64_t)L.pe_seq * L.pe_d * 4, 256);

@@ -39,8 +39,8 @@ constexpr int STG_BYTES = 2 * STG_HALF_BYTES;              // w tile + delta til
 constexpr int ACC_COLS = 128, TMEM_COLS = 2 * ACC_COLS;
 constexpr int N_EPI_WARPS = 8;
 
-// MODE 0 forward, 2 wgrad, 1 dgrad against a QUEUED weight version (weight stashing, tau_bkwd = tau_fwd: a plain bf16 operand; the
-// corrected dgrad has kernels of its own).  MODE 2: four warps sum the columns of dz, the bias gradient, from the A tiles in shared
+// MODE 0 forward, 2 wgrad, 1 dgrad against a plain bf16 operand: a queued weight version (weight stashing, corrected weights that the update
+// wrote out) or, on CTA pairs, the corrected weights in scratch.  Elsewhere umma_dgrad_kernel forms the corrected operand.  MODE 2: four warps sum the columns of dz, the bias gradient, from the A tiles in shared
 // memory.  FUSE (MODE 2): the update is applied in the epilogue; the bias gradients belong to the backward phase (bias_grad_kernel).
 template <int MODE, bool FUSE> struct Cfg {
   static constexpr int kStages = 4;                        // operand ring depth
@@ -837,9 +837,9 @@ umma_pair_gemm_kernel(TickArgs t, const CUtensorMap* __restrict__ maps, const in
 }
 
 // ---- dgrad with reuse of the corrected operand -----------------------------------------------------------
-// D[T,in] = dz[T,out] * Wc[out,in].  With thousands of rows the fp32 w and delta tiles (64 KB per k-block) and
-// their conversion would be repeated for every 128-row tile; here one CTA computes up to four 128-row tiles
-// against the SAME converted tile: per k-block the staging ring receives w and delta once, the transform warps
+// D[T,in] = dz[T,out] * Wc[out,in], launches of fewer than 256 rows or columns (the others: corr_weights_kernel below).  The fp32 w and
+// delta tiles (64 KB per k-block) and their conversion would be repeated for every 128-row tile; here one CTA computes up to
+// four 128-row tiles against the SAME converted tile: per k-block the staging ring receives w and delta once, the transform warps
 // write bf16(w - gap*delta) once, and the MMA warp issues one product per row tile into its own accumulator
 // (4 x 128 TMEM columns).  Traffic per 128x128x64 product drops from 80 KB to 32 KB.
 constexpr int DG_MG = 4;                                   // row tiles per B tile

@@ -736,7 +736,8 @@ cudaError_t launch_ce_loss(const TickArgs& t, int dtype, cudaStream_t stream) {
 }
 
 // ---- pre-op backward --------------------------------------------------------------------------------------------
-// These launches are plain: none starts before its predecessor, the stage's dgrad, has ended (their successors may start early).
+// These launches are plain (their successors may start early), but for LayerNorm launches of one stage of which an SM holds two blocks
+// and no more (launch_ln_fused): none else starts before its predecessor, the stage's dgrad, has ended.
 // Blocks that become resident during a predecessor's tail crowd on the SMs that are free first and stay there; with the rows
 // of a LayerNorm backward that costs more than the launch: an update of a 2-layer encoder of width 1280 (2048 rows) takes
 // 1189 us with early launches here and 1140 without, of 4 layers of width 512 (1024 rows) 907 and 897, of the encoder of
